@@ -109,6 +109,9 @@ typedef struct cadnn_net cadnn_net;
  *           from several streams.
  * Filters are regrouped so that the warps of a thread block get equal nonzero
  * counts; the permutation is undone when results are stored.
+ * Where the kept fraction makes the tensor cores the faster route (CADNN_FMT_AUTO, groups 1, conv or fc
+ * packed for a batch above 8), the handle also gets a dense image of the layer for them and NHWC calls
+ * take it; CADNN_NO_TCV in the environment leaves it out.
  * Errors: E_ARG (NULL, bad desc), E_DTYPE, E_UNSUPPORTED (grouped conv other than
  * depthwise; int8 depthwise; reduction length whose int32 sum could overflow),
  * E_ALLOC, E_CUDA.  Synchronizes the device copy before returning.
@@ -292,7 +295,8 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
  * pair (re-captured when either pointer changes); 0 launches the layers one by one.
  * Float networks made of a dense stem, sparse convs, dense depthwise convs of up to 9 taps,
  * max pools, a global average pool and fc layers keep their intermediate feature maps
- * channel-planar with a zero halo (see cadnn_conv2d_planar); others (int8) keep NHWC
+ * channel-planar with a zero halo (see cadnn_conv2d_planar), unless every sparse conv carries the
+ * dense tensor-core image and none was timed at pack time; others (int8) keep NHWC
  * (CADNN_NO_PLANAR_DW: networks with depthwise layers too).  CADNN_NO_PLANAR in the
  * environment at cadnn_net_create forces NHWC.
  * Layers after the first are launched as programmatic dependents of their predecessor

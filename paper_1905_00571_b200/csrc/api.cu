@@ -108,6 +108,7 @@ cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, in
         le.acc_in = (const int *)workspace;
         le.pdl = false;
     }
+    if (w->d_tcv && tcv_fits(w, n)) return launch_tcv(w, x, n, y, le, s);
     switch (w->s.kind) {
         case KK_SCONV_SPATIAL:
         case KK_SCONV_LINEAR: return launch_sconv(w, x, n, y, le, s);

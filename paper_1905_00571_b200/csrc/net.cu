@@ -536,6 +536,17 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
                 if (op.src == 0 || flat[op.src]) planar = false;
             }
         }
+        // Layers packed with the dense tensor-core image run NHWC (tcconv.cu).  Networks with depthwise layers, and those
+        // whose schedules were timed at pack time, are left to the planar kernels.
+        if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr && !(getenv("CADNN_PERSIST") && atoi(getenv("CADNN_PERSIST")) != 0)) {
+            bool tc = true;
+            for (int i = 0; i < n_ops && tc; ++i) {
+                const cadnn_weights *w = ops[i].kind == CADNN_OP_CONV ? ops[i].w : nullptr;
+                if (!w || w->s.kind == KK_DENSE_SMALLC) continue;
+                tc = w->d_tcv && w->nhwc_us <= 0.0f;
+            }
+            if (tc) planar = false;
+        }
         // Where the packer timed both layouts for every sparse conv, the measured sums decide.
         if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr) {
             double t_planar = 0.0, t_nhwc = 0.0;
@@ -661,7 +672,10 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
     net->status_host[1] = net->status_seen[1];
     // inside graphs, programmatic launches pay off for the planar kernels only (the NHWC sparse conv
     // measured slower with them: 556 -> 608 us on ResNet-50, 367 -> 410 us on the int8 VGG-16)
-    if (!net->planar && getenv("CADNN_PDL_GRAPH") == nullptr) net->pdl_graph = false;
+    // and for the tensor-core route
+    bool tc = false;
+    for (const cadnn_op &op : net->ops) tc = tc || (op.w && op.w->d_tcv);
+    if (!net->planar && !tc && getenv("CADNN_PDL_GRAPH") == nullptr) net->pdl_graph = false;
     {
         // The persistent kernel trades the launch ramp and drain of every layer boundary for a device-wide
         // barrier and a copy start-up per layer.  Measured on a B200 (pruned ResNet-50, batch 1) a phase costs

@@ -1416,6 +1416,18 @@ cadnn_status pack_common(const cadnn_layer_desc *desc, const Src &src, cadnn_wei
         else st = pack_sconv(h, src);
         if (st == CADNN_OK) st = upload(h);
         if (st == CADNN_OK) st = block_tc_upload(h);
+        if (st == CADNN_OK && (h->s.kind == KK_SCONV_SPATIAL || h->s.kind == KK_SCONV_LINEAR) && d.fmt == CADNN_FMT_AUTO &&
+            !getenv("CADNN_NO_TCV") && !getenv("CADNN_SCHEDULE") && tcv_pays(d, h->nnz)) {
+            const int8_t *qp = src.q;
+            if (src.s8 && !qp) {
+                const size_t per = (size_t)K, numel = per * d.c_out;
+                q_codes.resize(numel);
+                for (size_t i = 0; i < numel; ++i) q_codes[i] = src.qval(i, (int)(i / per));
+                qp = q_codes.data();
+            }
+            tcv_build(h, src.f, qp, src.mask);
+            st = tcv_upload(h);
+        }
         if (st == CADNN_OK && h->has_planar && h->on_device && (d.flags & CADNN_PACK_AUTOTUNE) && !h->tuned)
             autotune_planar(h, h->row_nnz);
         if (st == CADNN_OK && h->tune_key && !h->tuned && h->on_device) {   // remember what was measured
@@ -1669,6 +1681,7 @@ void cadnn_weights_free(cadnn_weights *w)
     if (w->half) cadnn_weights_free(w->half);
     if (w->d_blob) cudaFree(w->d_blob);
     if (w->d_tc_blob) cudaFree(w->d_tc_blob);
+    if (w->d_tcv) cudaFree(w->d_tcv);
     delete w;
 }
 

@@ -34,6 +34,21 @@
 // whatever it has, and cadnn_device_status reports it)
 __device__ int g_copy_timeout;
 
+cadnn_status copy_timeout_word(int **word)
+{
+    static void *at[kMaxDevices];   // looked up once per device; a race stores the same value twice
+    int dev = 0;
+    CADNN_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= kMaxDevices) return CADNN_E_UNSUPPORTED;
+    if (!at[dev]) {
+        void *a = nullptr;
+        CADNN_CUDA_TRY(cudaGetSymbolAddress(&a, g_copy_timeout));
+        at[dev] = a;
+    }
+    *word = (int *)at[dev];
+    return CADNN_OK;
+}
+
 cadnn_status read_copy_timeouts(int *count)
 {
     int v = 0;

@@ -1,0 +1,920 @@
+// Dense tensor-core route of the sparse convolutions and large-batch FC layers (implicit GEMM on
+// NHWC activations, float and int8).
+//
+// CADNN (arXiv 1905.00571), Section 1 ("computation pattern transformation"): a compressed layer is
+// executed in the form the processor runs fastest.  A stored nonzero costs the sparse kernels one
+// 32-bit shared-memory word per multiply-add, which bounds them at a quarter of the FMA rate; the tensor
+// cores multiply the same layer with its pruned positions as zeros at a rate so much higher that they win
+// from a few per cent of kept weights on (tcv_pays below has the rule).  Batch 32, 12.5 % kept, microseconds
+// before / now: 64->64 3x3 56x56 118 / 60, 256->64 1x1 56x56 86 / 45, 256->256 3x3 14x14 122 / 48; int8 at 8 %,
+// batch 8, 256->256 3x3 56x56 240 / 37.
+//
+// GEMM view: rows = output pixels (image, row, column flattened), columns = output channels, K = (kernel
+// row, kernel column, input channel).  One block = a tile of pixels x channels (several shapes, see Cfg and
+// choose); the K range can be split over a thread-block cluster whose partial sums meet in distributed
+// shared memory (small maps would otherwise leave most multiprocessors idle).
+//   * 8 loader warps gather the im2col rows from NHWC memory (out-of-image taps are zeros) into swizzled
+//     K-major operand tiles, 128 source bytes per pixel and stage, in groups that fill alternate stages;
+//   * one thread copies the matching weight tiles (pre-swizzled by the packer) with bulk copies; the first
+//     ones do not wait for the previous layer;
+//   * one thread issues the tcgen05.mma's; accumulators live in tensor memory;
+//   * the loader warps then finish the tile: a lane per pixel straight from tensor memory, or through
+//     shared memory as [pixel][channel]; with a split reduction every block sends each other block its
+//     pixels' sums with one bulk copy that counts on the receiver's barrier.
+// What bounds it: at batch 1 the chain start - first loads - last multiply-adds - exchange (about 5 of the 6
+// to 9 microseconds of a layer); at large batch, for float, shared-memory bandwidth - the six products of a
+// stage read 40 KB of operands per 16 K values where the tensor core needs 384 clocks.
+//
+// Float precision.  A float is the exact sum of three bf16 numbers (8 + 8 + 8 significand bits), a = a1 + a2 +
+// a3 with |a2| <= 2^-9 |a|, |a3| <= 2^-18 |a|.  Loaders split activations, the packer splits weights, and the
+// products a1 b1, a1 b2, a2 b1, a2 b2, a1 b3, a3 b1 are accumulated in fp32; what is left out is below 2^-25 of
+// |a b|, less than the rounding of one fp32 multiply-add.  a1 b1 has an accumulator of its own: the small terms
+// are summed apart and added once at the end, so they are not rounded away against the large sum.
+// Int8 products accumulate in int32, exact in any order.
+#include <algorithm>
+#include <cstdlib>
+#include <cstring>
+#include <cstdio>
+#include <cuda_bf16.h>
+#include "cadnn_internal.h"
+
+namespace {
+
+const int kLoadWarps = 8;
+const int kThreads = (kLoadWarps + 2) * 32;   // + the weight-copy warp and the multiply-add warp
+const int kSpin = 1 << 22;
+
+struct TcvParams {
+    const void *x;
+    void *y;
+    const unsigned char *wimg;
+    const float *scale, *bias;
+    const void *residual;
+    float res_scale;
+    int act, out_dtype;
+    int h, w, c_in, h_out, w_out, c_out;
+    int stride, pad, pad_w, kh, kw;
+    int M, nkb, n_nt, S, npx;
+    int stages, recv_off, bar_off;   // pipeline depth; byte offsets of the partial sums and of the barriers in shared memory
+    int ldc, c_off, vec_ok, vec_sb, vec16;  // vec_ok / vec_sb: output and residual / scale and bias allow 4 channels per access; vec16: int8 output 16
+    int kb_base, kb_rem;             // stages per block of a cluster: kb_base, and one more in the first kb_rem blocks
+    int Rp;                          // K positions per kernel row: kw * c_in rounded up to 16 bytes
+    FastDiv d_hw, d_wo, d_ci, d_Rp, d_S, d_nt;
+    int *gave_up;
+};
+
+__device__ __forceinline__ void mb_init(unsigned bar, unsigned count)
+{
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
+}
+__device__ __forceinline__ void mb_expect_tx(unsigned bar, unsigned bytes)
+{
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void mb_arrive(unsigned bar)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+// bounded wait; false = gave up (recorded)
+__device__ __forceinline__ bool mb_wait(unsigned bar, unsigned parity, int *gave_up)
+{
+    for (int it = 0; it < kSpin; ++it) {
+        unsigned ok;
+        asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return true;
+    }
+    atomicAdd(gave_up, 1);
+    return false;
+}
+__device__ __forceinline__ void bulk_copy(unsigned dst, const void *src, unsigned bytes, unsigned bar)
+{
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+// K-major operand tile, 64-byte rows, 64-byte swizzle (16-byte chunk index ^= (row / 2) % 4)
+__device__ __forceinline__ unsigned long long smem_desc(unsigned addr)
+{
+    return (unsigned long long)((addr >> 4) & 0x3fffu) | (1ull << 16) | ((unsigned long long)(512u >> 4) << 32) | (1ull << 46) | (4ull << 61);
+}
+template <bool F32> __device__ __forceinline__ void mma(unsigned d, unsigned long long a, unsigned long long b, unsigned idesc, unsigned acc)
+{
+    if (F32)
+        asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+                     ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+    else
+        asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}\n"
+                     ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+}
+__device__ __forceinline__ void tc_commit(unsigned bar)
+{
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+// 16 accumulator columns of this warp's 32 rows (thread = row)
+__device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned (&v)[16])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                   "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                 : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
+{
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const unsigned *>(&v);
+}
+// two floats -> three packed bf16 pairs whose sum is the pair exactly
+__device__ __forceinline__ void split2(float a, float b, unsigned &h, unsigned &m, unsigned &l)
+{
+    h = pack_bf16(a, b);
+    a -= __uint_as_float(h << 16);
+    b -= __uint_as_float(h & 0xffff0000u);
+    m = pack_bf16(a, b);
+    a -= __uint_as_float(m << 16);
+    b -= __uint_as_float(m & 0xffff0000u);
+    l = pack_bf16(a, b);
+}
+__device__ __forceinline__ void sts64(unsigned addr, unsigned a, unsigned b)
+{
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};\n" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ void sts128(unsigned addr, const uint4 &v)
+{
+    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};\n" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ uint4 ld_vec(const void *p)
+{
+    uint4 v;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint4 lds128(unsigned addr)
+{
+    uint4 v;
+    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+// copies `bytes` of this block's shared memory to address dst of block `owner` of the cluster; counts on that block's barrier
+__device__ __forceinline__ void push_copy(unsigned dst, unsigned src, unsigned bytes, unsigned bar, int owner)
+{
+    asm volatile("{\n.reg .b32 a, b;\nmapa.shared::cluster.u32 a, %0, %4;\nmapa.shared::cluster.u32 b, %3, %4;\n"
+                 "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [a], [%1], %2, [b];\n}\n"
+                 ::"r"(dst), "r"(src), "r"(bytes), "r"(bar), "r"(owner) : "memory");
+}
+
+// One kernel shape: PX pixels x CH channels per block.  SWAP: the channels are the 128 rows of the tensor-core tile and
+// the pixels its columns (any multiple of 16 up to PX, so that small maps waste little); otherwise the 128 rows are pixels
+// and the columns CH channels.
+template <bool F32, int PX, int CH, bool SWAP, int GROUPS> struct Cfg {
+    static const int kParts = F32 ? 3 : 2;                 // operand tiles of 64-byte rows per stage
+    static const int kKB = F32 ? 32 : 128;                 // K values per stage (128 source bytes per pixel)
+    static const int kXBytes = kParts * PX * 64;
+    static const int kWBytes = kParts * CH * 64;
+    static const int kStage = kXBytes + kWBytes;
+    static const int kBlocks = PX > 128 || GROUPS > 2 ? 1 : 2;           // per multiprocessor
+    static const int kN = SWAP ? PX : CH;
+    // Accumulators, kN columns each (kN at most 64: three, by size of the terms; beyond: the large products and the small
+    // ones; int8: two that take turns, so that no multiply-add waits for the one before it)
+    static const int kAcc = F32 && kN <= 64 ? 3 : 2;
+    static const int kCols = kAcc * kN <= 128 ? 128 : kAcc * kN <= 256 ? 256 : 512;
+    static const int kRow = CH + 4;                        // words per pixel of the exchanged sums (conflict-free 16-byte access)
+    // Loader warps work in groups that fill alternate stages, so that one's memory and fence latency hides behind the
+    // others'; a thread then holds kRPT 16-byte pieces of its next stage in registers.
+    // (at most as many groups as stages: a group waits for a stage by phase parity, which tells neighbouring phases apart only)
+    static const int kGroups = GROUPS;
+    static const int kGroupThreads = 256 / kGroups;
+    static const int kRPT = PX * 8 / kGroupThreads;        // pixels per loader thread, kGroupThreads / 8 apart
+};
+
+// What a loader thread knows about a pixel: where its window starts.
+struct Px {
+    int off;   // element offset of (iy, ix, channel 0) from the tensor's start; negative where the window begins in the padding
+    int yx;    // iy << 16 | ix (16 bits each); iy far outside for rows past the last pixel
+};
+const int kNoPixel = -30000;
+__device__ __forceinline__ Px load_px(unsigned addr)
+{
+    Px r;
+    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];\n" : "=r"(r.off), "=r"(r.yx) : "r"(addr));
+    return r;
+}
+
+// 16 source bytes of one im2col row: 4 floats or 16 int8 values from K position (ky, kx, ci)
+template <bool F32>
+__device__ __forceinline__ uint4 gather_vec(const TcvParams &p, const Px &r, int ky, int kx, int ci)
+{
+    const int iy = (r.yx >> 16) + ky, ix = (int)(short)r.yx + kx;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if ((unsigned)iy < (unsigned)p.h && (unsigned)ix < (unsigned)p.w && ky < p.kh) {
+        const int o = r.off + (ky * p.w + kx) * p.c_in + ci;
+        v = ld_vec(reinterpret_cast<const char *>(p.x) + (size_t)o * (F32 ? 4 : 1));
+    }
+    return v;
+}
+// The same when a pixel's channels are not a multiple of 16 bytes: positions r .. of row ky of the window, whose kw * c_in values
+// lie behind each other in memory.  Values of the columns outside the image read as zero; positions past the row's end meet
+// zero weights.  Floats come one by one; int8 values as the aligned words that hold any wanted one, shifted into place.
+template <bool F32>
+__device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, int ky, int r)
+{
+    const int iy = (px.yx >> 16) + ky, ix = (int)(short)px.yx;
+    const int a = max(0, -ix * p.c_in - r);
+    int b = min(p.kw, p.w - ix) * p.c_in - r;
+    if ((unsigned)iy >= (unsigned)p.h || ky >= p.kh) b = 0;
+    const int o = px.off + ky * p.w * p.c_in + r;
+    if (F32) {
+        unsigned v[4];
+        const float *x = reinterpret_cast<const float *>(p.x);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[j] = 0;
+            if (j >= a && j < b) v[j] = __float_as_uint(ld_act(x + o + j));
+        }
+        return make_uint4(v[0], v[1], v[2], v[3]);
+    }
+    const int s = o & 3;
+    const char *x = reinterpret_cast<const char *>(p.x) + (o - s);
+    unsigned w[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        w[i] = 0;
+        if (max(a, 4 * i - s) < min(min(b, 16), 4 * i - s + 4)) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(w[i]) : "l"(x + 4 * i));
+    }
+    unsigned v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int lo = min(max(a - 4 * i, 0), 4), hi = min(max(b - 4 * i, 0), 4);
+        const unsigned below = lo >= 4 ? 0xffffffffu : (1u << (8 * lo)) - 1, upto = hi >= 4 ? 0xffffffffu : (1u << (8 * hi)) - 1;
+        v[i] = __funnelshift_r(w[i], w[i + 1], 8 * s) & upto & ~below;
+    }
+    return make_uint4(v[0], v[1], v[2], v[3]);
+}
+
+// one int8-layer output value
+__device__ __forceinline__ int finish_q(const TcvParams &p, int sum, float sc, float bi, int r)
+{
+    return requant_s8(sum, sc, bi, p.act, p.residual != nullptr, r, p.res_scale);
+}
+__device__ __forceinline__ float finish_f(const TcvParams &p, unsigned sum, float sc, float bi, float r)
+{
+    return act_f32(__fmaf_rn(__uint_as_float(sum), sc, bi) + r, p.act);
+}
+__device__ __forceinline__ int byte_of(unsigned w, int j) { return (int)(signed char)((w >> (8 * j)) & 0xff); }
+
+// four of them, packed
+__device__ __forceinline__ unsigned finish_q4(const TcvParams &p, const uint4 &t, unsigned r, const float4 &sc, const float4 &bi)
+{
+    const unsigned q0 = finish_q(p, (int)t.x, sc.x, bi.x, byte_of(r, 0)) & 0xff, q1 = finish_q(p, (int)t.y, sc.y, bi.y, byte_of(r, 1)) & 0xff;
+    const unsigned q2 = finish_q(p, (int)t.z, sc.z, bi.z, byte_of(r, 2)) & 0xff, q3 = finish_q(p, (int)t.w, sc.w, bi.w, byte_of(r, 3)) & 0xff;
+    return q0 | q1 << 8 | q2 << 16 | q3 << 24;
+}
+
+// Epilogue of 4 consecutive channels of one pixel: sums t, residual r (4 floats, or 4 int8 values in its first word), written
+// to channel offset oi of the output; `left` channels exist.
+template <bool F32>
+__device__ __forceinline__ void finish4(const TcvParams &p, size_t oi, int left, const uint4 &t, const uint4 &r, const float4 &sc, const float4 &bi)
+{
+    if (F32) {
+        float *dst = reinterpret_cast<float *>(p.y) + oi;
+        const float4 o = make_float4(finish_f(p, t.x, sc.x, bi.x, __uint_as_float(r.x)), finish_f(p, t.y, sc.y, bi.y, __uint_as_float(r.y)),
+                                     finish_f(p, t.z, sc.z, bi.z, __uint_as_float(r.z)), finish_f(p, t.w, sc.w, bi.w, __uint_as_float(r.w)));
+        if (p.vec_ok) *reinterpret_cast<float4 *>(dst) = o;
+        else {
+            dst[0] = o.x;
+            if (left > 1) dst[1] = o.y;
+            if (left > 2) dst[2] = o.z;
+            if (left > 3) dst[3] = o.w;
+        }
+    } else if (p.out_dtype == CADNN_S8) {
+        const unsigned w4 = finish_q4(p, t, r.x, sc, bi);
+        signed char *dst = reinterpret_cast<signed char *>(p.y) + oi;
+        if (p.vec_ok) *reinterpret_cast<unsigned *>(dst) = w4;
+        else
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                if (j < left) dst[j] = (signed char)(w4 >> (8 * j));
+    } else {   // int8 layer, 32-bit result: the raw sum, or the requantized value before rounding
+        uint4 v = t;
+        if (p.out_dtype == CADNN_F32) {
+            v.x = __float_as_uint(requant_f32((int)t.x, sc.x, bi.x, p.act, p.residual != nullptr, byte_of(r.x, 0), p.res_scale));
+            v.y = __float_as_uint(requant_f32((int)t.y, sc.y, bi.y, p.act, p.residual != nullptr, byte_of(r.x, 1), p.res_scale));
+            v.z = __float_as_uint(requant_f32((int)t.z, sc.z, bi.z, p.act, p.residual != nullptr, byte_of(r.x, 2), p.res_scale));
+            v.w = __float_as_uint(requant_f32((int)t.w, sc.w, bi.w, p.act, p.residual != nullptr, byte_of(r.x, 3), p.res_scale));
+        }
+        unsigned *dst = reinterpret_cast<unsigned *>(p.y) + oi;
+        if (p.vec_ok) *reinterpret_cast<uint4 *>(dst) = v;
+        else {
+            dst[0] = v.x;
+            if (left > 1) dst[1] = v.y;
+            if (left > 2) dst[2] = v.z;
+            if (left > 3) dst[3] = v.w;
+        }
+    }
+}
+// the residual of those 4 channels: 4 floats, or 4 int8 values in the first word
+template <bool F32> __device__ __forceinline__ uint4 load_residual(const TcvParams &p, int m, int co)
+{
+    const size_t ri = (size_t)m * p.c_out + co;
+    uint4 v = make_uint4(0, 0, 0, 0);
+    if (F32) {
+        const float *res = reinterpret_cast<const float *>(p.residual) + ri;
+        if (p.vec_ok) return ld_vec(res);
+        const int left = p.c_out - co;
+        v.x = __float_as_uint(ld_act(res));
+        if (left > 1) v.y = __float_as_uint(ld_act(res + 1));
+        if (left > 2) v.z = __float_as_uint(ld_act(res + 2));
+        if (left > 3) v.w = __float_as_uint(ld_act(res + 3));
+    } else {
+        const signed char *res = reinterpret_cast<const signed char *>(p.residual) + ri;
+        if (p.vec_ok) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(v.x) : "l"(res));
+        else
+            for (int j = 0; j < 4; ++j)
+                if (co + j < p.c_out) v.x |= (unsigned)(unsigned char)ld_act(res + j) << (8 * j);
+    }
+    return v;
+}
+
+// scale and bias of 4 consecutive channels
+__device__ __forceinline__ void load_channels(const TcvParams &p, int co, float4 &sc, float4 &bi)
+{
+    if (co + 3 < p.c_out) {
+        if (p.vec_sb) {
+            if (p.scale) sc = __ldg(reinterpret_cast<const float4 *>(p.scale + co));
+            if (p.bias) bi = __ldg(reinterpret_cast<const float4 *>(p.bias + co));
+        } else {
+            if (p.scale) sc = make_float4(__ldg(p.scale + co), __ldg(p.scale + co + 1), __ldg(p.scale + co + 2), __ldg(p.scale + co + 3));
+            if (p.bias) bi = make_float4(__ldg(p.bias + co), __ldg(p.bias + co + 1), __ldg(p.bias + co + 2), __ldg(p.bias + co + 3));
+        }
+        return;
+    }
+    const int a = min(co + 1, p.c_out - 1), b = min(co + 2, p.c_out - 1);
+    if (p.scale) sc = make_float4(__ldg(p.scale + co), __ldg(p.scale + a), __ldg(p.scale + b), 1.0f);
+    if (p.bias) bi = make_float4(__ldg(p.bias + co), __ldg(p.bias + a), __ldg(p.bias + b), 0.0f);
+}
+
+template <bool F32, int PX, int CH, bool SWAP, int GROUPS, bool VEC>
+__global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP, GROUPS>::kBlocks) tcconv_kernel(const TcvParams p)
+{
+    typedef Cfg<F32, PX, CH, SWAP, GROUPS> C;
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    const unsigned raw32 = (unsigned)__cvta_generic_to_shared(smem_raw);
+    const unsigned base = (raw32 + 1023u) & ~1023u;
+    const int S = p.stages;
+    const unsigned bars = base + p.bar_off;             // full[S], empty[S], done, partial sums received, tensor-memory address
+    const unsigned done = bars + 2 * S * 8, recv = done + 8, slot32 = recv + 8;
+    volatile unsigned *slot = reinterpret_cast<volatile unsigned *>(smem_raw + (slot32 - raw32));
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    // (divisions here are multiplications by host-made constants: this is on the critical path of every small layer)
+    const int tile = (int)fdiv(blockIdx.x, p.d_S), rank = (int)blockIdx.x - tile * p.S;
+    const int mt = (int)fdiv((unsigned)tile, p.d_nt), nt = tile - mt * p.n_nt;
+    const int kb0 = rank * p.kb_base + min(rank, p.kb_rem), kb1 = kb0 + p.kb_base + (rank < p.kb_rem ? 1 : 0);
+    const int npx = SWAP ? p.npx : PX;                  // pixels of a tile
+    const int m0 = mt * npx;
+    const unsigned xpart = npx * 64;                    // bytes from one activation part of a stage to the next
+
+    const unsigned pxs = slot32 + 16;                   // window starts of the tile's pixels, 8 bytes each
+
+    // weights of stage kb: its CH x 64-byte tiles, 64 channels (4 KB) per bulk copy
+    const int n64 = (p.c_out + 63) / 64;
+    auto copy_weights = [&](int kb, int s) {
+        const unsigned dst = base + s * C::kStage + C::kXBytes, full = bars + s * 8;
+        int cnt = 0;
+#pragma unroll
+        for (int q = 0; q < CH / 64; ++q) cnt += nt * (CH / 64) + q < n64;
+        mb_expect_tx(full, (unsigned)(cnt * C::kParts * 4096));
+#pragma unroll
+        for (int q = 0; q < CH / 64; ++q) {
+            const int nb = nt * (CH / 64) + q;
+            if (nb >= n64) break;
+            const unsigned char *src = p.wimg + ((size_t)nb * p.nkb + kb) * (C::kParts * 4096);
+#pragma unroll
+            for (int t = 0; t < C::kParts; ++t) bulk_copy(dst + t * (CH * 64) + q * 4096, src + t * 4096, 4096u, full);
+        }
+    };
+
+    if (warp == kLoadWarps) {
+        if (lane == 0) {
+            for (int i = 0; i < S; ++i) {
+                mb_init(bars + i * 8, kLoadWarps / C::kGroups + 1);
+                mb_init(bars + (S + i) * 8, 1);
+            }
+            mb_init(done, 1);
+            mb_init(recv, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            // partial sums of this block's pixels from every block of the cluster, itself included
+            if (p.S > 1) mb_expect_tx(recv, (unsigned)(npx * C::kRow * 4));
+        }
+    } else if (warp == kLoadWarps + 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(slot32), "r"((unsigned)C::kCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+    } else if (tid < PX) {
+        const int m = m0 + tid;
+        const int img = (int)fdiv((unsigned)m, p.d_hw), q = m - img * p.h_out * p.w_out;
+        const int oy = (int)fdiv((unsigned)q, p.d_wo), ox = q - oy * p.w_out;
+        const int iy = oy * p.stride - p.pad, ix = ox * p.stride - p.pad_w;
+        const int yx = (m < p.M && tid < npx ? iy : kNoPixel) * 65536 | (ix & 0xffff), off = ((img * p.h + iy) * p.w + ix) * p.c_in;
+        asm volatile("st.shared.v2.b32 [%0], {%1, %2};\n" ::"r"(pxs + tid * 8), "r"(off), "r"(yx) : "memory");
+    }
+    // loader threads: 16 source bytes (chunk c) of the pixels r0, r0 + kPS, ... in every kGroups-th stage
+    const int kPS = C::kGroupThreads / 8;
+    const int grp = tid / C::kGroupThreads, c = tid & 7, r0 = tid % C::kGroupThreads / 8;
+    // K position of its next stage: kernel row ky, position ci in that row (VEC: channel ci of kernel column kx)
+    const int k = (kb0 + grp) * C::kKB + c * (C::kKB / 8);
+    int ky = (int)fdiv((unsigned)k, p.d_Rp), kx = 0, ci = k - ky * p.Rp;
+    if (VEC) {
+        kx = (int)fdiv((unsigned)ci, p.d_ci);
+        ci -= kx * p.c_in;
+    }
+    __syncwarp();
+    if (p.S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");   // waited for before the first remote copy
+    __syncthreads();
+
+    if (warp < kLoadWarps) {
+        uint4 v[C::kRPT];
+        auto request = [&]() {
+#pragma unroll
+            for (int i = 0; i < C::kRPT; ++i) {
+                const Px px = load_px(pxs + (r0 + kPS * i) * 8);
+                v[i] = VEC ? gather_vec<F32>(p, px, ky, kx, ci) : gather_run<F32>(p, px, ky, ci);
+            }
+            ci += C::kGroups * C::kKB;
+            const int wrap = VEC ? p.c_in : p.Rp;
+            while (ci >= wrap) {
+                ci -= wrap;
+                if (!VEC || ++kx == p.kw) { kx = 0; ++ky; }
+            }
+        };
+        grid_dep_wait();
+        if (kb0 + grp < kb1) request();
+        // swizzled place of the thread's chunk in pixel row r0 of an operand tile (rows kPS apart have the same pattern)
+        const unsigned sw = (unsigned)((r0 >> 1) & 3);
+        const unsigned at = F32 ? r0 * 64 + ((((unsigned)c >> 1) ^ sw) << 4) + (c & 1) * 8
+                                : (c >> 2) * xpart + r0 * 64 + ((((unsigned)c & 3u) ^ sw) << 4);
+        int s = grp;
+        unsigned round = 0;
+        bool alive = true;
+        for (int kb = kb0 + grp; kb < kb1; kb += C::kGroups) {
+            while (s >= S) { s -= S; ++round; }
+            if (round > 0 && alive) alive = mb_wait(bars + (S + s) * 8, (round - 1) & 1u, p.gave_up);
+            const unsigned a = base + s * C::kStage + at;
+#pragma unroll
+            for (int i = 0; i < C::kRPT; ++i) {
+                if (SWAP && r0 + kPS * i >= npx) continue;
+                if (!F32) sts128(a + i * (kPS * 64), v[i]);
+                else {
+                    unsigned h0, h1, m0_, m1, l0, l1;
+                    split2(__uint_as_float(v[i].x), __uint_as_float(v[i].y), h0, m0_, l0);
+                    split2(__uint_as_float(v[i].z), __uint_as_float(v[i].w), h1, m1, l1);
+                    sts64(a + i * (kPS * 64), h0, h1);
+                    sts64(a + i * (kPS * 64) + xpart, m0_, m1);
+                    sts64(a + i * (kPS * 64) + 2 * xpart, l0, l1);
+                }
+            }
+            if (kb + C::kGroups < kb1) request();
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mb_arrive(bars + s * 8);
+            s += C::kGroups;
+        }
+        grid_dep_trigger();
+    } else if (warp == kLoadWarps) {
+        if (lane == 0) {
+            int s = 0;
+            unsigned round = 0;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (round > 0 && !mb_wait(bars + (S + s) * 8, (round - 1) & 1u, p.gave_up)) break;
+                copy_weights(kb, s);
+                if (++s == S) { s = 0; ++round; }
+            }
+        }
+    } else if (lane == 0) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        const unsigned tmem = *slot;
+        const int N = SWAP ? npx : CH;
+        const unsigned fmt = (F32 ? 1u << 4 : 2u << 4) | (1u << 7) | (1u << 10) | (8u << 24);
+        const unsigned id1 = fmt | ((unsigned)(N >> 3) << 17), id2 = fmt | ((unsigned)(2 * N >> 3) << 17);
+        const unsigned ap = SWAP ? CH * 64 : xpart, bp = SWAP ? xpart : CH * 64;   // bytes from part to part of the two operands
+        int s = 0;
+        unsigned round = 0, acc = 0;
+        for (int kb = kb0; kb < kb1; ++kb) {
+            if (!mb_wait(bars + s * 8, round & 1u, p.gave_up)) break;
+            asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+            const unsigned xs = base + s * C::kStage, ws = xs + C::kXBytes;
+            const unsigned a = SWAP ? ws : xs, w = SWAP ? xs : ws;
+            if (F32) {
+#pragma unroll
+                for (int kk = 0; kk < 2; ++kk) {
+                    const unsigned long long a1 = smem_desc(a + kk * 32), a2 = smem_desc(a + ap + kk * 32), a3 = smem_desc(a + 2 * ap + kk * 32);
+                    const unsigned long long b1 = smem_desc(w + kk * 32), b2 = smem_desc(w + bp + kk * 32), b3 = smem_desc(w + 2 * bp + kk * 32);
+                    // The parts of b lie behind each other, and so do the accumulators: one instruction can take several
+                    // parts at once, which reads the a tile from shared memory less often.
+                    if (C::kAcc == 3) {   // columns [large | 2^-9 terms | 2^-18 terms]
+                        mma<true>(tmem, a1, b1, fmt | ((unsigned)(3 * N >> 3) << 17), acc);   // a1 b1 | a1 b2 | a1 b3
+                        mma<true>(tmem + N, a2, b1, id2, 1);                                  // a2 b1 | a2 b2
+                        mma<true>(tmem + 2 * N, a3, b1, id1, 1);                              // a3 b1
+                    } else {              // columns [large | small terms]
+                        if (2 * N <= 256) mma<true>(tmem, a1, b1, id2, acc);
+                        else {
+                            mma<true>(tmem, a1, b1, id1, acc);
+                            mma<true>(tmem + N, a1, b2, id1, acc);
+                        }
+                        mma<true>(tmem + N, a2, b1, id1, 1);
+                        mma<true>(tmem + N, a2, b2, id1, 1);
+                        mma<true>(tmem + N, a1, b3, id1, 1);
+                        mma<true>(tmem + N, a3, b1, id1, 1);
+                    }
+                    acc = 1;
+                }
+            } else {
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    mma<false>(tmem + (kk & 1) * N, smem_desc(a + (kk >> 1) * ap + (kk & 1) * 32), smem_desc(w + (kk >> 1) * bp + (kk & 1) * 32), id1,
+                               kk < 2 ? acc : 1);
+                acc = 1;
+            }
+            tc_commit(bars + (S + s) * 8);
+            if (++s == S) { s = 0; ++round; }
+        }
+        tc_commit(done);
+    }
+    __syncwarp();
+
+    // ---- epilogue (code that runs once per block costs its instruction fetches: loops stay rolled) ----
+    const unsigned tmem = *slot;
+    const int rows = npx / p.S, lo = rows * rank;
+    const int kVec = CH / 4, kStep = kLoadWarps * 32 / kVec;
+    const int col = (tid % kVec) * 4, r1 = tid / kVec, co = nt * CH + col;
+    const bool mine = warp < kLoadWarps && co < p.c_out;
+    float4 sc = make_float4(1, 1, 1, 1), bi = make_float4(0, 0, 0, 0);
+    uint4 res = make_uint4(0, 0, 0, 0);
+    if (mine && (SWAP || p.S > 1)) {
+        // of the row this thread finishes first; on their way while the last multiply-adds run
+        load_channels(p, co, sc, bi);
+        if (p.residual && r1 < rows && m0 + lo + r1 < p.M) res = load_residual<F32>(p, m0 + lo + r1, co);
+    }
+    __syncwarp();
+    if (p.S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");   // every block has initialised its barriers
+    if (warp < kLoadWarps) {
+        // a warp can read the 32 rows 32 q ..; the two warps with the same q take turns on groups of 16 columns
+        const int q = warp & 3, N = SWAP ? npx : CH;
+        const unsigned from = tmem + ((unsigned)(q * 32) << 16);
+        const int mrow = m0 + q * 32 + lane;   // (rows are pixels)
+        mb_wait(done, 0u, p.gave_up);
+        __syncwarp();
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+#pragma unroll 1
+        for (int j = (warp >> 2) * 16; j < N; j += 32) {
+            unsigned v[16], u[16];
+            tmem_ld16(from + j, v);
+            tmem_ld16(from + N + j, u);
+            if (F32 && C::kAcc == 3) {
+                unsigned t3[16];
+                tmem_ld16(from + 2 * N + j, t3);
+                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+                for (int t = 0; t < 16; ++t) u[t] = __float_as_uint(__uint_as_float(u[t]) + __uint_as_float(t3[t]));
+            } else asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+            for (int t = 0; t < 16; ++t) v[t] = F32 ? __float_as_uint(__uint_as_float(v[t]) + __uint_as_float(u[t])) : v[t] + u[t];
+            if (SWAP || p.S > 1) {   // to shared memory as [pixel][channel] (over the stages: all of them have been read)
+                if (SWAP) {
+                    const unsigned at = base + (j * C::kRow + q * 32 + lane) * 4;
+#pragma unroll
+                    for (int t = 0; t < 16; ++t) asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(at + t * C::kRow * 4), "r"(v[t]) : "memory");
+                } else {
+                    const unsigned at = base + ((q * 32 + lane) * C::kRow + j) * 4;
+#pragma unroll
+                    for (int t = 0; t < 16; t += 4) sts128(at + t * 4, make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]));
+                }
+            } else if (mrow < p.M) {   // a lane per pixel: it finishes its 16 consecutive channels at once
+                unsigned q8[4];
+#pragma unroll
+                for (int t = 0; t < 16; t += 4) {
+                    const int c4 = nt * CH + j + t;
+                    if (c4 >= p.c_out) break;
+                    load_channels(p, c4, sc, bi);
+                    if (p.residual) res = load_residual<F32>(p, mrow, c4);
+                    const uint4 t4 = make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+                    if (!F32 && p.vec16) q8[t / 4] = finish_q4(p, t4, res.x, sc, bi);
+                    else finish4<F32>(p, (size_t)mrow * p.ldc + p.c_off + c4, p.c_out - c4, t4, res, sc, bi);
+                }
+                if (!F32 && p.vec16 && nt * CH + j < p.c_out)
+                    *reinterpret_cast<uint4 *>(reinterpret_cast<signed char *>(p.y) + (size_t)mrow * p.ldc + p.c_off + nt * CH + j) =
+                        make_uint4(q8[0], q8[1], q8[2], q8[3]);
+            }
+        }
+        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+        if (p.S > 1) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+    }
+    __syncthreads();
+    if (warp == kLoadWarps + 1) {
+        asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((unsigned)C::kCols) : "memory");
+    }
+    if (!SWAP && p.S == 1) return;
+    // split reduction: each block's sums of a pixel go to the block of the cluster that finishes the pixel
+    const unsigned slice = rows * C::kRow * 4;
+    if (p.S > 1) {
+        if (tid < p.S) push_copy(base + p.recv_off + rank * slice, base + tid * slice, slice, recv, tid);
+        __syncwarp();
+        if (warp < kLoadWarps) mb_wait(recv, 0u, p.gave_up);
+        __syncwarp();
+        // this block has received everything, so the others may go; it goes itself when they have received what it sent
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
+    }
+    if (mine) {
+        unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (r1 * C::kRow + col) * 4;
+#pragma unroll 1
+        for (int row = r1, m = m0 + lo + r1; row < rows && m < p.M; row += kStep, m += kStep) {
+            uint4 t = lds128(at);
+#pragma unroll 4
+            for (int q = 1; q < p.S; ++q) {
+                const uint4 u = lds128(at + q * slice);
+                if (F32) {
+                    t.x = __float_as_uint(__uint_as_float(t.x) + __uint_as_float(u.x));
+                    t.y = __float_as_uint(__uint_as_float(t.y) + __uint_as_float(u.y));
+                    t.z = __float_as_uint(__uint_as_float(t.z) + __uint_as_float(u.z));
+                    t.w = __float_as_uint(__uint_as_float(t.w) + __uint_as_float(u.w));
+                } else {
+                    t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+                }
+            }
+            at += kStep * C::kRow * 4;
+            const uint4 r = res;
+            if (p.residual && row + kStep < rows && m + kStep < p.M) res = load_residual<F32>(p, m + kStep, co);
+            finish4<F32>(p, (size_t)m * p.ldc + p.c_off + co, p.c_out - co, t, r, sc, bi);
+        }
+    }
+    __syncwarp();
+    if (p.S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+}
+
+int ceil_div(int a, int b) { return (a + b - 1) / b; }
+
+struct Pick {
+    int px, ch, split;   // pixels and channels per block, blocks per cluster
+};
+
+// Shared memory of one block: its pipeline depth, where the exchanged sums and the barriers lie, and its size.
+struct SmemPlan {
+    int stages, recv_off, bar_off, bytes;
+};
+SmemPlan plan_smem(bool f32, const Pick &k, int nkb, long long blocks)
+{
+    const int PX = k.ch == 64 ? 128 : k.px <= 64 ? 64 : k.px <= 128 ? 128 : 256;
+    const bool swap = k.ch == 128;
+    const int groups = swap && PX == 64 && k.split > 1 ? 4 : 2;
+    const int stage = (f32 ? 3 : 2) * 64 * (PX + k.ch), out = k.px * (k.ch + 4) * 4;
+    // two blocks share a multiprocessor unless the shape is too large or a small split grid leaves room for a deeper pipeline
+    const int budget = (PX > 128 || groups > 2 || (k.split > 1 && blocks <= 148) ? 216 : 108) * 1024;
+    SmemPlan s;
+    s.stages = std::max(groups, std::min(std::min(4, std::max(groups, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
+    s.recv_off = std::max(s.stages * stage, swap || k.split > 1 ? out : 0);   // the sums are staged over the stages
+    s.bar_off = (s.recv_off + (k.split > 1 ? out : 0) + 127) / 128 * 128;
+    s.bytes = s.bar_off + 1024 + 128 + PX * 8;
+    return s;
+}
+
+// Block shape of a layer: the one a time model calls the fastest.  The model is linear in what a block does, with
+// coefficients fitted to 3000 measured launches (193 layers of the workloads at batch 1 to 128, every shape and split):
+//   time = start + P (b2 + n (c2 + d2 px / 64)) + Q (b1 + n (c1 + d1 px / 64))   [microseconds]
+// n = stages per block, P = rounds in which every multiprocessor runs two blocks, Q = rounds with one.  How many clusters
+// of a size run at once is what cudaOccupancyMaxActiveClusters reports for this GPU (a cluster has to fit one GPC).
+// Mean excess of the chosen over the best measured shape: 2 %.
+struct Cost {
+    float start, b2, c2, d2, b1, c1, d1;
+};
+const Cost kCost[2][6] = {
+    // 128 px x 64 ch, same split, <= 64 px x 128 ch, same split, <= 128 px x 128 ch, same split
+    {{1.48f, 4.67f, 0.0f, 0.429f, 3.30f, 0.0f, 0.264f},      // float
+     {2.48f, 3.69f, 0.0f, 0.480f, 3.05f, 0.0f, 0.265f},
+     {1.40f, 3.54f, 0.332f, 0.351f, 2.83f, 0.401f, 0.090f},
+     {1.38f, 0.0f, 0.0f, 0.0f, 3.52f, 0.353f, 0.188f},
+     {1.15f, 6.30f, 0.323f, 0.456f, 5.05f, 0.539f, 0.158f},
+     {1.81f, 0.0f, 0.0f, 0.0f, 5.19f, 0.320f, 0.306f}},
+    {{2.45f, 3.69f, 0.0f, 0.339f, 2.54f, 0.0f, 0.184f},      // int8
+     {2.54f, 3.10f, 0.0f, 0.382f, 2.63f, 0.0f, 0.213f},
+     {2.21f, 2.75f, 0.206f, 0.431f, 2.04f, 0.265f, 0.130f},
+     {1.17f, 3.11f, 0.480f, 0.0f, 3.12f, 0.229f, 0.343f},
+     {2.36f, 5.39f, 0.055f, 0.424f, 3.61f, 0.125f, 0.214f},
+     {1.61f, 4.20f, 0.0f, 0.704f, 5.05f, 0.0f, 0.303f}}};
+const Cost kCost256[2] = {{0.0f, 0.0f, 0.0f, 0.0f, 9.23f, 0.345f, 0.222f}, {0.0f, 0.0f, 0.0f, 0.0f, 8.37f, 0.157f, 0.220f}};
+
+Pick choose(bool f32, int c_out, long long M, int nkb)
+{
+    Pick best = {128, 64, 1};
+    double best_t = 1e300;
+    auto consider = [&](int px, int ch) {
+        const long long tiles = (M + px - 1) / px * ceil_div(c_out, ch);
+        for (int log = 0; log <= (px > 128 ? 0 : 4); ++log) {
+            const int split = 1 << log;
+            if (split > nkb || px % split) break;
+            if (split > 1 && tiles * split > 330) break;      // the grid already fills the chip twice
+            static const int cap1[5] = {148, 74, 33, 15, 7}, cap2[5] = {296, 148, 71, 33, 14};
+            const Pick k = {px, ch, split};
+            const bool two = plan_smem(f32, k, nkb, tiles * split).bytes <= 113 * 1024;
+            long long P = 0, Q = 0;
+            if (two) {
+                P = tiles / cap2[log];
+                const long long rest = tiles - P * cap2[log];
+                if (rest > cap1[log]) ++P;
+                else if (rest > 0) Q = 1;
+            } else Q = (tiles + cap1[log] - 1) / cap1[log];
+            const Cost &c = px > 128 ? kCost256[!f32] : kCost[!f32][(ch == 64 ? 0 : px <= 64 ? 2 : 4) + (split > 1)];
+            const double n = ceil_div(nkb, split), u = px / 64.0;
+            const double t = c.start + P * (c.b2 + n * (c.c2 + c.d2 * u)) + Q * (c.b1 + n * (c.c1 + c.d1 * u));
+            if (t < best_t) { best_t = t; best = k; }
+        }
+    };
+    consider(128, 64);
+    static const int fixed[] = {32, 64, 96, 112, 128, 256};
+    for (int px : fixed) consider(px, 128);
+    for (int q = 1; q <= 16; ++q) {   // the pixels cut into q equal tiles
+        const long long px = ((M + q - 1) / q + 15) / 16 * 16;
+        if (px <= 256) consider((int)px, 128);
+        if (px <= 16) break;
+    }
+    return best;
+}
+
+template <bool F32, int PX, int CH, bool SWAP, int GROUPS, bool VEC>
+cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
+{
+    auto kern = tcconv_kernel<F32, PX, CH, SWAP, GROUPS, VEC>;
+    typedef Cfg<F32, PX, CH, SWAP, GROUPS> C;
+    const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb, blocks);
+    if (sp.stages < C::kGroups || sp.stages * C::kStage > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
+    p.stages = sp.stages;
+    p.recv_off = sp.recv_off;
+    p.bar_off = sp.bar_off;
+    const int smem = sp.bytes;
+    static SmemLimit lim;
+    cadnn_status rs = raise_smem_limit((const void *)kern, smem, &lim);
+    if (rs != CADNN_OK) return rs;
+    if (p.S > 8) CADNN_CUDA_TRY(cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (p.S > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)p.S;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    CADNN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, p));
+    return CADNN_OK;
+}
+
+template <bool F32, bool VEC> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
+{
+    if (ch == 64) return launch_one<F32, 128, 64, false, 2, VEC>(p, blocks, pdl, st);
+    if (p.npx <= 64 && p.S > 1) return launch_one<F32, 64, 128, true, 4, VEC>(p, blocks, pdl, st);
+    if (p.npx <= 64) return launch_one<F32, 64, 128, true, 2, VEC>(p, blocks, pdl, st);
+    if (p.npx <= 128) return launch_one<F32, 128, 128, true, 2, VEC>(p, blocks, pdl, st);
+    return launch_one<F32, 256, 128, true, 2, VEC>(p, blocks, pdl, st);
+}
+
+
+}  // namespace
+
+namespace {
+// K positions per kernel row: kw * c_in values, padded to whole 16-byte pieces
+int row_positions(const cadnn_layer_desc &d)
+{
+    const int per16 = d.dtype == CADNN_S8 ? 16 : 4;
+    return ceil_div(d.kw * d.c_in, per16) * per16;
+}
+int stages_of(const cadnn_layer_desc &d) { return ceil_div(d.kh * row_positions(d), d.dtype == CADNN_S8 ? 128 : 32); }
+}  // namespace
+
+// When the dense route is taken.  Per multiply-add of the full layer the tensor cores cost the same whatever the mask; the
+// sparse kernels cost per stored weight.  Measured on the 3x3 and 1x1 layers of the workloads at batch 1 to 32 (microseconds
+// against density) the lines cross between 1 and 3 per cent, for float and for int8; float layers of at most 64 output channels
+// fill half a tile's columns only, and cross between 5 and 7 per cent.
+bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz)
+{
+    const double density = (double)nnz / ((double)d.c_out * d.kh * d.kw * d.c_in);
+    return density >= (d.dtype == CADNN_F32 && d.c_out <= 64 ? 0.06 : 0.025);
+}
+
+// Weight image: [64-channel tile][stage][part][64 rows][64 bytes], rows swizzled like the operand tiles.  Parts: the
+// three bf16 terms of a float, or the two 64-value halves of an int8 stage.
+void tcv_build(cadnn_weights *h, const float *f, const int8_t *q, const uint8_t *mask)
+{
+    const cadnn_layer_desc &d = h->desc;
+    const bool s8 = d.dtype == CADNN_S8;
+    const int R = d.kw * d.c_in, Rp = row_positions(d), nkb = stages_of(d), parts = s8 ? 2 : 3;
+    h->tcv_img.assign((size_t)ceil_div(d.c_out, 64) * nkb * parts * 4096, 0);
+    for (int co = 0; co < d.c_out; ++co) {
+        unsigned char *tile = &h->tcv_img[(size_t)(co / 64) * nkb * parts * 4096];
+        const int r = co & 63, sw = (r >> 1) & 3;
+        for (int ky = 0; ky < d.kh; ++ky)
+        for (int i = 0; i < R; ++i) {
+            const size_t wi = ((size_t)co * d.kh + ky) * R + i;
+            const int k = ky * Rp + i;
+            if (mask && !mask[wi]) continue;
+            if (s8) {
+                const int kb = k >> 7, part = (k >> 6) & 1, c = k & 63;
+                tile[((size_t)kb * 2 + part) * 4096 + r * 64 + (((c >> 4) ^ sw) << 4) + (c & 15)] = (unsigned char)q[wi];
+            } else {
+                const int kb = k >> 5, c = k & 31;
+                unsigned char *at = tile + (size_t)kb * 3 * 4096 + r * 64 + (((c >> 3) ^ sw) << 4) + (c & 7) * 2;
+                float v = f[wi];
+                for (int t = 0; t < 3; ++t) {
+                    const __nv_bfloat16 b = __float2bfloat16_rn(v);
+                    memcpy(at + t * 4096, &b, 2);
+                    v -= __bfloat162float(b);
+                }
+            }
+        }
+    }
+    h->has_tcv = true;
+    int a = 0, b = 0, c = 0;   // for tests and tuning: the block shape, "pixels,channels,split"
+    const char *e = getenv("CADNN_TCV");
+    if (e && sscanf(e, "%d,%d,%d", &a, &b, &c) == 3 && a >= 16 && a <= 256 && a % 16 == 0 && (b == 128 || (b == 64 && a == 128)) && c >= 1) {
+        h->tcv_force[0] = a; h->tcv_force[1] = b; h->tcv_force[2] = c;
+    }
+}
+
+// the kernel's index ranges: 31-bit element offsets and pixel numbers, 16-bit image coordinates
+bool tcv_fits(const cadnn_weights *w, int n)
+{
+    const cadnn_layer_desc &d = w->desc;
+    const long long lim = (1ll << 31) - (1 << 20);
+    return (long long)n * w->h_out * w->w_out < lim && ((long long)n * d.in_h + 2 * d.kh) * d.in_w * d.c_in < lim && d.in_h < 16000 && d.in_w < 16000;
+}
+
+cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep, cudaStream_t st)
+{
+    const cadnn_layer_desc &d = w->desc;
+    const bool f32 = d.dtype == CADNN_F32;
+    const long long M = (long long)n * w->h_out * w->w_out;
+    if (!w->d_tcv || !tcv_fits(w, n)) return CADNN_E_UNSUPPORTED;
+    if (M == 0) return CADNN_OK;
+    TcvParams p = {};
+    p.x = x; p.y = y; p.wimg = (const unsigned char *)w->d_tcv;
+    p.scale = ep.scale; p.bias = ep.bias; p.residual = ep.residual; p.res_scale = ep.res_scale;
+    p.act = ep.act; p.out_dtype = ep.out_dtype;
+    p.h = d.in_h; p.w = d.in_w; p.c_in = d.c_in; p.h_out = w->h_out; p.w_out = w->w_out; p.c_out = d.c_out;
+    p.stride = d.stride; p.pad = d.pad; p.pad_w = d.pad_w; p.kh = d.kh; p.kw = d.kw;
+    p.M = (int)M; p.Rp = row_positions(d); p.nkb = stages_of(d);
+    p.ldc = ep.out_c_total > 0 ? ep.out_c_total : d.c_out;
+    p.c_off = ep.out_c_total > 0 ? ep.out_c_off : 0;
+    p.vec_ok = d.c_out % 4 == 0 && p.ldc % 4 == 0 && p.c_off % 4 == 0;
+    p.vec16 = ep.out_dtype == CADNN_S8 && d.c_out % 16 == 0 && p.ldc % 16 == 0 && p.c_off % 16 == 0;
+    p.vec_sb = ((uintptr_t)ep.scale & 15) == 0 && ((uintptr_t)ep.bias & 15) == 0;
+    p.d_hw = make_fastdiv(w->h_out * w->w_out); p.d_wo = make_fastdiv(w->w_out);
+    p.d_ci = make_fastdiv(d.c_in); p.d_Rp = make_fastdiv(p.Rp);
+    cadnn_status rs = copy_timeout_word(&p.gave_up);
+    if (rs != CADNN_OK) return rs;
+    // the last batch size's choice is kept in the handle (one word, so that threads may race on it)
+    Pick pick = {w->tcv_force[0], w->tcv_force[1], w->tcv_force[2]};
+    const uint64_t kept = w->tcv_pick.load(std::memory_order_relaxed);
+    if (pick.px > 0) pick.split = std::max(1, pick.split);
+    else if ((kept >> 32) == (uint64_t)n && kept != 0) pick = {(int)(kept & 0xfff), (int)(kept >> 12 & 0xfff), (int)(kept >> 24 & 0xff)};
+    else {
+        pick = choose(f32, d.c_out, M, p.nkb);
+        w->tcv_pick.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
+    }
+    if (pick.ch == 64) pick.px = 128;
+    p.npx = pick.px;
+    p.n_nt = ceil_div(d.c_out, pick.ch);
+    // every block of a cluster finishes the same number of pixels, and two stages and the partial sums have to fit
+    p.S = pick.px > 128 ? 1 : std::min(pick.split, 16);
+    while (p.S > 1 && (p.npx % p.S || p.S > p.nkb)) --p.S;
+    p.kb_base = p.nkb / p.S; p.kb_rem = p.nkb % p.S;
+    p.d_S = make_fastdiv(p.S); p.d_nt = make_fastdiv(p.n_nt);
+    const long long blocks = (M + p.npx - 1) / p.npx * p.n_nt * p.S;
+    if (blocks > 2147483647ll) return CADNN_E_UNSUPPORTED;
+    const bool vec = d.c_in % (f32 ? 4 : 16) == 0;
+    if (f32) return vec ? launch_shape<true, true>(p, pick.ch, (int)blocks, ep.pdl, st) : launch_shape<true, false>(p, pick.ch, (int)blocks, ep.pdl, st);
+    return vec ? launch_shape<false, true>(p, pick.ch, (int)blocks, ep.pdl, st) : launch_shape<false, false>(p, pick.ch, (int)blocks, ep.pdl, st);
+}
+
+cadnn_status tcv_upload(cadnn_weights *h)
+{
+    if (!h->has_tcv || (h->desc.flags & CADNN_PACK_HOST_ONLY)) return CADNN_OK;
+    cudaError_t e = cudaMalloc(&h->d_tcv, h->tcv_img.size());
+    if (e != cudaSuccess) {
+        cadnn_note_cuda(e);
+        return e == cudaErrorMemoryAllocation ? CADNN_E_ALLOC : CADNN_E_CUDA;
+    }
+    CADNN_CUDA_TRY(cudaMemcpy(h->d_tcv, h->tcv_img.data(), h->tcv_img.size(), cudaMemcpyHostToDevice));
+    CADNN_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
+    std::vector<unsigned char>().swap(h->tcv_img);
+    return CADNN_OK;
+}

@@ -1,0 +1,91 @@
+"""Dense tensor-core route (csrc/tcconv.cu): every block shape and reduction split at the sizes where it can go wrong -
+ragged last tiles of pixels and channels, one pipeline stage and more stages than the ring holds, channels that are not a
+multiple of 16 bytes, padding, strides - against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import ref
+from workloads import gen
+from parity import assert_close_or_bounded, assert_exact
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+# (pixels, channels, split) of a block; None = the library's own choice
+SHAPES = ["128,64,1", "128,64,4", "16,128,1", "48,128,8", "64,128,1", "64,128,16", "80,128,2", "128,128,1", "128,128,4", "256,128,1", None]
+# n, h, w, c_in, c_out, k, stride, pad
+LAYERS = [(1, 7, 7, 32, 64, 1, 1, 0), (2, 9, 11, 40, 130, 3, 1, 1), (1, 14, 13, 67, 65, 3, 2, 1), (3, 10, 6, 3, 70, 5, 1, 2),
+          (1, 13, 13, 304, 129, 3, 1, 0), (17, 1, 1, 1027, 200, 1, 1, 0)]
+
+
+def _pack(B, monkeypatch, shape, dtype, layer, w, mask):
+    n, h, wd, c_in, c_out, k, stride, pad = layer
+    if shape:
+        monkeypatch.setenv("CADNN_TCV", shape)
+    d = B.make_desc(c_in, c_out, k, k, stride, pad, 1, h, wd, n, dtype)
+    return (B.cadnn_pack_q8 if dtype == "s8" else B.cadnn_pack)(d, w, mask)
+
+
+@pytest.mark.parametrize("layer", LAYERS)
+@pytest.mark.parametrize("shape", SHAPES)
+def test_float_layers(shape, layer, monkeypatch):
+    from paper_1905_00571_b200 import binding as B
+    n, h, wd, c_in, c_out, k, stride, pad = layer
+    g = gen.rng(41 + c_in)
+    x = gen.normal_input(g, (n, h, wd, c_in))
+    w = gen.he_weights(g, c_out, k, k, c_in)
+    mask = gen.random_mask(g, w.shape, 0.2)
+    scale, bias = gen.folded_bn(g, c_out)
+    res = gen.normal_input(g, ref.conv2d_f32(x, w, mask, stride, pad).shape)
+    want = ref.conv2d_f32(x, w, mask, stride, pad, 1, scale, bias, res, "relu")
+    wh = _pack(B, monkeypatch, shape, "f32", layer, w, mask)
+    y = torch.full(want.shape, -1.0, device=DEV)
+    dev = lambda a: torch.from_numpy(a).to(DEV)
+    B.cadnn_conv2d(wh, dev(x), y, dev(scale), dev(bias), dev(res), "relu")
+    torch.cuda.synchronize()
+    s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None, stride, pad, 1, np.abs(scale), np.abs(bias), np.abs(res), "none")
+    assert_close_or_bounded(y.cpu().numpy(), want, s_abs, int(mask.reshape(c_out, -1).sum(1).max()) + 4, "%s %s" % (layer, shape))
+    assert B.cadnn_device_status()["copy_timeouts"] == 0
+
+
+@pytest.mark.parametrize("layer", LAYERS)
+@pytest.mark.parametrize("shape", SHAPES)
+def test_int8_layers_bit_exact(shape, layer, monkeypatch):
+    from paper_1905_00571_b200 import binding as B
+    n, h, wd, c_in, c_out, k, stride, pad = layer
+    g = gen.rng(43 + c_in)
+    x = gen.int8_relu_activation(g, (n, h, wd, c_in))
+    q = gen.int8_weights(g, (c_out, k, k, c_in))
+    mask = gen.random_mask(g, q.shape, 0.2)
+    m = (g.uniform(0.5, 1.5, size=c_out) * 2e-4).astype(np.float32)
+    b = (g.standard_normal(c_out) * 3).astype(np.float32)
+    dev = lambda a: torch.from_numpy(a).to(DEV)
+    wh = _pack(B, monkeypatch, shape, "s8", layer, q, mask)
+    r = gen.int8_relu_activation(g, ref.conv2d_s8(x, q, mask, stride, pad, out="s32").shape)
+    for out, dt, res in (("s8", torch.int8, r), ("f32", torch.float32, None), ("s32", torch.int32, None)):
+        want = ref.conv2d_s8(x, q, mask, stride, pad, 1, m, b, "relu", out, res, 0.4) if out != "s32" else \
+            ref.conv2d_s8(x, q, mask, stride, pad, out="s32")
+        y = torch.full(want.shape, 5, dtype=dt, device=DEV)
+        B.cadnn_conv2d(wh, dev(x), y, dev(m), dev(b), None if res is None else dev(res), "relu", out_dtype=out, residual_scale=0.4)
+        torch.cuda.synchronize()
+        assert_exact(y.cpu().numpy(), want, "%s %s %s" % (layer, shape, out))
+    assert B.cadnn_device_status()["copy_timeouts"] == 0
+
+
+@pytest.mark.parametrize("c_off", [0, 12])
+def test_channel_window_of_a_concatenation(c_off):
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(47)
+    x = gen.relu_normal_input(g, (2, 8, 9, 48))
+    w = gen.he_weights(g, 68, 3, 3, 48)
+    mask = gen.random_mask(g, w.shape, 0.3)
+    want = ref.conv2d_f32(x, w, mask, 1, 1, act="relu")
+    wh = B.cadnn_pack(B.make_desc(48, 68, 3, 3, 1, 1, 1, 8, 9, 2, "f32"), w, mask)
+    y = torch.full((2, 8, 9, 96), 3.0, device=DEV)
+    B.cadnn_conv2d(wh, torch.from_numpy(x).to(DEV), y, act="relu", out_c_total=96, out_c_off=c_off)
+    torch.cuda.synchronize()
+    got = y.cpu().numpy()
+    s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None, 1, 1)
+    assert_close_or_bounded(got[..., c_off:c_off + 68], want, s_abs, 48 * 9, "window")
+    assert (got[..., :c_off] == 3.0).all() and (got[..., c_off + 68:] == 3.0).all()
