@@ -16,6 +16,7 @@ if not os.path.exists(LIB_PATH):
     raise ImportError("libcadnn.so is missing: run `python -m paper_1905_00571_b200.build` "
                       "(or __graft_entry__.build()) first; there is no fallback implementation")
 _lib = ctypes.CDLL(LIB_PATH)
+from . import _fastcall  # noqa: E402  (native marshalling of the calls made per layer or image; built with the library)
 
 OK = 0
 F32, S8, S32 = 0, 1, 2
@@ -228,17 +229,8 @@ def _epilogue(scale, bias, residual, act, out_dtype, out_c_total=0, out_c_off=0,
                     float(residual_scale))
 
 
-def cadnn_conv2d(w, x, y, scale=None, bias=None, residual=None, act="none", out_dtype=None, stream=None,
-                 out_c_total=0, out_c_off=0, residual_scale=0.0):
-    """x, y: torch CUDA tensors, NHWC contiguous; y is written in place (channels [out_c_off, out_c_off + c_out)
-    of it when out_c_total > 0)."""
-    n, h, wd = int(x.shape[0]), int(x.shape[1]), int(x.shape[2])
-    if out_dtype is None:
-        out_dtype = w.desc.dtype
-    ep = _epilogue(scale, bias, residual, act, out_dtype, out_c_total, out_c_off, residual_scale)
-    _check(_lib.cadnn_conv2d(w.handle, _dev_ptr(x), n, h, wd, _dev_ptr(y), ctypes.byref(ep), _stream(stream)),
-           "cadnn_conv2d")
-    return y
+_fastcall.setup(_check, ACT, DTYPE)
+cadnn_conv2d = _fastcall.cadnn_conv2d
 
 
 def cadnn_weights_workspace_bytes(w, n):
@@ -276,13 +268,7 @@ def cadnn_conv2d_planar(w, x, y, scale=None, bias=None, residual=None, act="none
     return y
 
 
-def cadnn_fc(w, x, y, scale=None, bias=None, residual=None, act="none", out_dtype=None, stream=None):
-    if out_dtype is None:
-        out_dtype = w.desc.dtype
-    ep = _epilogue(scale, bias, residual, act, out_dtype)
-    _check(_lib.cadnn_fc(w.handle, _dev_ptr(x), int(x.shape[0]), _dev_ptr(y), ctypes.byref(ep), _stream(stream)),
-           "cadnn_fc")
-    return y
+cadnn_fc = _fastcall.cadnn_fc
 
 
 def cadnn_maxpool2d(x, y, k, stride, pad=0, stream=None):
@@ -336,19 +322,8 @@ def cadnn_net_create(ops, n, h, w, c, in_dtype, keep=None):
     return Net(out, keep)
 
 
-def cadnn_forward(net, x, y, use_graph=True, stream=None):
-    _check(_lib.cadnn_forward(net.handle, _dev_ptr(x), _dev_ptr(y), 1 if use_graph else 0, _stream(stream)),
-           "cadnn_forward")
-    return y
-
-
-def cadnn_forward_host(net, x_host, y_host, use_graph=True, stream=None):
-    """x_host, y_host: CPU torch tensors (pinned recommended) or numpy arrays; blocks until y_host is filled."""
-    xp = x_host.data_ptr() if hasattr(x_host, "data_ptr") else x_host.ctypes.data
-    yp = y_host.data_ptr() if hasattr(y_host, "data_ptr") else y_host.ctypes.data
-    _check(_lib.cadnn_forward_host(net.handle, ctypes.c_void_p(xp), ctypes.c_void_p(yp), 1 if use_graph else 0,
-                                   _stream(stream)), "cadnn_forward_host")
-    return y_host
+cadnn_forward = _fastcall.cadnn_forward
+cadnn_forward_host = _fastcall.cadnn_forward_host
 
 
 STATIC_WORKSPACE_BYTES = 32 << 20

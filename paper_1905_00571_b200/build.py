@@ -3,10 +3,13 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libcadnn.so")
+FAST = os.path.join(HERE, "_fastcall" + sysconfig.get_config_var("EXT_SUFFIX"))   # native argument marshalling of the binding
+FAST_SOURCE = os.path.join(HERE, "csrc", "fastcall.c")
 SOURCES = sorted(glob.glob(os.path.join(HERE, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(HERE, "csrc", "*.h"))) + [os.path.join(ROOT, "include", "cadnn.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
@@ -14,14 +17,23 @@ NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", 
 
 
 def stale():
-    if not os.path.exists(LIB):
+    if not os.path.exists(LIB) or not os.path.exists(FAST):
         return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(FAST))
+    return any(os.path.getmtime(f) > t for f in SOURCES + HEADERS + [FAST_SOURCE])
+
+
+def build_fast():
+    """Compile the CPython extension against the library next to it."""
+    tmp = FAST + ".tmp%d" % os.getpid()
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-fPIC", "-shared", "-I" + sysconfig.get_paths()["include"],
+                           "-I" + os.path.join(ROOT, "include"), FAST_SOURCE, "-o", tmp, "-L" + HERE, "-l:" + os.path.basename(LIB),
+                           "-Wl,-rpath,$ORIGIN"])
+    os.replace(tmp, FAST)
 
 
 def build(force=False, verbose=False):
-    """Compile every .cu under csrc/ into libcadnn.so; returns its path."""
+    """Compile every .cu under csrc/ into libcadnn.so, and the binding's extension; returns the library's path."""
     if not force and not stale():
         return LIB
     nvcc = os.environ.get("NVCC", "nvcc")
@@ -43,6 +55,7 @@ def build(force=False, verbose=False):
     tmp = LIB + ".tmp%d" % os.getpid()
     subprocess.check_call([nvcc, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", tmp] + objs)
     os.replace(tmp, LIB)
+    build_fast()
     return LIB
 
 
