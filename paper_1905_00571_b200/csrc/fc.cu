@@ -30,39 +30,59 @@ __device__ __forceinline__ float fc_act(float z, int act)
     return z;
 }
 
+// four stored values and their column indices
+template <typename XT> struct Quad {
+    uint4 v;   // four floats, or four int8 values in the first word
+    uint2 i;
+    __device__ __forceinline__ void load(const FcParams &p, int q)
+    {
+        if (sizeof(XT) == 1) v.x = __ldg(reinterpret_cast<const unsigned *>(p.vals) + q);
+        else v = __ldg(reinterpret_cast<const uint4 *>(p.vals) + q);
+        i = __ldg(reinterpret_cast<const uint2 *>(p.idx) + q);
+    }
+};
+
+// What bounds it at batch 1: the chain row bounds - stored values - gather - reduction.  The bounds and a lane's first two
+// quads of values do not depend on the previous layer and are fetched before the wait for it; later ones are requested two
+// steps ahead of their use.
 template <typename XT, int NB>
 __global__ void __launch_bounds__(256) fc_spmv_kernel(const FcParams p)
 {
     typedef typename std::conditional<sizeof(XT) == 1, int, float>::type AT;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int row = blockIdx.x * kWarpsPerBlock + warp;
+    const int co = row < p.c_pad ? p.perm[row] : -1;
+    // rows are padded to whole quads of entries: a lane fetches four values and four column indices per step
+    int qbeg = 0, qend = 0;
+    if (co >= 0) {
+        qbeg = p.ptr[row] >> 2;
+        qend = p.ptr[row + 1] >> 2;
+    }
+    Quad<XT> first[2];
+    if (qbeg + lane < qend) first[0].load(p, qbeg + lane);
+    if (qbeg + lane + 32 < qend) first[1].load(p, qbeg + lane + 32);
     grid_dep_wait();
     grid_dep_trigger();
-    if (row >= p.c_pad) return;
-    const int co = p.perm[row];
     if (co < 0) return;
-    const int beg = p.ptr[row], end = p.ptr[row + 1];
     const XT *x = reinterpret_cast<const XT *>(p.x);
-    // rows are padded to whole quads of entries: a lane fetches four values and their four column indices per step
-    const int qbeg = beg >> 2, qend = end >> 2;
     for (int b0 = 0; b0 < p.n; b0 += NB) {
         AT acc[NB];
 #pragma unroll
         for (int b = 0; b < NB; ++b) acc[b] = 0;
+        Quad<XT> cur = first[0], next = first[1];
         for (int q = qbeg + lane; q < qend; q += 32) {
+            const Quad<XT> e = cur;
+            cur = next;
+            if (q + 64 < qend) next.load(p, q + 64);
             AT wv[4];
             if (sizeof(XT) == 1) {
-                const int w4 = __ldg(reinterpret_cast<const int *>(p.vals) + q);
-                wv[0] = (AT)(signed char)(w4 & 0xff);
-                wv[1] = (AT)(signed char)((w4 >> 8) & 0xff);
-                wv[2] = (AT)(signed char)((w4 >> 16) & 0xff);
-                wv[3] = (AT)(signed char)((w4 >> 24) & 0xff);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) wv[v] = (AT)(signed char)((e.v.x >> (8 * v)) & 0xff);
             } else {
-                const float4 w4 = __ldg(reinterpret_cast<const float4 *>(p.vals) + q);
-                wv[0] = (AT)w4.x; wv[1] = (AT)w4.y; wv[2] = (AT)w4.z; wv[3] = (AT)w4.w;
+                wv[0] = (AT)__uint_as_float(e.v.x); wv[1] = (AT)__uint_as_float(e.v.y);
+                wv[2] = (AT)__uint_as_float(e.v.z); wv[3] = (AT)__uint_as_float(e.v.w);
             }
-            const uint2 i4 = __ldg(reinterpret_cast<const uint2 *>(p.idx) + q);
-            const int k[4] = {(int)(i4.x & 0xffffu), (int)(i4.x >> 16), (int)(i4.y & 0xffffu), (int)(i4.y >> 16)};
+            const int k[4] = {(int)(e.i.x & 0xffffu), (int)(e.i.x >> 16), (int)(e.i.y & 0xffffu), (int)(e.i.y >> 16)};
 #pragma unroll
             for (int b = 0; b < NB; ++b)
                 if (b0 + b < p.n) {
