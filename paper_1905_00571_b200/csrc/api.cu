@@ -68,6 +68,17 @@ cadnn_status check_epilogue(const cadnn_weights *w, const cadnn_epilogue *ep, La
     return CADNN_OK;
 }
 
+// Layer calls of the tensor-core and small-batch fc kernels are programmatic dependents of whatever their stream runs before:
+// these kernels touch activations, residual, scale, bias and output only behind their wait for it, and their start-up (about
+// a microsecond) overlaps its end.  Not while a stream is being captured: the caller's graph may join branches there.
+bool overlap_start(const cadnn_weights *w, cudaStream_t s)
+{
+    if (!w || !(w->d_tcv || w->s.kind == KK_FC_SPMV)) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) { cudaGetLastError(); return false; }
+    return st == cudaStreamCaptureStatusNone;
+}
+
 }  // namespace
 
 cadnn_status check_layer_call(const cadnn_weights *w, bool has_residual, int act, int out_dtype, int out_c_total, int out_c_off)
@@ -124,7 +135,7 @@ extern "C" {
 cadnn_status cadnn_conv2d(const cadnn_weights *w, const void *x, int n, int h, int wd, void *y,
                           const cadnn_epilogue *ep, void *stream)
 {
-    return conv2d_impl(w, x, n, h, wd, y, ep, false, (cudaStream_t)stream);
+    return conv2d_impl(w, x, n, h, wd, y, ep, overlap_start(w, (cudaStream_t)stream), (cudaStream_t)stream);
 }
 
 cadnn_status cadnn_weights_workspace_bytes(const cadnn_weights *w, int n, int64_t *bytes)

@@ -166,13 +166,11 @@ __device__ __forceinline__ void push_copy(unsigned dst, unsigned src, unsigned b
 // One kernel shape: PX pixels x CH channels per block.  SWAP: the channels are the 128 rows of the tensor-core tile and
 // the pixels its columns (any multiple of 16 up to PX, so that small maps waste little); otherwise the 128 rows are pixels
 // and the columns CH channels.
-template <bool F32, int PX, int CH, bool SWAP, int GROUPS> struct Cfg {
+template <bool F32, int PX, int CH, bool SWAP> struct Cfg {
     static const int kParts = F32 ? 3 : 2;                 // operand tiles of 64-byte rows per stage
     static const int kKB = F32 ? 32 : 128;                 // K values per stage (128 source bytes per pixel)
-    static const int kXBytes = kParts * PX * 64;
     static const int kWBytes = kParts * CH * 64;
-    static const int kStage = kXBytes + kWBytes;
-    static const int kBlocks = PX > 128 || GROUPS > 2 ? 1 : 2;           // per multiprocessor
+    static const int kBlocks = PX > 128 ? 1 : 2;           // per multiprocessor
     static const int kN = SWAP ? PX : CH;
     // Accumulators, kN columns each (kN at most 64: three, by size of the terms; beyond: the large products and the small
     // ones; int8: two that take turns, so that no multiply-add waits for the one before it)
@@ -181,8 +179,8 @@ template <bool F32, int PX, int CH, bool SWAP, int GROUPS> struct Cfg {
     static const int kRow = CH + 4;                        // words per pixel of the exchanged sums (conflict-free 16-byte access)
     // Loader warps work in groups that fill alternate stages, so that one's memory and fence latency hides behind the
     // others'; a thread then holds kRPT 16-byte pieces of its next stage in registers.
-    // (at most as many groups as stages: a group waits for a stage by phase parity, which tells neighbouring phases apart only)
-    static const int kGroups = GROUPS;
+    // (At most as many groups as stages: a group waits for a stage by phase parity, which tells neighbouring phases apart only.)
+    static const int kGroups = 2;
     static const int kGroupThreads = 256 / kGroups;
     static const int kRPT = PX * 8 / kGroupThreads;        // pixels per loader thread, kGroupThreads / 8 apart
 };
@@ -353,10 +351,10 @@ __device__ __forceinline__ void load_channels(const TcvParams &p, int co, float4
     if (p.bias) bi = make_float4(__ldg(p.bias + co), __ldg(p.bias + a), __ldg(p.bias + b), 0.0f);
 }
 
-template <bool F32, int PX, int CH, bool SWAP, int GROUPS, bool VEC>
-__global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP, GROUPS>::kBlocks) tcconv_kernel(const TcvParams p)
+template <bool F32, int PX, int CH, bool SWAP, bool VEC>
+__global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcconv_kernel(const TcvParams p)
 {
-    typedef Cfg<F32, PX, CH, SWAP, GROUPS> C;
+    typedef Cfg<F32, PX, CH, SWAP> C;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const unsigned raw32 = (unsigned)__cvta_generic_to_shared(smem_raw);
     const unsigned base = (raw32 + 1023u) & ~1023u;
@@ -373,13 +371,14 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP, GROUPS>::kBlo
     const int npx = SWAP ? p.npx : PX;                  // pixels of a tile
     const int m0 = mt * npx;
     const unsigned xpart = npx * 64;                    // bytes from one activation part of a stage to the next
+    const unsigned xbytes = C::kParts * xpart, stage = xbytes + C::kWBytes;
 
     const unsigned pxs = slot32 + 16;                   // window starts of the tile's pixels, 8 bytes each
 
     // weights of stage kb: its CH x 64-byte tiles, 64 channels (4 KB) per bulk copy
     const int n64 = (p.c_out + 63) / 64;
     auto copy_weights = [&](int kb, int s) {
-        const unsigned dst = base + s * C::kStage + C::kXBytes, full = bars + s * 8;
+        const unsigned dst = base + s * stage + xbytes, full = bars + s * 8;
         int cnt = 0;
 #pragma unroll
         for (int q = 0; q < CH / 64; ++q) cnt += nt * (CH / 64) + q < n64;
@@ -460,7 +459,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP, GROUPS>::kBlo
         for (int kb = kb0 + grp; kb < kb1; kb += C::kGroups) {
             while (s >= S) { s -= S; ++round; }
             if (round > 0 && alive) alive = mb_wait(bars + (S + s) * 8, (round - 1) & 1u, p.gave_up);
-            const unsigned a = base + s * C::kStage + at;
+            const unsigned a = base + s * stage + at;
 #pragma unroll
             for (int i = 0; i < C::kRPT; ++i) {
                 if (SWAP && r0 + kPS * i >= npx) continue;
@@ -503,7 +502,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP, GROUPS>::kBlo
         for (int kb = kb0; kb < kb1; ++kb) {
             if (!mb_wait(bars + s * 8, round & 1u, p.gave_up)) break;
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            const unsigned xs = base + s * C::kStage, ws = xs + C::kXBytes;
+            const unsigned xs = base + s * stage, ws = xs + xbytes;
             const unsigned a = SWAP ? ws : xs, w = SWAP ? xs : ws;
             if (F32) {
 #pragma unroll
@@ -663,16 +662,14 @@ struct Pick {
 struct SmemPlan {
     int stages, recv_off, bar_off, bytes;
 };
-SmemPlan plan_smem(bool f32, const Pick &k, int nkb, long long blocks)
+SmemPlan plan_smem(bool f32, const Pick &k, int nkb)
 {
     const int PX = k.ch == 64 ? 128 : k.px <= 64 ? 64 : k.px <= 128 ? 128 : 256;
     const bool swap = k.ch == 128;
-    const int groups = swap && PX == 64 && k.split > 1 ? 4 : 2;
-    const int stage = (f32 ? 3 : 2) * 64 * (PX + k.ch), out = k.px * (k.ch + 4) * 4;
-    // two blocks share a multiprocessor unless the shape is too large or a small split grid leaves room for a deeper pipeline
-    const int budget = (PX > 128 || groups > 2 || (k.split > 1 && blocks <= 148) ? 216 : 108) * 1024;
+    const int stage = (f32 ? 3 : 2) * 64 * (k.px + k.ch), out = k.px * (k.ch + 4) * 4;
+    const int budget = (PX > 128 ? 216 : 108) * 1024;   // two blocks share a multiprocessor but for the largest shape
     SmemPlan s;
-    s.stages = std::max(groups, std::min(std::min(4, std::max(groups, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
+    s.stages = std::max(2, std::min(std::min(4, std::max(2, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
     s.recv_off = std::max(s.stages * stage, swap || k.split > 1 ? out : 0);   // the sums are staged over the stages
     s.bar_off = (s.recv_off + (k.split > 1 ? out : 0) + 127) / 128 * 128;
     s.bytes = s.bar_off + 1024 + 128 + PX * 8;
@@ -680,29 +677,34 @@ SmemPlan plan_smem(bool f32, const Pick &k, int nkb, long long blocks)
 }
 
 // Block shape of a layer: the one a time model calls the fastest.  The model is linear in what a block does, with
-// coefficients fitted to 3000 measured launches (193 layers of the workloads at batch 1 to 128, every shape and split):
+// coefficients fitted to 2000 measured shapes (193 layers of the workloads at batch 1 to 128, launched back to back as
+// programmatic dependents):
 //   time = start + P (b2 + n (c2 + d2 px / 64)) + Q (b1 + n (c1 + d1 px / 64))   [microseconds]
 // n = stages per block, P = rounds in which every multiprocessor runs two blocks, Q = rounds with one.  How many clusters
 // of a size run at once is what cudaOccupancyMaxActiveClusters reports for this GPU (a cluster has to fit one GPC).
-// Mean excess of the chosen over the best measured shape: 2 %.
+// Mean excess of the chosen over the best measured shape: 1 %.
 struct Cost {
     float start, b2, c2, d2, b1, c1, d1;
 };
-const Cost kCost[2][6] = {
-    // 128 px x 64 ch, same split, <= 64 px x 128 ch, same split, <= 128 px x 128 ch, same split
-    {{1.48f, 4.67f, 0.0f, 0.429f, 3.30f, 0.0f, 0.264f},      // float
-     {2.48f, 3.69f, 0.0f, 0.480f, 3.05f, 0.0f, 0.265f},
-     {1.40f, 3.54f, 0.332f, 0.351f, 2.83f, 0.401f, 0.090f},
-     {1.38f, 0.0f, 0.0f, 0.0f, 3.52f, 0.353f, 0.188f},
-     {1.15f, 6.30f, 0.323f, 0.456f, 5.05f, 0.539f, 0.158f},
-     {1.81f, 0.0f, 0.0f, 0.0f, 5.19f, 0.320f, 0.306f}},
-    {{2.45f, 3.69f, 0.0f, 0.339f, 2.54f, 0.0f, 0.184f},      // int8
-     {2.54f, 3.10f, 0.0f, 0.382f, 2.63f, 0.0f, 0.213f},
-     {2.21f, 2.75f, 0.206f, 0.431f, 2.04f, 0.265f, 0.130f},
-     {1.17f, 3.11f, 0.480f, 0.0f, 3.12f, 0.229f, 0.343f},
-     {2.36f, 5.39f, 0.055f, 0.424f, 3.61f, 0.125f, 0.214f},
-     {1.61f, 4.20f, 0.0f, 0.704f, 5.05f, 0.0f, 0.303f}}};
-const Cost kCost256[2] = {{0.0f, 0.0f, 0.0f, 0.0f, 9.23f, 0.345f, 0.222f}, {0.0f, 0.0f, 0.0f, 0.0f, 8.37f, 0.157f, 0.220f}};
+const Cost kCost[2][9] = {   // float, int8; 128 px x 64 ch, then up to 32, 64 and 128 px x 128 ch, each unsplit and split; 256 px x 128 ch
+    {{0.352f, 4.72f, 0.0f, 0.427f, 3.63f, 0.0f, 0.257f},
+     {1.82f, 4.04f, 0.0f, 0.401f, 2.66f, 0.0f, 0.276f},
+     {0.0124f, 3.2f, 0.535f, 0.0f, 2.9f, 0.413f, 0.0802f},
+     {0.638f, 3.09f, 0.397f, 0.373f, 2.52f, 0.388f, 0.172f},
+     {0.292f, 4.27f, 0.648f, 0.0f, 3.56f, 0.353f, 0.121f},
+     {1.63f, 4.0f, 0.0f, 0.68f, 2.55f, 0.301f, 0.202f},
+     {0.295f, 5.99f, 0.279f, 0.503f, 5.18f, 0.542f, 0.159f},
+     {1.08f, 0.0f, 0.0f, 0.0f, 5.04f, 0.306f, 0.315f},
+     {0.0f, 0.0f, 0.0f, 0.0f, 8.54f, 0.23f, 0.23f}},
+    {{1.08f, 3.82f, 0.0f, 0.341f, 3.02f, 0.0f, 0.19f},
+     {1.66f, 3.38f, 0.0f, 0.359f, 2.54f, 0.0f, 0.21f},
+     {0.77f, 2.49f, 0.441f, 0.0f, 2.06f, 0.286f, 0.155f},
+     {2.89f, 0.537f, 0.223f, 0.597f, 0.0f, 0.259f, 0.315f},
+     {1.42f, 2.99f, 0.6f, 0.0f, 2.4f, 0.219f, 0.146f},
+     {2.78f, 2.79f, 0.0f, 0.485f, 1.17f, 0.1f, 0.332f},
+     {2.35f, 5.49f, 0.0f, 0.425f, 2.9f, 0.118f, 0.217f},
+     {0.844f, 5.77f, 0.0f, 0.481f, 4.73f, 0.0f, 0.349f},
+     {0.0f, 0.0f, 0.0f, 0.0f, 7.55f, 0.0461f, 0.249f}}};
 
 Pick choose(bool f32, int c_out, long long M, int nkb)
 {
@@ -716,7 +718,7 @@ Pick choose(bool f32, int c_out, long long M, int nkb)
             if (split > 1 && tiles * split > 330) break;      // the grid already fills the chip twice
             static const int cap1[5] = {148, 74, 33, 15, 7}, cap2[5] = {296, 148, 71, 33, 14};
             const Pick k = {px, ch, split};
-            const bool two = plan_smem(f32, k, nkb, tiles * split).bytes <= 113 * 1024;
+            const bool two = plan_smem(f32, k, nkb).bytes <= 113 * 1024;
             long long P = 0, Q = 0;
             if (two) {
                 P = tiles / cap2[log];
@@ -724,7 +726,7 @@ Pick choose(bool f32, int c_out, long long M, int nkb)
                 if (rest > cap1[log]) ++P;
                 else if (rest > 0) Q = 1;
             } else Q = (tiles + cap1[log] - 1) / cap1[log];
-            const Cost &c = px > 128 ? kCost256[!f32] : kCost[!f32][(ch == 64 ? 0 : px <= 64 ? 2 : 4) + (split > 1)];
+            const Cost &c = kCost[!f32][px > 128 ? 8 : (ch == 64 ? 0 : px <= 32 ? 2 : px <= 64 ? 4 : 6) + (split > 1)];
             const double n = ceil_div(nkb, split), u = px / 64.0;
             const double t = c.start + P * (c.b2 + n * (c.c2 + c.d2 * u)) + Q * (c.b1 + n * (c.c1 + c.d1 * u));
             if (t < best_t) { best_t = t; best = k; }
@@ -741,13 +743,13 @@ Pick choose(bool f32, int c_out, long long M, int nkb)
     return best;
 }
 
-template <bool F32, int PX, int CH, bool SWAP, int GROUPS, bool VEC>
+template <bool F32, int PX, int CH, bool SWAP, bool VEC>
 cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
 {
-    auto kern = tcconv_kernel<F32, PX, CH, SWAP, GROUPS, VEC>;
-    typedef Cfg<F32, PX, CH, SWAP, GROUPS> C;
-    const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb, blocks);
-    if (sp.stages < C::kGroups || sp.stages * C::kStage > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
+    auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC>;
+    typedef Cfg<F32, PX, CH, SWAP> C;
+    const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb);
+    if (sp.stages < C::kGroups || sp.stages * C::kParts * 64 * (p.npx + CH) > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
     p.stages = sp.stages;
     p.recv_off = sp.recv_off;
     p.bar_off = sp.bar_off;
@@ -781,11 +783,10 @@ cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
 
 template <bool F32, bool VEC> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
 {
-    if (ch == 64) return launch_one<F32, 128, 64, false, 2, VEC>(p, blocks, pdl, st);
-    if (p.npx <= 64 && p.S > 1) return launch_one<F32, 64, 128, true, 4, VEC>(p, blocks, pdl, st);
-    if (p.npx <= 64) return launch_one<F32, 64, 128, true, 2, VEC>(p, blocks, pdl, st);
-    if (p.npx <= 128) return launch_one<F32, 128, 128, true, 2, VEC>(p, blocks, pdl, st);
-    return launch_one<F32, 256, 128, true, 2, VEC>(p, blocks, pdl, st);
+    if (ch == 64) return launch_one<F32, 128, 64, false, VEC>(p, blocks, pdl, st);
+    if (p.npx <= 64) return launch_one<F32, 64, 128, true, VEC>(p, blocks, pdl, st);
+    if (p.npx <= 128) return launch_one<F32, 128, 128, true, VEC>(p, blocks, pdl, st);
+    return launch_one<F32, 256, 128, true, VEC>(p, blocks, pdl, st);
 }
 
 
