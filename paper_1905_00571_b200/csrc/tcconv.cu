@@ -20,7 +20,7 @@
 //   * one thread issues the tcgen05.mma's; accumulators live in tensor memory;
 //   * the loader warps then finish the tile: a lane per pixel straight from tensor memory, or through
 //     shared memory as [pixel][channel]; with a split reduction every block sends each other block its
-//     pixels' sums with one bulk copy that counts on the receiver's barrier.
+//     pixels' sums from registers, counted on the receiver's barrier.
 // What bounds it: at batch 1 the chain start - first loads - last multiply-adds - exchange (about 5 of the 6
 // to 9 microseconds of a layer); at large batch, for float, shared-memory bandwidth - the six products of a
 // stage read 40 KB of operands per 16 K values where the tensor core needs 384 clocks.
@@ -59,7 +59,7 @@ struct TcvParams {
     int ldc, c_off, vec_ok, vec_sb, vec16;  // vec_ok / vec_sb: output and residual / scale and bias allow 4 channels per access; vec16: int8 output 16
     int kb_base, kb_rem;             // stages per block of a cluster: kb_base, and one more in the first kb_rem blocks
     int Rp;                          // K positions per kernel row: kw * c_in rounded up to 16 bytes
-    FastDiv d_hw, d_wo, d_ci, d_Rp, d_S, d_nt;
+    FastDiv d_hw, d_wo, d_ci, d_Rp, d_S, d_nt, d_rows;
     int *gave_up;
 };
 
@@ -155,8 +155,22 @@ __device__ __forceinline__ uint4 lds128(unsigned addr)
     asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
     return v;
 }
-// copies `bytes` of this block's shared memory to address dst of block `owner` of the cluster; counts on that block's barrier
-__device__ __forceinline__ void push_copy(unsigned dst, unsigned src, unsigned bytes, unsigned bar, int owner)
+// U values to address `addr` (as this block sees it) of block `owner` of the cluster; they count on that block's barrier
+template <int U> __device__ __forceinline__ void send(unsigned addr, unsigned bar, int owner, const unsigned *v)
+{
+    unsigned a, b;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(a) : "r"(addr), "r"(owner));
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(b) : "r"(bar), "r"(owner));
+    if (U == 4)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];\n"
+                     ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(b) : "memory");
+    else if (U == 2)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];\n" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(b) : "memory");
+    else asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];\n" ::"r"(a), "r"(v[0]), "r"(b) : "memory");
+}
+
+// copies `bytes` of this block's shared memory to address dst of block `owner`; counts on that block's barrier
+__device__ __forceinline__ void send_bulk(unsigned dst, unsigned src, unsigned bytes, unsigned bar, int owner)
 {
     asm volatile("{\n.reg .b32 a, b;\nmapa.shared::cluster.u32 a, %0, %4;\nmapa.shared::cluster.u32 b, %3, %4;\n"
                  "cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [a], [%1], %2, [b];\n}\n"
@@ -170,7 +184,8 @@ template <bool F32, int PX, int CH, bool SWAP> struct Cfg {
     static const int kParts = F32 ? 3 : 2;                 // operand tiles of 64-byte rows per stage
     static const int kKB = F32 ? 32 : 128;                 // K values per stage (128 source bytes per pixel)
     static const int kWBytes = kParts * CH * 64;
-    static const int kBlocks = PX > 128 ? 1 : 2;           // per multiprocessor
+    // blocks per multiprocessor the registers, tensor memory and shared memory are cut for
+    static const int kBlocks = PX > 128 ? 1 : 2;
     static const int kN = SWAP ? PX : CH;
     // Accumulators, kN columns each (kN at most 64: three, by size of the terms; beyond: the large products and the small
     // ones; int8: two that take turns, so that no multiply-add waits for the one before it)
@@ -351,6 +366,80 @@ __device__ __forceinline__ void load_channels(const TcvParams &p, int co, float4
     if (p.bias) bi = make_float4(__ldg(p.bias + co), __ldg(p.bias + a), __ldg(p.bias + b), 0.0f);
 }
 
+// Epilogue of channel ch for U consecutive pixels from m on: sums t, residuals r
+template <bool F32, int U>
+__device__ __forceinline__ void finish_column(const TcvParams &p, int m, int ch, const unsigned (&t)[U], const unsigned (&r)[U], float sc, float bi)
+{
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+        if (m + i >= p.M) break;
+        const size_t oi = (size_t)(m + i) * p.ldc + p.c_off + ch;
+        if (F32) reinterpret_cast<float *>(p.y)[oi] = finish_f(p, t[i], sc, bi, __uint_as_float(r[i]));
+        else if (p.out_dtype == CADNN_S8) reinterpret_cast<signed char *>(p.y)[oi] = (signed char)finish_q(p, (int)t[i], sc, bi, (int)r[i]);
+        else
+            reinterpret_cast<unsigned *>(p.y)[oi] = p.out_dtype == CADNN_S32 ? t[i]
+                : __float_as_uint(requant_f32((int)t[i], sc, bi, p.act, p.residual != nullptr, (int)r[i], p.res_scale));
+    }
+}
+template <bool F32, int U> __device__ __forceinline__ void load_column_residual(const TcvParams &p, int m, int ch, unsigned (&r)[U])
+{
+#pragma unroll
+    for (int i = 0; i < U; ++i) {
+        r[i] = 0;
+        if (!p.residual || m + i >= p.M) continue;
+        const size_t ri = (size_t)(m + i) * p.c_out + ch;
+        if (F32) r[i] = __float_as_uint(ld_act(reinterpret_cast<const float *>(p.residual) + ri));
+        else r[i] = (unsigned)(int)ld_act(reinterpret_cast<const signed char *>(p.residual) + ri);
+    }
+}
+// Split tile whose rows are channels: a thread takes channel ch (of the tile) and every second group of U pixels of this
+// block's share.  Partial sums lie as [sender][group][channel][U], so that loads and stores of a warp are contiguous.
+template <bool F32, int U>
+__device__ __forceinline__ void finish_split_columns(const TcvParams &p, unsigned at, int rows, int m0, int co, int ch, int first, unsigned bar)
+{
+    const int groups = rows / U;
+    const bool mine = co < p.c_out;
+    float sc = 1.0f, bi = 0.0f;
+    unsigned r[U];
+    if (mine) {
+        if (p.scale) sc = __ldg(p.scale + co);
+        if (p.bias) bi = __ldg(p.bias + co);
+        if (first < groups) load_column_residual<F32, U>(p, m0 + first * U, co, r);
+    }
+    mb_wait(bar, 0u, p.gave_up);
+    if (!mine) return;
+#pragma unroll 1
+    for (int g = first; g < groups; g += 2) {
+        unsigned t[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) t[i] = 0;
+        const unsigned from = at + (g * 128 + ch) * (U * 4);
+#pragma unroll 4
+        for (int q = 0; q < p.S; ++q) {
+            unsigned v[4];
+            const unsigned a = from + q * (rows * 128 * 4);
+            if (U == 4) {
+                const uint4 w = lds128(a);
+                v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+            } else if (U == 2) asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];\n" : "=r"(v[0]), "=r"(v[1]) : "r"(a) : "memory");
+            else asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(v[0]) : "r"(a) : "memory");
+#pragma unroll
+            for (int i = 0; i < U; ++i) t[i] = F32 ? __float_as_uint(__uint_as_float(t[i]) + __uint_as_float(v[i])) : t[i] + v[i];
+        }
+        finish_column<F32, U>(p, m0 + g * U, co, t, r, sc, bi);
+        if (g + 2 < groups) load_column_residual<F32, U>(p, m0 + (g + 2) * U, co, r);
+    }
+}
+template <int U>
+__device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, unsigned bar, int rank, int rows, int j, int ch, const unsigned (&v)[16])
+{
+#pragma unroll
+    for (int t = 0; t < 16; t += U) {
+        const int owner = (int)fdiv((unsigned)(j + t), p.d_rows), row = (j + t) - owner * rows;
+        send<U>(at + ((rank * (rows / U) + row / U) * 128 + ch) * (U * 4), bar, owner, v + t);
+    }
+}
+
 template <bool F32, int PX, int CH, bool SWAP, bool VEC>
 __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcconv_kernel(const TcvParams p)
 {
@@ -404,7 +493,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
             asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             // partial sums of this block's pixels from every block of the cluster, itself included
-            if (p.S > 1) mb_expect_tx(recv, (unsigned)(npx * C::kRow * 4));
+            if (p.S > 1) mb_expect_tx(recv, (unsigned)(npx * (F32 ? CH : C::kRow) * 4));
         }
     } else if (warp == kLoadWarps + 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(slot32), "r"((unsigned)C::kCols) : "memory");
@@ -550,7 +639,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
     const bool mine = warp < kLoadWarps && co < p.c_out;
     float4 sc = make_float4(1, 1, 1, 1), bi = make_float4(0, 0, 0, 0);
     uint4 res = make_uint4(0, 0, 0, 0);
-    if (mine && (SWAP || p.S > 1)) {
+    if (mine && (SWAP ? !F32 || p.S == 1 : p.S > 1)) {
         // of the row this thread finishes first; on their way while the last multiply-adds run
         load_channels(p, co, sc, bi);
         if (p.residual && r1 < rows && m0 + lo + r1 < p.M) res = load_residual<F32>(p, m0 + lo + r1, co);
@@ -579,7 +668,17 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
             } else asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
             for (int t = 0; t < 16; ++t) v[t] = F32 ? __float_as_uint(__uint_as_float(v[t]) + __uint_as_float(u[t])) : v[t] + u[t];
-            if (SWAP || p.S > 1) {   // to shared memory as [pixel][channel] (over the stages: all of them have been read)
+            if (F32 && p.S > 1) {   // each pixel's sums to the block of the cluster that finishes it
+                if (SWAP) {
+                    if (rows % 4 == 0) send_columns<4>(p, base + p.recv_off, recv, rank, rows, j, q * 32 + lane, v);
+                    else if (rows % 2 == 0) send_columns<2>(p, base + p.recv_off, recv, rank, rows, j, q * 32 + lane, v);
+                    else send_columns<1>(p, base + p.recv_off, recv, rank, rows, j, q * 32 + lane, v);
+                } else {
+                    const int px = q * 32 + lane, owner = (int)fdiv((unsigned)px, p.d_rows), row = rank * rows + px - owner * rows;
+#pragma unroll
+                    for (int t = 0; t < 16; t += 4) send<4>(base + p.recv_off + (row * C::kRow + j + t) * 4, recv, owner, v + t);
+                }
+            } else if (SWAP || p.S > 1) {   // to shared memory as [pixel][channel] (over the stages: all of them have been read)
                 if (SWAP) {
                     const unsigned at = base + (j * C::kRow + q * 32 + lane) * 4;
 #pragma unroll
@@ -607,7 +706,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-        if (p.S > 1) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
+        if (!F32 && p.S > 1) asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
     }
     __syncthreads();
     if (warp == kLoadWarps + 1) {
@@ -615,10 +714,22 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((unsigned)C::kCols) : "memory");
     }
     if (!SWAP && p.S == 1) return;
-    // split reduction: each block's sums of a pixel go to the block of the cluster that finishes the pixel
-    const unsigned slice = rows * C::kRow * 4;
-    if (p.S > 1) {
-        if (tid < p.S) push_copy(base + p.recv_off + rank * slice, base + tid * slice, slice, recv, tid);
+    const unsigned slice = rows * C::kRow * 4;   // partial sums of one sender (as [pixel][channel])
+    if (F32) {
+        if (warp >= kLoadWarps) return;
+        if (SWAP && p.S > 1) {
+            const int ch = tid & 127;
+            const unsigned at = base + p.recv_off;
+            if (rows % 4 == 0) finish_split_columns<F32, 4>(p, at, rows, m0 + lo, nt * CH + ch, ch, tid >> 7, recv);
+            else if (rows % 2 == 0) finish_split_columns<F32, 2>(p, at, rows, m0 + lo, nt * CH + ch, ch, tid >> 7, recv);
+            else finish_split_columns<F32, 1>(p, at, rows, m0 + lo, nt * CH + ch, ch, tid >> 7, recv);
+            return;
+        }
+        if (p.S > 1) mb_wait(recv, 0u, p.gave_up);
+    } else if (p.S > 1) {
+        // Int8 layers exchange through staged tiles and bulk copies: packed stores need 4 channels in a thread, and the register
+        // route's code costs them a third resident block per multiprocessor (int8 ResNet-50, batch 8: 421 against 451 us).
+        if (tid < p.S) send_bulk(base + p.recv_off + rank * slice, base + tid * slice, slice, recv, tid);
         __syncwarp();
         if (warp < kLoadWarps) mb_wait(recv, 0u, p.gave_up);
         __syncwarp();
@@ -648,8 +759,10 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
             finish4<F32>(p, (size_t)m * p.ldc + p.c_off + co, p.c_out - co, t, r, sc, bi);
         }
     }
-    __syncwarp();
-    if (p.S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    if (!F32 && p.S > 1) {
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    }
 }
 
 int ceil_div(int a, int b) { return (a + b - 1) / b; }
@@ -670,7 +783,8 @@ SmemPlan plan_smem(bool f32, const Pick &k, int nkb)
     const int budget = (PX > 128 ? 216 : 108) * 1024;   // two blocks share a multiprocessor but for the largest shape
     SmemPlan s;
     s.stages = std::max(2, std::min(std::min(4, std::max(2, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
-    s.recv_off = std::max(s.stages * stage, swap || k.split > 1 ? out : 0);   // the sums are staged over the stages
+    // sums staged over the stages: unsplit tiles whose rows are channels, and int8 split tiles
+    s.recv_off = std::max(s.stages * stage, (swap && k.split == 1) || (!f32 && k.split > 1) ? out : 0);
     s.bar_off = (s.recv_off + (k.split > 1 ? out : 0) + 127) / 128 * 128;
     s.bytes = s.bar_off + 1024 + 128 + PX * 8;
     return s;
@@ -898,7 +1012,7 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     p.S = pick.px > 128 ? 1 : std::min(pick.split, 16);
     while (p.S > 1 && (p.npx % p.S || p.S > p.nkb)) --p.S;
     p.kb_base = p.nkb / p.S; p.kb_rem = p.nkb % p.S;
-    p.d_S = make_fastdiv(p.S); p.d_nt = make_fastdiv(p.n_nt);
+    p.d_S = make_fastdiv(p.S); p.d_nt = make_fastdiv(p.n_nt); p.d_rows = make_fastdiv(p.npx / p.S);
     const long long blocks = (M + p.npx - 1) / p.npx * p.n_nt * p.S;
     if (blocks > 2147483647ll) return CADNN_E_UNSUPPORTED;
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0;
