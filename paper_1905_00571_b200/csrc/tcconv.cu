@@ -638,11 +638,21 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
     const int col = (tid % kVec) * 4, r1 = tid / kVec, co = nt * CH + col;
     const bool mine = warp < kLoadWarps && co < p.c_out;
     float4 sc = make_float4(1, 1, 1, 1), bi = make_float4(0, 0, 0, 0);
-    uint4 res = make_uint4(0, 0, 0, 0);
+    // residuals of the next kAhead rows: a tile with few stages is bound by how many of these loads are in flight
+    const int kAhead = F32 ? 4 : 1;   // (int8: 4 bytes a load, and registers that keep a third block resident count more)
+    uint4 res[kAhead];
+    auto load_rows = [&](int row) {
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            const int m = m0 + lo + row + i * kStep;
+            res[i] = make_uint4(0, 0, 0, 0);
+            if (p.residual && row + i * kStep < rows && m < p.M) res[i] = load_residual<F32>(p, m, co);
+        }
+    };
     if (mine && (SWAP ? !F32 || p.S == 1 : p.S > 1)) {
-        // of the row this thread finishes first; on their way while the last multiply-adds run
+        // of the rows this thread finishes first; on their way while the last multiply-adds run
         load_channels(p, co, sc, bi);
-        if (p.residual && r1 < rows && m0 + lo + r1 < p.M) res = load_residual<F32>(p, m0 + lo + r1, co);
+        load_rows(r1);
     }
     __syncwarp();
     if (p.S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");   // every block has initialised its barriers
@@ -695,10 +705,10 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
                     const int c4 = nt * CH + j + t;
                     if (c4 >= p.c_out) break;
                     load_channels(p, c4, sc, bi);
-                    if (p.residual) res = load_residual<F32>(p, mrow, c4);
+                    if (p.residual) res[0] = load_residual<F32>(p, mrow, c4);
                     const uint4 t4 = make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]);
-                    if (!F32 && p.vec16) q8[t / 4] = finish_q4(p, t4, res.x, sc, bi);
-                    else finish4<F32>(p, (size_t)mrow * p.ldc + p.c_off + c4, p.c_out - c4, t4, res, sc, bi);
+                    if (!F32 && p.vec16) q8[t / 4] = finish_q4(p, t4, res[0].x, sc, bi);
+                    else finish4<F32>(p, (size_t)mrow * p.ldc + p.c_off + c4, p.c_out - c4, t4, res[0], sc, bi);
                 }
                 if (!F32 && p.vec16 && nt * CH + j < p.c_out)
                     *reinterpret_cast<uint4 *>(reinterpret_cast<signed char *>(p.y) + (size_t)mrow * p.ldc + p.c_off + nt * CH + j) =
@@ -739,24 +749,31 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
     if (mine) {
         unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (r1 * C::kRow + col) * 4;
 #pragma unroll 1
-        for (int row = r1, m = m0 + lo + r1; row < rows && m < p.M; row += kStep, m += kStep) {
-            uint4 t = lds128(at);
+        for (int row = r1; row < rows; row += kAhead * kStep) {
+            uint4 r[kAhead];
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) r[i] = res[i];
+            if (row + kAhead * kStep < rows) load_rows(row + kAhead * kStep);
+#pragma unroll
+            for (int i = 0; i < kAhead; ++i) {
+                const int m = m0 + lo + row + i * kStep;
+                if (row + i * kStep >= rows || m >= p.M) break;
+                uint4 t = lds128(at);
 #pragma unroll 4
-            for (int q = 1; q < p.S; ++q) {
-                const uint4 u = lds128(at + q * slice);
-                if (F32) {
-                    t.x = __float_as_uint(__uint_as_float(t.x) + __uint_as_float(u.x));
-                    t.y = __float_as_uint(__uint_as_float(t.y) + __uint_as_float(u.y));
-                    t.z = __float_as_uint(__uint_as_float(t.z) + __uint_as_float(u.z));
-                    t.w = __float_as_uint(__uint_as_float(t.w) + __uint_as_float(u.w));
-                } else {
-                    t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+                for (int q = 1; q < p.S; ++q) {
+                    const uint4 u = lds128(at + q * slice);
+                    if (F32) {
+                        t.x = __float_as_uint(__uint_as_float(t.x) + __uint_as_float(u.x));
+                        t.y = __float_as_uint(__uint_as_float(t.y) + __uint_as_float(u.y));
+                        t.z = __float_as_uint(__uint_as_float(t.z) + __uint_as_float(u.z));
+                        t.w = __float_as_uint(__uint_as_float(t.w) + __uint_as_float(u.w));
+                    } else {
+                        t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+                    }
                 }
+                at += kStep * C::kRow * 4;
+                finish4<F32>(p, (size_t)m * p.ldc + p.c_off + co, p.c_out - co, t, r[i], sc, bi);
             }
-            at += kStep * C::kRow * 4;
-            const uint4 r = res;
-            if (p.residual && row + kStep < rows && m + kStep < p.M) res = load_residual<F32>(p, m + kStep, co);
-            finish4<F32>(p, (size_t)m * p.ldc + p.c_off + co, p.c_out - co, t, r, sc, bi);
         }
     }
     if (!F32 && p.S > 1) {
