@@ -267,6 +267,8 @@ __global__ void __launch_bounds__(128) block_tc_kernel(const TcParams p, const _
         if (have) {
             tc_ld32(tmem + ((unsigned)(warp * 32) << 16) + half * 32, v);
             asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+#pragma unroll
+            for (int j = 0; j < 32; ++j) asm volatile("" : "+r"(v[j]));   // the loaded registers are not to be used ahead of the wait
         } else {
 #pragma unroll
             for (int j = 0; j < 32; ++j) v[j] = 0;

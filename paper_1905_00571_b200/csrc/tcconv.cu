@@ -40,8 +40,6 @@
 
 namespace {
 
-const int kLoadWarps = 8;
-const int kThreads = (kLoadWarps + 2) * 32;   // + the weight-copy warp and the multiply-add warp
 const int kSpin = 1 << 22;
 
 struct TcvParams {
@@ -119,6 +117,14 @@ __device__ __forceinline__ void tmem_ld16(unsigned taddr, unsigned (&v)[16])
                    "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                  : "r"(taddr) : "memory");
 }
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory"); }
+// Keeps uses of the registers a tcgen05.ld fills behind the wait before this call: nothing else tells the compiler that they
+// are not valid earlier.
+__device__ __forceinline__ void tmem_arrived(unsigned (&v)[16])
+{
+    asm volatile("" : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]),
+                      "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]));
+}
 __device__ __forceinline__ unsigned pack_bf16(float lo, float hi)
 {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -192,11 +198,13 @@ template <bool F32, int PX, int CH, bool SWAP> struct Cfg {
     static const int kAcc = F32 && kN <= 64 ? 3 : 2;
     static const int kCols = kAcc * kN <= 128 ? 128 : kAcc * kN <= 256 ? 256 : 512;
     static const int kRow = CH + 4;                        // words per pixel of the exchanged sums (conflict-free 16-byte access)
+    static const int kLoadWarps = PX > 128 ? 16 : 8;
+    static const int kThreads = (kLoadWarps + 2) * 32;     // + the weight-copy warp and the multiply-add warp
     // Loader warps work in groups that fill alternate stages, so that one's memory and fence latency hides behind the
     // others'; a thread then holds kRPT 16-byte pieces of its next stage in registers.
     // (At most as many groups as stages: a group waits for a stage by phase parity, which tells neighbouring phases apart only.)
     static const int kGroups = 2;
-    static const int kGroupThreads = 256 / kGroups;
+    static const int kGroupThreads = kLoadWarps * 32 / kGroups;
     static const int kRPT = PX * 8 / kGroupThreads;        // pixels per loader thread, kGroupThreads / 8 apart
 };
 
@@ -441,9 +449,10 @@ __device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, un
 }
 
 template <bool F32, int PX, int CH, bool SWAP, bool VEC>
-__global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcconv_kernel(const TcvParams p)
+__global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP>::kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcconv_kernel(const TcvParams p)
 {
     typedef Cfg<F32, PX, CH, SWAP> C;
+    const int kLoadWarps = C::kLoadWarps;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const unsigned raw32 = (unsigned)__cvta_generic_to_shared(smem_raw);
     const unsigned base = (raw32 + 1023u) & ~1023u;
@@ -641,6 +650,8 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
     // residuals of the next kAhead rows: a tile with few stages is bound by how many of these loads are in flight
     const int kAhead = F32 ? 4 : 1;   // (int8: 4 bytes a load, and registers that keep a third block resident count more)
     uint4 res[kAhead];
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) res[i] = make_uint4(0, 0, 0, 0);
     auto load_rows = [&](int row) {
 #pragma unroll
         for (int i = 0; i < kAhead; ++i) {
@@ -657,7 +668,7 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
     __syncwarp();
     if (p.S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");   // every block has initialised its barriers
     if (warp < kLoadWarps) {
-        // a warp can read the 32 rows 32 q ..; the two warps with the same q take turns on groups of 16 columns
+        // a warp can read the 32 rows 32 q ..; the warps with the same q take turns on groups of 16 columns
         const int q = warp & 3, N = SWAP ? npx : CH;
         const unsigned from = tmem + ((unsigned)(q * 32) << 16);
         const int mrow = m0 + q * 32 + lane;   // (rows are pixels)
@@ -665,17 +676,23 @@ __global__ void __launch_bounds__(kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcc
         __syncwarp();
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
 #pragma unroll 1
-        for (int j = (warp >> 2) * 16; j < N; j += 32) {
+        for (int j = (warp >> 2) * 16; j < N; j += kLoadWarps * 4) {
             unsigned v[16], u[16];
             tmem_ld16(from + j, v);
             tmem_ld16(from + N + j, u);
             if (F32 && C::kAcc == 3) {
                 unsigned t3[16];
                 tmem_ld16(from + 2 * N + j, t3);
-                asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+                tmem_wait();
+                tmem_arrived(u);
+                tmem_arrived(t3);
 #pragma unroll
                 for (int t = 0; t < 16; ++t) u[t] = __float_as_uint(__uint_as_float(u[t]) + __uint_as_float(t3[t]));
-            } else asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
+            } else {
+                tmem_wait();
+                tmem_arrived(u);
+            }
+            tmem_arrived(v);
 #pragma unroll
             for (int t = 0; t < 16; ++t) v[t] = F32 ? __float_as_uint(__uint_as_float(v[t]) + __uint_as_float(u[t])) : v[t] + u[t];
             if (F32 && p.S > 1) {   // each pixel's sums to the block of the cluster that finishes it
@@ -891,7 +908,7 @@ cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
     if (p.S > 8) CADNN_CUDA_TRY(cudaFuncSetAttribute((const void *)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)blocks, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.blockDim = dim3(C::kThreads, 1, 1);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[2];

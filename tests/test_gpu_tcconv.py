@@ -49,6 +49,25 @@ def test_float_layers(shape, layer, monkeypatch):
     assert B.cadnn_device_status()["copy_timeouts"] == 0
 
 
+@pytest.mark.parametrize("shape", SHAPES)
+def test_all_terms_of_the_float_products_arrive(shape, monkeypatch):
+    """The smallest of the split products weigh 2^-18: a result that misses them is off by 5e-6 (2-norm), one with all of them
+    by about 1e-7."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(45)
+    layer = (2, 12, 13, 64, 130, 3, 1, 1)
+    n, h, wd, c_in, c_out, k, stride, pad = layer
+    x = gen.relu_normal_input(g, (n, h, wd, c_in))
+    w = gen.he_weights(g, c_out, k, k, c_in)
+    mask = gen.random_mask(g, w.shape, 0.2)
+    want = ref.conv2d_f32(x, w, mask, stride, pad).astype(np.float64)
+    wh = _pack(B, monkeypatch, shape, "f32", layer, w, mask)
+    y = torch.zeros(want.shape, device=DEV)
+    B.cadnn_conv2d(wh, torch.from_numpy(x).to(DEV), y)
+    torch.cuda.synchronize()
+    assert np.linalg.norm(y.cpu().numpy() - want) < 5e-7 * np.linalg.norm(want)
+
+
 @pytest.mark.parametrize("layer", LAYERS)
 @pytest.mark.parametrize("shape", SHAPES)
 def test_int8_layers_bit_exact(shape, layer, monkeypatch):
