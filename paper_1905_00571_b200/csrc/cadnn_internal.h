@@ -146,8 +146,6 @@ struct cadnn_weights {
     const int32_t *d_tc_grp_ptr = nullptr;
 
     // dense tensor-core image (tcconv.cu): built when the layer's density makes that route the faster one
-    bool has_tcv = false;
-    std::vector<unsigned char> tcv_img;   // host copy, dropped after the upload
     void *d_tcv = nullptr;
     int tcv_force[3] = {0, 0, 0};          // CADNN_TCV at pack time: pixels, channels, split (0 = choose)
     mutable std::atomic<uint64_t> tcv_pick{0};   // block shape of the last batch size (tcconv.cu)
@@ -247,8 +245,7 @@ cadnn_status block_tc_upload(cadnn_weights *h);
 cadnn_status launch_block_tc(const cadnn_weights *w, const void *x, int n, int *acc, void *y, const LaunchEpilogue *le, cudaStream_t st);
 // dense tensor-core route (tcconv.cu)
 bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz);
-void tcv_build(cadnn_weights *h, const float *f, const int8_t *q, const uint8_t *mask);
-cadnn_status tcv_upload(cadnn_weights *h);
+cadnn_status tcv_build(cadnn_weights *h);
 bool tcv_fits(const cadnn_weights *w, int n);   // the batch is within the kernel's index ranges
 cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep, cudaStream_t st);
 cadnn_status copy_timeout_word(int **word);   // device address of the copy give-up counter

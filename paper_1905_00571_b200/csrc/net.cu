@@ -8,6 +8,7 @@
 #include <new>
 #include <vector>
 #include <cstdio>
+#include <cstring>
 #include "cadnn_internal.h"
 
 struct SlotInfo {
@@ -45,6 +46,8 @@ struct cadnn_net {
     // device staging for cadnn_forward_host
     void *stage_x = nullptr, *stage_y = nullptr;
     int64_t in_bytes = 0, out_bytes = 0;
+    // small outputs: pinned host memory into which the last kernel of a host forward writes the output, then the give-up counter
+    int *deliver_host = nullptr;
     // int32 sums of block-structured layers (tensor-core blocks), shared by all such ops of the net
     void *tc_ws = nullptr;
     int64_t tc_ws_bytes = 0;
@@ -156,7 +159,8 @@ cadnn_status run_all(cadnn_net *net, const void *x, void *y, cudaStream_t st, bo
 // issued on a second stream, forked from and joined back to the captured one with events, so
 // that in the graph it is a parallel branch.  At batch 1 no single layer fills the device, so
 // the branch runs beside the block's first convs instead of in front of them.
-cadnn_status run_all_forked(cadnn_net *net, const void *x, void *y, cudaStream_t st, cudaStream_t side, bool pdl)
+// *chain: the last launch on st was an op with nothing to wait for behind it.
+cadnn_status run_all_forked(cadnn_net *net, const void *x, void *y, cudaStream_t st, cudaStream_t side, bool pdl, bool *chain)
 {
     const int n_ops = (int)net->ops.size();
     std::vector<cudaEvent_t> join(n_ops, nullptr);   // recorded on the side stream after op i
@@ -206,7 +210,11 @@ cadnn_status run_all_forked(cadnn_net *net, const void *x, void *y, cudaStream_t
     }
     // branches nobody read still have to end inside the capture
     for (int j = 0; j < n_ops; ++j)
-        if (join[j] && cudaStreamWaitEvent(st, join[j], 0) != cudaSuccess && rs == CADNN_OK) rs = CADNN_E_CUDA;
+        if (join[j]) {
+            first = true;
+            if (cudaStreamWaitEvent(st, join[j], 0) != cudaSuccess && rs == CADNN_OK) rs = CADNN_E_CUDA;
+        }
+    *chain = !first;
     for (cudaEvent_t e : events) cudaEventDestroy(e);
     if (rs == CADNN_E_CUDA) cadnn_note_cuda(cudaGetLastError());
     return rs;
@@ -355,9 +363,32 @@ void drop_graph(cadnn_net::GraphCache &gc)
     gc.graph = nullptr;
 }
 
+// Output and give-up counter to pinned host memory: one small kernel behind the last layer in place of two copies, each of
+// which costs the tail of a host forward several microseconds (for outputs of up to kDeliverBytes).
+const int64_t kDeliverBytes = 64 * 1024;
+__global__ void deliver_kernel(const int *y, int words, const int *gave_up, int *host)
+{
+    grid_dep_wait();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < words; i += gridDim.x * blockDim.x) host[i] = y[i];
+    if (blockIdx.x == 0 && threadIdx.x == 0) host[words] = *gave_up;
+}
+cadnn_status launch_deliver(cadnn_net *net, bool pdl, cudaStream_t st)
+{
+    int *word = nullptr;
+    cadnn_status s = copy_timeout_word(&word);
+    if (s != CADNN_OK) return s;
+    const int words = (int)((net->out_bytes + 3) / 4);
+    return launch_kernel(deliver_kernel, (words + 1023) / 1024, 256, 0, pdl, st, (const int *)net->stage_y, words, (const int *)word, net->deliver_host);
+}
+
+// slot 1: a host forward (with deliver_host, the output is delivered behind the last layer)
 cadnn_status forward_impl(cadnn_net *net, const void *x, void *y, int use_graph, cudaStream_t st, int slot)
 {
-    if (!use_graph) return run_all(net, x, y, st, net->use_pdl);
+    const bool deliver = slot == 1 && net->deliver_host;
+    if (!use_graph) {
+        cadnn_status s = run_all(net, x, y, st, net->use_pdl);
+        return s == CADNN_OK && deliver ? launch_deliver(net, net->use_pdl, st) : s;
+    }
     cadnn_net::GraphCache &gc = net->cache[slot];
     if (!gc.exec || gc.x != x || gc.y != y) {
         drop_graph(gc);
@@ -379,6 +410,7 @@ cadnn_status forward_impl(cadnn_net *net, const void *x, void *y, int use_graph,
         if (net->fork_branches)
             for (; n_sides < kSides; ++n_sides)
                 if (cudaStreamCreateWithFlags(&sides[n_sides], cudaStreamNonBlocking) != cudaSuccess) { cudaGetLastError(); break; }
+        bool chain = false;
         if (n_sides == 0) s = run_all(net, x, y, cap, net->pdl_graph);
         else {
             // networks with concatenations have branches of several ops (measured on Inception-V3, batch 1: 0.78 ms
@@ -388,9 +420,10 @@ cadnn_status forward_impl(cadnn_net *net, const void *x, void *y, int use_graph,
             for (const cadnn_op &op : net->ops) concat = concat || op.dst_c_total > 0;
             const char *force = getenv("CADNN_GRAPH_LANES");   // "1": general scheduler always, "0": never
             if (force) concat = atoi(force) != 0;
-            if (net->persist || !concat) s = run_all_forked(net, x, y, cap, sides[0], net->pdl_graph);
+            if (net->persist || !concat) s = run_all_forked(net, x, y, cap, sides[0], net->pdl_graph, &chain);
             else s = run_all_dag(net, x, y, cap, sides, n_sides, net->pdl_graph);
         }
+        if (s == CADNN_OK && deliver) s = launch_deliver(net, net->pdl_graph && chain, cap);
         e = cudaStreamEndCapture(cap, &gc.graph);
         for (int k = 0; k < n_sides; ++k) cudaStreamDestroy(sides[k]);
         if (own) cudaStreamDestroy(cap);
@@ -707,13 +740,25 @@ cadnn_status cadnn_forward_host(cadnn_net *net, const void *x_host, void *y_host
             return e == cudaErrorMemoryAllocation ? CADNN_E_ALLOC : CADNN_E_CUDA;
         }
     }
+    if (!net->deliver_host && net->out_bytes <= kDeliverBytes && !net->persist &&
+        cudaHostAlloc((void **)&net->deliver_host, (size_t)net->out_bytes + 16, cudaHostAllocDefault) != cudaSuccess) {
+        cudaGetLastError();
+        net->deliver_host = nullptr;
+        return CADNN_E_ALLOC;
+    }
     CADNN_CUDA_TRY(cudaMemcpyAsync(net->stage_x, x_host, (size_t)net->in_bytes, cudaMemcpyHostToDevice, st));
     cadnn_status s = forward_impl(net, net->stage_x, net->stage_y, use_graph, st, 1);
     if (s != CADNN_OK) return s;
-    CADNN_CUDA_TRY(cudaMemcpyAsync(y_host, net->stage_y, (size_t)net->out_bytes, cudaMemcpyDeviceToHost, st));
-    s = queue_status_read(net, st);
-    if (s != CADNN_OK) return s;
+    if (!net->deliver_host) {
+        CADNN_CUDA_TRY(cudaMemcpyAsync(y_host, net->stage_y, (size_t)net->out_bytes, cudaMemcpyDeviceToHost, st));
+        s = queue_status_read(net, st);
+        if (s != CADNN_OK) return s;
+    }
     CADNN_CUDA_TRY(cudaStreamSynchronize(st));
+    if (net->deliver_host) {
+        memcpy(y_host, net->deliver_host, (size_t)net->out_bytes);
+        net->status_host[0] = net->deliver_host[(net->out_bytes + 3) / 4];
+    }
     return status_moved(net) ? CADNN_E_DEVICE_STATUS : CADNN_OK;
 }
 
@@ -851,6 +896,7 @@ void cadnn_net_free(cadnn_net *net)
     if (net->flush) cudaFree(net->flush);
     if (net->tc_ws) cudaFree(net->tc_ws);
     if (net->status_host) cudaFreeHost(net->status_host);
+    if (net->deliver_host) cudaFreeHost(net->deliver_host);
     persist_free(net->persist);
     delete net;
 }

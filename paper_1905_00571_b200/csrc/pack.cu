@@ -1349,7 +1349,8 @@ cadnn_status pack_dense(cadnn_weights *h, const Src &src, int kind)
     return CADNN_OK;
 }
 
-cadnn_status pack_common(const cadnn_layer_desc *desc, const Src &src, cadnn_weights **out)
+// dense_route: the handle may get the dense tensor-core image (the planar-only form of a stride-2 layer has no use for one)
+cadnn_status pack_common(const cadnn_layer_desc *desc, const Src &src, cadnn_weights **out, bool dense_route = true)
 {
     if (!desc || !out || (!src.f && !src.q)) return CADNN_E_ARG;
     cadnn_layer_desc dn = *desc;
@@ -1416,18 +1417,9 @@ cadnn_status pack_common(const cadnn_layer_desc *desc, const Src &src, cadnn_wei
         else st = pack_sconv(h, src);
         if (st == CADNN_OK) st = upload(h);
         if (st == CADNN_OK) st = block_tc_upload(h);
-        if (st == CADNN_OK && (h->s.kind == KK_SCONV_SPATIAL || h->s.kind == KK_SCONV_LINEAR || h->s.kind == KK_DENSE_SMALLC) && d.fmt == CADNN_FMT_AUTO &&
-            !getenv("CADNN_NO_TCV") && !getenv("CADNN_SCHEDULE") && tcv_pays(d, h->nnz)) {
-            const int8_t *qp = src.q;
-            if (src.s8 && !qp) {
-                const size_t per = (size_t)K, numel = per * d.c_out;
-                q_codes.resize(numel);
-                for (size_t i = 0; i < numel; ++i) q_codes[i] = src.qval(i, (int)(i / per));
-                qp = q_codes.data();
-            }
-            tcv_build(h, src.f, qp, src.mask);
-            st = tcv_upload(h);
-        }
+        if (st == CADNN_OK && dense_route && (h->s.kind == KK_SCONV_SPATIAL || h->s.kind == KK_SCONV_LINEAR || h->s.kind == KK_DENSE_SMALLC) &&
+            d.fmt == CADNN_FMT_AUTO && !getenv("CADNN_NO_TCV") && !getenv("CADNN_SCHEDULE") && tcv_pays(d, h->nnz))
+            st = tcv_build(h);
         if (st == CADNN_OK && h->has_planar && h->on_device && (d.flags & CADNN_PACK_AUTOTUNE) && !h->tuned)
             autotune_planar(h, h->row_nnz);
         if (st == CADNN_OK && h->tune_key && !h->tuned && h->on_device) {   // remember what was measured
@@ -1475,7 +1467,7 @@ cadnn_status pack_common(const cadnn_layer_desc *desc, const Src &src, cadnn_wei
             sc.f = wc.data();
             sc.mask = mc.data();
             cadnn_weights *child = nullptr;
-            if (pack_common(&dc, sc, &child) == CADNN_OK) {
+            if (pack_common(&dc, sc, &child, false) == CADNN_OK) {
                 if (child->has_planar && child->h_out == h->h_out && child->w_out == h->w_out) h->half = child;
                 else cadnn_weights_free(child);
             }

@@ -825,7 +825,7 @@ SmemPlan plan_smem(bool f32, const Pick &k, int nkb)
 }
 
 // Block shape of a layer: the one a time model calls the fastest.  The model is linear in what a block does, with
-// coefficients fitted to 2000 measured shapes (193 layers of the workloads at batch 1 to 128, launched back to back as
+// coefficients fitted to 3900 measured shapes (212 layers of the workloads at batch 1 to 128, launched back to back as
 // programmatic dependents):
 //   time = start + P (b2 + n (c2 + d2 px / 64)) + Q (b1 + n (c1 + d1 px / 64))   [microseconds]
 // n = stages per block, P = rounds in which every multiprocessor runs two blocks, Q = rounds with one.  How many clusters
@@ -835,24 +835,24 @@ struct Cost {
     float start, b2, c2, d2, b1, c1, d1;
 };
 const Cost kCost[2][9] = {   // float, int8; 128 px x 64 ch, then up to 32, 64 and 128 px x 128 ch, each unsplit and split; 256 px x 128 ch
-    {{0.352f, 4.72f, 0.0f, 0.427f, 3.63f, 0.0f, 0.257f},
-     {1.82f, 4.04f, 0.0f, 0.401f, 2.66f, 0.0f, 0.276f},
-     {0.0124f, 3.2f, 0.535f, 0.0f, 2.9f, 0.413f, 0.0802f},
-     {0.638f, 3.09f, 0.397f, 0.373f, 2.52f, 0.388f, 0.172f},
-     {0.292f, 4.27f, 0.648f, 0.0f, 3.56f, 0.353f, 0.121f},
-     {1.63f, 4.0f, 0.0f, 0.68f, 2.55f, 0.301f, 0.202f},
-     {0.295f, 5.99f, 0.279f, 0.503f, 5.18f, 0.542f, 0.159f},
-     {1.08f, 0.0f, 0.0f, 0.0f, 5.04f, 0.306f, 0.315f},
-     {0.0f, 0.0f, 0.0f, 0.0f, 8.54f, 0.23f, 0.23f}},
-    {{1.08f, 3.82f, 0.0f, 0.341f, 3.02f, 0.0f, 0.19f},
-     {1.66f, 3.38f, 0.0f, 0.359f, 2.54f, 0.0f, 0.21f},
-     {0.77f, 2.49f, 0.441f, 0.0f, 2.06f, 0.286f, 0.155f},
-     {2.89f, 0.537f, 0.223f, 0.597f, 0.0f, 0.259f, 0.315f},
-     {1.42f, 2.99f, 0.6f, 0.0f, 2.4f, 0.219f, 0.146f},
-     {2.78f, 2.79f, 0.0f, 0.485f, 1.17f, 0.1f, 0.332f},
-     {2.35f, 5.49f, 0.0f, 0.425f, 2.9f, 0.118f, 0.217f},
-     {0.844f, 5.77f, 0.0f, 0.481f, 4.73f, 0.0f, 0.349f},
-     {0.0f, 0.0f, 0.0f, 0.0f, 7.55f, 0.0461f, 0.249f}}};
+    {{0.385f, 4.84f, 0.0f, 0.421f, 3.61f, 0.0f, 0.257f},
+     {1.3f, 5.25f, 0.0f, 0.429f, 3.28f, 0.0f, 0.28f},
+     {0.0f, 3.35f, 0.522f, 0.0f, 2.99f, 0.415f, 0.0615f},
+     {0.641f, 2.81f, 0.413f, 0.303f, 2.26f, 0.41f, 0.0958f},
+     {0.166f, 4.49f, 0.634f, 0.0f, 3.79f, 0.36f, 0.11f},
+     {1.03f, 3.89f, 0.115f, 0.561f, 2.63f, 0.324f, 0.169f},
+     {0.172f, 6.37f, 0.26f, 0.501f, 5.52f, 0.54f, 0.156f},
+     {0.76f, 0.0f, 0.0f, 0.0f, 4.85f, 0.322f, 0.301f},
+     {0.0f, 0.0f, 0.0f, 0.0f, 6.52f, 0.435f, 0.162f}},
+    {{1.19f, 3.83f, 0.0f, 0.353f, 2.85f, 0.0f, 0.191f},
+     {1.68f, 3.44f, 0.0f, 0.358f, 2.44f, 0.0f, 0.216f},
+     {0.927f, 2.42f, 0.445f, 0.0f, 1.83f, 0.28f, 0.167f},
+     {2.83f, 0.611f, 0.216f, 0.605f, 0.0f, 0.259f, 0.309f},
+     {1.24f, 3.19f, 0.602f, 0.0f, 2.64f, 0.215f, 0.147f},
+     {2.71f, 2.82f, 0.0f, 0.505f, 1.18f, 0.119f, 0.305f},
+     {2.74f, 4.88f, 0.0f, 0.452f, 2.61f, 0.108f, 0.224f},
+     {0.507f, 5.89f, 0.0f, 0.563f, 4.98f, 0.0f, 0.356f},
+     {0.0f, 11.6f, 0.0f, 0.578f, 6.35f, 0.0f, 0.21f}}};
 
 Pick choose(bool f32, int c_out, long long M, int nkb)
 {
@@ -881,7 +881,7 @@ Pick choose(bool f32, int c_out, long long M, int nkb)
         }
     };
     consider(128, 64);
-    static const int fixed[] = {32, 64, 96, 112, 128, 256};
+    static const int fixed[] = {32, 64, 96, 112, 128, 192, 208, 224, 256};
     for (int px : fixed) consider(px, 128);
     for (int q = 1; q <= 16; ++q) {   // the pixels cut into q equal tiles
         const long long px = ((M + q - 1) / q + 15) / 16 * 16;
@@ -960,43 +960,119 @@ bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz)
     return density >= (d.dtype == CADNN_F32 && d.c_out <= 64 ? 0.06 : 0.025);
 }
 
-// Weight image: [64-channel tile][stage][part][64 rows][64 bytes], rows swizzled like the operand tiles.  Parts: the
-// three bf16 terms of a float, or the two 64-value halves of an int8 stage.
-void tcv_build(cadnn_weights *h, const float *f, const int8_t *q, const uint8_t *mask)
+namespace {
+
+// Where weight (output channel co, kernel row ky, position i = kx * c_in + ci of that row) lies in the image
+// [64-channel tile][stage][part][64 rows][64 bytes], rows swizzled like the operand tiles.  Parts: the three bf16 terms of a
+// float, or the two 64-value halves of an int8 stage.
+struct ImageDims {
+    int nkb, Rp;
+};
+__host__ __device__ inline size_t image_at(const ImageDims &d, bool f32, int co, int ky, int i)
+{
+    const int k = ky * d.Rp + i, r = co & 63, sw = (r >> 1) & 3;
+    const size_t tile = (size_t)(co >> 6) * d.nkb;
+    if (f32) {
+        const int c = k & 31;
+        return (tile + (k >> 5)) * 3 * 4096 + r * 64 + (((c >> 3) ^ sw) << 4) + (c & 7) * 2;
+    }
+    const int c = k & 63;
+    return ((tile + (k >> 7)) * 2 + ((k >> 6) & 1)) * 4096 + r * 64 + (((c >> 4) ^ sw) << 4) + (c & 15);
+}
+__host__ __device__ inline void image_put(unsigned char *image, const ImageDims &d, int co, int ky, int i, float v)
+{
+    __nv_bfloat16 *at = reinterpret_cast<__nv_bfloat16 *>(image + image_at(d, true, co, ky, i));
+    for (int t = 0; t < 3; ++t) {
+        const __nv_bfloat16 b = __float2bfloat16_rn(v);
+        at[t * 2048] = b;
+        v -= __bfloat162float(b);
+    }
+}
+
+// The image written on the device from the sparse image that is there already (tiled CSR records: a header of row starts,
+// then {value, tile offset} entries): one warp per (channel chunk, packed row).  Padding entries have the value 0, as the
+// image has everywhere else.
+struct ExpandParams {
+    const uint32_t *ent;
+    const int32_t *perm;
+    unsigned char *image;
+    ImageDims dims;
+    int n_chunks, c_pad, n_groups, G, hdr_words, block_words, CIc, PPb, pitch, half, linear, s8, c_in;
+};
+__global__ void __launch_bounds__(256) expand_kernel(const ExpandParams p)
+{
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int c = blockIdx.y;
+    if (row >= p.c_pad) return;
+    const int co = p.perm[row];
+    if (co < 0) return;
+    const uint32_t *blk = p.ent + ((size_t)c * p.n_groups + row / p.G) * p.block_words, *ents = blk + p.hdr_words;
+    const int first = (int)blk[row % p.G], last = (int)blk[row % p.G + 1];
+    for (int e = first + lane; e < last; e += 32) {
+        uint32_t off, bits;
+        if (p.s8) {
+            bits = ents[e] & 0xffu;
+            off = ents[e] >> 8;
+        } else {
+            bits = ents[2 * (size_t)e];
+            off = ents[2 * (size_t)e + 1];
+        }
+        if ((bits << 1) == 0) continue;   // +-0
+        const int cl = (int)(off % (uint32_t)p.PPb) / (p.s8 ? 1 : 4), t = (int)(off / (uint32_t)p.PPb);
+        int kx = 0, ky = 0;
+        if (!p.linear) {
+            const int pos = t % p.pitch;
+            ky = t / p.pitch;
+            kx = p.half ? (pos >= p.half ? 2 * (pos - p.half) + 1 : 2 * pos) : pos;
+        }
+        const int i = kx * p.c_in + c * p.CIc + cl;
+        if (p.s8) p.image[image_at(p.dims, false, co, ky, i)] = (unsigned char)bits;
+        else image_put(p.image, p.dims, co, ky, i, __uint_as_float(bits));
+    }
+}
+
+}  // namespace
+
+// Builds the dense image of a handle whose sparse (or dense stem) image is on the device.
+cadnn_status tcv_build(cadnn_weights *h)
 {
     const cadnn_layer_desc &d = h->desc;
-    const bool s8 = d.dtype == CADNN_S8;
-    const int R = d.kw * d.c_in, Rp = row_positions(d), nkb = stages_of(d), parts = s8 ? 2 : 3;
-    h->tcv_img.assign((size_t)ceil_div(d.c_out, 64) * nkb * parts * 4096, 0);
-    for (int co = 0; co < d.c_out; ++co) {
-        unsigned char *tile = &h->tcv_img[(size_t)(co / 64) * nkb * parts * 4096];
-        const int r = co & 63, sw = (r >> 1) & 3;
-        for (int ky = 0; ky < d.kh; ++ky)
-        for (int i = 0; i < R; ++i) {
-            const size_t wi = ((size_t)co * d.kh + ky) * R + i;
-            const int k = ky * Rp + i;
-            if (mask && !mask[wi]) continue;
-            if (s8) {
-                const int kb = k >> 7, part = (k >> 6) & 1, c = k & 63;
-                tile[((size_t)kb * 2 + part) * 4096 + r * 64 + (((c >> 4) ^ sw) << 4) + (c & 15)] = (unsigned char)q[wi];
-            } else {
-                const int kb = k >> 5, c = k & 31;
-                unsigned char *at = tile + (size_t)kb * 3 * 4096 + r * 64 + (((c >> 3) ^ sw) << 4) + (c & 7) * 2;
-                float v = f[wi];
-                for (int t = 0; t < 3; ++t) {
-                    const __nv_bfloat16 b = __float2bfloat16_rn(v);
-                    memcpy(at + t * 4096, &b, 2);
-                    v -= __bfloat162float(b);
-                }
-            }
-        }
-    }
-    h->has_tcv = true;
     int a = 0, b = 0, c = 0;   // for tests and tuning: the block shape, "pixels,channels,split"
     const char *e = getenv("CADNN_TCV");
     if (e && sscanf(e, "%d,%d,%d", &a, &b, &c) == 3 && a >= 16 && a <= 256 && a % 16 == 0 && (b == 128 || (b == 64 && a == 128)) && c >= 1) {
         h->tcv_force[0] = a; h->tcv_force[1] = b; h->tcv_force[2] = c;
     }
+    if (d.flags & CADNN_PACK_HOST_ONLY) return CADNN_OK;
+    const bool s8 = d.dtype == CADNN_S8;
+    const ImageDims dims = {stages_of(d), row_positions(d)};
+    const size_t bytes = (size_t)ceil_div(d.c_out, 64) * dims.nkb * (s8 ? 2 : 3) * 4096;
+    const cudaError_t er = cudaMalloc(&h->d_tcv, bytes);
+    if (er != cudaSuccess) {
+        cadnn_note_cuda(er);
+        return er == cudaErrorMemoryAllocation ? CADNN_E_ALLOC : CADNN_E_CUDA;
+    }
+    if (h->s.kind == KK_DENSE_SMALLC) {   // few weights, kept tap-major: written on the host
+        std::vector<unsigned char> image(bytes, 0);
+        for (int co = 0; co < d.c_out; ++co)
+            for (int ky = 0; ky < d.kh; ++ky)
+                for (int i = 0; i < d.kw * d.c_in; ++i)
+                    image_put(image.data(), dims, co, ky, i, h->dense_f[((size_t)ky * d.kw * d.c_in + i) * d.c_out + co]);
+        CADNN_CUDA_TRY(cudaMemcpy(h->d_tcv, image.data(), bytes, cudaMemcpyHostToDevice));
+    } else {
+        CADNN_CUDA_TRY(cudaMemsetAsync(h->d_tcv, 0, bytes, cudaStreamLegacy));
+        const Schedule &s = h->s;
+        ExpandParams p;
+        p.ent = h->d_ent; p.perm = h->d_perm; p.image = (unsigned char *)h->d_tcv; p.dims = dims;
+        p.n_chunks = s.n_chunks; p.c_pad = h->c_pad; p.n_groups = s.n_groups; p.G = s.G;
+        p.hdr_words = (s.G + 1 + 3) / 4 * 4;
+        p.block_words = p.hdr_words + s.max_entries * (s8 ? 1 : 2);
+        p.CIc = s.CIc; p.PPb = s.PPb; p.pitch = std::max(1, s.pitch); p.half = s.half;
+        p.linear = s.kind == KK_SCONV_LINEAR; p.s8 = s8; p.c_in = d.c_in;
+        expand_kernel<<<dim3((unsigned)ceil_div(h->c_pad, 8), (unsigned)s.n_chunks), 256, 0, cudaStreamLegacy>>>(p);
+        CADNN_CUDA_TRY(cudaGetLastError());
+    }
+    CADNN_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
+    return CADNN_OK;
 }
 
 // the kernel's index ranges: 31-bit element offsets and pixel numbers, 16-bit image coordinates
@@ -1052,18 +1128,4 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0;
     if (f32) return vec ? launch_shape<true, true>(p, pick.ch, (int)blocks, ep.pdl, st) : launch_shape<true, false>(p, pick.ch, (int)blocks, ep.pdl, st);
     return vec ? launch_shape<false, true>(p, pick.ch, (int)blocks, ep.pdl, st) : launch_shape<false, false>(p, pick.ch, (int)blocks, ep.pdl, st);
-}
-
-cadnn_status tcv_upload(cadnn_weights *h)
-{
-    if (!h->has_tcv || (h->desc.flags & CADNN_PACK_HOST_ONLY)) return CADNN_OK;
-    cudaError_t e = cudaMalloc(&h->d_tcv, h->tcv_img.size());
-    if (e != cudaSuccess) {
-        cadnn_note_cuda(e);
-        return e == cudaErrorMemoryAllocation ? CADNN_E_ALLOC : CADNN_E_CUDA;
-    }
-    CADNN_CUDA_TRY(cudaMemcpy(h->d_tcv, h->tcv_img.data(), h->tcv_img.size(), cudaMemcpyHostToDevice));
-    CADNN_CUDA_TRY(cudaStreamSynchronize(cudaStreamLegacy));
-    std::vector<unsigned char>().swap(h->tcv_img);
-    return CADNN_OK;
 }
