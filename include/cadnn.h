@@ -296,7 +296,8 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
  * Float networks made of a dense stem, sparse convs, dense depthwise convs of up to 9 taps,
  * max pools, a global average pool and fc layers keep their intermediate feature maps
  * channel-planar with a zero halo (see cadnn_conv2d_planar), unless every sparse conv carries the
- * dense tensor-core image and none was timed at pack time; others (int8) keep NHWC
+ * dense tensor-core image and none was timed at pack time (networks with depthwise layers: and the
+ * network is large); others (int8) keep NHWC
  * (CADNN_NO_PLANAR_DW: networks with depthwise layers too).  CADNN_NO_PLANAR in the
  * environment at cadnn_net_create forces NHWC.
  * Layers after the first are launched as programmatic dependents of their predecessor

@@ -569,16 +569,23 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
                 if (op.src == 0 || flat[op.src]) planar = false;
             }
         }
-        // Layers packed with the dense tensor-core image run NHWC (tcconv.cu).  Networks with depthwise layers, and those
-        // whose schedules were timed at pack time, are left to the planar kernels.
+        // Layers packed with the dense tensor-core image run NHWC (tcconv.cu), unless their schedules were timed at pack time.
+        // Networks with depthwise layers do so above 150 million multiply-adds of kept weights: up to there the planar kernels'
+        // shorter start-up makes up for their rate (MobileNet-V2, planar / NHWC: batch 1 225 / 225 us, batch 2 304 / 262, batch 16
+        // 1060 / 662; half width at 160 x 160, batch 1: 159 / 198).
         if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr && !(getenv("CADNN_PERSIST") && atoi(getenv("CADNN_PERSIST")) != 0)) {
-            bool tc = true;
+            bool tc = true, dw = false;
+            double macs = 0.0;
             for (int i = 0; i < n_ops && tc; ++i) {
                 const cadnn_weights *w = ops[i].kind == CADNN_OP_CONV ? ops[i].w : nullptr;
-                if (!w || w->s.kind == KK_DENSE_SMALLC) continue;
-                tc = w->d_tcv && w->nhwc_us <= 0.0f;
+                if (!w) continue;
+                if (w->s.kind == KK_DW) dw = true;
+                else if (w->s.kind != KK_DENSE_SMALLC) {
+                    tc = w->d_tcv && w->nhwc_us <= 0.0f;
+                    macs += (double)w->nnz * w->h_out * w->w_out * n;
+                }
             }
-            if (tc) planar = false;
+            if (tc && (!dw || macs > 150e6)) planar = false;
         }
         // Where the packer timed both layouts for every sparse conv, the measured sums decide.
         if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr) {
