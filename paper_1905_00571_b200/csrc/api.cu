@@ -96,7 +96,7 @@ cadnn_status check_layer_call(const cadnn_weights *w, bool has_residual, int act
 }
 
 cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, int wd, void *y, const cadnn_epilogue *ep,
-                         bool pdl, cudaStream_t s, void *workspace, int64_t workspace_bytes)
+                         bool pdl, cudaStream_t s, void *workspace, int64_t workspace_bytes, const Prefetch *prefetch)
 {
     if (!w || !x || !y || n < 0) return CADNN_E_ARG;
     if (!w->on_device) return CADNN_E_ARG;
@@ -106,6 +106,7 @@ cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, in
     cadnn_status st = check_epilogue(w, ep, le);
     if (st != CADNN_OK) return st;
     le.pdl = pdl;
+    le.prefetch = prefetch;
     if (w->has_tc && w->nnz == w->tc_nnz) {
         // every stored weight sits in a dense block: the tensor-core kernel finishes the layer
         return launch_block_tc(w, x, n, nullptr, y, &le, s);
@@ -119,7 +120,7 @@ cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, in
         le.acc_in = (const int *)workspace;
         le.pdl = false;
     }
-    if (w->d_tcv && tcv_fits(w, n)) return launch_tcv(w, x, n, y, le, s);
+    if (w->d_tcv && tcv_fits(w, n) && (w->s.kind != KK_FC_SPMV || tcv_fc_pays(w, n))) return launch_tcv(w, x, n, y, le, s);
     switch (w->s.kind) {
         case KK_SCONV_SPATIAL:
         case KK_SCONV_LINEAR: return launch_sconv(w, x, n, y, le, s);

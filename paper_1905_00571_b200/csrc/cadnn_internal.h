@@ -147,6 +147,7 @@ struct cadnn_weights {
 
     // dense tensor-core image (tcconv.cu): built when the layer's density makes that route the faster one
     void *d_tcv = nullptr;
+    size_t tcv_bytes = 0;
     int tcv_force[3] = {0, 0, 0};          // CADNN_TCV at pack time: pixels, channels, split (0 = choose)
     mutable std::atomic<uint64_t> tcv_pick{0};   // block shape of the last batch size (tcconv.cu)
 
@@ -158,6 +159,13 @@ struct cadnn_weights {
     const int32_t *d_ptr = nullptr;
     const int32_t *d_perm = nullptr;
     const float *d_dense = nullptr;
+};
+
+// Weights that kernels launched a little later will read: a tensor-core layer of a network asks for them to be brought into L2.
+struct Prefetch {
+    static const int kMax = 4;
+    const void *at[kMax] = {nullptr, nullptr, nullptr, nullptr};
+    unsigned long long bytes[kMax] = {0, 0, 0, 0};
 };
 
 struct LaunchEpilogue {
@@ -176,6 +184,7 @@ struct LaunchEpilogue {
     // (parity_planes_bytes below gives its size); parity_mask = planes wanted, bit (row parity * 2 + column parity)
     float *parity_y = nullptr;
     int parity_mask = 0;
+    const Prefetch *prefetch = nullptr;   // dense tensor-core route
 };
 
 // Parity planes of an h x w map of c channels: plane (py * 2 + px) holds the pixels (2 i + py, 2 j + px) at (i, j) of a
@@ -246,6 +255,7 @@ cadnn_status launch_block_tc(const cadnn_weights *w, const void *x, int n, int *
 // dense tensor-core route (tcconv.cu)
 bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz);
 cadnn_status tcv_build(cadnn_weights *h);
+bool tcv_fc_pays(const cadnn_weights *w, int n);   // a small-batch fc layer runs faster dense
 bool tcv_fits(const cadnn_weights *w, int n);   // the batch is within the kernel's index ranges
 cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep, cudaStream_t st);
 cadnn_status copy_timeout_word(int **word);   // device address of the copy give-up counter
@@ -306,7 +316,7 @@ cadnn_status launch_gavgpool(const float *x, int n, int h, int wd, int c, float 
 
 // layer entry shared by the public calls and the network runner
 cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, int wd, void *y, const cadnn_epilogue *ep,
-                         bool pdl, cudaStream_t st, void *workspace = nullptr, int64_t workspace_bytes = 0);
+                         bool pdl, cudaStream_t st, void *workspace = nullptr, int64_t workspace_bytes = 0, const Prefetch *prefetch = nullptr);
 
 #ifdef __CUDACC__
 // Division by a runtime constant as multiply-high and shift (the divisor is fixed per

@@ -35,6 +35,7 @@ struct cadnn_net {
     PersistPlan *persist = nullptr;
     int persist_first = -1, persist_last = -1;
     int64_t workspace = 0;
+    std::vector<Prefetch> ahead;   // per op: weights its kernel brings into L2 for later ops
     std::vector<char> use_half;   // per op: a stride-2 conv that runs as its stride-1 form over its input's parity planes
     // graph cache: [0] caller's device pointers, [1] the net's own staging buffers
     struct GraphCache {
@@ -118,8 +119,9 @@ cadnn_status run_op(cadnn_net *net, const cadnn_op &op, const void *x, void *y, 
         ep.out_c_total = op.dst_c_total;
         ep.out_c_off = op.dst_c_off;
         ep.residual_scale = op.res_scale;
-        if (op.kind == CADNN_OP_FC) return conv2d_impl(op.w, src, si.n, 1, 1, dst, &ep, pdl, st);
-        return conv2d_impl(op.w, src, si.n, si.h, si.w, dst, &ep, pdl, st, net->tc_ws, net->tc_ws_bytes);
+        const Prefetch *ahead = net->ahead.empty() ? nullptr : &net->ahead[(size_t)(&op - net->ops.data())];
+        if (op.kind == CADNN_OP_FC) return conv2d_impl(op.w, src, si.n, 1, 1, dst, &ep, pdl, st, nullptr, 0, ahead);
+        return conv2d_impl(op.w, src, si.n, si.h, si.w, dst, &ep, pdl, st, net->tc_ws, net->tc_ws_bytes, ahead);
     }
     if (op.kind == CADNN_OP_MAXPOOL || op.kind == CADNN_OP_AVGPOOL)
         return launch_pool_window(src, si.n, si.h, si.w, si.c, op.pool_k, op.pool_stride, op.pool_pad, si.dtype,
@@ -515,6 +517,36 @@ cadnn_status plan_parity_planes(cadnn_net *net)
     return CADNN_OK;
 }
 
+// Which weights each tensor-core op brings into L2 while it runs: those of the ops behind the next tensor-core op, up to the one
+// after it.  The dense images of a network do not all stay in L2 (ResNet-50: 141 MB), and at batch 1 a layer's few blocks
+// cannot keep enough loads in flight to hide HBM (512->512 3x3 7x7: 6 us instead of 3 in the network).
+void plan_prefetch(cadnn_net *net)
+{
+    const int n_ops = (int)net->ops.size();
+    auto tc = [&](int i) { return net->ops[i].w && net->ops[i].w->d_tcv; };
+    net->ahead.assign(n_ops, Prefetch());
+    if (net->planar) return;
+    for (int i = 0; i < n_ops; ++i) {
+        if (!tc(i)) continue;
+        int j = i + 1;
+        while (j < n_ops && !tc(j)) ++j;
+        int used = 0;
+        for (int k = j + 1; k < n_ops && used < Prefetch::kMax; ++k) {
+            const cadnn_weights *w = net->ops[k].w;
+            Prefetch &a = net->ahead[i];
+            if (tc(k)) {
+                a.at[used] = w->d_tcv;
+                a.bytes[used++] = w->tcv_bytes;
+                break;
+            }
+            if (w && w->s.kind == KK_FC_SPMV) {   // values and column indices lie behind each other
+                a.at[used] = w->d_vals;
+                a.bytes[used++] = (unsigned long long)((const char *)w->d_offs - (const char *)w->d_vals) + w->offs.size() * 2;
+            }
+        }
+    }
+}
+
 }  // namespace
 
 extern "C" {
@@ -690,6 +722,7 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
         cadnn_net_free(net);
         return st;
     }
+    plan_prefetch(net);
     if (net->tc_ws_bytes > 0) {
         cudaError_t e = cudaMalloc(&net->tc_ws, (size_t)net->tc_ws_bytes);
         if (e != cudaSuccess) {

@@ -1458,6 +1458,7 @@ cadnn_status pack_common(const cadnn_layer_desc *desc, const Src &src, cadnn_wei
         else st = pack_sconv(h, src);
         if (st == CADNN_OK) st = upload(h);
         if (st == CADNN_OK) st = block_tc_upload(h);
+        if (st == CADNN_OK && h->s.kind == KK_FC_SPMV && !getenv("CADNN_NO_TCV") && tcv_fc_pays(h, std::max(1, d.batch_hint))) st = tcv_build(h);
         if (st == CADNN_OK && dense_route && (h->s.kind == KK_SCONV_SPATIAL || h->s.kind == KK_SCONV_LINEAR || h->s.kind == KK_DENSE_SMALLC) &&
             d.fmt == CADNN_FMT_AUTO && !getenv("CADNN_NO_TCV") && !getenv("CADNN_SCHEDULE") && tcv_pays(d, h->nnz))
             st = tcv_build(h);

@@ -108,3 +108,34 @@ def test_channel_window_of_a_concatenation(c_off):
     s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None, 1, 1)
     assert_close_or_bounded(got[..., c_off:c_off + 68], want, s_abs, 48 * 9, "window")
     assert (got[..., :c_off] == 3.0).all() and (got[..., c_off + 68:] == 3.0).all()
+
+
+@pytest.mark.parametrize("dtype", ["f32", "s8"])
+def test_small_batch_fc_takes_the_dense_route_where_it_pays(dtype):
+    """Packed for a batch of 8 (row CSR): 7 images run dense, one image sparse, both against the oracle."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(49)
+    c_in, c_out = 1027, 1201
+    mask = gen.random_mask(g, (c_out, 1, 1, c_in), 0.5)
+    dev = lambda a: torch.from_numpy(a).to(DEV)
+    d = B.make_desc(c_in, c_out, batch_hint=8, dtype=dtype)
+    for n in (7, 1):
+        if dtype == "s8":
+            x = gen.int8_relu_activation(g, (n, c_in))
+            q = gen.int8_weights(g, (c_out, 1, 1, c_in))
+            m = (g.uniform(0.5, 1.5, size=c_out) * 2e-4).astype(np.float32)
+            b = (g.standard_normal(c_out) * 3).astype(np.float32)
+            want = ref.fc_s8(x, q.reshape(c_out, c_in), mask.reshape(c_out, c_in), m, b, "relu", "s8")
+            y = torch.zeros((n, c_out), dtype=torch.int8, device=DEV)
+            B.cadnn_fc(B.cadnn_pack_q8(d, q, mask), dev(x), y, dev(m), dev(b), act="relu")
+            torch.cuda.synchronize()
+            assert_exact(y.cpu().numpy(), want, "fc s8, batch %d" % n)
+        else:
+            x = gen.normal_input(g, (n, 1, 1, c_in))
+            w = gen.he_weights(g, c_out, 1, 1, c_in)
+            want = ref.conv2d_f32(x, w, mask).reshape(n, c_out)
+            s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None).reshape(n, c_out)
+            y = torch.zeros((n, c_out), device=DEV)
+            B.cadnn_fc(B.cadnn_pack(d, w, mask), dev(x.reshape(n, c_in)), y)
+            torch.cuda.synchronize()
+            assert_close_or_bounded(y.cpu().numpy(), want, s_abs, c_in, "fc f32, batch %d" % n)
