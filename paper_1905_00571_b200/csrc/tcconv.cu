@@ -187,12 +187,14 @@ __device__ __forceinline__ void send_bulk(unsigned dst, unsigned src, unsigned b
 // One kernel shape: PX pixels x CH channels per block.  SWAP: the channels are the 128 rows of the tensor-core tile and
 // the pixels its columns (any multiple of 16 up to PX, so that small maps waste little); otherwise the 128 rows are pixels
 // and the columns CH channels.
-template <bool F32, int PX, int CH, bool SWAP> struct Cfg {
+template <bool F32, int PX, int CH, bool SWAP, bool VEC> struct Cfg {
     static const int kParts = F32 ? 3 : 2;                 // operand tiles of 64-byte rows per stage
     static const int kKB = F32 ? 32 : 128;                 // K values per stage (128 source bytes per pixel)
     static const int kWBytes = kParts * CH * 64;
-    // blocks per multiprocessor the registers, tensor memory and shared memory are cut for
-    static const int kBlocks = PX > 128 ? 1 : 2;
+    // Blocks per multiprocessor the registers are cut for (tensor memory and shared memory for one or two).  Int8 tiles of layers
+    // with few stages are small enough for three (int8 ResNet-50, batch 32: 963 us with 62 to 78 registers and one residual row
+    // ahead, 923 us with 64 and two; four rows 947, eight 998).
+    static const int kBlocks = PX > 128 ? 1 : F32 || !VEC ? 2 : 3;
     static const int kN = SWAP ? PX : CH;
     // Accumulators, kN columns each (kN at most 64: three, by size of the terms; beyond: the large products and the small
     // ones; int8: two that take turns, so that no multiply-add waits for the one before it)
@@ -450,9 +452,9 @@ __device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, un
 }
 
 template <bool F32, int PX, int CH, bool SWAP, bool VEC>
-__global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP>::kThreads, Cfg<F32, PX, CH, SWAP>::kBlocks) tcconv_kernel(const TcvParams p)
+__global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32, PX, CH, SWAP, VEC>::kBlocks) tcconv_kernel(const TcvParams p)
 {
-    typedef Cfg<F32, PX, CH, SWAP> C;
+    typedef Cfg<F32, PX, CH, SWAP, VEC> C;
     const int kLoadWarps = C::kLoadWarps;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const unsigned raw32 = (unsigned)__cvta_generic_to_shared(smem_raw);
@@ -656,7 +658,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP>::kThreads, Cfg<F32, PX,
     const bool mine = warp < kLoadWarps && co < p.c_out;
     float4 sc = make_float4(1, 1, 1, 1), bi = make_float4(0, 0, 0, 0);
     // residuals of the next kAhead rows: a tile with few stages is bound by how many of these loads are in flight
-    const int kAhead = F32 ? 4 : 1;   // (int8: 4 bytes a load, and registers that keep a third block resident count more)
+    const int kAhead = F32 ? 4 : PX > 64 ? 2 : 1;   // (int8: registers that keep a third block resident count more)
     uint4 res[kAhead];
 #pragma unroll
     for (int i = 0; i < kAhead; ++i) res[i] = make_uint4(0, 0, 0, 0);
@@ -903,7 +905,7 @@ template <bool F32, int PX, int CH, bool SWAP, bool VEC>
 cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
 {
     auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC>;
-    typedef Cfg<F32, PX, CH, SWAP> C;
+    typedef Cfg<F32, PX, CH, SWAP, VEC> C;
     const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb);
     if (sp.stages < C::kGroups || sp.stages * C::kParts * 64 * (p.npx + CH) > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
     p.stages = sp.stages;
