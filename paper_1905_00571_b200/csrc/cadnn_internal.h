@@ -168,6 +168,14 @@ struct Prefetch {
     unsigned long long bytes[kMax] = {0, 0, 0, 0};
 };
 
+// a depthwise layer that follows a planar sparse conv
+struct FusedDw {
+    const cadnn_weights *w;
+    const float *scale, *bias;
+    float *y;
+    int act;
+};
+
 struct LaunchEpilogue {
     const float *scale = nullptr;
     const float *bias = nullptr;
@@ -185,6 +193,7 @@ struct LaunchEpilogue {
     float *parity_y = nullptr;
     int parity_mask = 0;
     const Prefetch *prefetch = nullptr;   // dense tensor-core route
+    const FusedDw *dw = nullptr;          // planar sparse convs (ps_fuses_dw): a depthwise layer over the output, done in the same launch
 };
 
 // Parity planes of an h x w map of c channels: plane (py * 2 + px) holds the pixels (2 i + py, 2 j + px) at (i, j) of a
@@ -243,6 +252,7 @@ cadnn_status launch_sconv_planar(const cadnn_weights *w, const void *x, int n, v
                                  cudaStream_t st);
 cadnn_status launch_sconv_planar_staged(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep,
                                         cudaStream_t st);
+bool ps_fuses_dw(const cadnn_weights *w, const cadnn_weights *dw);   // whether LaunchEpilogue.dw can be given
 bool dw_planar_ok(const cadnn_weights *w);   // a depthwise layer the planar layout can run (float, <= 9 taps, pad within the halo)
 cadnn_status launch_dw_planar(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep,
                               cudaStream_t st);

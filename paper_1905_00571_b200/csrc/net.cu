@@ -70,7 +70,18 @@ void *slot_ptr(cadnn_net *net, int slot, const void *x, void *y)
     return net->slots[slot].ptr;
 }
 
-cadnn_status run_op(cadnn_net *net, const cadnn_op &op, const void *x, void *y, cudaStream_t st, bool pdl = false)
+// op i is a planar sparse conv whose launch also runs op i + 1, the depthwise layer that reads it
+bool runs_next(const cadnn_net *net, int i)
+{
+    if (!net->planar || i + 1 >= (int)net->ops.size()) return false;
+    const cadnn_op &op = net->ops[i], &nx = net->ops[i + 1];
+    if (op.kind != CADNN_OP_CONV || nx.kind != CADNN_OP_CONV || op.w->s.kind == KK_DENSE_SMALLC || op.w->s.kind == KK_DW) return false;
+    return nx.src == op.dst && nx.res < 0 && !net->slots[op.dst].par_ptr && !((size_t)i < net->use_half.size() && net->use_half[i]) &&
+           ps_fuses_dw(op.w, nx.w);
+}
+
+// with_next: runs_next holds for op, and the next op is run as well
+cadnn_status run_op(cadnn_net *net, const cadnn_op &op, const void *x, void *y, cudaStream_t st, bool pdl = false, bool with_next = false)
 {
     const SlotInfo &si = net->slots[op.src];
     const void *src = slot_ptr(net, op.src, x, y);
@@ -85,6 +96,13 @@ cadnn_status run_op(cadnn_net *net, const cadnn_op &op, const void *x, void *y, 
             le.out_dtype = CADNN_F32;
             le.pdl = pdl;
             le.early_trigger = net->early_trigger;
+            FusedDw dw;
+            if (with_next) {
+                const cadnn_op &nx = (&op)[1];
+                dw.w = nx.w; dw.scale = nx.scale; dw.bias = nx.bias; dw.act = nx.act;
+                dw.y = (float *)slot_ptr(net, nx.dst, x, y);
+                le.dw = &dw;
+            }
             const SlotInfo &so = net->slots[op.dst];
             if (so.par_ptr) {
                 le.parity_y = (float *)so.par_ptr;
@@ -149,9 +167,11 @@ cadnn_status run_all(cadnn_net *net, const void *x, void *y, cudaStream_t st, bo
             first = true;
             continue;
         }
-        cadnn_status s = run_op(net, net->ops[i], x, y, st, pdl && !first);
+        const bool two = runs_next(net, i);
+        cadnn_status s = run_op(net, net->ops[i], x, y, st, pdl && !first, two);
         if (s != CADNN_OK) return s;
         first = false;
+        i += two;
     }
     return CADNN_OK;
 }
@@ -206,8 +226,10 @@ cadnn_status run_all_forked(cadnn_net *net, const void *x, void *y, cudaStream_t
             rs = run_op(net, op, x, y, side, false);
             if (rs == CADNN_OK && cudaEventRecord(join[i], side) != cudaSuccess) rs = CADNN_E_CUDA;
         } else {
-            rs = run_op(net, op, x, y, st, pdl && !first);
+            const bool two = runs_next(net, i);
+            rs = run_op(net, op, x, y, st, pdl && !first, two);
             first = false;
+            i += two;
         }
     }
     // branches nobody read still have to end inside the capture
@@ -805,7 +827,10 @@ cadnn_status cadnn_forward_host(cadnn_net *net, const void *x_host, void *y_host
 cadnn_status cadnn_net_info(const cadnn_net *net, int *n_launches, int64_t *workspace_bytes)
 {
     if (!net) return CADNN_E_ARG;
-    if (n_launches) *n_launches = (int)net->ops.size() - (net->persist ? net->persist_last - net->persist_first : 0);
+    if (n_launches) {
+        *n_launches = (int)net->ops.size() - (net->persist ? net->persist_last - net->persist_first : 0);
+        for (int i = 0; i < (int)net->ops.size(); ++i) *n_launches -= runs_next(net, i);
+    }
     if (workspace_bytes) *workspace_bytes = net->workspace;
     return CADNN_OK;
 }

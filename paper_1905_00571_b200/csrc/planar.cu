@@ -357,7 +357,7 @@ cadnn_status launch_gavgpool_planar(const float *x, int n, int h, int wd, int c,
 bool dw_planar_ok(const cadnn_weights *w)
 {
     const cadnn_layer_desc &d = w->desc;
-    return w->s.kind == KK_DW && d.dtype == CADNN_F32 && d.kh * d.kw <= 9 && d.pad <= kPlanarHalo &&
+    return w->s.kind == KK_DW && d.dtype == CADNN_F32 && d.kh * d.kw <= 9 && d.pad <= kPlanarHalo && d.pad_w == d.pad &&
            d.kh - 1 - d.pad <= kPlanarHalo && d.kw - 1 - d.pad <= kPlanarHalo && w->d_dense != nullptr;
 }
 

@@ -71,6 +71,16 @@ cadnn_status write_copy_timeouts(int value)
 
 namespace {
 
+// Depthwise layer finished behind a conv whose blocks hold whole planes (ps_fuses_dw)
+struct DwTail {
+    const float *wt;       // [kh * kw][c]
+    const float *scale, *bias;
+    float *y;
+    int off;               // byte offset of the planes in shared memory: [G][pitch], then 12 words per filter: taps, scale, bias
+    int kh, kw, stride, off0, w_out, wp_out, pitch_out, qtot, act;
+    FastDiv d_wp_out;
+};
+
 struct PsParams {
     const float *x;
     float *y;
@@ -94,6 +104,7 @@ struct PsParams {
     int early_trigger;     // as a programmatic primary: let the next layer's prologue start at once
     int RB, nb, bar_off;   // TMA staging: rows per box, boxes per chunk, byte offset of the stage barriers
     FastDiv d_groups, d_tiles, d_wp, d_wp_out, d_l4;
+    DwTail dw;             // depthwise layer over this one's output (dw.y null = none)
     ParityPlanes par;      // second copy of the output for a stride-2 reader (par.y null = none)
 };
 
@@ -213,8 +224,48 @@ __device__ __forceinline__ void ps_compute_chunk(const PsParams &p, const unsign
     }
 }
 
+// Depthwise layer over the planes of this warp's filters, which the epilogue has just left in shared memory (the sums of
+// dw_planar_kernel in the same order, from the same values).  Such a layer is all latency (launch, one round trip to L2, a
+// few multiply-adds: 5 us alone); behind the conv it costs about 2.  MobileNet-V2, batch 1, where ten of the seventeen
+// depthwise layers follow a conv of one tile: 225 / 209 us; at 160 x 160 pixels 197 / 183.
+template <int RPW>
+__device__ __forceinline__ void ps_dw_tail(const PsParams &p, unsigned char *smem, int lane, int rslot, unsigned img, const int (&co_of)[RPW])
+{
+    const float *planes = reinterpret_cast<const float *>(smem + p.dw.off);
+    __syncwarp();
+#pragma unroll 1
+    for (int j = 0; j < RPW; ++j) {
+        const int slot = rslot * RPW + j, co = co_of[j];
+        if (co < 0) continue;
+        const float *plane = planes + slot * p.pitch_out, *k12 = planes + p.G * p.pitch_out + slot * 12;
+        float *dst = p.dw.y + ((size_t)img * p.c_out + co) * p.dw.pitch_out + kPlanarHalo * p.dw.wp_out;
+        float wv[9];
+        int off[9];
+        const int taps = p.dw.kh * p.dw.kw;
+        int ky = 0, kx = 0;
+#pragma unroll
+        for (int k = 0; k < 9; ++k) {
+            wv[k] = k12[k];
+            off[k] = k < taps ? ky * p.wp_out + kx : 0;
+            if (++kx == p.dw.kw) { kx = 0; ++ky; }
+        }
+        const float sc = k12[9], bi = k12[10];
+#pragma unroll 2
+        for (int i = lane; i < p.dw.qtot; i += 32) {
+            const int oy = (int)fdiv((unsigned)i, p.dw.d_wp_out), ox = i - oy * p.dw.wp_out - kPlanarHalo;
+            if (ox < 0 || ox >= p.dw.w_out) continue;
+            const float *at = plane + (oy * p.dw.stride + p.dw.off0) * p.wp_out + ox * p.dw.stride + p.dw.off0;
+            float acc = 0.0f;
+#pragma unroll
+            for (int k = 0; k < 9; ++k)
+                if (k < taps) acc = fmaf(wv[k], at[off[k]], acc);
+            dst[i] = ps_act(fmaf(acc, sc, bi), p.dw.act);
+        }
+    }
+}
+
 // partial sums of the warps that share a filter, epilogue, stores
-template <int T, int RPW>
+template <int T, int RPW, bool DW = false>
 __device__ __forceinline__ void ps_block_tail(const PsParams &p, unsigned char *smem, int lane, int rslot, int slice, int KS,
                                               unsigned img, int q0, unsigned okmask, const int (&co_of)[RPW],
                                               const float (&sc)[RPW], const float (&bi)[RPW], float (&acc)[RPW][T],
@@ -288,6 +339,7 @@ __device__ __forceinline__ void ps_block_tail(const PsParams &p, unsigned char *
                     else if (p.residual) z += p.residual[oi];
                     z = ps_act(z, p.act);
                     p.y[oi] = z;
+                    if (DW) reinterpret_cast<float *>(smem + p.dw.off)[(rslot * RPW + j) * p.pitch_out + q0 + lane + 32 * t] = z;
                     if (p.par.y) {
                         const int q = q0 + lane + 32 * t;
                         const int row = (int)fdiv((unsigned)q, p.d_wp_out);
@@ -297,6 +349,7 @@ __device__ __forceinline__ void ps_block_tail(const PsParams &p, unsigned char *
             }
         }
     }
+    if (DW && slice == 0) ps_dw_tail<RPW>(p, smem, lane, rslot, img, co_of);
     if (KC > 1) cluster_sync();   // peers may still be reading this block's partial sums
 }
 
@@ -448,7 +501,7 @@ __device__ __forceinline__ void ps_tma_issue(const PsParams &p, const CUtensorMa
     }
 }
 
-template <int T, int RPW, bool ROWS>
+template <int T, int RPW, bool ROWS, bool DW>
 __global__ void __launch_bounds__(512) sconv_planar_tma_kernel(const PsParams p, const __grid_constant__ CUtensorMap tmap)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -519,6 +572,23 @@ __global__ void __launch_bounds__(512) sconv_planar_tma_kernel(const PsParams p,
 #pragma unroll
         for (int t = 0; t < T; ++t) acc[j][t] = 0.0f;
 
+    if (DW && slice == 0) {
+        // planes read as zero where the conv stores nothing; taps, scale and bias of the depthwise layer
+        float *planes = reinterpret_cast<float *>(smem + p.dw.off);
+#pragma unroll
+        for (int j = 0; j < RPW; ++j) {
+            const int slot = rslot * RPW + j, co = co_of[j], taps = p.dw.kh * p.dw.kw;
+            for (int i = lane; i < p.pitch_out; i += 32) planes[slot * p.pitch_out + i] = 0.0f;
+            if (lane < 12 && co >= 0) {
+                float v = 0.0f;
+                if (lane < taps) v = __ldg(p.dw.wt + (size_t)lane * p.c_out + co);
+                else if (lane == 9) v = p.dw.scale ? __ldg(p.dw.scale + co) : 1.0f;
+                else if (lane == 10) v = p.dw.bias ? __ldg(p.dw.bias + co) : 0.0f;
+                planes[p.G * p.pitch_out + slot * 12 + lane] = v;
+            }
+        }
+    }
+
     grid_dep_wait();   // x (and the residual) are final from here on
     if (warp == 0 && lane < npre) ps_tma_issue(p, &tmap, smem32, lane, c_first + lane, grp, (int)img * p.c_in, xq, false, true, [] {});
     float sc[RPW], bi[RPW];
@@ -556,7 +626,7 @@ __global__ void __launch_bounds__(512) sconv_planar_tma_kernel(const PsParams p,
             parity ^= 1u;
         }
     }
-    ps_block_tail<T, RPW>(p, smem, lane, rslot, slice, KS, img, q0, okmask, co_of, sc, bi, acc, KC, rank,
+    ps_block_tail<T, RPW, DW>(p, smem, lane, rslot, slice, KS, img, q0, okmask, co_of, sc, bi, acc, KC, rank,
                           p.residual ? res : nullptr);
 }
 
@@ -564,10 +634,11 @@ template <int T, int RPW>
 cadnn_status ps_launch_one(const PsParams &p, const CUtensorMap *map, int blocks, int threads, int smem, bool pdl, cudaStream_t st)
 {
     if (map) {
-        auto kern = p.R > 0 ? sconv_planar_tma_kernel<T, RPW, true> : sconv_planar_tma_kernel<T, RPW, false>;
-        static SmemLimit lim[2];   // per instantiation (row-tile / linear), per device
+        auto kern = p.R > 0 ? sconv_planar_tma_kernel<T, RPW, true, false>
+                  : p.dw.y ? sconv_planar_tma_kernel<T, RPW, false, true> : sconv_planar_tma_kernel<T, RPW, false, false>;
+        static SmemLimit lim[3];   // per instantiation (row-tile / linear / with a depthwise layer), per device
         if (smem > 48 * 1024) {
-            cadnn_status rs = raise_smem_limit((const void *)kern, smem, &lim[p.R > 0 ? 1 : 0]);
+            cadnn_status rs = raise_smem_limit((const void *)kern, smem, &lim[p.R > 0 ? 1 : p.dw.y ? 2 : 0]);
             if (rs != CADNN_OK) return rs;
         }
         cudaLaunchConfig_t cfg = {};
@@ -666,6 +737,17 @@ bool encode_nhwc_s8_tiles_map(void *map, const void *base, int c, int w, int h, 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Whether a depthwise layer over w's output can run in the same launch: every block holds whole planes of its filters (one tile per
+// image, no cluster whose blocks finish different filters), with shared memory left for them.  Planes of several tiles would have to
+// overlap: tried, 160 x 160 pixels gained 2 %, 250 x 250 and 224 x 224 lost 1.
+bool ps_fuses_dw(const cadnn_weights *w, const cadnn_weights *dw)
+{
+    const PsSchedule &s = w->ps;
+    return w->has_ps && w->use_ps && s.tma && s.R == 0 && s.tiles == 1 && s.KC <= 1 && dw_planar_ok(dw) && dw->desc.c_out == w->desc.c_out &&
+           dw->desc.in_h == w->h_out && dw->desc.in_w == w->w_out &&
+           (s.smem_bytes + 15) / 16 * 16 + s.G * (planar_pitch(w->h_out, w->w_out) + 12) * 4 <= 220 * 1024;
+}
+
 cadnn_status launch_sconv_planar_staged(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep,
                                         cudaStream_t st)
 {
@@ -701,6 +783,20 @@ cadnn_status launch_sconv_planar_staged(const cadnn_weights *w, const void *x, i
     if (blocks <= 0) return CADNN_OK;
     if (blocks > 2147483647LL) return CADNN_E_UNSUPPORTED;
     const int threads = s.NW * 32;
+    int smem = s.smem_bytes;
+    p.dw = DwTail();
+    if (ep.dw) {
+        const cadnn_weights *v = ep.dw->w;
+        if (!ps_fuses_dw(w, v)) return CADNN_E_UNSUPPORTED;
+        DwTail &t = p.dw;
+        t.wt = v->d_dense; t.scale = ep.dw->scale; t.bias = ep.dw->bias; t.y = ep.dw->y; t.act = ep.dw->act;
+        t.kh = v->desc.kh; t.kw = v->desc.kw; t.stride = v->desc.stride; t.off0 = kPlanarHalo - v->desc.pad;
+        t.w_out = v->w_out; t.wp_out = v->w_out + 2 * kPlanarHalo; t.pitch_out = planar_pitch(v->h_out, v->w_out);
+        t.qtot = v->h_out * t.wp_out;
+        t.d_wp_out = make_fastdiv(t.wp_out);
+        t.off = (smem + 15) / 16 * 16;
+        smem = t.off + s.G * (p.pitch_out + 12) * 4;
+    }
     CUtensorMap map;
     const CUtensorMap *mp = nullptr;
     if (s.tma) {
@@ -721,10 +817,10 @@ cadnn_status launch_sconv_planar_staged(const cadnn_weights *w, const void *x, i
         p.RB = 0; p.nb = 0; p.bar_off = 0;
     }
     switch (s.T) {
-        case 1: return ps_launch_rpw<1>(p, mp, s.RPW, (int)blocks, threads, s.smem_bytes, ep.pdl, st);
-        case 2: return ps_launch_rpw<2>(p, mp, s.RPW, (int)blocks, threads, s.smem_bytes, ep.pdl, st);
-        case 4: return ps_launch_rpw<4>(p, mp, s.RPW, (int)blocks, threads, s.smem_bytes, ep.pdl, st);
-        case 8: return ps_launch_rpw<8>(p, mp, s.RPW, (int)blocks, threads, s.smem_bytes, ep.pdl, st);
+        case 1: return ps_launch_rpw<1>(p, mp, s.RPW, (int)blocks, threads, smem, ep.pdl, st);
+        case 2: return ps_launch_rpw<2>(p, mp, s.RPW, (int)blocks, threads, smem, ep.pdl, st);
+        case 4: return ps_launch_rpw<4>(p, mp, s.RPW, (int)blocks, threads, smem, ep.pdl, st);
+        case 8: return ps_launch_rpw<8>(p, mp, s.RPW, (int)blocks, threads, smem, ep.pdl, st);
     }
     return CADNN_E_UNSUPPORTED;
 }
