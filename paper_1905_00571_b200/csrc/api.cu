@@ -96,7 +96,7 @@ cadnn_status check_layer_call(const cadnn_weights *w, bool has_residual, int act
 }
 
 cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, int wd, void *y, const cadnn_epilogue *ep,
-                         bool pdl, cudaStream_t s, void *workspace, int64_t workspace_bytes, const Prefetch *prefetch)
+                         bool pdl, cudaStream_t s, void *workspace, int64_t workspace_bytes, const Prefetch *prefetch, void *pooled)
 {
     if (!w || !x || !y || n < 0) return CADNN_E_ARG;
     if (!w->on_device) return CADNN_E_ARG;
@@ -107,6 +107,7 @@ cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, in
     if (st != CADNN_OK) return st;
     le.pdl = pdl;
     le.prefetch = prefetch;
+    le.pooled = pooled;
     if (w->has_tc && w->nnz == w->tc_nnz) {
         // every stored weight sits in a dense block: the tensor-core kernel finishes the layer
         return launch_block_tc(w, x, n, nullptr, y, &le, s);

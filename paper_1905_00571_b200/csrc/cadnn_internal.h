@@ -193,6 +193,7 @@ struct LaunchEpilogue {
     float *parity_y = nullptr;
     int parity_mask = 0;
     const Prefetch *prefetch = nullptr;   // dense tensor-core route
+    void *pooled = nullptr;               // the same: where the 2 x 2 max pool of the output goes as well (tcv_pools), null = nowhere
     const FusedDw *dw = nullptr;          // planar sparse convs (ps_fuses_dw): a depthwise layer over the output, done in the same launch
 };
 
@@ -267,6 +268,7 @@ bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz);
 cadnn_status tcv_build(cadnn_weights *h);
 bool tcv_fc_pays(const cadnn_weights *w, int n);   // a small-batch fc layer runs faster dense
 bool tcv_fits(const cadnn_weights *w, int n);   // the batch is within the kernel's index ranges
+bool tcv_pools(const cadnn_weights *w, int n);   // LaunchEpilogue.pooled can be given
 cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep, cudaStream_t st);
 cadnn_status copy_timeout_word(int **word);   // device address of the copy give-up counter
 cadnn_status read_tc_timeouts(int *count);
@@ -326,7 +328,8 @@ cadnn_status launch_gavgpool(const float *x, int n, int h, int wd, int c, float 
 
 // layer entry shared by the public calls and the network runner
 cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, int wd, void *y, const cadnn_epilogue *ep,
-                         bool pdl, cudaStream_t st, void *workspace = nullptr, int64_t workspace_bytes = 0, const Prefetch *prefetch = nullptr);
+                         bool pdl, cudaStream_t st, void *workspace = nullptr, int64_t workspace_bytes = 0, const Prefetch *prefetch = nullptr,
+                         void *pooled = nullptr);
 
 #ifdef __CUDACC__
 // Division by a runtime constant as multiply-high and shift (the divisor is fixed per

@@ -36,6 +36,7 @@ struct cadnn_net {
     int persist_first = -1, persist_last = -1;
     int64_t workspace = 0;
     std::vector<Prefetch> ahead;   // per op: weights its kernel brings into L2 for later ops
+    std::vector<char> with_next;   // per op: its launch also runs the op behind it (plan_pairs)
     std::vector<char> use_half;   // per op: a stride-2 conv that runs as its stride-1 form over its input's parity planes
     // graph cache: [0] caller's device pointers, [1] the net's own staging buffers
     struct GraphCache {
@@ -70,17 +71,29 @@ void *slot_ptr(cadnn_net *net, int slot, const void *x, void *y)
     return net->slots[slot].ptr;
 }
 
-// op i is a planar sparse conv whose launch also runs op i + 1, the depthwise layer that reads it
-bool runs_next(const cadnn_net *net, int i)
+// Pairs of ops that one launch runs: a planar sparse conv and the depthwise layer that reads it, or an int8 conv on the tensor
+// cores and the 2 x 2 max pool that reads it.  The first one's tensor is written all the same.  (Not in networks with concatenations,
+// whose graphs order ops one by one.)
+void plan_pairs(cadnn_net *net)
 {
-    if (!net->planar || i + 1 >= (int)net->ops.size()) return false;
-    const cadnn_op &op = net->ops[i], &nx = net->ops[i + 1];
-    if (op.kind != CADNN_OP_CONV || nx.kind != CADNN_OP_CONV || op.w->s.kind == KK_DENSE_SMALLC || op.w->s.kind == KK_DW) return false;
-    return nx.src == op.dst && nx.res < 0 && !net->slots[op.dst].par_ptr && !((size_t)i < net->use_half.size() && net->use_half[i]) &&
-           ps_fuses_dw(op.w, nx.w);
+    net->with_next.assign(net->ops.size(), 0);
+    for (const cadnn_op &op : net->ops)
+        if (op.dst_c_total > 0) return;
+    if (getenv("CADNN_GRAPH_LANES")) return;
+    for (size_t i = 0; i + 1 < net->ops.size(); ++i) {
+        const cadnn_op &op = net->ops[i], &nx = net->ops[i + 1];
+        if (op.kind != CADNN_OP_CONV || nx.src != op.dst || op.dst == net->out_slot) continue;
+        if (net->planar) {
+            net->with_next[i] = nx.kind == CADNN_OP_CONV && nx.res < 0 && op.w->s.kind != KK_DENSE_SMALLC && op.w->s.kind != KK_DW &&
+                                !net->slots[op.dst].par_ptr && !(i < net->use_half.size() && net->use_half[i]) && ps_fuses_dw(op.w, nx.w);
+        } else {
+            net->with_next[i] = nx.kind == CADNN_OP_MAXPOOL && nx.pool_k == 2 && nx.pool_stride == 2 && nx.pool_pad == 0 && nx.dst != net->out_slot &&
+                                op.res < 0 && op.out_dtype == CADNN_S8 && tcv_pools(op.w, net->slots[op.src].n);
+        }
+    }
 }
 
-// with_next: runs_next holds for op, and the next op is run as well
+// with_next: the op behind is run as well (plan_pairs)
 cadnn_status run_op(cadnn_net *net, const cadnn_op &op, const void *x, void *y, cudaStream_t st, bool pdl = false, bool with_next = false)
 {
     const SlotInfo &si = net->slots[op.src];
@@ -139,7 +152,8 @@ cadnn_status run_op(cadnn_net *net, const cadnn_op &op, const void *x, void *y, 
         ep.residual_scale = op.res_scale;
         const Prefetch *ahead = net->ahead.empty() ? nullptr : &net->ahead[(size_t)(&op - net->ops.data())];
         if (op.kind == CADNN_OP_FC) return conv2d_impl(op.w, src, si.n, 1, 1, dst, &ep, pdl, st, nullptr, 0, ahead);
-        return conv2d_impl(op.w, src, si.n, si.h, si.w, dst, &ep, pdl, st, net->tc_ws, net->tc_ws_bytes, ahead);
+        return conv2d_impl(op.w, src, si.n, si.h, si.w, dst, &ep, pdl, st, net->tc_ws, net->tc_ws_bytes, ahead,
+                           with_next ? slot_ptr(net, (&op)[1].dst, x, y) : nullptr);
     }
     if (op.kind == CADNN_OP_MAXPOOL || op.kind == CADNN_OP_AVGPOOL)
         return launch_pool_window(src, si.n, si.h, si.w, si.c, op.pool_k, op.pool_stride, op.pool_pad, si.dtype,
@@ -167,7 +181,7 @@ cadnn_status run_all(cadnn_net *net, const void *x, void *y, cudaStream_t st, bo
             first = true;
             continue;
         }
-        const bool two = runs_next(net, i);
+        const bool two = net->with_next[i];
         cadnn_status s = run_op(net, net->ops[i], x, y, st, pdl && !first, two);
         if (s != CADNN_OK) return s;
         first = false;
@@ -226,7 +240,7 @@ cadnn_status run_all_forked(cadnn_net *net, const void *x, void *y, cudaStream_t
             rs = run_op(net, op, x, y, side, false);
             if (rs == CADNN_OK && cudaEventRecord(join[i], side) != cudaSuccess) rs = CADNN_E_CUDA;
         } else {
-            const bool two = runs_next(net, i);
+            const bool two = net->with_next[i];
             rs = run_op(net, op, x, y, st, pdl && !first, two);
             first = false;
             i += two;
@@ -745,6 +759,7 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
         return st;
     }
     plan_prefetch(net);
+    plan_pairs(net);
     if (net->tc_ws_bytes > 0) {
         cudaError_t e = cudaMalloc(&net->tc_ws, (size_t)net->tc_ws_bytes);
         if (e != cudaSuccess) {
@@ -829,7 +844,7 @@ cadnn_status cadnn_net_info(const cadnn_net *net, int *n_launches, int64_t *work
     if (!net) return CADNN_E_ARG;
     if (n_launches) {
         *n_launches = (int)net->ops.size() - (net->persist ? net->persist_last - net->persist_first : 0);
-        for (int i = 0; i < (int)net->ops.size(); ++i) *n_launches -= runs_next(net, i);
+        for (char two : net->with_next) *n_launches -= two;
     }
     if (workspace_bytes) *workspace_bytes = net->workspace;
     return CADNN_OK;

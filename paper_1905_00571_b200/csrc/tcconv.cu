@@ -58,6 +58,7 @@ struct TcvParams {
     int kb_base, kb_rem;             // stages per block of a cluster: kb_base, and one more in the first kb_rem blocks
     int Rp;                          // K positions per kernel row: kw * c_in rounded up to 16 bytes
     FastDiv d_hw, d_wo, d_ci, d_Rp, d_S, d_nt, d_rows;
+    signed char *pooled;             // int8: the 2 x 2 max pool of the output, written beside it; h_out, w_out, d_hw and d_wo are then the pool's
     int *gave_up;
     Prefetch ahead;
 };
@@ -275,6 +276,15 @@ __device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, in
     return make_uint4(v[0], v[1], v[2], v[3]);
 }
 
+// With a pool the pixels of a tile are numbered by window: pixel m is number m % 4 of window m / 4 (maps of even size, so that the
+// windows of all images form rows of w_out).  Its place among the output's pixels:
+template <bool POOL> __device__ __forceinline__ int place_of(const TcvParams &p, int m)
+{
+    if (!POOL) return m;
+    const int g = m >> 2, r = (int)fdiv((unsigned)g, p.d_wo);
+    return (2 * r + ((m >> 1) & 1)) * (2 * p.w_out) + 2 * (g - r * p.w_out) + (m & 1);
+}
+
 // one int8-layer output value
 __device__ __forceinline__ int finish_q(const TcvParams &p, int sum, float sc, float bi, int r)
 {
@@ -451,7 +461,8 @@ __device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, un
     }
 }
 
-template <bool F32, int PX, int CH, bool SWAP, bool VEC>
+// (POOL is an instantiation of its own: as a branch at run time it cost int8 ResNet-50, which has no such pool, 0.7 %.)
+template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL>
 __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32, PX, CH, SWAP, VEC>::kBlocks) tcconv_kernel(const TcvParams p)
 {
     typedef Cfg<F32, PX, CH, SWAP, VEC> C;
@@ -513,8 +524,13 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
     } else if (tid < PX) {
         const int m = m0 + tid;
-        const int img = (int)fdiv((unsigned)m, p.d_hw), q = m - img * p.h_out * p.w_out;
-        const int oy = (int)fdiv((unsigned)q, p.d_wo), ox = q - oy * p.w_out;
+        const int at = POOL ? m >> 2 : m;
+        const int img = (int)fdiv((unsigned)at, p.d_hw), q = at - img * p.h_out * p.w_out;
+        int oy = (int)fdiv((unsigned)q, p.d_wo), ox = q - oy * p.w_out;
+        if (POOL) {
+            oy = 2 * oy + ((m >> 1) & 1);
+            ox = 2 * ox + (m & 1);
+        }
         const int iy = oy * p.stride - p.pad, ix = ox * p.stride - p.pad_w;
         const int yx = (m < p.M && tid < npx ? iy : kNoPixel) * 65536 | (ix & 0xffff), off = ((img * p.h + iy) * p.w + ix) * p.c_in;
         asm volatile("st.shared.v2.b32 [%0], {%1, %2};\n" ::"r"(pxs + tid * 8), "r"(off), "r"(yx) : "memory");
@@ -737,9 +753,19 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                     if (!F32 && p.vec16) q8[t / 4] = finish_q4(p, t4, res[0].x, sc, bi);
                     else finish4<F32>(p, (size_t)mrow * p.ldc + p.c_off + c4, p.c_out - c4, t4, res[0], sc, bi);
                 }
-                if (!F32 && p.vec16 && nt * CH + j < p.c_out)
-                    *reinterpret_cast<uint4 *>(reinterpret_cast<signed char *>(p.y) + (size_t)mrow * p.ldc + p.c_off + nt * CH + j) =
+                if (!F32 && p.vec16 && nt * CH + j < p.c_out) {
+                    *reinterpret_cast<uint4 *>(reinterpret_cast<signed char *>(p.y) + (size_t)place_of<POOL>(p, mrow) * p.ldc + p.c_off + nt * CH + j) =
                         make_uint4(q8[0], q8[1], q8[2], q8[3]);
+                    if (POOL) {   // the four lanes of a window
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            q8[t] = __vmaxs4(q8[t], __shfl_xor_sync(15u << (lane & 28), q8[t], 1));
+                            q8[t] = __vmaxs4(q8[t], __shfl_xor_sync(15u << (lane & 28), q8[t], 2));
+                        }
+                        if ((lane & 3) == 0)
+                            *reinterpret_cast<uint4 *>(p.pooled + (size_t)(mrow >> 2) * p.c_out + nt * CH + j) = make_uint4(q8[0], q8[1], q8[2], q8[3]);
+                    }
+                }
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -773,7 +799,27 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         // this block has received everything, so the others may go; it goes itself when they have received what it sent
         asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
     }
-    if (mine) {
+    if (POOL && mine) {   // a thread takes the four pixels of a window
+#pragma unroll 1
+        for (int g = r1; 4 * g < rows && m0 + lo + 4 * g < p.M; g += kStep) {
+            const unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (4 * g * C::kRow + col) * 4;
+            const int m = m0 + lo + 4 * g;
+            unsigned best = 0x80808080u;
+#pragma unroll 1
+            for (int i = 0; i < 4; ++i) {
+                uint4 t = lds128(at + i * C::kRow * 4);
+#pragma unroll 4
+                for (int q = 1; q < p.S; ++q) {
+                    const uint4 u = lds128(at + i * C::kRow * 4 + q * slice);
+                    t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+                }
+                const unsigned v = finish_q4(p, t, 0, sc, bi);
+                *reinterpret_cast<unsigned *>(reinterpret_cast<signed char *>(p.y) + (size_t)place_of<POOL>(p, m + i) * p.c_out + co) = v;
+                best = __vmaxs4(best, v);
+            }
+            *reinterpret_cast<unsigned *>(p.pooled + (size_t)(m >> 2) * p.c_out + co) = best;
+        }
+    } else if (mine) {
         unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (r1 * C::kRow + col) * 4;
 #pragma unroll 1
         for (int row = r1; row < rows; row += kAhead * kStep) {
@@ -901,10 +947,10 @@ Pick choose(bool f32, int c_out, long long M, int nkb)
     return best;
 }
 
-template <bool F32, int PX, int CH, bool SWAP, bool VEC>
+template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL>
 cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
 {
-    auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC>;
+    auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC, POOL>;
     typedef Cfg<F32, PX, CH, SWAP, VEC> C;
     const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb);
     if (sp.stages < C::kGroups || sp.stages * C::kParts * 64 * (p.npx + CH) > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
@@ -939,12 +985,12 @@ cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
     return CADNN_OK;
 }
 
-template <bool F32, bool VEC> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
+template <bool F32, bool VEC, bool POOL = false> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
 {
-    if (ch == 64) return launch_one<F32, 128, 64, false, VEC>(p, blocks, pdl, st);
-    if (p.npx <= 64) return launch_one<F32, 64, 128, true, VEC>(p, blocks, pdl, st);
-    if (p.npx <= 128) return launch_one<F32, 128, 128, true, VEC>(p, blocks, pdl, st);
-    return launch_one<F32, 256, 128, true, VEC>(p, blocks, pdl, st);
+    if (ch == 64) return launch_one<F32, 128, 64, false, VEC, POOL>(p, blocks, pdl, st);
+    if (p.npx <= 64) return launch_one<F32, 64, 128, true, VEC, POOL>(p, blocks, pdl, st);
+    if (p.npx <= 128) return launch_one<F32, 128, 128, true, VEC, POOL>(p, blocks, pdl, st);
+    return launch_one<F32, 256, 128, true, VEC, POOL>(p, blocks, pdl, st);
 }
 
 
@@ -1128,6 +1174,15 @@ bool tcv_fits(const cadnn_weights *w, int n)
     return (long long)n * w->h_out * w->w_out < lim && ((long long)n * d.in_h + 2 * d.kh) * d.in_w * d.c_in < lim && d.in_h < 16000 && d.in_w < 16000;
 }
 
+// Whether the layer's launch can write the 2 x 2 max pool of its output too (int8 outputs without residual, whole channel pieces).
+// The pool is then no launch of its own and reads nothing; int8 VGG-16 has five of them: batch 1 152.1 / 141.4 us, batch 4
+// 318 / 313, batch 16 906 / 894.
+bool tcv_pools(const cadnn_weights *w, int n)
+{
+    return w->d_tcv && w->desc.dtype == CADNN_S8 && w->s.kind != KK_FC_SPMV && w->h_out % 2 == 0 && w->w_out % 2 == 0 && w->desc.c_out % 16 == 0 &&
+           tcv_fits(w, n);
+}
+
 cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep, cudaStream_t st)
 {
     const cadnn_layer_desc &d = w->desc;
@@ -1146,8 +1201,14 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     p.c_off = ep.out_c_total > 0 ? ep.out_c_off : 0;
     p.vec_ok = d.c_out % 4 == 0 && p.ldc % 4 == 0 && p.c_off % 4 == 0;
     p.vec16 = ep.out_dtype == CADNN_S8 && d.c_out % 16 == 0 && p.ldc % 16 == 0 && p.c_off % 16 == 0;
+    if (ep.pooled) {
+        if (!tcv_pools(w, n) || ep.residual || ep.out_dtype != CADNN_S8 || ep.out_c_total > 0) return CADNN_E_UNSUPPORTED;
+        p.pooled = (signed char *)ep.pooled;
+        p.h_out /= 2;
+        p.w_out /= 2;
+    }
     p.vec_sb = ((uintptr_t)ep.scale & 15) == 0 && ((uintptr_t)ep.bias & 15) == 0;
-    p.d_hw = make_fastdiv(w->h_out * w->w_out); p.d_wo = make_fastdiv(w->w_out);
+    p.d_hw = make_fastdiv(p.h_out * p.w_out); p.d_wo = make_fastdiv(p.w_out);
     p.d_ci = make_fastdiv(d.c_in); p.d_Rp = make_fastdiv(p.Rp);
     if (ep.prefetch) p.ahead = *ep.prefetch;
     cadnn_status rs = copy_timeout_word(&p.gave_up);
@@ -1166,12 +1227,15 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     p.n_nt = ceil_div(d.c_out, pick.ch);
     // every block of a cluster finishes the same number of pixels, and two stages and the partial sums have to fit
     p.S = pick.px > 128 ? 1 : std::min(pick.split, 16);
-    while (p.S > 1 && (p.npx % p.S || p.S > p.nkb)) --p.S;
+    // (with a pool: whole windows)
+    while (p.S > 1 && (p.npx % p.S || p.S > p.nkb || (p.pooled && p.npx / p.S % 4))) --p.S;
     p.kb_base = p.nkb / p.S; p.kb_rem = p.nkb % p.S;
     p.d_S = make_fastdiv(p.S); p.d_nt = make_fastdiv(p.n_nt); p.d_rows = make_fastdiv(p.npx / p.S);
     const long long blocks = (M + p.npx - 1) / p.npx * p.n_nt * p.S;
     if (blocks > 2147483647ll) return CADNN_E_UNSUPPORTED;
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0;
-    if (f32) return vec ? launch_shape<true, true>(p, pick.ch, (int)blocks, ep.pdl, st) : launch_shape<true, false>(p, pick.ch, (int)blocks, ep.pdl, st);
-    return vec ? launch_shape<false, true>(p, pick.ch, (int)blocks, ep.pdl, st) : launch_shape<false, false>(p, pick.ch, (int)blocks, ep.pdl, st);
+    const int n_blocks = (int)blocks;
+    if (f32) return vec ? launch_shape<true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<true, false>(p, pick.ch, n_blocks, ep.pdl, st);
+    if (p.pooled) return vec ? launch_shape<false, true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
+    return vec ? launch_shape<false, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, false>(p, pick.ch, n_blocks, ep.pdl, st);
 }
