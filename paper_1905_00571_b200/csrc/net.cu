@@ -28,6 +28,7 @@ struct cadnn_net {
     int out_slot = -1;
     bool use_pdl = true;   // layers after the first launch as programmatic dependents
     bool pdl_graph = true;       // ... also inside captured graphs
+    bool link_graph = false;     // ... across the graph's branches too (link_programmatic)
     bool early_trigger = false;
     bool fork_branches = true;   // graph capture: ops off the critical path become parallel branches
     bool planar = false;   // intermediate feature maps are channel-planar with a zero halo (planar.cu)
@@ -419,6 +420,32 @@ cadnn_status launch_deliver(cadnn_net *net, bool pdl, cudaStream_t st)
     return launch_kernel(deliver_kernel, (words + 1023) / 1024, 256, 0, pdl, st, (const int *)net->stage_y, words, (const int *)word, net->deliver_host);
 }
 
+// Edges between kernels that the capture left plain - into a branch, out of it, at a join - become programmatic: the kernel behind
+// starts while the one before drains, and waits for it (for all kernels it has edges from) where it first touches activations, as
+// every layer kernel does.  Joins used to cost a full launch behind the last producer: Inception-V3, batch 1, 453 / 449 us; ResNet-50
+// 318 / 316, int8 216 / 214.5, batch 2 259 / 255.  From batch 4 on the waiting blocks take places that the other branch's could use
+// (ResNet-50 at 25 %, batch 8: 775 / 779).
+cudaError_t link_programmatic(cudaGraph_t graph)
+{
+    size_t n = 0;
+    cudaError_t e = cudaGraphGetEdges_v2(graph, nullptr, nullptr, nullptr, &n);
+    if (e != cudaSuccess || n == 0) return e;
+    std::vector<cudaGraphNode_t> from(n), to(n);
+    std::vector<cudaGraphEdgeData> data(n);
+    e = cudaGraphGetEdges_v2(graph, from.data(), to.data(), data.data(), &n);
+    for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
+        cudaGraphNodeType a, b;
+        if ((e = cudaGraphNodeGetType(from[i], &a)) != cudaSuccess || (e = cudaGraphNodeGetType(to[i], &b)) != cudaSuccess) break;
+        if (a != cudaGraphNodeTypeKernel || b != cudaGraphNodeTypeKernel || data[i].type != cudaGraphDependencyTypeDefault) continue;
+        cudaGraphEdgeData programmatic = {};
+        programmatic.type = cudaGraphDependencyTypeProgrammatic;
+        programmatic.from_port = cudaGraphKernelNodePortProgrammatic;
+        e = cudaGraphRemoveDependencies_v2(graph, &from[i], &to[i], &data[i], 1);
+        if (e == cudaSuccess) e = cudaGraphAddDependencies_v2(graph, &from[i], &to[i], &programmatic, 1);
+    }
+    return e;
+}
+
 // slot 1: a host forward (with deliver_host, the output is delivered behind the last layer)
 cadnn_status forward_impl(cadnn_net *net, const void *x, void *y, int use_graph, cudaStream_t st, int slot)
 {
@@ -467,6 +494,7 @@ cadnn_status forward_impl(cadnn_net *net, const void *x, void *y, int use_graph,
         if (own) cudaStreamDestroy(cap);
         if (s != CADNN_OK) { drop_graph(gc); return s; }
         if (e != cudaSuccess) { drop_graph(gc); return cadnn_note_cuda(e); }
+        if (net->link_graph && (e = link_programmatic(gc.graph)) != cudaSuccess) { drop_graph(gc); return cadnn_note_cuda(e); }
         e = cudaGraphInstantiate(&gc.exec, gc.graph, 0);
         if (e != cudaSuccess) { drop_graph(gc); return cadnn_note_cuda(e); }
         gc.x = x;
@@ -795,6 +823,9 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
         const char *pe = getenv("CADNN_PERSIST");   // "1": on; unset / "0": off
         if (net->planar && pe && atoi(pe) != 0) plan_persistent(net);
     }
+    // (the persistent kernel and the block tensor-core kernel have no wait of their own)
+    net->link_graph = net->pdl_graph && !net->persist && n <= 2;
+    for (const cadnn_op &op : net->ops) net->link_graph = net->link_graph && !(op.w && op.w->has_tc);
     *out = net;
     return CADNN_OK;
 }
