@@ -68,12 +68,18 @@ cadnn_status check_epilogue(const cadnn_weights *w, const cadnn_epilogue *ep, La
     return CADNN_OK;
 }
 
+// The NHWC calls of n images that run on the dense tensor-core route (the others take the kernel of the handle's schedule)
+bool takes_dense(const cadnn_weights *w, int n)
+{
+    return w->d_tcv && tcv_fits(w, n) && (w->s.kind != KK_FC_SPMV || tcv_fc_pays(w, n));
+}
+
 // Layer calls of the tensor-core and small-batch fc kernels are programmatic dependents of whatever their stream runs before:
 // these kernels touch activations, residual, scale, bias and output only behind their wait for it, and their start-up (about
 // a microsecond) overlaps its end.  Not while a stream is being captured: the caller's graph may join branches there.
-bool overlap_start(const cadnn_weights *w, cudaStream_t s)
+bool overlap_start(const cadnn_weights *w, int n, cudaStream_t s)
 {
-    if (!w || !(w->d_tcv || w->s.kind == KK_FC_SPMV)) return false;
+    if (!w || !(takes_dense(w, n) || w->s.kind == KK_FC_SPMV)) return false;   // (sconv_kernel reads scale and bias before its wait)
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &st) != cudaSuccess) { cudaGetLastError(); return false; }
     return st == cudaStreamCaptureStatusNone;
@@ -121,7 +127,7 @@ cadnn_status conv2d_impl(const cadnn_weights *w, const void *x, int n, int h, in
         le.acc_in = (const int *)workspace;
         le.pdl = false;
     }
-    if (w->d_tcv && tcv_fits(w, n) && (w->s.kind != KK_FC_SPMV || tcv_fc_pays(w, n))) return launch_tcv(w, x, n, y, le, s);
+    if (takes_dense(w, n)) return launch_tcv(w, x, n, y, le, s);
     switch (w->s.kind) {
         case KK_SCONV_SPATIAL:
         case KK_SCONV_LINEAR: return launch_sconv(w, x, n, y, le, s);
@@ -137,7 +143,7 @@ extern "C" {
 cadnn_status cadnn_conv2d(const cadnn_weights *w, const void *x, int n, int h, int wd, void *y,
                           const cadnn_epilogue *ep, void *stream)
 {
-    return conv2d_impl(w, x, n, h, wd, y, ep, overlap_start(w, (cudaStream_t)stream), (cudaStream_t)stream);
+    return conv2d_impl(w, x, n, h, wd, y, ep, overlap_start(w, n, (cudaStream_t)stream), (cudaStream_t)stream);
 }
 
 cadnn_status cadnn_weights_workspace_bytes(const cadnn_weights *w, int n, int64_t *bytes)

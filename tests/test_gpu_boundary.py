@@ -89,3 +89,32 @@ def test_graph_replays_read_fresh_input_contents():
             torch.cuda.synchronize()
             want, _ = oracle_forward.forward(m, x)
             assert_close_f32(y.cpu().numpy(), want, "%s replay with seed %d" % (m.name, seed), floor=NET_FLOOR)
+
+
+def test_scale_written_by_the_call_before_a_batch_beyond_the_dense_index_range():
+    """A batch of 2^31 input elements runs on the sparse kernel although the handle has a dense image.  That kernel fetches
+    scale and bias ahead of any wait, so its launch must not overlap the call that writes them (here an fc layer, which lets
+    its dependents start before it stores)."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(61)
+    c_in, c_out, hw = 32, 16, 64
+    n = 2 ** 31 // (hw * hw * c_in)
+    q = gen.int8_weights(g, (c_out, 1, 1, c_in))
+    wh = B.cadnn_pack_q8(B.make_desc(c_in, c_out, 1, 1, 1, 0, 1, hw, hw, 1, "s8"), q, gen.random_mask(g, q.shape, 0.5))
+    # the fc layer: scale = 1e-3 for every channel, from 4096 inputs of one
+    wf = np.full((c_out, 1, 1, 4096), 1e-3 / 4096, np.float32)
+    fc = B.cadnn_pack(B.make_desc(4096, c_out, batch_hint=1), wf, None)
+    ones = torch.ones((1, 4096), device=DEV)
+    x = torch.randint(-127, 128, (n, hw, hw, c_in), dtype=torch.int8, device=DEV)
+    y = torch.zeros((n, hw, hw, c_out), dtype=torch.int8, device=DEV)
+    for _ in range(3):
+        scale = torch.full((1, c_out), 50.0, device=DEV)   # saturates every output, should a block read it too early
+        torch.cuda.synchronize()
+        B.cadnn_fc(fc, ones, scale)
+        B.cadnn_conv2d(wh, x, y, scale=scale, out_dtype="s8")
+        torch.cuda.synchronize()
+        for lo in (0, n // 2, n - 2):   # small calls of the same layer: the dense route, exact as well
+            want = torch.zeros((2, hw, hw, c_out), dtype=torch.int8, device=DEV)
+            B.cadnn_conv2d(wh, x[lo:lo + 2].contiguous(), want, scale=scale, out_dtype="s8")
+            torch.cuda.synchronize()
+            assert torch.equal(y[lo:lo + 2], want) and int(want.abs().max()) < 127
