@@ -185,6 +185,13 @@ __device__ __forceinline__ void send_bulk(unsigned dst, unsigned src, unsigned b
                  ::"r"(dst), "r"(src), "r"(bytes), "r"(bar), "r"(owner) : "memory");
 }
 
+const int kTensorColumns = 512;   // of a multiprocessor
+constexpr int accumulators(bool f32, int n) { return f32 && n <= 64 ? 3 : 2; }
+constexpr int tensor_columns(bool f32, int n)
+{
+    return accumulators(f32, n) * n <= 128 ? 128 : accumulators(f32, n) * n <= 256 ? 256 : 512;
+}
+
 // One kernel shape: PX pixels x CH channels per block.  SWAP: the channels are the 128 rows of the tensor-core tile and
 // the pixels its columns (any multiple of 16 up to PX, so that small maps waste little); otherwise the 128 rows are pixels
 // and the columns CH channels.
@@ -192,15 +199,16 @@ template <bool F32, int PX, int CH, bool SWAP, bool VEC> struct Cfg {
     static const int kParts = F32 ? 3 : 2;                 // operand tiles of 64-byte rows per stage
     static const int kKB = F32 ? 32 : 128;                 // K values per stage (128 source bytes per pixel)
     static const int kWBytes = kParts * CH * 64;
-    // Blocks per multiprocessor the registers are cut for (tensor memory and shared memory for one or two).  Int8 tiles of layers
-    // with few stages are small enough for three (int8 ResNet-50, batch 32: 963 us with 62 to 78 registers and one residual row
-    // ahead, 923 us with 64 and two; four rows 947, eight 998).
-    static const int kBlocks = PX > 128 ? 1 : F32 || !VEC ? 2 : 3;
     static const int kN = SWAP ? PX : CH;
     // Accumulators, kN columns each (kN at most 64: three, by size of the terms; beyond: the large products and the small
     // ones; int8: two that take turns, so that no multiply-add waits for the one before it)
-    static const int kAcc = F32 && kN <= 64 ? 3 : 2;
-    static const int kCols = kAcc * kN <= 128 ? 128 : kAcc * kN <= 256 ? 256 : 512;
+    static const int kAcc = accumulators(F32, kN);
+    static const int kCols = tensor_columns(F32, kN);
+    // Blocks per multiprocessor the registers are cut for (more than tensor memory holds would wait in tcgen05.alloc).  Int8 tiles
+    // of 128 columns and layers with few stages are small enough for three (int8 ResNet-50, batch 32: 963 us with 62 to 78
+    // registers and one residual row ahead, 923 us with 64 and two; four rows 947, eight 998).
+    static const int kBlocks = PX > 128 ? 1 : F32 || !VEC || 3 * kCols > kTensorColumns ? 2 : 3;
+    static_assert(kBlocks * kCols <= kTensorColumns, "a block would wait for tensor memory that its neighbours hold");
     static const int kRow = CH + 4;                        // words per pixel of the exchanged sums (conflict-free 16-byte access)
     static const int kLoadWarps = PX > 128 ? 16 : 8;
     static const int kThreads = (kLoadWarps + 2) * 32;     // + the weight-copy warp and the multiply-add warp
@@ -855,30 +863,52 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
     }
 }
 
-int ceil_div(int a, int b) { return (a + b - 1) / b; }
+constexpr int ceil_div(int a, int b) { return (a + b - 1) / b; }
 
 struct Pick {
     int px, ch, split;   // pixels and channels per block, blocks per cluster
 };
 
+const int kSmemOfSm = 228 * 1024, kSmemReserved = 1024;   // shared memory of a multiprocessor, and what the system takes of it per block
+
 // Shared memory of one block: its pipeline depth, where the exchanged sums and the barriers lie, and its size.
 struct SmemPlan {
     int stages, recv_off, bar_off, bytes;
 };
-SmemPlan plan_smem(bool f32, const Pick &k, int nkb)
+constexpr int tile_pixels(const Pick &k) { return k.ch == 64 ? 128 : k.px <= 64 ? 64 : k.px <= 128 ? 128 : 256; }   // PX of the kernel shape
+constexpr SmemPlan plan_smem(bool f32, const Pick &k, int nkb)
 {
-    const int PX = k.ch == 64 ? 128 : k.px <= 64 ? 64 : k.px <= 128 ? 128 : 256;
+    const int PX = tile_pixels(k);
     const bool swap = k.ch == 128;
     const int stage = (f32 ? 3 : 2) * 64 * (k.px + k.ch), out = k.px * (k.ch + 4) * 4;
     const int budget = (PX > 128 ? 216 : 108) * 1024;   // two blocks share a multiprocessor but for the largest shape
-    SmemPlan s;
+    SmemPlan s = {};
     s.stages = std::max(2, std::min(std::min(4, std::max(2, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
     // sums staged over the stages: unsplit tiles whose rows are channels, and int8 split tiles
     s.recv_off = std::max(s.stages * stage, (swap && k.split == 1) || (!f32 && k.split > 1) ? out : 0);
     s.bar_off = (s.recv_off + (k.split > 1 ? out : 0) + 127) / 128 * 128;
     s.bytes = s.bar_off + 1024 + 128 + PX * 8;
+    // Blocks of a cluster wait for each other while they hold tensor memory.  Were more of them resident than it has columns for,
+    // two clusters could each hold what the other's last block waits for; so a block of c columns takes more than c / 640 of the
+    // multiprocessor's shared memory, and five quarters of the columns never fit.  (Other blocks hold columns too, but finish by
+    // themselves.)
+    if (k.split > 1) s.bytes = std::max(s.bytes, (tensor_columns(f32, swap ? PX : k.ch) / 128 * kSmemOfSm / 5 - kSmemReserved + 128) & ~127);
     return s;
 }
+constexpr bool clusters_find_tensor_memory()
+{
+    for (int f32 = 0; f32 < 2; ++f32)
+        for (int px = 16; px <= 128; px += 16)
+            for (int ch = 64; ch <= 128; ch += 64)
+                for (int split = 2; split <= 16; ++split)
+                    for (int nkb = split; nkb <= 5 * split; ++nkb) {
+                        const Pick k = {ch == 64 ? 128 : px, ch, split};
+                        if (5 * (plan_smem(f32, k, nkb).bytes + kSmemReserved) <= tensor_columns(f32, ch == 64 ? 64 : tile_pixels(k)) / 128 * kSmemOfSm)
+                            return false;
+                    }
+    return true;
+}
+static_assert(clusters_find_tensor_memory(), "clusters of split tiles could wait for each other's tensor memory");
 
 // Block shape of a layer: the one a time model calls the fastest.  The model is linear in what a block does, with
 // coefficients fitted to 3900 measured shapes (212 layers of the workloads at batch 1 to 128, launched back to back as
