@@ -56,6 +56,7 @@ struct TcvParams {
     int stages, recv_off, bar_off;   // pipeline depth; byte offsets of the partial sums and of the barriers in shared memory
     int ldc, c_off, vec_ok, vec_sb, vec16;  // vec_ok / vec_sb: output and residual / scale and bias allow 4 channels per access; vec16: int8 output 16
     int kb_base, kb_rem;             // stages per block of a cluster: kb_base, and one more in the first kb_rem blocks
+    int whole, tail;                 // int8 input: bytes of its whole 4-byte words, and bytes behind them
     int Rp;                          // K positions per kernel row: kw * c_in rounded up to 16 bytes
     FastDiv d_hw, d_wo, d_ci, d_Rp, d_S, d_nt, d_rows;
     signed char *pooled;             // int8: the 2 x 2 max pool of the output, written beside it; h_out, w_out, d_hw and d_wo are then the pool's
@@ -247,8 +248,9 @@ __device__ __forceinline__ uint4 gather_vec(const TcvParams &p, const Px &r, int
 }
 // The same when a pixel's channels are not a multiple of 16 bytes: positions r .. of row ky of the window, whose kw * c_in values
 // lie behind each other in memory.  Values of the columns outside the image read as zero; positions past the row's end meet
-// zero weights.  Floats come one by one; int8 values as the aligned words that hold any wanted one, shifted into place.
-template <bool F32>
+// zero weights.  Floats come one by one; int8 values as the aligned words that hold any wanted one, shifted into place
+// (TAIL: the tensor's last word is not whole, and its bytes are left to patch_tail).
+template <bool F32, bool TAIL>
 __device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, int ky, int r)
 {
     const int iy = (px.yx >> 16) + ky, ix = (int)(short)px.yx;
@@ -266,6 +268,7 @@ __device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, in
         }
         return make_uint4(v[0], v[1], v[2], v[3]);
     }
+    if (TAIL) b = min(b, p.whole - o);
     const int s = o & 3;
     const char *x = reinterpret_cast<const char *>(p.x) + (o - s);
     unsigned w[5];
@@ -282,6 +285,18 @@ __device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, in
         v[i] = __funnelshift_r(w[i], w[i + 1], 8 * s) & upto & ~below;
     }
     return make_uint4(v[0], v[1], v[2], v[3]);
+}
+// The bytes behind the tensor's last whole word, written over the zeros that gather_run gave for them (addr: where its 16 bytes lie
+// in shared memory).
+__device__ __forceinline__ void patch_tail(const TcvParams &p, const Px &px, int ky, int r, unsigned addr)
+{
+    const int iy = (px.yx >> 16) + ky, ix = (int)(short)px.yx;
+    if ((unsigned)iy >= (unsigned)p.h || ky >= p.kh) return;
+    const int a = max(0, -ix * p.c_in - r), b = min(min(p.kw, p.w - ix) * p.c_in - r, 16);
+    const int at = p.whole - (px.off + ky * p.w * p.c_in + r);   // position of the first of them
+    for (int j = 0; j < p.tail; ++j)
+        if (at + j >= a && at + j < b)
+            asm volatile("st.shared.u8 [%0], %1;\n" ::"r"(addr + at + j), "r"((int)ld_act(reinterpret_cast<const signed char *>(p.x) + p.whole + j)) : "memory");
 }
 
 // With a pool the pixels of a tile are numbered by window: pixel m is number m % 4 of window m / 4 (maps of even size, so that the
@@ -469,8 +484,9 @@ __device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, un
     }
 }
 
-// (POOL is an instantiation of its own: as a branch at run time it cost int8 ResNet-50, which has no such pool, 0.7 %.)
-template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL>
+// (POOL and TAIL are instantiations of their own: as branches at run time they cost the int8 ResNet-50, which has neither such a pool
+// nor such a tensor, 0.7 and 0.4 %.)
+template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL, bool TAIL>
 __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32, PX, CH, SWAP, VEC>::kBlocks) tcconv_kernel(const TcvParams p)
 {
     typedef Cfg<F32, PX, CH, SWAP, VEC> C;
@@ -563,7 +579,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
 #pragma unroll
             for (int i = 0; i < C::kRPT; ++i) {
                 const Px px = load_px(pxs + (r0 + kPS * i) * 8);
-                v[i] = VEC ? gather_vec<F32>(p, px, ky, kx, ci) : gather_run<F32>(p, px, ky, ci);
+                v[i] = VEC ? gather_vec<F32>(p, px, ky, kx, ci) : gather_run<F32, TAIL>(p, px, ky, ci);
             }
             ci += C::kGroups * C::kKB;
             const int wrap = VEC ? p.c_in : p.Rp;
@@ -597,6 +613,12 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                     sts64(a + i * (kPS * 64) + xpart, m0_, m1);
                     sts64(a + i * (kPS * 64) + 2 * xpart, l0, l1);
                 }
+            }
+            if (TAIL) {
+                const int k = kb * C::kKB + c * (C::kKB / 8), row = (int)fdiv((unsigned)k, p.d_Rp);
+#pragma unroll 1
+                for (int i = 0; i < C::kRPT && (!SWAP || r0 + kPS * i < npx); ++i)
+                    patch_tail(p, load_px(pxs + (r0 + kPS * i) * 8), row, k - row * p.Rp, a + i * (kPS * 64));
             }
             if (kb + C::kGroups < kb1) request();
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
@@ -977,10 +999,10 @@ Pick choose(bool f32, int c_out, long long M, int nkb)
     return best;
 }
 
-template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL>
+template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL, bool TAIL>
 cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
 {
-    auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC, POOL>;
+    auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC, POOL, TAIL>;
     typedef Cfg<F32, PX, CH, SWAP, VEC> C;
     const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb);
     if (sp.stages < C::kGroups || sp.stages * C::kParts * 64 * (p.npx + CH) > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
@@ -1015,14 +1037,13 @@ cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
     return CADNN_OK;
 }
 
-template <bool F32, bool VEC, bool POOL = false> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
+template <bool F32, bool VEC, bool POOL = false, bool TAIL = false> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
 {
-    if (ch == 64) return launch_one<F32, 128, 64, false, VEC, POOL>(p, blocks, pdl, st);
-    if (p.npx <= 64) return launch_one<F32, 64, 128, true, VEC, POOL>(p, blocks, pdl, st);
-    if (p.npx <= 128) return launch_one<F32, 128, 128, true, VEC, POOL>(p, blocks, pdl, st);
-    return launch_one<F32, 256, 128, true, VEC, POOL>(p, blocks, pdl, st);
+    if (ch == 64) return launch_one<F32, 128, 64, false, VEC, POOL, TAIL>(p, blocks, pdl, st);
+    if (p.npx <= 64) return launch_one<F32, 64, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);
+    if (p.npx <= 128) return launch_one<F32, 128, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);
+    return launch_one<F32, 256, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);
 }
-
 
 }  // namespace
 
@@ -1226,6 +1247,8 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     p.act = ep.act; p.out_dtype = ep.out_dtype;
     p.h = d.in_h; p.w = d.in_w; p.c_in = d.c_in; p.h_out = w->h_out; p.w_out = w->w_out; p.c_out = d.c_out;
     p.stride = d.stride; p.pad = d.pad; p.pad_w = d.pad_w; p.kh = d.kh; p.kw = d.kw;
+    const long long in_bytes = (long long)n * d.in_h * d.in_w * d.c_in;   // (of int8)
+    p.whole = (int)(in_bytes & ~3ll); p.tail = (int)(in_bytes & 3);
     p.M = (int)M; p.Rp = row_positions(d); p.nkb = stages_of(d);
     p.ldc = ep.out_c_total > 0 ? ep.out_c_total : d.c_out;
     p.c_off = ep.out_c_total > 0 ? ep.out_c_off : 0;
@@ -1266,6 +1289,9 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0;
     const int n_blocks = (int)blocks;
     if (f32) return vec ? launch_shape<true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<true, false>(p, pick.ch, n_blocks, ep.pdl, st);
+    if (p.tail && !vec)
+        return p.pooled ? launch_shape<false, false, true, true>(p, pick.ch, n_blocks, ep.pdl, st)
+                        : launch_shape<false, false, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
     if (p.pooled) return vec ? launch_shape<false, true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
     return vec ? launch_shape<false, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, false>(p, pick.ch, n_blocks, ep.pdl, st);
 }

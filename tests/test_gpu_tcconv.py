@@ -139,3 +139,23 @@ def test_small_batch_fc_takes_the_dense_route_where_it_pays(dtype):
             B.cadnn_fc(B.cadnn_pack(d, w, mask), dev(x.reshape(n, c_in)), y)
             torch.cuda.synchronize()
             assert_close_or_bounded(y.cpu().numpy(), want, s_abs, c_in, "fc f32, batch %d" % n)
+
+
+@pytest.mark.parametrize("shape", ["128,64,1", "16,128,1", "128,128,1", "256,128,1", None])
+@pytest.mark.parametrize("h,w,c_in,k", [(5, 5, 1, 3), (3, 5, 3, 3), (7, 3, 7, 1), (5, 7, 9, 3), (9, 1, 35, 1), (6, 7, 3, 5)])
+def test_int8_tensors_that_end_inside_a_word(h, w, c_in, k, shape, monkeypatch):
+    """Sizes of 1, 2 and 3 modulo 4 bytes: the last bytes are fetched one by one, nothing behind the tensor is read, and they
+    take part in the result (bytes of another value follow them here)."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(59 + c_in)
+    size = h * w * c_in
+    x = np.ascontiguousarray(gen.int8_image(g, (1, h, w, c_in)))
+    q = gen.int8_weights(g, (70, k, k, c_in))
+    want = ref.conv2d_s8(x, q, None, 1, k // 2, out="s32")
+    wh = _pack(B, monkeypatch, shape, "s8", (1, h, w, c_in, 70, k, 1, k // 2), q, None)
+    flat = torch.full((size + 64,), 77, dtype=torch.int8, device=DEV)
+    flat[:size] = torch.from_numpy(x.reshape(-1)).to(DEV)
+    y = torch.zeros(want.shape, dtype=torch.int32, device=DEV)
+    B.cadnn_conv2d(wh, flat[:size].view(1, h, w, c_in), y, out_dtype="s32")
+    torch.cuda.synchronize()
+    assert_exact(y.cpu().numpy(), want, "%d bytes" % size)
