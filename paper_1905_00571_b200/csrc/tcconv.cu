@@ -246,6 +246,13 @@ __device__ __forceinline__ uint4 gather_vec(const TcvParams &p, const Px &r, int
     }
     return v;
 }
+// mask of the bytes n .. of a word, empty from n = 4 on (the instruction takes shifts beyond the width as the width)
+__device__ __forceinline__ unsigned from_byte(int n)
+{
+    unsigned m;
+    asm("shl.b32 %0, 0xffffffff, %1;\n" : "=r"(m) : "r"(8 * n));
+    return m;
+}
 // The same when a pixel's channels are not a multiple of 16 bytes: positions r .. of row ky of the window, whose kw * c_in values
 // lie behind each other in memory.  Values of the columns outside the image read as zero; positions past the row's end meet
 // zero weights.  Floats come one by one; int8 values as the aligned words that hold any wanted one, shifted into place
@@ -271,18 +278,17 @@ __device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, in
     if (TAIL) b = min(b, p.whole - o);
     const int s = o & 3;
     const char *x = reinterpret_cast<const char *>(p.x) + (o - s);
+    const int first = a + s, end = a < min(b, 16) ? min(b, 16) + s : 0;   // the wanted bytes of those words
     unsigned w[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
         w[i] = 0;
-        if (max(a, 4 * i - s) < min(min(b, 16), 4 * i - s + 4)) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(w[i]) : "l"(x + 4 * i));
+        if (4 * i + 4 > first && 4 * i < end) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(w[i]) : "l"(x + 4 * i));
     }
     unsigned v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        const int lo = min(max(a - 4 * i, 0), 4), hi = min(max(b - 4 * i, 0), 4);
-        const unsigned below = lo >= 4 ? 0xffffffffu : (1u << (8 * lo)) - 1, upto = hi >= 4 ? 0xffffffffu : (1u << (8 * hi)) - 1;
-        v[i] = __funnelshift_r(w[i], w[i + 1], 8 * s) & upto & ~below;
+        v[i] = __funnelshift_r(w[i], w[i + 1], 8 * s) & from_byte(max(a - 4 * i, 0)) & ~from_byte(max(b - 4 * i, 0));
     }
     return make_uint4(v[0], v[1], v[2], v[3]);
 }
@@ -294,6 +300,7 @@ __device__ __forceinline__ void patch_tail(const TcvParams &p, const Px &px, int
     if ((unsigned)iy >= (unsigned)p.h || ky >= p.kh) return;
     const int a = max(0, -ix * p.c_in - r), b = min(min(p.kw, p.w - ix) * p.c_in - r, 16);
     const int at = p.whole - (px.off + ky * p.w * p.c_in + r);   // position of the first of them
+#pragma unroll 1
     for (int j = 0; j < p.tail; ++j)
         if (at + j >= a && at + j < b)
             asm volatile("st.shared.u8 [%0], %1;\n" ::"r"(addr + at + j), "r"((int)ld_act(reinterpret_cast<const signed char *>(p.x) + p.whole + j)) : "memory");
@@ -1041,8 +1048,8 @@ template <bool F32, bool VEC, bool POOL = false, bool TAIL = false> cadnn_status
 {
     if (ch == 64) return launch_one<F32, 128, 64, false, VEC, POOL, TAIL>(p, blocks, pdl, st);
     if (p.npx <= 64) return launch_one<F32, 64, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);
-    if (p.npx <= 128) return launch_one<F32, 128, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);
-    return launch_one<F32, 256, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);
+    if (TAIL || p.npx <= 128) return launch_one<F32, 128, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);   // (256 pixels would spill registers)
+    return launch_one<F32, 256, 128, true, VEC, POOL, false>(p, blocks, pdl, st);
 }
 
 }  // namespace
@@ -1275,7 +1282,8 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
         pick = choose(f32, d.c_out, M, p.nkb);
         w->tcv_pick.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
     }
-    if (pick.ch == 64) pick.px = 128;
+    const bool vec = d.c_in % (f32 ? 4 : 16) == 0, run_tail = !f32 && !vec && p.tail;
+    if (pick.ch == 64 || (run_tail && pick.px > 128)) pick.px = 128;
     p.npx = pick.px;
     p.n_nt = ceil_div(d.c_out, pick.ch);
     // every block of a cluster finishes the same number of pixels, and two stages and the partial sums have to fit
@@ -1286,10 +1294,9 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     p.d_S = make_fastdiv(p.S); p.d_nt = make_fastdiv(p.n_nt); p.d_rows = make_fastdiv(p.npx / p.S);
     const long long blocks = (M + p.npx - 1) / p.npx * p.n_nt * p.S;
     if (blocks > 2147483647ll) return CADNN_E_UNSUPPORTED;
-    const bool vec = d.c_in % (f32 ? 4 : 16) == 0;
     const int n_blocks = (int)blocks;
     if (f32) return vec ? launch_shape<true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<true, false>(p, pick.ch, n_blocks, ep.pdl, st);
-    if (p.tail && !vec)
+    if (run_tail)
         return p.pooled ? launch_shape<false, false, true, true>(p, pick.ch, n_blocks, ep.pdl, st)
                         : launch_shape<false, false, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
     if (p.pooled) return vec ? launch_shape<false, true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
