@@ -1176,7 +1176,7 @@ bool tcv_fc_pays(const cadnn_weights *w, int n)
     return n >= 3 && 3.7 + dense_mb / (f32 ? 7.0 : 8.0) < 2.5 + 1.6e-6 * n * (double)w->nnz;
 }
 
-// Builds the dense image of a handle whose sparse (or dense stem) image is on the device.
+// Builds the dense image of a handle whose sparse (or dense stem) image is on the device, where there is memory for it.
 cadnn_status tcv_build(cadnn_weights *h)
 {
     const cadnn_layer_desc &d = h->desc;
@@ -1189,12 +1189,14 @@ cadnn_status tcv_build(cadnn_weights *h)
     const bool s8 = d.dtype == CADNN_S8;
     const ImageDims dims = {stages_of(d), row_positions(d)};
     const size_t bytes = (size_t)ceil_div(d.c_out, 64) * dims.nkb * (s8 ? 2 : 3) * 4096;
-    h->tcv_bytes = bytes;
     const cudaError_t er = cudaMalloc(&h->d_tcv, bytes);
-    if (er != cudaSuccess) {
-        cadnn_note_cuda(er);
-        return er == cudaErrorMemoryAllocation ? CADNN_E_ALLOC : CADNN_E_CUDA;
+    if (er == cudaErrorMemoryAllocation) {   // the layer runs without it
+        cudaGetLastError();
+        h->d_tcv = nullptr;
+        return CADNN_OK;
     }
+    CADNN_CUDA_TRY(er);
+    h->tcv_bytes = bytes;
     if (h->s.kind == KK_DENSE_SMALLC) {   // few weights, kept tap-major: written on the host
         std::vector<unsigned char> image(bytes, 0);
         for (int co = 0; co < d.c_out; ++co)

@@ -159,3 +159,31 @@ def test_int8_tensors_that_end_inside_a_word(h, w, c_in, k, shape, monkeypatch):
     B.cadnn_conv2d(wh, flat[:size].view(1, h, w, c_in), y, out_dtype="s32")
     torch.cuda.synchronize()
     assert_exact(y.cpu().numpy(), want, "%d bytes" % size)
+
+
+def test_no_memory_for_the_dense_image_leaves_the_sparse_route():
+    """The dense image (200 MB here) is optional: with 100 MB of device memory left the layer packs all the same, and computes
+    what it computes with the image."""
+    from paper_1905_00571_b200 import binding as B
+    g = np.random.default_rng(63)
+    n, c_in, c_out = 16, 8192, 4096
+    w = g.standard_normal((c_out, 1, 1, c_in), dtype=np.float32) * np.float32(0.02)
+    mask = (g.random(w.shape, dtype=np.float32) < 0.03).astype(np.uint8)
+    x = torch.from_numpy(g.standard_normal((n, c_in), dtype=np.float32)).to(DEV)
+    d = B.make_desc(c_in, c_out, batch_hint=n)
+    y = [torch.zeros((n, c_out), device=DEV) for _ in range(2)]
+    B.cadnn_fc(B.cadnn_pack(d, w, mask), x, y[0])
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - (100 << 20), dtype=torch.uint8, device=DEV)
+    try:
+        wh = B.cadnn_pack(d, w, mask)
+    finally:
+        del hog
+        torch.cuda.empty_cache()
+    B.cadnn_fc(wh, x, y[1])
+    torch.cuda.synchronize()
+    # two sums of at most 330 products in different orders: each within 330 * 2^-24 of sum |w x|
+    s_abs = x.abs().cpu().numpy().astype(np.float64) @ np.abs(w * mask).reshape(c_out, c_in).astype(np.float64).T
+    terms = int(mask.reshape(c_out, -1).sum(1).max())
+    assert (np.abs(y[0].cpu().numpy().astype(np.float64) - y[1].cpu().numpy()) <= 2 * terms * 2.0 ** -24 * s_abs).all()
