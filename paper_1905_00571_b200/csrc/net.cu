@@ -49,7 +49,8 @@ struct cadnn_net {
     // device staging for cadnn_forward_host
     void *stage_x = nullptr, *stage_y = nullptr;
     int64_t in_bytes = 0, out_bytes = 0;
-    // small outputs: pinned host memory into which the last kernel of a host forward writes the output, then the give-up counter
+    // small outputs: pinned host memory (behind status_host) into which the last kernel of a host forward writes the output, then
+    // the give-up counter
     int *deliver_host = nullptr;
     // int32 sums of block-structured layers (tensor-core blocks), shared by all such ops of the net
     void *tc_ws = nullptr;
@@ -797,11 +798,13 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
         }
         net->workspace += net->tc_ws_bytes;
     }
-    if (cudaHostAlloc((void **)&net->status_host, 2 * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
+    const bool deliver = net->out_bytes <= kDeliverBytes;
+    if (cudaHostAlloc((void **)&net->status_host, deliver ? (size_t)net->out_bytes + 32 : 2 * sizeof(int), cudaHostAllocDefault) != cudaSuccess) {
         cudaGetLastError();
         cadnn_net_free(net);
         return CADNN_E_ALLOC;
     }
+    if (deliver) net->deliver_host = net->status_host + 4;
     if (read_copy_timeouts(&net->status_seen[0]) != CADNN_OK || read_barrier_timeouts(&net->status_seen[1]) != CADNN_OK) {
         cadnn_net_free(net);
         return CADNN_E_CUDA;
@@ -823,6 +826,7 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
         const char *pe = getenv("CADNN_PERSIST");   // "1": on; unset / "0": off
         if (net->planar && pe && atoi(pe) != 0) plan_persistent(net);
     }
+    if (net->persist) net->deliver_host = nullptr;
     // (the persistent kernel and the block tensor-core kernel have no wait of their own)
     net->link_graph = net->pdl_graph && !net->persist && n <= 2;
     for (const cadnn_op &op : net->ops) net->link_graph = net->link_graph && !(op.w && op.w->has_tc);
@@ -847,12 +851,6 @@ cadnn_status cadnn_forward_host(cadnn_net *net, const void *x_host, void *y_host
             cadnn_note_cuda(e);
             return e == cudaErrorMemoryAllocation ? CADNN_E_ALLOC : CADNN_E_CUDA;
         }
-    }
-    if (!net->deliver_host && net->out_bytes <= kDeliverBytes && !net->persist &&
-        cudaHostAlloc((void **)&net->deliver_host, (size_t)net->out_bytes + 16, cudaHostAllocDefault) != cudaSuccess) {
-        cudaGetLastError();
-        net->deliver_host = nullptr;
-        return CADNN_E_ALLOC;
     }
     CADNN_CUDA_TRY(cudaMemcpyAsync(net->stage_x, x_host, (size_t)net->in_bytes, cudaMemcpyHostToDevice, st));
     cadnn_status s = forward_impl(net, net->stage_x, net->stage_y, use_graph, st, 1);
@@ -1007,7 +1005,6 @@ void cadnn_net_free(cadnn_net *net)
     if (net->flush) cudaFree(net->flush);
     if (net->tc_ws) cudaFree(net->tc_ws);
     if (net->status_host) cudaFreeHost(net->status_host);
-    if (net->deliver_host) cudaFreeHost(net->deliver_host);
     persist_free(net->persist);
     delete net;
 }

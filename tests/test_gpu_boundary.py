@@ -118,3 +118,24 @@ def test_scale_written_by_the_call_before_a_batch_beyond_the_dense_index_range()
             B.cadnn_conv2d(wh, x[lo:lo + 2].contiguous(), want, scale=scale, out_dtype="s8")
             torch.cuda.synchronize()
             assert torch.equal(y[lo:lo + 2], want) and int(want.abs().max()) < 127
+
+
+@pytest.mark.parametrize("hw,c_out", [(5, 3), (64, 16), (64, 17)])
+def test_host_forwards_of_small_and_large_outputs(hw, c_out):
+    """Outputs of up to 64 KB are written to pinned host memory by a last kernel (75 bytes and exactly 64 KB here), larger ones
+    are copied; both equal the device forward, with and without a graph."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(67)
+    q = gen.int8_weights(g, (c_out, 1, 1, 16))
+    m = torch.full((c_out,), 1e-2, device=DEV)
+    wh = B.cadnn_pack_q8(B.make_desc(16, c_out, 1, 1, 1, 0, 1, hw, hw, 1, "s8"), q, None)
+    ops = [B.Op(B.OP_CONV, wh.handle, 0, 1, -1, m.data_ptr(), None, 0, B.S8, 0, 0, 0)]
+    net = B.cadnn_net_create(ops, 1, hw, hw, 16, "s8", keep=(wh, m))
+    want = torch.zeros((1, hw, hw, c_out), dtype=torch.int8, device=DEV)
+    got = torch.zeros((1, hw, hw, c_out), dtype=torch.int8).pin_memory()
+    for i, graph in enumerate((True, True, False)):
+        x = torch.from_numpy(gen.int8_image(g, (1, hw, hw, 16)))
+        B.cadnn_forward(net, x.to(DEV), want, False, None)
+        torch.cuda.synchronize()
+        B.cadnn_forward_host(net, x.pin_memory(), got, graph)
+        assert torch.equal(got, want.cpu()) and int(want.abs().max()) > 0, i
