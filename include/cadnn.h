@@ -123,8 +123,9 @@ cadnn_status cadnn_pack(const cadnn_layer_desc *desc, const float *w_ohwi, const
 cadnn_status cadnn_pack_q8(const cadnn_layer_desc *desc, const int8_t *q_ohwi, const uint8_t *mask,
                            cadnn_weights **out);
 
-/* nnz = kept positions; packed_bytes = bytes of the device image; fmt = cadnn_fmt used.
- * Any output pointer may be NULL. */
+/* nnz = kept positions; packed_bytes = bytes of all device images of the handle (compressed, channel-planar and its
+ * parity form, dense blocks, dense image; a host-only pack counts what it would upload, without the dense image);
+ * fmt = cadnn_fmt used.  Any output pointer may be NULL. */
 cadnn_status cadnn_weights_info(const cadnn_weights *w, int64_t *nnz, int64_t *packed_bytes, int *fmt);
 
 /*

@@ -181,7 +181,7 @@ cadnn_status upload(cadnn_weights *h)
     size_t b_pse = h->ps_ent.size() * 4, b_psp = h->ps_perm.size() * 4;
     size_t o_ple = o_ent + al(b_ent), o_plp = o_ple + al(b_ple), o_plo = o_plp + al(b_plp), o_pse = o_plo + al(b_plo);
     size_t o_psp = o_pse + al(b_pse), total = o_psp + al(b_psp);
-    h->packed_bytes = (int64_t)(b_vals + b_offs + b_ptr + b_perm + b_dense + b_ent);
+    h->packed_bytes = (int64_t)(b_vals + b_offs + b_ptr + b_perm + b_dense + b_ent + b_ple + b_plp + b_plo + b_pse + b_psp);
     if (h->desc.flags & CADNN_PACK_HOST_ONLY) return CADNN_OK;
     if (total == 0) total = 256;
     CADNN_CUDA_TRY(cudaGetDevice(&h->device));
@@ -1555,7 +1555,7 @@ cadnn_status cadnn_weights_info(const cadnn_weights *w, int64_t *nnz, int64_t *p
 {
     if (!w) return CADNN_E_ARG;
     if (nnz) *nnz = w->nnz;
-    if (packed_bytes) *packed_bytes = w->packed_bytes;
+    if (packed_bytes) *packed_bytes = w->packed_bytes + (int64_t)w->tcv_bytes + (w->half ? w->half->packed_bytes : 0);
     if (fmt) *fmt = w->fmt;
     return CADNN_OK;
 }

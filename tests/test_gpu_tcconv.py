@@ -181,9 +181,37 @@ def test_no_memory_for_the_dense_image_leaves_the_sparse_route():
     finally:
         del hog
         torch.cuda.empty_cache()
+    assert B.cadnn_weights_info(wh)["packed_bytes"] < 100 << 20
     B.cadnn_fc(wh, x, y[1])
     torch.cuda.synchronize()
     # two sums of at most 330 products in different orders: each within 330 * 2^-24 of sum |w x|
     s_abs = x.abs().cpu().numpy().astype(np.float64) @ np.abs(w * mask).reshape(c_out, c_in).astype(np.float64).T
     terms = int(mask.reshape(c_out, -1).sum(1).max())
     assert (np.abs(y[0].cpu().numpy().astype(np.float64) - y[1].cpu().numpy()) <= 2 * terms * 2.0 ** -24 * s_abs).all()
+
+
+@pytest.mark.parametrize("kind", ["conv f32", "conv stride 2", "conv s8", "fc f32", "fc s8, small batch"])
+def test_reported_bytes_cover_the_device_memory_of_a_handle(kind):
+    """packed_bytes against the fall of the device's free memory over twenty handles.  An allocation
+    takes at most 2 MB more than asked for, and a handle has three: its images, its dense image, its parity form."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(65)
+    s8 = "s8" in kind
+    if kind.startswith("fc"):
+        d, shape = B.make_desc(2048, 1000, batch_hint=8 if "small" in kind else 32, dtype="s8" if s8 else "f32"), (1000, 1, 1, 2048)
+    else:
+        d, shape = B.make_desc(256, 250, 3, 3, 2 if "2" in kind.split()[-1] else 1, 1, 1, 14, 14, 1, "s8" if s8 else "f32"), (250, 3, 3, 256)
+    w = gen.int8_weights(g, shape) if s8 else gen.he_weights(g, *shape)
+    mask = gen.random_mask(g, shape, 0.3)
+    pack = B.cadnn_pack_q8 if s8 else B.cadnn_pack
+    first = pack(d, w, mask)
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    n = 20
+    handles = [pack(d, w, mask) for _ in range(n)]
+    used = (free - torch.cuda.mem_get_info()[0]) / n
+    told = B.cadnn_weights_info(handles[0])["packed_bytes"]
+    assert told == B.cadnn_weights_info(first)["packed_bytes"]
+    dense = (250 + 63) // 64 * 64 * 9 * 256 * (1 if s8 else 6) if kind.startswith("conv") else 1024 * 2048 * (1 if s8 else 6)
+    assert told >= dense, (told, dense)
+    assert told <= used + 2 ** 21 and used <= told + 3 * 2 ** 21, (told, used)
