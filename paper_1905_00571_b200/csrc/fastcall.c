@@ -5,6 +5,7 @@
  */
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
+#include <limits.h>
 #include "cadnn.h"
 
 static PyObject *g_check, *g_act, *g_dtype;            /* binding._check, binding.ACT, binding.DTYPE */
@@ -38,12 +39,18 @@ static int parse(PyObject *const *args, Py_ssize_t nargs, PyObject *kwnames, con
     return 0;
 }
 
+/* (the C ABI takes int: what does not fit is refused, not cut) */
 static int as_int(PyObject *o, int dflt, int *v)
 {
     if (!o) { *v = dflt; return 0; }
     const long l = PyLong_AsLong(o);
+    if (l == -1 && PyErr_Occurred()) return -1;
+    if (l < INT_MIN || l > INT_MAX) {
+        PyErr_Format(PyExc_OverflowError, "%ld does not fit a C int", l);
+        return -1;
+    }
     *v = (int)l;
-    return l == -1 && PyErr_Occurred() ? -1 : 0;
+    return 0;
 }
 
 /* device pointer of a tensor (None = NULL) */
@@ -86,11 +93,8 @@ static int shape_dims(PyObject *t, int *d, int want)
         Py_DECREF(f);
         return -1;
     }
-    for (int i = 0; i < want; ++i) {
-        const long v = PyLong_AsLong(PySequence_Fast_GET_ITEM(f, i));
-        if (v == -1 && PyErr_Occurred()) { Py_DECREF(f); return -1; }
-        d[i] = (int)v;
-    }
+    for (int i = 0; i < want; ++i)
+        if (as_int(PySequence_Fast_GET_ITEM(f, i), 0, &d[i])) { Py_DECREF(f); return -1; }
     Py_DECREF(f);
     return 0;
 }

@@ -197,3 +197,28 @@ def test_parity_form_of_a_stride2_layer_is_the_same_layer(B, k, h, w):
     got = ref.conv2d_f32(planes, w2, m2, 1, pad)
     assert got.shape == want.shape
     np.testing.assert_allclose(got, want, rtol=1e-6, atol=1e-6)
+
+
+class _FakeTensor:
+    def __init__(self, *shape):
+        self.shape = shape
+
+    def data_ptr(self):
+        return 0
+
+
+def test_numbers_beyond_a_c_int_are_refused_by_the_marshalling(B):
+    """2^32 + 1 images are not one image: sizes and counts that do not fit the ABI's int raise instead of being cut to 32 bits."""
+    wh = _host_pack(B, np.ones((8, 1, 1, 8), np.float32), None, 1, 1, 0)
+    y = _FakeTensor(1, 8)
+    for bad in (2 ** 32 + 1, 2 ** 31, -2 ** 31 - 1):
+        with pytest.raises(OverflowError):
+            B.cadnn_fc(wh, _FakeTensor(bad, 8), y, stream=0)
+        with pytest.raises(OverflowError):
+            B.cadnn_conv2d(wh, _FakeTensor(1, bad, 1, 8), y, stream=0)
+        with pytest.raises(OverflowError):
+            B.cadnn_conv2d(wh, _FakeTensor(1, 1, 1, 8), y, stream=0, out_c_total=bad)
+        with pytest.raises(OverflowError):
+            B.cadnn_fc(wh, _FakeTensor(1, 8), y, stream=0, act=bad)
+    with pytest.raises(B.CadnnError):   # one image passes the marshalling; the host-only handle is refused behind it
+        B.cadnn_fc(wh, _FakeTensor(1, 8), y, stream=0)
