@@ -73,7 +73,7 @@ struct TuneRecord {
     Schedule s;
     PsSchedule ps;
     int pl_T, pl_NW, pl_RPW, pl_KSW, pl_D, use_ps;
-    float pl_us, ps_us, nhwc_us;
+    float pl_us, ps_us, nhwc_us, tcv_us;
 };
 
 struct cadnn_weights {
@@ -120,7 +120,8 @@ struct cadnn_weights {
     bool use_ps = false;             // the network runner prefers it over the direct planar kernel
     PsSchedule ps;
     float ps_us = -1.0f, pl_us = -1.0f;   // measured time of the staged / direct planar kernel (autotune), microseconds
-    float nhwc_us = -1.0f;                // ... and of the NHWC kernel
+    float nhwc_us = -1.0f;                // ... of the NHWC sparse kernel
+    float tcv_us = -1.0f;                 // ... and of the dense tensor-core kernel
     std::vector<uint32_t> ps_ent;
     std::vector<int32_t> ps_perm;    // packed row -> output channel, -1 = padding row
     const uint32_t *d_ps_ent = nullptr;
@@ -145,7 +146,8 @@ struct cadnn_weights {
     const int32_t *d_tc_grp = nullptr;
     const int32_t *d_tc_grp_ptr = nullptr;
 
-    // dense tensor-core image (tcconv.cu): built when the layer's density makes that route the faster one
+    // dense tensor-core image (tcconv.cu): there when that route is the faster one, by the layer's density or, where both kernels
+    // were timed, by their times
     void *d_tcv = nullptr;
     size_t tcv_bytes = 0;
     int tcv_force[3] = {0, 0, 0};          // CADNN_TCV at pack time: pixels, channels, split (0 = choose)
@@ -266,6 +268,7 @@ cadnn_status launch_block_tc(const cadnn_weights *w, const void *x, int n, int *
 // dense tensor-core route (tcconv.cu)
 bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz);
 cadnn_status tcv_build(cadnn_weights *h);
+void tcv_drop(cadnn_weights *h);   // frees the dense image
 bool tcv_fc_pays(const cadnn_weights *w, int n);   // a small-batch fc layer runs faster dense
 bool tcv_fits(const cadnn_weights *w, int n);   // the batch is within the kernel's index ranges
 bool tcv_pools(const cadnn_weights *w, int n);   // LaunchEpilogue.pooled can be given

@@ -666,7 +666,7 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
                 if (op.src == 0 || flat[op.src]) planar = false;
             }
         }
-        // Layers packed with the dense tensor-core image run NHWC (tcconv.cu), unless their schedules were timed at pack time.
+        // Layers packed with the dense tensor-core image run NHWC (tcconv.cu); for those timed at pack time the times decide below.
         // Networks with depthwise layers do so above 150 million multiply-adds of kept weights: up to there the planar kernels'
         // shorter start-up makes up for their rate (MobileNet-V2, planar / NHWC: batch 1 225 / 225 us, batch 2 304 / 262, batch 16
         // 1060 / 662; half width at 160 x 160, batch 1: 159 / 198).
@@ -684,7 +684,8 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
             }
             if (tc && (!dw || macs > 150e6)) planar = false;
         }
-        // Where the packer timed both layouts for every sparse conv, the measured sums decide.
+        // Where the packer timed both layouts for every sparse conv, the measured sums decide: planar, and NHWC by the kernel that
+        // would run there (a handle keeps a dense image only where that kernel was the faster one).
         if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr) {
             double t_planar = 0.0, t_nhwc = 0.0;
             bool all = true;
@@ -696,9 +697,10 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
                     const float th = (w->half->has_ps && w->half->use_ps) ? w->half->ps_us : w->half->pl_us;
                     if (th > 0.0f && (tp <= 0.0f || th < tp)) tp = th;
                 }
-                if (tp <= 0.0f || w->nhwc_us <= 0.0f) { all = false; break; }
+                const float tn = w->d_tcv ? w->tcv_us : w->nhwc_us;
+                if (tp <= 0.0f || tn <= 0.0f) { all = false; break; }
                 t_planar += tp;
-                t_nhwc += w->nhwc_us;
+                t_nhwc += tn;
             }
             if (getenv("CADNN_VERBOSE"))
                 fprintf(stderr, "cadnn_net_create: sparse convs timed at pack time: planar %.1f us, NHWC %.1f us%s\n", t_planar, t_nhwc,

@@ -1123,6 +1123,29 @@ void autotune_ps(cadnn_weights *h, const PsRows &rows, const std::vector<int64_t
     if (best_us > 0.0f) h->ps_us = best_us;
 }
 
+// Time the dense tensor-core kernel the way the others are timed (a launch waits for the one before it).
+void time_dense(cadnn_weights *h)
+{
+    const cadnn_layer_desc &d = h->desc;
+    const int batch = std::max(1, d.batch_hint);
+    const size_t esz = d.dtype == CADNN_S8 ? 1 : 4;
+    const size_t xb = std::max<size_t>(256, (size_t)batch * d.in_h * d.in_w * d.c_in * esz), yb = std::max<size_t>(256, (size_t)batch * h->h_out * h->w_out * d.c_out * esz);
+    void *x = nullptr, *y = nullptr;
+    cudaStream_t st = nullptr;
+    if (tcv_fits(h, batch) && cudaMalloc(&x, xb) == cudaSuccess && cudaMalloc(&y, yb) == cudaSuccess &&
+        cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking) == cudaSuccess) {
+        cudaMemsetAsync(x, 0, xb, st);
+        LaunchEpilogue ep;
+        ep.out_dtype = d.dtype;
+        ep.act = CADNN_ACT_RELU;
+        h->tcv_us = time_launches([&]() { return launch_tcv(h, x, batch, y, ep, st); }, st, batch >= 16 ? 4 : 16, 4);
+    }
+    if (st) cudaStreamDestroy(st);
+    if (x) cudaFree(x);
+    if (y) cudaFree(y);
+    cudaGetLastError();
+}
+
 // ---- schedule cache -------------------------------------------------------------------------
 // Section 4, "Optimization parameters selection": the parameters of a layer are searched once.
 // With CADNN_TUNE_CACHE=<file> in the environment the measured choices of every layer packed
@@ -1143,6 +1166,7 @@ uint64_t tune_key(const cadnn_layer_desc &d, const std::vector<int64_t> &row_nnz
         mix((uint64_t)(int64_t)v);
     mix(sizeof(Schedule));
     mix(sizeof(PsSchedule));
+    mix(sizeof(TuneRecord));
     for (int64_t v : row_nnz) mix((uint64_t)v);
     return hsh;
 }
@@ -1460,18 +1484,26 @@ cadnn_status pack_common(const cadnn_layer_desc *desc, const Src &src, cadnn_wei
         if (st == CADNN_OK) st = block_tc_upload(h);
         if (st == CADNN_OK && h->s.kind == KK_FC_SPMV && !getenv("CADNN_NO_TCV") && tcv_fc_pays(h, std::max(1, d.batch_hint))) st = tcv_build(h);
         if (st == CADNN_OK && dense_route && (h->s.kind == KK_SCONV_SPATIAL || h->s.kind == KK_SCONV_LINEAR || h->s.kind == KK_DENSE_SMALLC) &&
-            d.fmt == CADNN_FMT_AUTO && !getenv("CADNN_NO_TCV") && !getenv("CADNN_SCHEDULE") && tcv_pays(d, h->nnz))
-            st = tcv_build(h);
+            d.fmt == CADNN_FMT_AUTO && !getenv("CADNN_NO_TCV") && !getenv("CADNN_SCHEDULE") && tcv_pays(d, h->nnz)) {
+            // a layer whose sparse kernel was timed keeps the dense image where that was timed faster
+            if (h->tuned) h->tcv_us = h->tuned->tcv_us;
+            auto sparse_wins = [&]() { return h->nhwc_us > 0.0f && h->tcv_us > 0.0f && h->nhwc_us <= h->tcv_us; };
+            if (!sparse_wins()) {
+                st = tcv_build(h);
+                if (st == CADNN_OK && h->d_tcv && h->nhwc_us > 0.0f && h->tcv_us <= 0.0f) time_dense(h);
+                if (sparse_wins()) tcv_drop(h);
+            }
+        }
         if (st == CADNN_OK && h->has_planar && h->on_device && (d.flags & CADNN_PACK_AUTOTUNE) && !h->tuned)
             autotune_planar(h, h->row_nnz);
-        if (st == CADNN_OK && h->tune_key && !h->tuned && h->on_device) {   // remember what was measured
+        if (st == CADNN_OK && h->tune_key && h->on_device && (!h->tuned || h->tuned->tcv_us < h->tcv_us)) {   // remember what was measured
             TuneRecord rec;
             memset(&rec, 0, sizeof(rec));
             rec.s = h->s;
             if (h->has_ps) rec.ps = h->ps; else rec.ps.T = 0;
             rec.pl_T = h->pl_T; rec.pl_NW = h->pl_NW; rec.pl_RPW = h->pl_RPW; rec.pl_KSW = h->pl_KSW; rec.pl_D = h->pl_D;
             rec.use_ps = (h->has_ps && h->use_ps) ? 1 : 0;
-            rec.pl_us = h->pl_us; rec.ps_us = h->ps_us; rec.nhwc_us = h->nhwc_us;
+            rec.pl_us = h->pl_us; rec.ps_us = h->ps_us; rec.nhwc_us = h->nhwc_us; rec.tcv_us = h->tcv_us;
             tune_store(h->tune_key, rec);
         }
         // A float stride-2 layer (3x3 with padding 1, or 1x1) also gets the form a network uses when the layer before it

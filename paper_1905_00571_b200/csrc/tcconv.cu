@@ -1226,6 +1226,13 @@ cadnn_status tcv_build(cadnn_weights *h)
     return CADNN_OK;
 }
 
+void tcv_drop(cadnn_weights *h)
+{
+    cudaFree(h->d_tcv);
+    h->d_tcv = nullptr;
+    h->tcv_bytes = 0;
+}
+
 // the kernel's index ranges: 31-bit element offsets and pixel numbers, 16-bit image coordinates
 bool tcv_fits(const cadnn_weights *w, int n)
 {

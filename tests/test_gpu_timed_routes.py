@@ -1,0 +1,82 @@
+"""Timed packs and the dense tensor-core route: the packer times that kernel too, a handle keeps the dense image where it was
+the faster one, and a network's layout follows from the times of the kernels that would run."""
+import struct
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import forward as oracle_forward
+from oracle import ref
+from workloads import gen, models
+from parity import assert_close_f32, assert_exact, NET_FLOOR
+from test_gpu_parity_planes import _conv
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def test_a_timed_network_takes_the_dense_route_where_it_is_faster():
+    """Two 3x3 layers that keep 40 % on 28 x 28 maps of 32 images: several times faster on the tensor cores than on either sparse
+    kernel, so the network runs NHWC whether its schedules were timed or not."""
+    from paper_1905_00571_b200 import binding as B
+    from paper_1905_00571_b200.network import PackedModel
+    g = gen.rng(71)
+    m = models.Model("timed_dense", "f32", (56, 56, 3), seed=71)
+    stem, hw = _conv(m, g, "stem", 0, 3, 64, 3, 2, 1, (56, 56), "relu", 1.0)
+    a, _ = _conv(m, g, "a", stem, 64, 128, 3, 1, 1, hw, "relu", 0.4)
+    b, _ = _conv(m, g, "b", a, 128, 128, 3, 1, 1, hw, "relu", 0.4)
+    pool = m.new_slot()
+    m.ops.append(models.Op("gavgpool", "pool", b, pool, c_in=128, c_out=128, in_hw=hw, out_hw=(1, 1)))
+    w = gen.he_weights(g, 10, 1, 1, 128)
+    m.ops.append(models.Op("fc", "fc", pool, m.new_slot(), -1, 128, 10, 1, 1, 0, 1, "none", w, None,
+                           np.ones(10, np.float32), np.zeros(10, np.float32), "f32", 1.0, (1, 1), (1, 1)))
+    x = models.make_input(m, 32)
+    want, _ = oracle_forward.forward(m, x)
+    for autotune in (False, True):
+        pm = PackedModel(m, 32, DEV, autotune=autotune)
+        assert not B.cadnn_net_layout(pm.net)["planar"], autotune
+        y = pm.new_output()
+        pm.forward(torch.from_numpy(x).to(DEV), y)
+        torch.cuda.synchronize()
+        assert_close_f32(y.cpu().numpy(), want, "logits, autotune %s" % autotune, floor=NET_FLOOR)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "s8"])
+def test_a_timed_handle_keeps_the_dense_image_only_where_it_was_faster(dtype, tmp_path, monkeypatch):
+    """The cache record's last number is the dense kernel's time: with a long one the handle holds no dense image and calls run the
+    sparse kernel, with a short one it does; a record without the time is completed; results are the layer's in each case."""
+    from paper_1905_00571_b200 import binding as B
+    cache = tmp_path / "tune.cache"
+    monkeypatch.setenv("CADNN_TUNE_CACHE", str(cache))
+    g = gen.rng(73)
+    x = gen.int8_relu_activation(g, (2, 9, 10, 72)) if dtype == "s8" else gen.relu_normal_input(g, (2, 9, 10, 72))
+    w = gen.int8_weights(g, (70, 3, 3, 72)) if dtype == "s8" else gen.he_weights(g, 70, 3, 3, 72)
+    mask = gen.random_mask(g, w.shape, 0.2)
+    want = ref.conv2d_s8(x, w, mask, 1, 1, out="s32") if dtype == "s8" else ref.conv2d_f32(x, w, mask, 1, 1, act="relu")
+    d = B.make_desc(72, 70, 3, 3, 1, 1, 1, 9, 10, 2, dtype, autotune=True)
+    pack = B.cadnn_pack_q8 if dtype == "s8" else B.cadnn_pack
+    dense = 128 * 9 * 72 * (1 if dtype == "s8" else 6)
+
+    def check(wh, what):
+        y = torch.zeros(want.shape, dtype=torch.int32 if dtype == "s8" else torch.float32, device=DEV)
+        if dtype == "s8":
+            B.cadnn_conv2d(wh, torch.from_numpy(x).to(DEV), y, out_dtype="s32")
+        else:
+            B.cadnn_conv2d(wh, torch.from_numpy(x).to(DEV), y, act="relu")
+        torch.cuda.synchronize()
+        (assert_exact if dtype == "s8" else assert_close_f32)(y.cpu().numpy(), want, what)
+        return B.cadnn_weights_info(wh)["packed_bytes"]
+
+    check(pack(d, w, mask), "timed")
+    key, record = cache.read_text().split()
+    told = {}
+    for us in (1e6, 1e-3):
+        cache.write_text("%s %s\n" % (key, record[:-8] + struct.pack("<f", us).hex()))
+        told[us] = check(pack(d, w, mask), "%g us" % us)
+        assert len(cache.read_text().splitlines()) == 1
+    assert told[1e-3] - told[1e6] >= dense
+    cache.write_text("%s %s\n" % (key, record[:-8] + struct.pack("<f", -1.0).hex()))
+    check(pack(d, w, mask), "no time recorded")
+    again = cache.read_text().split()
+    assert again[2] == key and struct.unpack("<f", bytes.fromhex(again[3][-8:]))[0] > 0.0
