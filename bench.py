@@ -158,6 +158,27 @@ def run_reference(args):
     print(json.dumps(line))
 
 
+def pack(model, batch, dev, x, flush, no_autotune, PackedModel):
+    """The packed network, and how its schedules were chosen: timed layer by layer at pack time, or by the packer's own rules where
+    the whole network measured faster that way (layers timed one by one do not show how far a kernel overlaps its neighbours)."""
+    import torch
+    best = None
+    for timed in ((False,) if no_autotune else (True, False)):
+        pm = PackedModel(model, batch, dev, autotune=timed)
+        y = pm.new_output()
+        ev = [(torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)) for _ in range(25)]
+        for a, b in ev:
+            flush.zero_()
+            a.record()
+            pm.forward(x, y)
+            b.record()
+        torch.cuda.synchronize()
+        ms = sorted(a.elapsed_time(b) for a, b in ev[5:])[10]
+        if best is None or ms < best[0]:
+            best = (ms, pm, "timed at pack time" if timed else "model")
+    return best[1], best[2]
+
+
 def run_ours(args):
     import torch
     from paper_1905_00571_b200 import dist, roofline
@@ -171,14 +192,14 @@ def run_ours(args):
     dev = torch.device("cuda", local)
     model, wname = build_model(args.workload)
     batch = args.batch
-    pm = PackedModel(model, batch, dev, autotune=not args.no_autotune)
     x_np = models.make_input(model, batch, seed=1000 + rank)
     x_host = torch.from_numpy(x_np).pin_memory()
-    y_host = torch.empty(pm.out_shape, dtype=pm.out_dtype).pin_memory()
     x = x_host.to(dev)
-    y = pm.new_output()
     flush = torch.empty(256 << 20, dtype=torch.uint8, device=dev)   # larger than the 126 MB L2
     stream = torch.cuda.current_stream()
+    pm, schedules = pack(model, batch, dev, x, flush, args.no_autotune, PackedModel)
+    y_host = torch.empty(pm.out_shape, dtype=pm.out_dtype).pin_memory()
+    y = pm.new_output()
     n_ops = len(model.ops)
     K, W = args.steps, args.warmup
 
@@ -288,7 +309,7 @@ def run_ours(args):
         from paper_1905_00571_b200 import binding as B
         planar = B.cadnn_net_layout(pm.net)["planar"]
         roof["cuda_kernels"] = (["sconv_planar_kernel", "sconv_planar_tma_kernel", "sconv_planar_staged_kernel"]
-                                if planar else ["sconv_kernel"])
+                                if planar else ["tcconv_kernel", "sconv_kernel"])   # with and without a dense image
     t_roof_nom = sum(r["t_roof_us"] for r in rows_nom)
     t_roof_meas = sum(r["t_roof_us"] for r in rows_meas)
     k3 = [(r, ms) for r, ms in zip(rows_nom, per) if r["family"] == "sconv_kxk" and r["nnz"] and r["name"] not in ("conv1", "stem")]
@@ -346,7 +367,7 @@ def run_ours(args):
                 "dtype": "f32" if model.dtype == "f32" else "s8", "data": "synthetic",
                 "config": {"workload": wname, "batch_per_gpu": batch, "parallelism": "replicas x%d" % world,
                            "l2": "flushed between iterations (256 MiB write)", "launch": "CUDA graph replay",
-                           "schedules": "model" if args.no_autotune else "timed at pack time"},
+                           "schedules": schedules},
                 "latency_ms": cold_ms, "latency_ms_warm_l2": warm_ms, "images_per_s_warm_l2": images / (warm_ms * 1e-3),
                 "sparse_roofline": sparse, "roofline": roof, "cpu_baseline": cpu_base,
                 "e2e": {"value": images / (e2e_ms * 1e-3), "unit": "images/s", "ms_per_step": e2e_ms,
