@@ -748,23 +748,27 @@ bool ps_eligible(const cadnn_layer_desc &d, bool s8)
     return (long long)planar_pitch(d.in_h, d.in_w) * d.c_in < (1LL << 31);
 }
 
-void ps_collect_rows(const cadnn_layer_desc &d, const Src &src, PsRows &r)
+// Read off the planar image, which has the kept weights in this order (build_planar_image): its offsets are ci planes, and the
+// tap from the corner of the padded frame.
+void ps_collect_rows(const cadnn_weights *h, const std::vector<int64_t> &row_nnz, PsRows &r)
 {
+    const cadnn_layer_desc &d = h->desc;
     const int wp = d.in_w + 2 * kPlanarHalo;
+    const uint32_t plane = (uint32_t)planar_pitch(d.in_h, d.in_w);
     r.ptr.assign(d.c_out + 1, 0);
+    for (int co = 0; co < d.c_out; ++co) r.ptr[co + 1] = r.ptr[co] + (int32_t)row_nnz[co];
+    r.ci.resize(r.ptr[d.c_out]);
+    r.tap.resize(r.ptr[d.c_out]);
+    r.v.resize(r.ptr[d.c_out]);
     for (int co = 0; co < d.c_out; ++co) {
-        r.ptr[co] = (int32_t)r.ci.size();
-        for (int ci = 0; ci < d.c_in; ++ci)
-            for (int ky = 0; ky < d.kh; ++ky)
-                for (int kx = 0; kx < d.kw; ++kx) {
-                    const size_t wi = (((size_t)co * d.kh + ky) * d.kw + kx) * d.c_in + ci;
-                    if (!src.kept(wi)) continue;
-                    r.ci.push_back(ci);
-                    r.tap.push_back((ky - d.pad) * wp + (kx - d.pad));
-                    r.v.push_back(src.fval(wi));
-                }
+        const uint32_t *e = h->pl_ent.data() + 2 * (size_t)h->pl_ptr[co];
+        for (int32_t i = r.ptr[co]; i < r.ptr[co + 1]; ++i, e += 2) {
+            const uint32_t ci = e[1] / plane;
+            r.ci[i] = (int32_t)ci;
+            r.tap[i] = (int32_t)(e[1] - ci * plane) - kPlanarHalo * (wp + 1);
+            memcpy(&r.v[i], &e[0], 4);
+        }
     }
-    r.ptr[d.c_out] = (int32_t)r.ci.size();
 }
 
 // derived fields of a staged-planar schedule from (T, RPW, NW, KS, CIc, stages); false if it cannot run
@@ -1244,7 +1248,7 @@ void pack_ps(cadnn_weights *h, const Src &src, const std::vector<int64_t> &row_n
     const cadnn_layer_desc &d = h->desc;
     if (!ps_eligible(d, src.s8) || getenv("CADNN_NO_STAGED")) return;
     PsRows rows;
-    ps_collect_rows(d, src, rows);
+    ps_collect_rows(h, row_nnz, rows);
     ps_default(d, h->nnz, h->ps);
     if (d.stride != 1) {   // row tiles are staged by TMA only
         h->ps.tma = 1;
