@@ -303,11 +303,10 @@ def run_ours(args):
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "traffic": None, "peak_source": peaks["source"]}
     roof.update(kernel=top, launches_per_step=ft["launches"], avg_launch_us=ft["ms"] * 1e3 / ft["launches"])
-    roof["traffic"] = recorded_traffic(args.workload, batch, top)
+    planar = B.cadnn_net_layout(pm.net)["planar"]
+    roof["traffic"] = recorded_traffic(args.workload, batch, top, planar)
     roof["algorithmic_bytes_per_launch"] = ft["bytes"] / ft["launches"]
     if top.startswith("sconv"):   # CUDA kernels behind the family in this net's layout
-        from paper_1905_00571_b200 import binding as B
-        planar = B.cadnn_net_layout(pm.net)["planar"]
         roof["cuda_kernels"] = (["sconv_planar_kernel", "sconv_planar_tma_kernel", "sconv_planar_staged_kernel"]
                                 if planar else ["tcconv_kernel", "sconv_kernel"])   # with and without a dense image
     t_roof_nom = sum(r["t_roof_us"] for r in rows_nom)
@@ -382,9 +381,10 @@ def run_ours(args):
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the dominant kernel family, from one ncu
 # pass over this command (summary and command line: profiles/resnet50_batch1_launch_list.md), valid for the kernel
-# sources whose digest is recorded with it.  The family's layers run in the three channel-planar sparse conv kernels,
-# which serve 1x1 and k x k layers alike: the figure is the mean over all 52 sparse conv launches of a step.
-TRAFFIC = {"workload": "resnet50", "batch": 1, "family": "sconv_1x1", "dram_bytes_per_launch": 1960049, "digest": "3e6cc2c9ca66921c"}
+# sources whose digest is recorded with it.  The family's layers run in the dense tensor-core kernel (NHWC networks),
+# which serves 1x1 and k x k layers alike: the figure is the mean over the 52 conv launches of a step behind the stem.
+TRAFFIC = {"workload": "resnet50", "batch": 1, "family": "sconv_1x1", "planar": False, "dram_bytes_per_launch": 4358786,
+           "digest": "8b302aa6540ede6c"}
 
 
 def kernel_sources_digest():
@@ -400,9 +400,9 @@ def kernel_sources_digest():
     return h.hexdigest()[:16]
 
 
-def recorded_traffic(workload, batch, family):
+def recorded_traffic(workload, batch, family, planar):
     t = TRAFFIC
-    if t["dram_bytes_per_launch"] is None or (t["workload"], t["batch"], t["family"]) != (workload, batch, family):
+    if t["dram_bytes_per_launch"] is None or (t["workload"], t["batch"], t["family"], t["planar"]) != (workload, batch, family, planar):
         return None
     return t["dram_bytes_per_launch"] if t["digest"] == kernel_sources_digest() else None
 

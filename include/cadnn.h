@@ -22,7 +22,9 @@
  *    passed as void*, NULL = the default stream).  No call synchronizes the
  *    device unless its comment says so.
  *  - Inputs must be finite; NaN / Inf behaviour is unspecified (a pruned weight
- *    contributes exactly 0 only for finite activations).
+ *    contributes exactly 0 only for finite activations).  The dense route of float layers
+ *    (cadnn_pack) takes weights and activations of magnitude up to 3.39e38; below 8e-34
+ *    they may lose their last bits there.
  *  - There is no CPU fallback: without a CUDA device every compute call fails
  *    with CADNN_E_CUDA.
  */
@@ -65,8 +67,10 @@ typedef enum {
 
 #define CADNN_PACK_HOST_ONLY 1 /* build the packed image on the host only (no device needed, no compute) */
 #define CADNN_PACK_AUTOTUNE 2  /* conv layers: time the candidate schedules on the current device (batch_hint
-                                  images of zeros, scratch buffers allocated and freed inside the call) and
-                                  keep the fastest, instead of trusting the packer's time model.  With
+                                  images of zeros, scratch buffers allocated and freed inside the call; the
+                                  dense tensor-core kernel among them) and keep the fastest, instead of
+                                  trusting the packer's rules.  A layer is timed by itself: how far a kernel
+                                  overlaps its neighbours in a network does not show.  With
                                   CADNN_TUNE_CACHE=<file> in the environment the choices are appended to that
                                   text file and a later pack of the same layer (geometry, batch hint, nonzeros
                                   per filter) reads them back instead of timing: tune once per machine, and a
@@ -109,9 +113,10 @@ typedef struct cadnn_net cadnn_net;
  *           from several streams.
  * Filters are regrouped so that the warps of a thread block get equal nonzero
  * counts; the permutation is undone when results are stored.
- * Where the kept fraction makes the tensor cores the faster route (CADNN_FMT_AUTO, groups 1, conv or fc
- * packed for a batch above 8), the handle also gets a dense image of the layer for them and NHWC calls
- * take it; CADNN_NO_TCV in the environment leaves it out.
+ * Where the kept fraction makes the tensor cores the faster route (CADNN_FMT_AUTO, groups 1, conv or fc; for an fc
+ * packed for a batch of up to 8, where the batch does), the handle also gets a dense image of the layer for them, if
+ * there is device memory for it, and NHWC calls take it; CADNN_NO_TCV in the environment leaves it out.  With
+ * CADNN_PACK_AUTOTUNE the times of both kernels decide.
  * Errors: E_ARG (NULL, bad desc), E_DTYPE, E_UNSUPPORTED (grouped conv other than
  * depthwise; int8 depthwise; reduction length whose int32 sum could overflow),
  * E_ALLOC, E_CUDA.  Synchronizes the device copy before returning.

@@ -424,8 +424,8 @@ cadnn_status launch_deliver(cadnn_net *net, bool pdl, cudaStream_t st)
 // Edges between kernels that the capture left plain - into a branch, out of it, at a join - become programmatic: the kernel behind
 // starts while the one before drains, and waits for it (for all kernels it has edges from) where it first touches activations, as
 // every layer kernel does.  Joins used to cost a full launch behind the last producer: Inception-V3, batch 1, 453 / 449 us; ResNet-50
-// 318 / 316, int8 216 / 214.5, batch 2 259 / 255.  From batch 4 on the waiting blocks take places that the other branch's could use
-// (ResNet-50 at 25 %, batch 8: 775 / 779).
+// 318 / 316, int8 216 / 214.5, batch 2 259 / 255.  At larger batches the waiting blocks take places that the other branch's could use
+// (ResNet-50 at 25 %, batch 8: 775 / 779; the line is drawn at batch 2, the last one measured to gain).
 cudaError_t link_programmatic(cudaGraph_t graph)
 {
     size_t n = 0;
@@ -668,8 +668,9 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
         }
         // Layers packed with the dense tensor-core image run NHWC (tcconv.cu); for those timed at pack time the times decide below.
         // Networks with depthwise layers do so above 150 million multiply-adds of kept weights: up to there the planar kernels'
-        // shorter start-up makes up for their rate (MobileNet-V2, planar / NHWC: batch 1 225 / 225 us, batch 2 304 / 262, batch 16
-        // 1060 / 662; half width at 160 x 160, batch 1: 159 / 198).
+        // shorter start-up and the depthwise layers they take along make up for their rate (MobileNet-V2, planar / NHWC: batch 1
+        // 208 / 223 us, batch 2 298 / 262, batch 16 962 / 661; half width at 160 x 160, batch 1 151 / 199, batch 2 166 / 209;
+        // MobileNet-V1, batch 1, 148 / 143).
         if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr && !(getenv("CADNN_PERSIST") && atoi(getenv("CADNN_PERSIST")) != 0)) {
             bool tc = true, dw = false;
             double macs = 0.0;

@@ -902,7 +902,8 @@ bool build_ps_image(cadnn_weights *h, const PsRows &rows, const std::vector<int6
 //   microseconds = 2.29 waves + perSM (0.206 + warps entries (0.00025 + 0.00101 T)) + 0.31 chunks + 0.24 KS
 // (perSM = blocks on the fullest multiprocessor, entries = nonzeros a warp walks, T = bands per lane).  The pick averages 4 %
 // above the fastest measured schedule; MobileNet-V2 at batch 1: 258 us with the rule of thumb
-// below, 225 us with this one, 210 us with timed schedules; MobileNet-V1 199, 148 and 137 us.
+// below, 225 us with this one, 210 us with timed schedules (208 and 207 since depthwise layers join the launch where the schedule
+// lets them); MobileNet-V1 199, 148 and 137 us.
 bool ps_model(const cadnn_layer_desc &d, int64_t nnz, PsSchedule &best)
 {
     const int batch = std::max(1, d.batch_hint);

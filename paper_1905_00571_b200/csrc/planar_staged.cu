@@ -227,7 +227,8 @@ __device__ __forceinline__ void ps_compute_chunk(const PsParams &p, const unsign
 // Depthwise layer over the planes of this warp's filters, which the epilogue has just left in shared memory (the sums of
 // dw_planar_kernel in the same order, from the same values).  Such a layer is all latency (launch, one round trip to L2, a
 // few multiply-adds: 5 us alone); behind the conv it costs about 2.  MobileNet-V2, batch 1, where ten of the seventeen
-// depthwise layers follow a conv of one tile: 225 / 209 us; at 160 x 160 pixels 197 / 183.
+// depthwise layers follow a conv of one tile: 225 / 208 us alone, 246 / 228 with three such networks in turn (whose maps do not
+// stay in L2 together); at 160 x 160 pixels 197 / 183.
 template <int RPW>
 __device__ __forceinline__ void ps_dw_tail(const PsParams &p, unsigned char *smem, int lane, int rslot, unsigned img, const int (&co_of)[RPW])
 {

@@ -26,7 +26,8 @@
 // stage read 40 KB of operands per 16 K values where the tensor core needs 384 clocks.
 //
 // Float precision.  A float is the exact sum of three bf16 numbers (8 + 8 + 8 significand bits), a = a1 + a2 +
-// a3 with |a2| <= 2^-9 |a|, |a3| <= 2^-18 |a|.  Loaders split activations, the packer splits weights, and the
+// a3 with |a2| <= 2^-9 |a|, |a3| <= 2^-18 |a|, from 2^-110 (8e-34) on (below, the third part loses bits under
+// bf16's smallest number, 2^-133) and up to 3.39e38 (beyond, the first part rounds to infinity).  Loaders split activations, the packer splits weights, and the
 // products a1 b1, a1 b2, a2 b1, a2 b2, a1 b3, a3 b1 are accumulated in fp32; what is left out is below 2^-25 of
 // |a b|, less than the rounding of one fp32 multiply-add.  a1 b1 has an accumulator of its own: the small terms
 // are summed apart and added once at the end, so they are not rounded away against the large sum.
@@ -944,7 +945,8 @@ static_assert(clusters_find_tensor_memory(), "clusters of split tiles could wait
 // programmatic dependents):
 //   time = start + P (b2 + n (c2 + d2 px / 64)) + Q (b1 + n (c1 + d1 px / 64))   [microseconds]
 // n = stages per block, P = rounds in which every multiprocessor runs two blocks, Q = rounds with one.  How many clusters
-// of a size run at once is what cudaOccupancyMaxActiveClusters reports for this GPU (a cluster has to fit one GPC).
+// of a size run at once (a cluster has to fit one GPC) is the table cap1 / cap2 in choose, as cudaOccupancyMaxActiveClusters
+// reported it on a B200.
 // Mean excess of the chosen over the best measured shape: 1 %.
 struct Cost {
     float start, b2, c2, d2, b1, c1, d1;
