@@ -240,7 +240,7 @@ def main():
             sys.stdout.flush()
             if args.layers:
                 lines = ["\n## per layer: batch %d, density %.3g\n" % (batch, dens),
-                         "| layer | kernel | in | c_in→c_out | k/s | nnz | µs | roofline µs | fraction | schedule |", "|---|---|---|---|---|---|---|---|---|---|"]
+                         "| layer | kernel | in | c_in→c_out | k/s | nnz | µs | roofline µs | fraction | schedule (of the sparse kernel; NHWC layers with a dense image run tcconv_kernel) |", "|---|---|---|---|---|---|---|---|---|---|"]
                 planar = B.cadnn_net_layout(pm.net)["planar"]
                 parity_ops = set(B.cadnn_net_parity_layers(pm.net, ops=True))
                 for i, (op, r, t) in enumerate(zip(model.ops, rows, per)):
