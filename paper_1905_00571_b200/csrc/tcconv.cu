@@ -55,7 +55,8 @@ struct TcvParams {
     int stride, pad, pad_w, kh, kw;
     int M, nkb, n_nt, S, npx;
     int stages, recv_off, bar_off;   // pipeline depth; byte offsets of the partial sums and of the barriers in shared memory
-    int ldc, c_off, vec_ok, vec_sb, vec16;  // vec_ok / vec_sb: output and residual / scale and bias allow 4 channels per access; vec16: int8 output 16
+    int res_tile;                    // int8: the residual of the block's outputs is brought into shared memory, this many bytes at a time (0: no residual)
+    int ldc, c_off, vec_ok;          // vec_ok: output and residual allow 4 channels per access
     int kb_base, kb_rem;             // stages per block of a cluster: kb_base, and one more in the first kb_rem blocks
     int whole, tail;                 // int8 input: bytes of its whole 4-byte words, and bytes behind them
     int Rp;                          // K positions per kernel row: kw * c_in rounded up to 16 bytes
@@ -159,6 +160,21 @@ __device__ __forceinline__ uint4 ld_vec(const void *p)
     asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
+// the same where `ok`, zeros elsewhere; a predicated load, so that several of a thread's are on their way at once
+__device__ __forceinline__ uint4 ld_vec_if(const void *p, bool ok)
+{
+    uint4 v;
+    asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %5, 0;\nmov.b32 %0, 0;\nmov.b32 %1, 0;\nmov.b32 %2, 0;\nmov.b32 %3, 0;\n"
+                 "@q ld.global.v4.b32 {%0, %1, %2, %3}, [%4];\n}\n"
+                 : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w) : "l"(p), "r"((int)ok));
+    return v;
+}
+__device__ __forceinline__ unsigned ld_word_if(const void *p, bool ok)
+{
+    unsigned v;
+    asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\nmov.b32 %0, 0;\n@q ld.global.b32 %0, [%1];\n}\n" : "=&r"(v) : "l"(p), "r"((int)ok));
+    return v;
+}
 __device__ __forceinline__ uint4 lds128(unsigned addr)
 {
     uint4 v;
@@ -177,6 +193,29 @@ template <int U> __device__ __forceinline__ void send(unsigned addr, unsigned ba
     else if (U == 2)
         asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];\n" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(b) : "memory");
     else asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];\n" ::"r"(a), "r"(v[0]), "r"(b) : "memory");
+}
+
+// 4 or 16 bytes of global memory to shared memory, waited for with copies_landed by the thread that asked for them
+__device__ __forceinline__ void copy4(unsigned dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy16(unsigned dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_landed() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
+__device__ __forceinline__ float lds32(unsigned addr)
+{
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 lds_float4(unsigned addr)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
+    return v;
 }
 
 // copies `bytes` of this block's shared memory to address dst of block `owner`; counts on that block's barrier
@@ -240,12 +279,9 @@ template <bool F32>
 __device__ __forceinline__ uint4 gather_vec(const TcvParams &p, const Px &r, int ky, int kx, int ci)
 {
     const int iy = (r.yx >> 16) + ky, ix = (int)(short)r.yx + kx;
-    uint4 v = make_uint4(0, 0, 0, 0);
-    if ((unsigned)iy < (unsigned)p.h && (unsigned)ix < (unsigned)p.w && ky < p.kh) {
-        const int o = r.off + (ky * p.w + kx) * p.c_in + ci;
-        v = ld_vec(reinterpret_cast<const char *>(p.x) + (size_t)o * (F32 ? 4 : 1));
-    }
-    return v;
+    const bool inside = (unsigned)iy < (unsigned)p.h && (unsigned)ix < (unsigned)p.w && ky < p.kh;
+    const int o = r.off + (ky * p.w + kx) * p.c_in + ci;
+    return ld_vec_if(reinterpret_cast<const char *>(p.x) + (long long)o * (F32 ? 4 : 1), inside);
 }
 // mask of the bytes n .. of a word, empty from n = 4 on (the instruction takes shifts beyond the width as the width)
 __device__ __forceinline__ unsigned from_byte(int n)
@@ -271,8 +307,7 @@ __device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, in
         const float *x = reinterpret_cast<const float *>(p.x);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            v[j] = 0;
-            if (j >= a && j < b) v[j] = __float_as_uint(ld_act(x + o + j));
+            v[j] = ld_word_if(x + o + j, j >= a && j < b);
         }
         return make_uint4(v[0], v[1], v[2], v[3]);
     }
@@ -283,8 +318,7 @@ __device__ __forceinline__ uint4 gather_run(const TcvParams &p, const Px &px, in
     unsigned w[5];
 #pragma unroll
     for (int i = 0; i < 5; ++i) {
-        w[i] = 0;
-        if (4 * i + 4 > first && 4 * i < end) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(w[i]) : "l"(x + 4 * i));
+        w[i] = ld_word_if(x + 4 * i, 4 * i + 4 > first && 4 * i < end);
     }
     unsigned v[4];
 #pragma unroll
@@ -377,109 +411,88 @@ __device__ __forceinline__ void finish4(const TcvParams &p, size_t oi, int left,
         }
     }
 }
-// the residual of those 4 channels: 4 floats, or 4 int8 values in the first word
-template <bool F32> __device__ __forceinline__ uint4 load_residual(const TcvParams &p, int m, int co)
+// the residual of those 4 channels of a float layer
+__device__ __forceinline__ uint4 load_residual(const TcvParams &p, int m, int co)
 {
-    const size_t ri = (size_t)m * p.c_out + co;
+    const float *res = reinterpret_cast<const float *>(p.residual) + (size_t)m * p.c_out + co;
+    if (p.vec_ok) return ld_vec(res);
     uint4 v = make_uint4(0, 0, 0, 0);
-    if (F32) {
-        const float *res = reinterpret_cast<const float *>(p.residual) + ri;
-        if (p.vec_ok) return ld_vec(res);
-        const int left = p.c_out - co;
-        v.x = __float_as_uint(ld_act(res));
-        if (left > 1) v.y = __float_as_uint(ld_act(res + 1));
-        if (left > 2) v.z = __float_as_uint(ld_act(res + 2));
-        if (left > 3) v.w = __float_as_uint(ld_act(res + 3));
-    } else {
-        const signed char *res = reinterpret_cast<const signed char *>(p.residual) + ri;
-        if (p.vec_ok) asm volatile("ld.global.b32 %0, [%1];\n" : "=r"(v.x) : "l"(res));
-        else
-            for (int j = 0; j < 4; ++j)
-                if (co + j < p.c_out) v.x |= (unsigned)(unsigned char)ld_act(res + j) << (8 * j);
-    }
+    const int left = p.c_out - co;
+    v.x = __float_as_uint(ld_act(res));
+    if (left > 1) v.y = __float_as_uint(ld_act(res + 1));
+    if (left > 2) v.z = __float_as_uint(ld_act(res + 2));
+    if (left > 3) v.w = __float_as_uint(ld_act(res + 3));
     return v;
 }
 
-// scale and bias of 4 consecutive channels
-__device__ __forceinline__ void load_channels(const TcvParams &p, int co, float4 &sc, float4 &bi)
-{
-    if (co + 3 < p.c_out) {
-        if (p.vec_sb) {
-            if (p.scale) sc = __ldg(reinterpret_cast<const float4 *>(p.scale + co));
-            if (p.bias) bi = __ldg(reinterpret_cast<const float4 *>(p.bias + co));
-        } else {
-            if (p.scale) sc = make_float4(__ldg(p.scale + co), __ldg(p.scale + co + 1), __ldg(p.scale + co + 2), __ldg(p.scale + co + 3));
-            if (p.bias) bi = make_float4(__ldg(p.bias + co), __ldg(p.bias + co + 1), __ldg(p.bias + co + 2), __ldg(p.bias + co + 3));
-        }
-        return;
-    }
-    const int a = min(co + 1, p.c_out - 1), b = min(co + 2, p.c_out - 1);
-    if (p.scale) sc = make_float4(__ldg(p.scale + co), __ldg(p.scale + a), __ldg(p.scale + b), 1.0f);
-    if (p.bias) bi = make_float4(__ldg(p.bias + co), __ldg(p.bias + a), __ldg(p.bias + b), 0.0f);
-}
-
-// Epilogue of channel ch for U consecutive pixels from m on: sums t, residuals r
-template <bool F32, int U>
+// Epilogue of channel ch of a float layer for U consecutive pixels from m on: sums t, residuals r
+template <int U>
 __device__ __forceinline__ void finish_column(const TcvParams &p, int m, int ch, const unsigned (&t)[U], const unsigned (&r)[U], float sc, float bi)
 {
+    float *y = reinterpret_cast<float *>(p.y) + (size_t)m * p.ldc + p.c_off + ch;
 #pragma unroll
-    for (int i = 0; i < U; ++i) {
-        if (m + i >= p.M) break;
-        const size_t oi = (size_t)(m + i) * p.ldc + p.c_off + ch;
-        if (F32) reinterpret_cast<float *>(p.y)[oi] = finish_f(p, t[i], sc, bi, __uint_as_float(r[i]));
-        else if (p.out_dtype == CADNN_S8) reinterpret_cast<signed char *>(p.y)[oi] = (signed char)finish_q(p, (int)t[i], sc, bi, (int)r[i]);
-        else
-            reinterpret_cast<unsigned *>(p.y)[oi] = p.out_dtype == CADNN_S32 ? t[i]
-                : __float_as_uint(requant_f32((int)t[i], sc, bi, p.act, p.residual != nullptr, (int)r[i], p.res_scale));
-    }
+    for (int i = 0; i < U; ++i)
+        if (m + i < p.M) y[(size_t)i * p.ldc] = finish_f(p, t[i], sc, bi, __uint_as_float(r[i]));
 }
-template <bool F32, int U> __device__ __forceinline__ void load_column_residual(const TcvParams &p, int m, int ch, unsigned (&r)[U])
+template <int U> __device__ __forceinline__ void load_column_residual(const TcvParams &p, int m, int ch, unsigned (&r)[U])
 {
 #pragma unroll
     for (int i = 0; i < U; ++i) {
         r[i] = 0;
-        if (!p.residual || m + i >= p.M) continue;
-        const size_t ri = (size_t)(m + i) * p.c_out + ch;
-        if (F32) r[i] = __float_as_uint(ld_act(reinterpret_cast<const float *>(p.residual) + ri));
-        else r[i] = (unsigned)(int)ld_act(reinterpret_cast<const signed char *>(p.residual) + ri);
+        if (p.residual && m + i < p.M) r[i] = __float_as_uint(ld_act(reinterpret_cast<const float *>(p.residual) + (size_t)(m + i) * p.c_out + ch));
     }
 }
 // Split tile whose rows are channels: a thread takes channel ch (of the tile) and every second group of U pixels of this
-// block's share.  Partial sums lie as [sender][group][channel][U], so that loads and stores of a warp are contiguous.
-template <bool F32, int U>
-__device__ __forceinline__ void finish_split_columns(const TcvParams &p, unsigned at, int rows, int m0, int co, int ch, int first, unsigned bar)
+// block's share, kBatch groups at a time.  Partial sums lie as [sender][group][channel][U], so that loads and stores of a warp are
+// contiguous.  The first batch's residuals are asked for by the caller, ahead of the last multiply-adds: 64 pixels split in two
+// (4 groups a thread) waited once per group for them, 2600 of the layer's 16000 clocks.
+const int kBatch = 4;
+template <int U>
+__device__ __forceinline__ void load_split_residual(const TcvParams &p, int m0, int co, int first, int groups, unsigned (&r)[16])
+{
+#pragma unroll
+    for (int k = 0; k < kBatch; ++k) {
+        unsigned v[U];
+#pragma unroll
+        for (int i = 0; i < U; ++i) v[i] = 0;
+        if (first + 2 * k < groups) load_column_residual<U>(p, m0 + (first + 2 * k) * U, co, v);
+#pragma unroll
+        for (int i = 0; i < U; ++i) r[k * U + i] = v[i];
+    }
+}
+template <int U>
+__device__ __forceinline__ void finish_split_columns(const TcvParams &p, unsigned at, int rows, int m0, int co, int ch, int first, float sc, float bi,
+                                                     unsigned (&r)[16])
 {
     const int groups = rows / U;
-    const bool mine = co < p.c_out;
-    float sc = 1.0f, bi = 0.0f;
-    unsigned r[U];
-    if (mine) {
-        if (p.scale) sc = __ldg(p.scale + co);
-        if (p.bias) bi = __ldg(p.bias + co);
-        if (first < groups) load_column_residual<F32, U>(p, m0 + first * U, co, r);
-    }
-    mb_wait(bar, 0u, p.gave_up);
-    if (!mine) return;
 #pragma unroll 1
-    for (int g = first; g < groups; g += 2) {
-        unsigned t[U];
+    for (int g0 = first; g0 < groups; g0 += 2 * kBatch) {
+        if (g0 != first) load_split_residual<U>(p, m0, co, g0, groups, r);
 #pragma unroll
-        for (int i = 0; i < U; ++i) t[i] = 0;
-        const unsigned from = at + (g * 128 + ch) * (U * 4);
+        for (int k = 0; k < kBatch; ++k) {
+            const int g = g0 + 2 * k;
+            if (g >= groups) break;
+            unsigned t[U], res[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                t[i] = 0;
+                res[i] = r[k * U + i];
+            }
+            const unsigned from = at + (g * 128 + ch) * (U * 4);
 #pragma unroll 4
-        for (int q = 0; q < p.S; ++q) {
-            unsigned v[4];
-            const unsigned a = from + q * (rows * 128 * 4);
-            if (U == 4) {
-                const uint4 w = lds128(a);
-                v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
-            } else if (U == 2) asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];\n" : "=r"(v[0]), "=r"(v[1]) : "r"(a) : "memory");
-            else asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(v[0]) : "r"(a) : "memory");
+            for (int q = 0; q < p.S; ++q) {
+                unsigned v[4];
+                const unsigned a = from + q * (rows * 128 * 4);
+                if (U == 4) {
+                    const uint4 w = lds128(a);
+                    v[0] = w.x; v[1] = w.y; v[2] = w.z; v[3] = w.w;
+                } else if (U == 2) asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];\n" : "=r"(v[0]), "=r"(v[1]) : "r"(a) : "memory");
+                else asm volatile("ld.shared.b32 %0, [%1];\n" : "=r"(v[0]) : "r"(a) : "memory");
 #pragma unroll
-            for (int i = 0; i < U; ++i) t[i] = F32 ? __float_as_uint(__uint_as_float(t[i]) + __uint_as_float(v[i])) : t[i] + v[i];
+                for (int i = 0; i < U; ++i) t[i] = __float_as_uint(__uint_as_float(t[i]) + __uint_as_float(v[i]));
+            }
+            finish_column<U>(p, m0 + g * U, co, t, res, sc, bi);
         }
-        finish_column<F32, U>(p, m0 + g * U, co, t, r, sc, bi);
-        if (g + 2 < groups) load_column_residual<F32, U>(p, m0 + (g + 2) * U, co, r);
     }
 }
 template <int U>
@@ -518,6 +531,9 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
     const unsigned xbytes = C::kParts * xpart, stage = xbytes + C::kWBytes;
 
     const unsigned pxs = slot32 + 16;                   // window starts of the tile's pixels, 8 bytes each
+    const unsigned consts = pxs + PX * 8;               // scale and bias of the tile's channels
+    const unsigned restile = consts + CH * 8;           // p.res_tile: the residual, CH bytes per pixel that this block finishes
+    const int rows = npx / p.S, lo = rows * rank;       // those pixels: rows of them from number lo of the tile on
 
     // weights of stage kb: its CH x 64-byte tiles, 64 channels (4 KB) per bulk copy
     const int n64 = (p.c_out + 63) / 64;
@@ -583,10 +599,21 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
 
     if (warp < kLoadWarps) {
         uint4 v[C::kRPT];
+        // Window starts stay in registers, and the loads are predicated: with the starts read from shared memory for every stage and
+        // the loads behind branches one piece was issued every 100 clocks, 430 of a stage's 1800 (64 pixels).
+        // (Where registers are short because three blocks share a multiprocessor, they are read ahead of each stage's loads.)
+        const bool kKeep = C::kBlocks < 3 || C::kRPT < 8;
+        Px start[C::kRPT];
+        auto read_starts = [&]() {
+#pragma unroll
+            for (int i = 0; i < C::kRPT; ++i) start[i] = load_px(pxs + (r0 + kPS * i) * 8);
+        };
+        if (kKeep) read_starts();
         auto request = [&]() {
+            if (!kKeep) read_starts();
 #pragma unroll
             for (int i = 0; i < C::kRPT; ++i) {
-                const Px px = load_px(pxs + (r0 + kPS * i) * 8);
+                const Px &px = start[i];
                 v[i] = VEC ? gather_vec<F32>(p, px, ky, kx, ci) : gather_run<F32, TAIL>(p, px, ky, ci);
             }
             ci += C::kGroups * C::kKB;
@@ -598,6 +625,26 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         };
         grid_dep_wait();
         if (kb0 + grp < kb1) request();
+        // What the epilogue needs, asked for now so that it has arrived by then (loading it there cost a round trip to L2 for every
+        // four channels or residual row: 64 -> 256 1x1 int8 with a residual, 128 x 128 tile, 9000 of 12500 clocks).
+        if (tid < CH) {
+            const int ch = nt * CH + tid;
+            const unsigned a = consts + tid * 4;
+            if (p.scale && ch < p.c_out) copy4(a, p.scale + ch);
+            else asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a), "f"(1.0f) : "memory");
+            if (p.bias && ch < p.c_out) copy4(a + CH * 4, p.bias + ch);
+            else asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a + CH * 4), "f"(0.0f) : "memory");
+        }
+        if (!F32 && p.res_tile >= 4) {
+            const int log = p.res_tile == 16 ? 4 : 2, per = CH >> log;
+            for (int i = tid; i < rows * per; i += kLoadWarps * 32) {
+                const int row = i / per, m = m0 + lo + row, at = (i - row * per) << log, ch = nt * CH + at;
+                if (m >= p.M || ch >= p.c_out) continue;
+                const char *src = reinterpret_cast<const char *>(p.residual) + (size_t)m * p.c_out + ch;
+                if (log == 4) copy16(restile + row * CH + at, src);
+                else copy4(restile + row * CH + at, src);
+            }
+        }
         // swizzled place of the thread's chunk in pixel row r0 of an operand tile (rows kPS apart have the same pattern)
         const unsigned sw = (unsigned)((r0 >> 1) & 3);
         const unsigned at = F32 ? r0 * 64 + ((((unsigned)c >> 1) ^ sw) << 4) + (c & 1) * 8
@@ -628,13 +675,32 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                 for (int i = 0; i < C::kRPT && (!SWAP || r0 + kPS * i < npx); ++i)
                     patch_tail(p, load_px(pxs + (r0 + kPS * i) * 8), row, k - row * p.Rp, a + i * (kPS * 64));
             }
-            if (kb + C::kGroups < kb1) request();
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
             __syncwarp();
             if (lane == 0) mb_arrive(bars + s * 8);
+            if (kb + C::kGroups < kb1) request();
             s += C::kGroups;
         }
         grid_dep_trigger();
+        if (!F32 && p.res_tile == 1) {   // channels of no multiple of 4: byte by byte, 16 on their way at once
+#pragma unroll 1
+            for (int i = tid; i < rows * CH; i += kLoadWarps * 32 * 16) {
+                int b[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const int at = i + k * kLoadWarps * 32, m = m0 + lo + at / CH, ch = nt * CH + at % CH;
+                    b[k] = 0;
+                    if (at < rows * CH && m < p.M && ch < p.c_out) b[k] = ld_act(reinterpret_cast<const signed char *>(p.residual) + (size_t)m * p.c_out + ch);
+                }
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const int at = i + k * kLoadWarps * 32;
+                    if (at < rows * CH) asm volatile("st.shared.u8 [%0], %1;\n" ::"r"(restile + at), "r"(b[k]) : "memory");
+                }
+            }
+        }
+        copies_landed();
+        asm volatile("bar.sync 1, %0;\n" ::"n"(C::kLoadWarps * 32) : "memory");
     } else if (warp == kLoadWarps) {
         if (lane > 0 && lane <= Prefetch::kMax && p.ahead.bytes[lane - 1]) {
             // this block's share of the weights of layers to come
@@ -706,36 +772,41 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
 
     // ---- epilogue (code that runs once per block costs its instruction fetches: loops stay rolled) ----
     const unsigned tmem = *slot;
-    const int rows = npx / p.S, lo = rows * rank;
     const int kVec = CH / 4, kStep = kLoadWarps * 32 / kVec;
     const int col = (tid % kVec) * 4, r1 = tid / kVec, co = nt * CH + col;
     const bool mine = warp < kLoadWarps && co < p.c_out;
-    float4 sc = make_float4(1, 1, 1, 1), bi = make_float4(0, 0, 0, 0);
-    // residuals of the next kAhead rows: a tile with few stages is bound by how many of these loads are in flight
-    const int kAhead = F32 ? 4 : PX > 64 ? 2 : 1;   // (int8: registers that keep a third block resident count more)
+    // (rows of the tile are channels:) this thread's channel in float tiles, and residuals of its next 16 pixels
+    const int lch = (warp & 3) * 32 + lane, cch = nt * CH + lch;
+    const bool column = F32 && SWAP && warp < kLoadWarps && cch < p.c_out;
+    unsigned rc[16];
+    // residuals of the next kAhead rows (four channels each)
+    const int kAhead = 4;
     uint4 res[kAhead];
-#pragma unroll
-    for (int i = 0; i < kAhead; ++i) res[i] = make_uint4(0, 0, 0, 0);
     auto load_rows = [&](int row) {
 #pragma unroll
         for (int i = 0; i < kAhead; ++i) {
             const int m = m0 + lo + row + i * kStep;
             res[i] = make_uint4(0, 0, 0, 0);
-            if (p.residual && row + i * kStep < rows && m < p.M) res[i] = load_residual<F32>(p, m, co);
+            if (p.residual && row + i * kStep < rows && m < p.M) res[i] = load_residual(p, m, co);
         }
     };
-    if (mine && (SWAP ? !F32 || p.S == 1 : p.S > 1)) {
-        // of the rows this thread finishes first; on their way while the last multiply-adds run
-        load_channels(p, co, sc, bi);
-        load_rows(r1);
-    }
+    // of the pixels this thread finishes first; on their way while the last multiply-adds run
+    if (F32 && SWAP) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) rc[i] = 0;
+        if (column && p.residual) {
+            if (p.S == 1) load_column_residual<16>(p, m0 + (warp >> 2) * 16, cch, rc);
+            else if (rows % 4 == 0) load_split_residual<4>(p, m0 + lo, cch, tid >> 7, rows / 4, rc);
+            else if (rows % 2 == 0) load_split_residual<2>(p, m0 + lo, cch, tid >> 7, rows / 2, rc);
+            else load_split_residual<1>(p, m0 + lo, cch, tid >> 7, rows, rc);
+        }
+    } else if (F32 && mine) load_rows(r1);
     __syncwarp();
     if (p.S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory");   // every block has initialised its barriers
     if (warp < kLoadWarps) {
         // a warp can read the 32 rows 32 q ..; the warps with the same q take turns on groups of 16 columns
         const int q = warp & 3, N = SWAP ? npx : CH;
         const unsigned from = tmem + ((unsigned)(q * 32) << 16);
-        const int mrow = m0 + q * 32 + lane;   // (rows are pixels)
         mb_wait(done, 0u, p.gave_up);
         __syncwarp();
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
@@ -761,49 +832,27 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
             for (int t = 0; t < 16; ++t) v[t] = F32 ? __float_as_uint(__uint_as_float(v[t]) + __uint_as_float(u[t])) : v[t] + u[t];
             if (F32 && p.S > 1) {   // each pixel's sums to the block of the cluster that finishes it
                 if (SWAP) {
-                    if (rows % 4 == 0) send_columns<4>(p, base + p.recv_off, recv, rank, rows, j, q * 32 + lane, v);
-                    else if (rows % 2 == 0) send_columns<2>(p, base + p.recv_off, recv, rank, rows, j, q * 32 + lane, v);
-                    else send_columns<1>(p, base + p.recv_off, recv, rank, rows, j, q * 32 + lane, v);
+                    if (rows % 4 == 0) send_columns<4>(p, base + p.recv_off, recv, rank, rows, j, lch, v);
+                    else if (rows % 2 == 0) send_columns<2>(p, base + p.recv_off, recv, rank, rows, j, lch, v);
+                    else send_columns<1>(p, base + p.recv_off, recv, rank, rows, j, lch, v);
                 } else {
                     const int px = q * 32 + lane, owner = (int)fdiv((unsigned)px, p.d_rows), row = rank * rows + px - owner * rows;
 #pragma unroll
                     for (int t = 0; t < 16; t += 4) send<4>(base + p.recv_off + (row * C::kRow + j + t) * 4, recv, owner, v + t);
                 }
-            } else if (SWAP || p.S > 1) {   // to shared memory as [pixel][channel] (over the stages: all of them have been read)
-                if (SWAP) {
-                    const unsigned at = base + (j * C::kRow + q * 32 + lane) * 4;
-#pragma unroll
-                    for (int t = 0; t < 16; ++t) asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(at + t * C::kRow * 4), "r"(v[t]) : "memory");
-                } else {
-                    const unsigned at = base + ((q * 32 + lane) * C::kRow + j) * 4;
-#pragma unroll
-                    for (int t = 0; t < 16; t += 4) sts128(at + t * 4, make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]));
+            } else if (F32 && SWAP) {   // 16 pixels of one channel, straight to memory: a warp writes 128 contiguous bytes of each pixel
+                if (column) {
+                    finish_column<16>(p, m0 + j, cch, v, rc, lds32(consts + lch * 4), lds32(consts + (CH + lch) * 4));
+                    if (p.residual && j + kLoadWarps * 4 < N) load_column_residual<16>(p, m0 + j + kLoadWarps * 4, cch, rc);
                 }
-            } else if (mrow < p.M) {   // a lane per pixel: it finishes its 16 consecutive channels at once
-                unsigned q8[4];
+            } else if (SWAP) {   // to shared memory as [pixel][channel] (over the stages: all of them have been read)
+                const unsigned at = base + (j * C::kRow + lch) * 4;
 #pragma unroll
-                for (int t = 0; t < 16; t += 4) {
-                    const int c4 = nt * CH + j + t;
-                    if (c4 >= p.c_out) break;
-                    load_channels(p, c4, sc, bi);
-                    if (p.residual) res[0] = load_residual<F32>(p, mrow, c4);
-                    const uint4 t4 = make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]);
-                    if (!F32 && p.vec16) q8[t / 4] = finish_q4(p, t4, res[0].x, sc, bi);
-                    else finish4<F32>(p, (size_t)mrow * p.ldc + p.c_off + c4, p.c_out - c4, t4, res[0], sc, bi);
-                }
-                if (!F32 && p.vec16 && nt * CH + j < p.c_out) {
-                    *reinterpret_cast<uint4 *>(reinterpret_cast<signed char *>(p.y) + (size_t)place_of<POOL>(p, mrow) * p.ldc + p.c_off + nt * CH + j) =
-                        make_uint4(q8[0], q8[1], q8[2], q8[3]);
-                    if (POOL) {   // the four lanes of a window
+                for (int t = 0; t < 16; ++t) asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(at + t * C::kRow * 4), "r"(v[t]) : "memory");
+            } else {
+                const unsigned at = base + ((q * 32 + lane) * C::kRow + j) * 4;
 #pragma unroll
-                        for (int t = 0; t < 4; ++t) {
-                            q8[t] = __vmaxs4(q8[t], __shfl_xor_sync(15u << (lane & 28), q8[t], 1));
-                            q8[t] = __vmaxs4(q8[t], __shfl_xor_sync(15u << (lane & 28), q8[t], 2));
-                        }
-                        if ((lane & 3) == 0)
-                            *reinterpret_cast<uint4 *>(p.pooled + (size_t)(mrow >> 2) * p.c_out + nt * CH + j) = make_uint4(q8[0], q8[1], q8[2], q8[3]);
-                    }
-                }
+                for (int t = 0; t < 16; t += 4) sts128(at + t * 4, make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]));
             }
         }
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -814,16 +863,18 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"((unsigned)C::kCols) : "memory");
     }
-    if (!SWAP && p.S == 1) return;
+    if (F32 && SWAP && p.S == 1) return;
     const unsigned slice = rows * C::kRow * 4;   // partial sums of one sender (as [pixel][channel])
     if (F32) {
         if (warp >= kLoadWarps) return;
         if (SWAP && p.S > 1) {
-            const int ch = tid & 127;
+            mb_wait(recv, 0u, p.gave_up);
+            if (!column) return;
             const unsigned at = base + p.recv_off;
-            if (rows % 4 == 0) finish_split_columns<F32, 4>(p, at, rows, m0 + lo, nt * CH + ch, ch, tid >> 7, recv);
-            else if (rows % 2 == 0) finish_split_columns<F32, 2>(p, at, rows, m0 + lo, nt * CH + ch, ch, tid >> 7, recv);
-            else finish_split_columns<F32, 1>(p, at, rows, m0 + lo, nt * CH + ch, ch, tid >> 7, recv);
+            const float sc = lds32(consts + lch * 4), bi = lds32(consts + (CH + lch) * 4);
+            if (rows % 4 == 0) finish_split_columns<4>(p, at, rows, m0 + lo, cch, lch, tid >> 7, sc, bi, rc);
+            else if (rows % 2 == 0) finish_split_columns<2>(p, at, rows, m0 + lo, cch, lch, tid >> 7, sc, bi, rc);
+            else finish_split_columns<1>(p, at, rows, m0 + lo, cch, lch, tid >> 7, sc, bi, rc);
             return;
         }
         if (p.S > 1) mb_wait(recv, 0u, p.gave_up);
@@ -837,53 +888,62 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         // this block has received everything, so the others may go; it goes itself when they have received what it sent
         asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");
     }
-    if (POOL && mine) {   // a thread takes the four pixels of a window
+    if (mine) {
+        const float4 sc = lds_float4(consts + col * 4), bi = lds_float4(consts + (CH + col) * 4);
+        if (POOL) {   // a thread takes the four pixels of a window
 #pragma unroll 1
-        for (int g = r1; 4 * g < rows && m0 + lo + 4 * g < p.M; g += kStep) {
-            const unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (4 * g * C::kRow + col) * 4;
-            const int m = m0 + lo + 4 * g;
-            unsigned best = 0x80808080u;
+            for (int g = r1; 4 * g < rows && m0 + lo + 4 * g < p.M; g += kStep) {
+                const unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (4 * g * C::kRow + col) * 4;
+                const int m = m0 + lo + 4 * g;
+                unsigned best = 0x80808080u;
 #pragma unroll 1
-            for (int i = 0; i < 4; ++i) {
-                uint4 t = lds128(at + i * C::kRow * 4);
+                for (int i = 0; i < 4; ++i) {
+                    uint4 t = lds128(at + i * C::kRow * 4);
 #pragma unroll 4
-                for (int q = 1; q < p.S; ++q) {
-                    const uint4 u = lds128(at + i * C::kRow * 4 + q * slice);
-                    t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
-                }
-                const unsigned v = finish_q4(p, t, 0, sc, bi);
-                *reinterpret_cast<unsigned *>(reinterpret_cast<signed char *>(p.y) + (size_t)place_of<POOL>(p, m + i) * p.c_out + co) = v;
-                best = __vmaxs4(best, v);
-            }
-            *reinterpret_cast<unsigned *>(p.pooled + (size_t)(m >> 2) * p.c_out + co) = best;
-        }
-    } else if (mine) {
-        unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (r1 * C::kRow + col) * 4;
-#pragma unroll 1
-        for (int row = r1; row < rows; row += kAhead * kStep) {
-            uint4 r[kAhead];
-#pragma unroll
-            for (int i = 0; i < kAhead; ++i) r[i] = res[i];
-            if (row + kAhead * kStep < rows) load_rows(row + kAhead * kStep);
-#pragma unroll
-            for (int i = 0; i < kAhead; ++i) {
-                const int m = m0 + lo + row + i * kStep;
-                if (row + i * kStep >= rows || m >= p.M) break;
-                uint4 t = lds128(at);
-#pragma unroll 4
-                for (int q = 1; q < p.S; ++q) {
-                    const uint4 u = lds128(at + q * slice);
-                    if (F32) {
-                        t.x = __float_as_uint(__uint_as_float(t.x) + __uint_as_float(u.x));
-                        t.y = __float_as_uint(__uint_as_float(t.y) + __uint_as_float(u.y));
-                        t.z = __float_as_uint(__uint_as_float(t.z) + __uint_as_float(u.z));
-                        t.w = __float_as_uint(__uint_as_float(t.w) + __uint_as_float(u.w));
-                    } else {
+                    for (int q = 1; q < p.S; ++q) {
+                        const uint4 u = lds128(at + i * C::kRow * 4 + q * slice);
                         t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
                     }
+                    const unsigned v = finish_q4(p, t, 0, sc, bi);
+                    *reinterpret_cast<unsigned *>(reinterpret_cast<signed char *>(p.y) + (size_t)place_of<POOL>(p, m + i) * p.c_out + co) = v;
+                    best = __vmaxs4(best, v);
                 }
-                at += kStep * C::kRow * 4;
-                finish4<F32>(p, (size_t)m * p.ldc + p.c_off + co, p.c_out - co, t, r[i], sc, bi);
+                *reinterpret_cast<unsigned *>(p.pooled + (size_t)(m >> 2) * p.c_out + co) = best;
+            }
+        } else {
+            unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (r1 * C::kRow + col) * 4;
+#pragma unroll 1
+            for (int row = r1; row < rows; row += F32 ? kAhead * kStep : kStep) {
+                uint4 r[kAhead];
+                if (F32) {
+#pragma unroll
+                    for (int i = 0; i < kAhead; ++i) r[i] = res[i];
+                    if (row + kAhead * kStep < rows) load_rows(row + kAhead * kStep);
+                }
+#pragma unroll
+                for (int i = 0; i < (F32 ? kAhead : 1); ++i) {
+                    const int m = m0 + lo + row + i * kStep;
+                    if (row + i * kStep >= rows || m >= p.M) break;
+                    uint4 t = lds128(at);
+                    if (!F32) {
+                        r[0] = make_uint4(0, 0, 0, 0);
+                        if (p.res_tile) r[0].x = __float_as_uint(lds32(restile + row * CH + col));
+                    }
+#pragma unroll 4
+                    for (int q = 1; q < p.S; ++q) {
+                        const uint4 u = lds128(at + q * slice);
+                        if (F32) {
+                            t.x = __float_as_uint(__uint_as_float(t.x) + __uint_as_float(u.x));
+                            t.y = __float_as_uint(__uint_as_float(t.y) + __uint_as_float(u.y));
+                            t.z = __float_as_uint(__uint_as_float(t.z) + __uint_as_float(u.z));
+                            t.w = __float_as_uint(__uint_as_float(t.w) + __uint_as_float(u.w));
+                        } else {
+                            t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
+                        }
+                    }
+                    at += kStep * C::kRow * 4;
+                    finish4<F32>(p, (size_t)m * p.ldc + p.c_off + co, p.c_out - co, t, r[i], sc, bi);
+                }
             }
         }
     }
@@ -906,18 +966,19 @@ struct SmemPlan {
     int stages, recv_off, bar_off, bytes;
 };
 constexpr int tile_pixels(const Pick &k) { return k.ch == 64 ? 128 : k.px <= 64 ? 64 : k.px <= 128 ? 128 : 256; }   // PX of the kernel shape
-constexpr SmemPlan plan_smem(bool f32, const Pick &k, int nkb)
+constexpr SmemPlan plan_smem(bool f32, const Pick &k, int nkb, bool res_tile)
 {
     const int PX = tile_pixels(k);
     const bool swap = k.ch == 128;
     const int stage = (f32 ? 3 : 2) * 64 * (k.px + k.ch), out = k.px * (k.ch + 4) * 4;
-    const int budget = (PX > 128 ? 216 : 108) * 1024;   // two blocks share a multiprocessor but for the largest shape
+    const int res = res_tile ? k.px / k.split * k.ch : 0;
+    const int budget = (PX > 128 ? 216 : 108) * 1024 - res;   // two blocks share a multiprocessor but for the largest shape
     SmemPlan s = {};
     s.stages = std::max(2, std::min(std::min(4, std::max(2, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
-    // sums staged over the stages: unsplit tiles whose rows are channels, and int8 split tiles
-    s.recv_off = std::max(s.stages * stage, (swap && k.split == 1) || (!f32 && k.split > 1) ? out : 0);
+    // sums staged over the stages: int8 tiles, and unsplit float tiles whose rows are pixels
+    s.recv_off = std::max(s.stages * stage, !f32 || (!swap && k.split == 1) ? out : 0);
     s.bar_off = (s.recv_off + (k.split > 1 ? out : 0) + 127) / 128 * 128;
-    s.bytes = s.bar_off + 1024 + 128 + PX * 8;
+    s.bytes = s.bar_off + 1024 + 128 + PX * 8 + k.ch * 8 + res;
     // Blocks of a cluster wait for each other while they hold tensor memory.  Were more of them resident than it has columns for,
     // two clusters could each hold what the other's last block waits for; so a block of c columns takes more than c / 640 of the
     // multiprocessor's shared memory, and five quarters of the columns never fit.  (Other blocks hold columns too, but finish by
@@ -933,7 +994,7 @@ constexpr bool clusters_find_tensor_memory()
                 for (int split = 2; split <= 16; ++split)
                     for (int nkb = split; nkb <= 5 * split; ++nkb) {
                         const Pick k = {ch == 64 ? 128 : px, ch, split};
-                        if (5 * (plan_smem(f32, k, nkb).bytes + kSmemReserved) <= tensor_columns(f32, ch == 64 ? 64 : tile_pixels(k)) / 128 * kSmemOfSm)
+                        if (5 * (plan_smem(f32, k, nkb, false).bytes + kSmemReserved) <= tensor_columns(f32, ch == 64 ? 64 : tile_pixels(k)) / 128 * kSmemOfSm)
                             return false;
                     }
     return true;
@@ -971,7 +1032,7 @@ const Cost kCost[2][9] = {   // float, int8; 128 px x 64 ch, then up to 32, 64 a
      {0.507f, 5.89f, 0.0f, 0.563f, 4.98f, 0.0f, 0.356f},
      {0.0f, 11.6f, 0.0f, 0.578f, 6.35f, 0.0f, 0.21f}}};
 
-Pick choose(bool f32, int c_out, long long M, int nkb)
+Pick choose(bool f32, int c_out, long long M, int nkb, bool res_tile)
 {
     Pick best = {128, 64, 1};
     double best_t = 1e300;
@@ -983,7 +1044,7 @@ Pick choose(bool f32, int c_out, long long M, int nkb)
             if (split > 1 && tiles * split > 330) break;      // the grid already fills the chip twice
             static const int cap1[5] = {148, 74, 33, 15, 7}, cap2[5] = {296, 148, 71, 33, 14};
             const Pick k = {px, ch, split};
-            const bool two = plan_smem(f32, k, nkb).bytes <= 113 * 1024;
+            const bool two = plan_smem(f32, k, nkb, res_tile).bytes <= 113 * 1024;
             long long P = 0, Q = 0;
             if (two) {
                 P = tiles / cap2[log];
@@ -1013,7 +1074,7 @@ cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
 {
     auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC, POOL, TAIL>;
     typedef Cfg<F32, PX, CH, SWAP, VEC> C;
-    const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb);
+    const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb, p.res_tile != 0);
     if (sp.stages < C::kGroups || sp.stages * C::kParts * 64 * (p.npx + CH) > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
     p.stages = sp.stages;
     p.recv_off = sp.recv_off;
@@ -1271,14 +1332,13 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     p.ldc = ep.out_c_total > 0 ? ep.out_c_total : d.c_out;
     p.c_off = ep.out_c_total > 0 ? ep.out_c_off : 0;
     p.vec_ok = d.c_out % 4 == 0 && p.ldc % 4 == 0 && p.c_off % 4 == 0;
-    p.vec16 = ep.out_dtype == CADNN_S8 && d.c_out % 16 == 0 && p.ldc % 16 == 0 && p.c_off % 16 == 0;
     if (ep.pooled) {
         if (!tcv_pools(w, n) || ep.residual || ep.out_dtype != CADNN_S8 || ep.out_c_total > 0) return CADNN_E_UNSUPPORTED;
         p.pooled = (signed char *)ep.pooled;
         p.h_out /= 2;
         p.w_out /= 2;
     }
-    p.vec_sb = ((uintptr_t)ep.scale & 15) == 0 && ((uintptr_t)ep.bias & 15) == 0;
+    p.res_tile = f32 || !ep.residual ? 0 : d.c_out % 16 == 0 ? 16 : d.c_out % 4 == 0 ? 4 : 1;
     p.d_hw = make_fastdiv(p.h_out * p.w_out); p.d_wo = make_fastdiv(p.w_out);
     p.d_ci = make_fastdiv(d.c_in); p.d_Rp = make_fastdiv(p.Rp);
     if (ep.prefetch) p.ahead = *ep.prefetch;
@@ -1290,7 +1350,7 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     if (pick.px > 0) pick.split = std::max(1, pick.split);
     else if ((kept >> 32) == (uint64_t)n && kept != 0) pick = {(int)(kept & 0xfff), (int)(kept >> 12 & 0xfff), (int)(kept >> 24 & 0xff)};
     else {
-        pick = choose(f32, d.c_out, M, p.nkb);
+        pick = choose(f32, d.c_out, M, p.nkb, p.res_tile != 0);
         w->tcv_pick.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
     }
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0, run_tail = !f32 && !vec && p.tail;

@@ -215,3 +215,41 @@ def test_reported_bytes_cover_the_device_memory_of_a_handle(kind):
     dense = (250 + 63) // 64 * 64 * 9 * 256 * (1 if s8 else 6) if kind.startswith("conv") else 1024 * 2048 * (1 if s8 else 6)
     assert told >= dense, (told, dense)
     assert told <= used + 2 ** 21 and used <= told + 3 * 2 ** 21, (told, used)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "s8"])
+@pytest.mark.parametrize("shape", ["48,128,16", "16,128,16", "112,128,16", "32,128,4", "128,64,2"])
+def test_shares_of_a_split_tile(shape, dtype, monkeypatch):
+    """A split tile's blocks finish 3, 1, 7, 8 and 64 pixels each (sums sent one, four, ... at a time, a block's own share stored),
+    with a residual that they ask for ahead, on a map whose last tile is ragged."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(53)
+    layer = (2, 11, 7, 64, 136, 3, 1, 1)
+    n, h, wd, c_in, c_out, k, stride, pad = layer
+    dev = lambda a: torch.from_numpy(a).to(DEV)
+    mask = gen.random_mask(g, (c_out, k, k, c_in), 0.2)
+    if dtype == "s8":   # 18 x 128 values of K: 64-channel stages of two taps
+        layer = (2, 11, 7, 256, 136, 3, 1, 1)
+        c_in, mask = 256, gen.random_mask(g, (c_out, k, k, 256), 0.2)
+        x, q = gen.int8_relu_activation(g, (n, h, wd, c_in)), gen.int8_weights(g, (c_out, k, k, c_in))
+        m = (g.uniform(0.5, 1.5, size=c_out) * 2e-4).astype(np.float32)
+        b = (g.standard_normal(c_out) * 3).astype(np.float32)
+        r = gen.int8_relu_activation(g, (n, h, wd, c_out))
+        want = ref.conv2d_s8(x, q, mask, stride, pad, 1, m, b, "relu", "s8", r, 0.4)
+        wh = _pack(B, monkeypatch, shape, dtype, layer, q, mask)
+        y = torch.full(want.shape, 5, dtype=torch.int8, device=DEV)
+        B.cadnn_conv2d(wh, dev(x), y, dev(m), dev(b), dev(r), "relu", out_dtype="s8", residual_scale=0.4)
+        torch.cuda.synchronize()
+        assert_exact(y.cpu().numpy(), want, shape)
+    else:
+        x, w = gen.relu_normal_input(g, (n, h, wd, c_in)), gen.he_weights(g, c_out, k, k, c_in)
+        scale, bias = gen.folded_bn(g, c_out)
+        r = gen.normal_input(g, (n, h, wd, c_out))
+        want = ref.conv2d_f32(x, w, mask, stride, pad, 1, scale, bias, r, "relu")
+        wh = _pack(B, monkeypatch, shape, dtype, layer, w, mask)
+        y = torch.full(want.shape, -1.0, device=DEV)
+        B.cadnn_conv2d(wh, dev(x), y, dev(scale), dev(bias), dev(r), "relu")
+        torch.cuda.synchronize()
+        s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None, stride, pad, 1, np.abs(scale), np.abs(bias), np.abs(r), "none")
+        assert_close_or_bounded(y.cpu().numpy(), want, s_abs, int(mask.reshape(c_out, -1).sum(1).max()) + 4, shape)
+    assert B.cadnn_device_status()["copy_timeouts"] == 0
