@@ -495,13 +495,22 @@ __device__ __forceinline__ void finish_split_columns(const TcvParams &p, unsigne
         }
     }
 }
+// (What stays in this block is stored, not sent: the link between multiprocessors carries about 15 bytes a clock out of each, and its
+// latency is the same for a block itself.  32 pixels x 128 channels split in 2 / 4 / 8, 224 blocks: 1830 / 1820 / 2240 clocks sent to
+// all, 1270 / 1430 / 1930 to the others.)
 template <int U>
 __device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, unsigned bar, int rank, int rows, int j, int ch, const unsigned (&v)[16])
 {
 #pragma unroll
     for (int t = 0; t < 16; t += U) {
         const int owner = (int)fdiv((unsigned)(j + t), p.d_rows), row = (j + t) - owner * rows;
-        send<U>(at + ((rank * (rows / U) + row / U) * 128 + ch) * (U * 4), bar, owner, v + t);
+        const unsigned a = at + ((rank * (rows / U) + row / U) * 128 + ch) * (U * 4);
+        if (owner == rank) {
+            if (U == 4) sts128(a, make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]));
+            else
+#pragma unroll
+                for (int i = 0; i < U; ++i) asm volatile("st.shared.b32 [%0], %1;\n" ::"r"(a + 4 * i), "r"(v[t + i]) : "memory");
+        } else send<U>(a, bar, owner, v + t);
     }
 }
 
@@ -563,8 +572,8 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
             mb_init(recv, 1);
             asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
             asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-            // partial sums of this block's pixels from every block of the cluster, itself included
-            if (p.S > 1) mb_expect_tx(recv, (unsigned)(npx * (F32 ? CH : C::kRow) * 4));
+            // partial sums of this block's pixels from every other block of the cluster
+            if (p.S > 1) mb_expect_tx(recv, (unsigned)((npx - rows) * (F32 ? CH : C::kRow) * 4));
         }
     } else if (warp == kLoadWarps + 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(slot32), "r"((unsigned)C::kCols) : "memory");
@@ -838,7 +847,11 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                 } else {
                     const int px = q * 32 + lane, owner = (int)fdiv((unsigned)px, p.d_rows), row = rank * rows + px - owner * rows;
 #pragma unroll
-                    for (int t = 0; t < 16; t += 4) send<4>(base + p.recv_off + (row * C::kRow + j + t) * 4, recv, owner, v + t);
+                    for (int t = 0; t < 16; t += 4) {
+                        const unsigned a = base + p.recv_off + (row * C::kRow + j + t) * 4;
+                        if (owner == rank) sts128(a, make_uint4(v[t], v[t + 1], v[t + 2], v[t + 3]));
+                        else send<4>(a, recv, owner, v + t);
+                    }
                 }
             } else if (F32 && SWAP) {   // 16 pixels of one channel, straight to memory: a warp writes 128 contiguous bytes of each pixel
                 if (column) {
@@ -881,7 +894,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
     } else if (p.S > 1) {
         // Int8 layers exchange through staged tiles and bulk copies: packed stores need 4 channels in a thread, and the register
         // route's code costs them a third resident block per multiprocessor (int8 ResNet-50, batch 8: 421 against 451 us).
-        if (tid < p.S) send_bulk(base + p.recv_off + rank * slice, base + tid * slice, slice, recv, tid);
+        if (tid < p.S && tid != rank) send_bulk(base + p.recv_off + rank * slice, base + tid * slice, slice, recv, tid);
         __syncwarp();
         if (warp < kLoadWarps) mb_wait(recv, 0u, p.gave_up);
         __syncwarp();
@@ -893,15 +906,15 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         if (POOL) {   // a thread takes the four pixels of a window
 #pragma unroll 1
             for (int g = r1; 4 * g < rows && m0 + lo + 4 * g < p.M; g += kStep) {
-                const unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (4 * g * C::kRow + col) * 4;
+                const unsigned in = (4 * g * C::kRow + col) * 4, at = base + p.recv_off + in, own = base + rank * slice + in;
                 const int m = m0 + lo + 4 * g;
                 unsigned best = 0x80808080u;
 #pragma unroll 1
                 for (int i = 0; i < 4; ++i) {
-                    uint4 t = lds128(at + i * C::kRow * 4);
+                    uint4 t = lds128(own + i * C::kRow * 4);
 #pragma unroll 4
                     for (int q = 1; q < p.S; ++q) {
-                        const uint4 u = lds128(at + i * C::kRow * 4 + q * slice);
+                        const uint4 u = lds128(at + i * C::kRow * 4 + (q <= rank ? q - 1 : q) * slice);
                         t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
                     }
                     const unsigned v = finish_q4(p, t, 0, sc, bi);
@@ -911,7 +924,9 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                 *reinterpret_cast<unsigned *>(p.pooled + (size_t)(m >> 2) * p.c_out + co) = best;
             }
         } else {
-            unsigned at = base + (p.S > 1 ? p.recv_off : 0) + (r1 * C::kRow + col) * 4;
+            // (this block's own sums: int8 where they were staged, float among the received ones)
+            unsigned at = base + p.recv_off + (r1 * C::kRow + col) * 4, own = at + rank * slice;
+            if (!F32 || p.S == 1) own -= p.recv_off;
 #pragma unroll 1
             for (int row = r1; row < rows; row += F32 ? kAhead * kStep : kStep) {
                 uint4 r[kAhead];
@@ -924,14 +939,14 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                 for (int i = 0; i < (F32 ? kAhead : 1); ++i) {
                     const int m = m0 + lo + row + i * kStep;
                     if (row + i * kStep >= rows || m >= p.M) break;
-                    uint4 t = lds128(at);
+                    uint4 t = lds128(own);
                     if (!F32) {
                         r[0] = make_uint4(0, 0, 0, 0);
                         if (p.res_tile) r[0].x = __float_as_uint(lds32(restile + row * CH + col));
                     }
 #pragma unroll 4
                     for (int q = 1; q < p.S; ++q) {
-                        const uint4 u = lds128(at + q * slice);
+                        const uint4 u = lds128(at + (q <= rank ? q - 1 : q) * slice);
                         if (F32) {
                             t.x = __float_as_uint(__uint_as_float(t.x) + __uint_as_float(u.x));
                             t.y = __float_as_uint(__uint_as_float(t.y) + __uint_as_float(u.y));
@@ -942,6 +957,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                         }
                     }
                     at += kStep * C::kRow * 4;
+                    own += kStep * C::kRow * 4;
                     finish4<F32>(p, (size_t)m * p.ldc + p.c_off + co, p.c_out - co, t, r[i], sc, bi);
                 }
             }
