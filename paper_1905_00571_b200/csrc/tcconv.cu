@@ -36,6 +36,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <cstdio>
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include "cadnn_internal.h"
 
@@ -44,6 +45,7 @@ namespace {
 const int kSpin = 1 << 22;
 
 struct TcvParams {
+    CUtensorMap pixels;              // Gather::kCopyEngine: the input as im2col rows
     const void *x;
     void *y;
     const unsigned char *wimg;
@@ -57,6 +59,7 @@ struct TcvParams {
     int stages, recv_off, bar_off;   // pipeline depth; byte offsets of the partial sums and of the barriers in shared memory
     int res_tile;                    // int8: the residual of the block's outputs is brought into shared memory, this many bytes at a time (0: no residual)
     int ldc, c_off, vec_ok;          // vec_ok: output and residual allow 4 channels per access
+    int odd_half;                    // copy engine: 1 if the last stage's second 64 positions lie beyond K
     int kb_base, kb_rem;             // stages per block of a cluster: kb_base, and one more in the first kb_rem blocks
     int whole, tail;                 // int8 input: bytes of its whole 4-byte words, and bytes behind them
     int Rp;                          // K positions per kernel row: kw * c_in rounded up to 16 bytes
@@ -94,6 +97,13 @@ __device__ __forceinline__ void bulk_copy(unsigned dst, const void *src, unsigne
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+// Rows of the im2col matrix by the copy engine: `pixels` output pixels from the one whose window starts at (w, h) of image n on (both
+// may lie in the padding), 64 channels from c on at window position (kx, ky), as 64-byte swizzled rows.
+__device__ __forceinline__ void copy_pixels(unsigned dst, const CUtensorMap *map, int c, int w, int h, int n, int kx, int ky, unsigned bar)
+{
+    asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2], {%7, %8};\n"
+                 ::"r"(dst), "l"(map), "r"(bar), "r"(c), "r"(w), "r"(h), "r"(n), "h"((unsigned short)kx), "h"((unsigned short)ky) : "memory");
 }
 // K-major operand tile, 64-byte rows, 64-byte swizzle (16-byte chunk index ^= (row / 2) % 4)
 __device__ __forceinline__ unsigned long long smem_desc(unsigned addr)
@@ -233,10 +243,14 @@ constexpr int tensor_columns(bool f32, int n)
     return accumulators(f32, n) * n <= 128 ? 128 : accumulators(f32, n) * n <= 256 ? 256 : 512;
 }
 
+// How the activations come into shared memory: values one by one or as shifted words (pixels of any number of channels), 16 bytes at a
+// time (whole 16-byte pieces of channels), or by the copy engine (int8, whole 64-channel rows).
+enum class Gather { kValues, kPieces, kCopyEngine };
+
 // One kernel shape: PX pixels x CH channels per block.  SWAP: the channels are the 128 rows of the tensor-core tile and
 // the pixels its columns (any multiple of 16 up to PX, so that small maps waste little); otherwise the 128 rows are pixels
 // and the columns CH channels.
-template <bool F32, int PX, int CH, bool SWAP, bool VEC> struct Cfg {
+template <bool F32, int PX, int CH, bool SWAP, Gather GATHER> struct Cfg {
     static const int kParts = F32 ? 3 : 2;                 // operand tiles of 64-byte rows per stage
     static const int kKB = F32 ? 32 : 128;                 // K values per stage (128 source bytes per pixel)
     static const int kWBytes = kParts * CH * 64;
@@ -248,7 +262,7 @@ template <bool F32, int PX, int CH, bool SWAP, bool VEC> struct Cfg {
     // Blocks per multiprocessor the registers are cut for (more than tensor memory holds would wait in tcgen05.alloc).  Int8 tiles
     // of 128 columns and layers with few stages are small enough for three (int8 ResNet-50, batch 32: 963 us with 62 to 78
     // registers and one residual row ahead, 923 us with 64 and two; four rows 947, eight 998).
-    static const int kBlocks = PX > 128 ? 1 : F32 || !VEC || 3 * kCols > kTensorColumns ? 2 : 3;
+    static const int kBlocks = PX > 128 ? 1 : F32 || GATHER == Gather::kValues || 3 * kCols > kTensorColumns ? 2 : 3;
     static_assert(kBlocks * kCols <= kTensorColumns, "a block would wait for tensor memory that its neighbours hold");
     static const int kRow = CH + 4;                        // words per pixel of the exchanged sums (conflict-free 16-byte access)
     static const int kLoadWarps = PX > 128 ? 16 : 8;
@@ -516,10 +530,11 @@ __device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, un
 
 // (POOL and TAIL are instantiations of their own: as branches at run time they cost the int8 ResNet-50, which has neither such a pool
 // nor such a tensor, 0.7 and 0.4 %.)
-template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL, bool TAIL>
-__global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32, PX, CH, SWAP, VEC>::kBlocks) tcconv_kernel(const TcvParams p)
+template <bool F32, int PX, int CH, bool SWAP, Gather GATHER, bool POOL, bool TAIL>
+__global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, GATHER>::kThreads, Cfg<F32, PX, CH, SWAP, GATHER>::kBlocks) tcconv_kernel(const __grid_constant__ TcvParams p)
 {
-    typedef Cfg<F32, PX, CH, SWAP, VEC> C;
+    const bool VEC = GATHER == Gather::kPieces, ENGINE = GATHER == Gather::kCopyEngine;
+    typedef Cfg<F32, PX, CH, SWAP, GATHER> C;
     const int kLoadWarps = C::kLoadWarps;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const unsigned raw32 = (unsigned)__cvta_generic_to_shared(smem_raw);
@@ -551,7 +566,9 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         int cnt = 0;
 #pragma unroll
         for (int q = 0; q < CH / 64; ++q) cnt += nt * (CH / 64) + q < n64;
-        mb_expect_tx(full, (unsigned)(cnt * C::kParts * 4096));
+        unsigned bytes = cnt * C::kParts * 4096;
+        if (ENGINE) bytes += 2 * kb + 1 < 2 * p.nkb - p.odd_half ? xbytes : xpart;
+        mb_expect_tx(full, bytes);
 #pragma unroll
         for (int q = 0; q < CH / 64; ++q) {
             const int nb = nt * (CH / 64) + q;
@@ -565,7 +582,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
     if (warp == kLoadWarps) {
         if (lane == 0) {
             for (int i = 0; i < S; ++i) {
-                mb_init(bars + i * 8, kLoadWarps / C::kGroups + 1);
+                mb_init(bars + i * 8, ENGINE ? 1 : kLoadWarps / C::kGroups + 1);
                 mb_init(bars + (S + i) * 8, 1);
             }
             mb_init(done, 1);
@@ -579,7 +596,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(slot32), "r"((unsigned)C::kCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
         asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    } else if (tid < PX) {
+    } else if (!ENGINE && tid < PX) {
         const int m = m0 + tid;
         const int at = POOL ? m >> 2 : m;
         const int img = (int)fdiv((unsigned)at, p.d_hw), q = at - img * p.h_out * p.w_out;
@@ -606,7 +623,33 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
     if (p.S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory");   // waited for before the first remote copy
     __syncthreads();
 
-    if (warp < kLoadWarps) {
+    // What the epilogue needs, asked for ahead so that it has arrived by then (loading it there cost a round trip to L2 for every four
+    // channels or residual row: 64 -> 256 1x1 int8 with a residual, 128 x 128 tile, 9000 of 12500 clocks).
+    auto request_epilogue = [&]() {
+        if (tid < CH) {
+            const int ch = nt * CH + tid;
+            const unsigned a = consts + tid * 4;
+            if (p.scale && ch < p.c_out) copy4(a, p.scale + ch);
+            else asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a), "f"(1.0f) : "memory");
+            if (p.bias && ch < p.c_out) copy4(a + CH * 4, p.bias + ch);
+            else asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a + CH * 4), "f"(0.0f) : "memory");
+        }
+        if (!F32 && p.res_tile >= 4) {
+            const int log = p.res_tile == 16 ? 4 : 2, per = CH >> log;
+            for (int i = tid; i < rows * per; i += kLoadWarps * 32) {
+                const int row = i / per, m = m0 + lo + row, at = (i - row * per) << log, ch = nt * CH + at;
+                if (m >= p.M || ch >= p.c_out) continue;
+                const char *src = reinterpret_cast<const char *>(p.residual) + (size_t)m * p.c_out + ch;
+                if (log == 4) copy16(restile + row * CH + at, src);
+                else copy4(restile + row * CH + at, src);
+            }
+        }
+    };
+    if (ENGINE && warp < kLoadWarps) {
+        grid_dep_wait();
+        request_epilogue();
+        grid_dep_trigger();
+    } else if (warp < kLoadWarps) {
         uint4 v[C::kRPT];
         // Window starts stay in registers, and the loads are predicated: with the starts read from shared memory for every stage and
         // the loads behind branches one piece was issued every 100 clocks, 430 of a stage's 1800 (64 pixels).
@@ -634,26 +677,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         };
         grid_dep_wait();
         if (kb0 + grp < kb1) request();
-        // What the epilogue needs, asked for now so that it has arrived by then (loading it there cost a round trip to L2 for every
-        // four channels or residual row: 64 -> 256 1x1 int8 with a residual, 128 x 128 tile, 9000 of 12500 clocks).
-        if (tid < CH) {
-            const int ch = nt * CH + tid;
-            const unsigned a = consts + tid * 4;
-            if (p.scale && ch < p.c_out) copy4(a, p.scale + ch);
-            else asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a), "f"(1.0f) : "memory");
-            if (p.bias && ch < p.c_out) copy4(a + CH * 4, p.bias + ch);
-            else asm volatile("st.shared.f32 [%0], %1;\n" ::"r"(a + CH * 4), "f"(0.0f) : "memory");
-        }
-        if (!F32 && p.res_tile >= 4) {
-            const int log = p.res_tile == 16 ? 4 : 2, per = CH >> log;
-            for (int i = tid; i < rows * per; i += kLoadWarps * 32) {
-                const int row = i / per, m = m0 + lo + row, at = (i - row * per) << log, ch = nt * CH + at;
-                if (m >= p.M || ch >= p.c_out) continue;
-                const char *src = reinterpret_cast<const char *>(p.residual) + (size_t)m * p.c_out + ch;
-                if (log == 4) copy16(restile + row * CH + at, src);
-                else copy4(restile + row * CH + at, src);
-            }
-        }
+        request_epilogue();
         // swizzled place of the thread's chunk in pixel row r0 of an operand tile (rows kPS apart have the same pattern)
         const unsigned sw = (unsigned)((r0 >> 1) & 3);
         const unsigned at = F32 ? r0 * 64 + ((((unsigned)c >> 1) ^ sw) << 4) + (c & 1) * 8
@@ -691,25 +715,6 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
             s += C::kGroups;
         }
         grid_dep_trigger();
-        if (!F32 && p.res_tile == 1) {   // channels of no multiple of 4: byte by byte, 16 on their way at once
-#pragma unroll 1
-            for (int i = tid; i < rows * CH; i += kLoadWarps * 32 * 16) {
-                int b[16];
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int at = i + k * kLoadWarps * 32, m = m0 + lo + at / CH, ch = nt * CH + at % CH;
-                    b[k] = 0;
-                    if (at < rows * CH && m < p.M && ch < p.c_out) b[k] = ld_act(reinterpret_cast<const signed char *>(p.residual) + (size_t)m * p.c_out + ch);
-                }
-#pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int at = i + k * kLoadWarps * 32;
-                    if (at < rows * CH) asm volatile("st.shared.u8 [%0], %1;\n" ::"r"(restile + at), "r"(b[k]) : "memory");
-                }
-            }
-        }
-        copies_landed();
-        asm volatile("bar.sync 1, %0;\n" ::"n"(C::kLoadWarps * 32) : "memory");
     } else if (warp == kLoadWarps) {
         if (lane > 0 && lane <= Prefetch::kMax && p.ahead.bytes[lane - 1]) {
             // this block's share of the weights of layers to come
@@ -719,11 +724,41 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
                              ::"l"((const char *)p.ahead.at[lane - 1] + lo), "r"((unsigned)(min(part, n - lo) & ~15ull)) : "memory");
         }
         if (lane == 0) {
-            int s = 0;
-            unsigned round = 0;
-            for (int kb = kb0; kb < kb1; ++kb) {
+            // where the window of the tile's first pixel starts, and the position of the next 64 values of K (copy engine)
+            const int at = POOL ? m0 >> 2 : m0, img = (int)fdiv((unsigned)at, p.d_hw), q = at - img * p.h_out * p.w_out;
+            const int oy = (int)fdiv((unsigned)q, p.d_wo), ox = q - oy * p.w_out, step = (POOL ? 2 : 1) * p.stride;
+            const int iy = oy * step - p.pad, ix = ox * step - p.pad_w;
+            int ky = (int)fdiv((unsigned)(kb0 * C::kKB), p.d_Rp), ci = kb0 * C::kKB - ky * p.Rp, kx = (int)fdiv((unsigned)ci, p.d_ci);
+            ci -= kx * p.c_in;
+            auto pixels = [&](int s) {
+#pragma unroll
+                for (int t = 0; t < 2; ++t) {
+                    if (ky == p.kh) break;
+                    const unsigned dst = base + s * stage + t * xpart;
+                    if (!POOL) copy_pixels(dst, &p.pixels, ci, ix, iy, img, kx, ky, bars + s * 8);
+                    else   // a quarter of the rows for each place in a window
+#pragma unroll
+                        for (int r = 0; r < 4; ++r)
+                            copy_pixels(dst + r * (xpart / 4), &p.pixels, ci, ix, iy, img, kx + (r & 1) * p.stride, ky + (r >> 1) * p.stride, bars + s * 8);
+                    ci += 64;
+                    if (ci == p.c_in) {
+                        ci = 0;
+                        if (++kx == p.kw) { kx = 0; ++ky; }
+                    }
+                }
+            };
+            const int ahead = ENGINE ? min(S, kb1 - kb0) : 0;
+            if (ENGINE) {   // weights do not wait for the previous layer
+                for (int i = 0; i < ahead; ++i) copy_weights(kb0 + i, i);
+                grid_dep_wait();
+                for (int i = 0; i < ahead; ++i) pixels(i);
+            }
+            int s = ahead == S ? 0 : ahead;
+            unsigned round = ahead == S;
+            for (int kb = kb0 + ahead; kb < kb1; ++kb) {
                 if (round > 0 && !mb_wait(bars + (S + s) * 8, (round - 1) & 1u, p.gave_up)) break;
                 copy_weights(kb, s);
+                if (ENGINE) pixels(s);
                 if (++s == S) { s = 0; ++round; }
             }
         }
@@ -778,6 +813,27 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         tc_commit(done);
     }
     __syncwarp();
+    if (warp < kLoadWarps) {
+        if (!F32 && p.res_tile == 1) {   // channels of no multiple of 4: byte by byte, 16 on their way at once
+#pragma unroll 1
+            for (int i = tid; i < rows * CH; i += kLoadWarps * 32 * 16) {
+                int b[16];
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const int at = i + k * kLoadWarps * 32, m = m0 + lo + at / CH, ch = nt * CH + at % CH;
+                    b[k] = 0;
+                    if (at < rows * CH && m < p.M && ch < p.c_out) b[k] = ld_act(reinterpret_cast<const signed char *>(p.residual) + (size_t)m * p.c_out + ch);
+                }
+#pragma unroll
+                for (int k = 0; k < 16; ++k) {
+                    const int at = i + k * kLoadWarps * 32;
+                    if (at < rows * CH) asm volatile("st.shared.u8 [%0], %1;\n" ::"r"(restile + at), "r"(b[k]) : "memory");
+                }
+            }
+        }
+        copies_landed();
+        asm volatile("bar.sync 1, %0;\n" ::"n"(C::kLoadWarps * 32) : "memory");
+    }
 
     // ---- epilogue (code that runs once per block costs its instruction fetches: loops stay rolled) ----
     const unsigned tmem = *slot;
@@ -906,15 +962,17 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, VEC>::kThreads, Cfg<F32
         if (POOL) {   // a thread takes the four pixels of a window
 #pragma unroll 1
             for (int g = r1; 4 * g < rows && m0 + lo + 4 * g < p.M; g += kStep) {
-                const unsigned in = (4 * g * C::kRow + col) * 4, at = base + p.recv_off + in, own = base + rank * slice + in;
+                // (the copy engine leaves a window's pixels a quarter of the tile apart)
+                const int next = ENGINE ? npx / 4 : 1;
+                const unsigned in = ((ENGINE ? g : 4 * g) * C::kRow + col) * 4, at = base + p.recv_off + in, own = base + rank * slice + in;
                 const int m = m0 + lo + 4 * g;
                 unsigned best = 0x80808080u;
 #pragma unroll 1
                 for (int i = 0; i < 4; ++i) {
-                    uint4 t = lds128(own + i * C::kRow * 4);
+                    uint4 t = lds128(own + i * next * C::kRow * 4);
 #pragma unroll 4
                     for (int q = 1; q < p.S; ++q) {
-                        const uint4 u = lds128(at + i * C::kRow * 4 + (q <= rank ? q - 1 : q) * slice);
+                        const uint4 u = lds128(at + i * next * C::kRow * 4 + (q <= rank ? q - 1 : q) * slice);
                         t.x += u.x; t.y += u.y; t.z += u.z; t.w += u.w;
                     }
                     const unsigned v = finish_q4(p, t, 0, sc, bi);
@@ -1085,11 +1143,11 @@ Pick choose(bool f32, int c_out, long long M, int nkb, bool res_tile)
     return best;
 }
 
-template <bool F32, int PX, int CH, bool SWAP, bool VEC, bool POOL, bool TAIL>
+template <bool F32, int PX, int CH, bool SWAP, Gather GATHER, bool POOL, bool TAIL>
 cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
 {
-    auto kern = tcconv_kernel<F32, PX, CH, SWAP, VEC, POOL, TAIL>;
-    typedef Cfg<F32, PX, CH, SWAP, VEC> C;
+    auto kern = tcconv_kernel<F32, PX, CH, SWAP, GATHER, POOL, TAIL>;
+    typedef Cfg<F32, PX, CH, SWAP, GATHER> C;
     const SmemPlan sp = plan_smem(F32, {p.npx, CH, p.S}, p.nkb, p.res_tile != 0);
     if (sp.stages < C::kGroups || sp.stages * C::kParts * 64 * (p.npx + CH) > sp.recv_off || p.npx > PX) return CADNN_E_UNSUPPORTED;
     p.stages = sp.stages;
@@ -1123,12 +1181,12 @@ cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
     return CADNN_OK;
 }
 
-template <bool F32, bool VEC, bool POOL = false, bool TAIL = false> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
+template <bool F32, Gather GATHER, bool POOL = false, bool TAIL = false> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
 {
-    if (ch == 64) return launch_one<F32, 128, 64, false, VEC, POOL, TAIL>(p, blocks, pdl, st);
-    if (p.npx <= 64) return launch_one<F32, 64, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);
-    if (TAIL || p.npx <= 128) return launch_one<F32, 128, 128, true, VEC, POOL, TAIL>(p, blocks, pdl, st);   // (256 pixels would spill registers)
-    return launch_one<F32, 256, 128, true, VEC, POOL, false>(p, blocks, pdl, st);
+    if (ch == 64) return launch_one<F32, 128, 64, false, GATHER, POOL, TAIL>(p, blocks, pdl, st);
+    if (p.npx <= 64) return launch_one<F32, 64, 128, true, GATHER, POOL, TAIL>(p, blocks, pdl, st);
+    if (TAIL || p.npx <= 128) return launch_one<F32, 128, 128, true, GATHER, POOL, TAIL>(p, blocks, pdl, st);   // (256 pixels would spill registers)
+    return launch_one<F32, 256, 128, true, GATHER, POOL, false>(p, blocks, pdl, st);
 }
 
 }  // namespace
@@ -1329,6 +1387,48 @@ bool tcv_pools(const cadnn_weights *w, int n)
            tcv_fits(w, n);
 }
 
+namespace {
+
+typedef CUresult (*EncodeIm2colFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *, const int *,
+                                   const int *, cuuint32_t, cuuint32_t, const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
+                                   CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+EncodeIm2colFn encode_im2col_fn()
+{
+    static const EncodeIm2colFn fn = []() -> EncodeIm2colFn {
+        void *ptr = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeIm2col", &ptr, cudaEnableDefault, &found) == cudaSuccess && found == cudaDriverEntryPointSuccess)
+            return (EncodeIm2colFn)ptr;
+        cudaGetLastError();
+        return nullptr;
+    }();
+    return fn;
+}
+
+// Whether the copy engine can gather an int8 layer's im2col rows: each 64 values of K are 64 channels of one window position, and the
+// geometry fits the tensor map's fields (corners of 8 bits, steps of up to 8 - twice the stride with a pool - and window offsets of 8).
+// It takes the address arithmetic, the loads and the stores off the loader warps and keeps every stage of the ring in flight: a
+// stage of the gather took 700 clocks whatever its pixels.
+bool engine_takes(const cadnn_layer_desc &d)
+{
+    return d.dtype == CADNN_S8 && d.c_in % 64 == 0 && d.stride <= 4 && d.pad <= 127 && d.pad_w <= 127 && d.kh <= 128 && d.kw <= 128 && encode_im2col_fn();
+}
+
+// The input of n images as im2col rows of 64 channels, `rows` output pixels per copy (`pooled`: every second one of every second row).
+bool encode_pixels(CUtensorMap *map, const cadnn_layer_desc &d, const void *x, int n, int rows, bool pooled)
+{
+    const cuuint64_t dims[4] = {(cuuint64_t)d.c_in, (cuuint64_t)d.in_w, (cuuint64_t)d.in_h, (cuuint64_t)n};
+    const cuuint64_t strides[3] = {dims[0], dims[0] * dims[1], dims[0] * dims[1] * dims[2]};
+    // the windows' first positions: from the padding to as far before the far padding's end as the window is wide
+    const int lower[2] = {-d.pad_w, -d.pad}, upper[2] = {d.pad_w - (d.kw - 1), d.pad - (d.kh - 1)};
+    const cuuint32_t step = (cuuint32_t)((pooled ? 2 : 1) * d.stride), steps[4] = {1, step, step, 1};
+    return encode_im2col_fn()(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void *>(x), dims, strides, lower, upper, 64, (cuuint32_t)rows, steps,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace
+
 cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, const LaunchEpilogue &ep, cudaStream_t st)
 {
     const cadnn_layer_desc &d = w->desc;
@@ -1345,6 +1445,7 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     const long long in_bytes = (long long)n * d.in_h * d.in_w * d.c_in;   // (of int8)
     p.whole = (int)(in_bytes & ~3ll); p.tail = (int)(in_bytes & 3);
     p.M = (int)M; p.Rp = row_positions(d); p.nkb = stages_of(d);
+    p.odd_half = (int)((long long)d.kh * p.Rp % 128 != 0);
     p.ldc = ep.out_c_total > 0 ? ep.out_c_total : d.c_out;
     p.c_off = ep.out_c_total > 0 ? ep.out_c_off : 0;
     p.vec_ok = d.c_out % 4 == 0 && p.ldc % 4 == 0 && p.c_off % 4 == 0;
@@ -1382,10 +1483,16 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     const long long blocks = (M + p.npx - 1) / p.npx * p.n_nt * p.S;
     if (blocks > 2147483647ll) return CADNN_E_UNSUPPORTED;
     const int n_blocks = (int)blocks;
-    if (f32) return vec ? launch_shape<true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<true, false>(p, pick.ch, n_blocks, ep.pdl, st);
+    if (f32) return vec ? launch_shape<true, Gather::kPieces>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<true, Gather::kValues>(p, pick.ch, n_blocks, ep.pdl, st);
     if (run_tail)
-        return p.pooled ? launch_shape<false, false, true, true>(p, pick.ch, n_blocks, ep.pdl, st)
-                        : launch_shape<false, false, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
-    if (p.pooled) return vec ? launch_shape<false, true, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
-    return vec ? launch_shape<false, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, false>(p, pick.ch, n_blocks, ep.pdl, st);
+        return p.pooled ? launch_shape<false, Gather::kValues, true, true>(p, pick.ch, n_blocks, ep.pdl, st)
+                        : launch_shape<false, Gather::kValues, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
+    // (With a pool the copies of one stage are quarters of the tile, which have to be whole groups of 8 swizzled rows, and blocks of a
+    // cluster would share out quarters of windows.)
+    if (engine_takes(d) && !(p.pooled && (p.S > 1 || p.npx % 32)) && encode_pixels(&p.pixels, d, x, n, p.pooled ? p.npx / 4 : p.npx, p.pooled != nullptr))
+        return p.pooled ? launch_shape<false, Gather::kCopyEngine, true>(p, pick.ch, n_blocks, ep.pdl, st)
+                        : launch_shape<false, Gather::kCopyEngine>(p, pick.ch, n_blocks, ep.pdl, st);
+    if (p.pooled)
+        return vec ? launch_shape<false, Gather::kPieces, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, Gather::kValues, true>(p, pick.ch, n_blocks, ep.pdl, st);
+    return vec ? launch_shape<false, Gather::kPieces>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, Gather::kValues>(p, pick.ch, n_blocks, ep.pdl, st);
 }

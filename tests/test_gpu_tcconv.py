@@ -253,3 +253,37 @@ def test_shares_of_a_split_tile(shape, dtype, monkeypatch):
         s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None, stride, pad, 1, np.abs(scale), np.abs(bias), np.abs(r), "none")
         assert_close_or_bounded(y.cpu().numpy(), want, s_abs, int(mask.reshape(c_out, -1).sum(1).max()) + 4, shape)
     assert B.cadnn_device_status()["copy_timeouts"] == 0
+
+
+# n, h, w, c_in, c_out, kh, kw, stride, pad, pad_w
+ENGINE_LAYERS = [(3, 9, 7, 64, 80, 3, 3, 1, 1, 1), (2, 13, 10, 192, 96, 1, 7, 1, 0, 3), (2, 10, 13, 64, 130, 7, 1, 1, 3, 0), (3, 15, 12, 128, 64, 3, 3, 2, 1, 1),
+                 (5, 9, 11, 64, 64, 1, 1, 2, 0, 0), (1, 8, 8, 64, 48, 5, 5, 1, 0, 0), (2, 6, 5, 128, 70, 3, 5, 1, 2, 0), (33, 1, 1, 320, 200, 1, 1, 1, 0, 0)]
+
+
+@pytest.mark.parametrize("shape", ["128,64,1", "48,128,1", "128,128,2", "256,128,1", None])
+@pytest.mark.parametrize("layer", ENGINE_LAYERS)
+def test_int8_rows_by_the_copy_engine(layer, shape, monkeypatch):
+    """Layers of whole 64-channel rows: tiles that begin and end inside a row of the map and run over images, rectangular windows with
+    different paddings, strides, a last stage of one half, against float64 sums and against the general gather (one channel more)."""
+    from paper_1905_00571_b200 import binding as B
+    n, h, wd, c_in, c_out, kh, kw, stride, pad, pad_w = layer
+    g = gen.rng(59 + c_in + kw)
+    x, q = gen.int8_relu_activation(g, (n, h, wd, c_in)), gen.int8_weights(g, (c_out, kh, kw, c_in))
+    mask = gen.random_mask(g, q.shape, 0.2)
+    if shape:
+        monkeypatch.setenv("CADNN_TCV", shape)
+    dev = lambda a: torch.from_numpy(a).to(DEV)
+    outs = []
+    for extra in (0, 1):   # an odd number of channels takes the general gather
+        xs, qs, ms = (np.pad(a, [(0, 0)] * 3 + [(0, extra)]) for a in (x, q, mask))
+        # (whole numbers below 2^53 in double: exact; the int8 oracle has one padding for both axes)
+        want = torch.nn.functional.conv2d(torch.from_numpy(xs).double().permute(0, 3, 1, 2), torch.from_numpy(qs * ms).double().permute(0, 3, 1, 2), None,
+                                          stride, (pad, pad_w)).permute(0, 2, 3, 1).to(torch.int32).numpy()
+        wh = B.cadnn_pack_q8(B.make_desc(c_in + extra, c_out, kh, kw, stride, pad, 1, h, wd, n, "s8", pad_w=pad_w), qs, ms)
+        y = torch.full(want.shape, 5, dtype=torch.int32, device=DEV)
+        B.cadnn_conv2d(wh, dev(xs), y, out_dtype="s32")
+        torch.cuda.synchronize()
+        assert_exact(y.cpu().numpy(), want, "%s %s" % (layer, shape))
+        outs.append(y.cpu().numpy())
+    assert (outs[0] == outs[1]).all()
+    assert B.cadnn_device_status()["copy_timeouts"] == 0
