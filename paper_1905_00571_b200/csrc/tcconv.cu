@@ -185,6 +185,10 @@ __device__ __forceinline__ unsigned ld_word_if(const void *p, bool ok)
     asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\nmov.b32 %0, 0;\n@q ld.global.b32 %0, [%1];\n}\n" : "=&r"(v) : "l"(p), "r"((int)ok));
     return v;
 }
+__device__ __forceinline__ void st_word_if(float *p, float v, bool ok)
+{
+    asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %2, 0;\n@q st.global.f32 [%0], %1;\n}\n" ::"l"(p), "f"(v), "r"((int)ok) : "memory");
+}
 __device__ __forceinline__ uint4 lds128(unsigned addr)
 {
     uint4 v;
@@ -364,23 +368,38 @@ template <bool POOL> __device__ __forceinline__ int place_of(const TcvParams &p,
     return (2 * r + ((m >> 1) & 1)) * (2 * p.w_out) + 2 * (g - r * p.w_out) + (m & 1);
 }
 
-// one int8-layer output value
-__device__ __forceinline__ int finish_q(const TcvParams &p, int sum, float sc, float bi, int r)
+// act_f32 and requant_s8 without branches: with them in, a value took about 60 clocks wherever 16 stood in a row (the activation is
+// a kernel argument, so each value jumped over what it did not need).  NaN and the sign of zero come out as they do there.
+__device__ __forceinline__ float activate(float z, int act)
 {
-    return requant_s8(sum, sc, bi, p.act, p.residual != nullptr, r, p.res_scale);
+    const bool none = act == CADNN_ACT_NONE;
+    const float top = act == CADNN_ACT_RELU6 ? 6.0f : __int_as_float(0x7f800000);
+    z = (z > 0.0f) | none ? z : 0.0f;
+    return z > top ? top : z;
+}
+// one int8-layer output value, in the low byte (the rest is undefined): the sum of a value of at most 127 and 1.5 x 2^23 has it
+// there, rounded half to even
+__device__ __forceinline__ unsigned finish_q(const TcvParams &p, int sum, float sc, float bi, int r)
+{
+    float t = __fmaf_rn(__int2float_rn(sum), sc, bi);
+    const float u = __fmaf_rn(__int2float_rn(r), p.res_scale, t);
+    t = p.residual ? u : t;
+    t = (t > 0.0f) | (p.act != CADNN_ACT_RELU) ? t : 0.0f;
+    t = fminf(fmaxf(t, -127.0f), 127.0f);
+    return __float_as_uint(t + 12582912.0f);
 }
 __device__ __forceinline__ float finish_f(const TcvParams &p, unsigned sum, float sc, float bi, float r)
 {
-    return act_f32(__fmaf_rn(__uint_as_float(sum), sc, bi) + r, p.act);
+    return activate(__fmaf_rn(__uint_as_float(sum), sc, bi) + r, p.act);
 }
 __device__ __forceinline__ int byte_of(unsigned w, int j) { return (int)(signed char)((w >> (8 * j)) & 0xff); }
 
 // four of them, packed
 __device__ __forceinline__ unsigned finish_q4(const TcvParams &p, const uint4 &t, unsigned r, const float4 &sc, const float4 &bi)
 {
-    const unsigned q0 = finish_q(p, (int)t.x, sc.x, bi.x, byte_of(r, 0)) & 0xff, q1 = finish_q(p, (int)t.y, sc.y, bi.y, byte_of(r, 1)) & 0xff;
-    const unsigned q2 = finish_q(p, (int)t.z, sc.z, bi.z, byte_of(r, 2)) & 0xff, q3 = finish_q(p, (int)t.w, sc.w, bi.w, byte_of(r, 3)) & 0xff;
-    return q0 | q1 << 8 | q2 << 16 | q3 << 24;
+    const unsigned q0 = finish_q(p, (int)t.x, sc.x, bi.x, byte_of(r, 0)), q1 = finish_q(p, (int)t.y, sc.y, bi.y, byte_of(r, 1));
+    const unsigned q2 = finish_q(p, (int)t.z, sc.z, bi.z, byte_of(r, 2)), q3 = finish_q(p, (int)t.w, sc.w, bi.w, byte_of(r, 3));
+    return __byte_perm(__byte_perm(q0, q1, 0x0040), __byte_perm(q2, q3, 0x0040), 0x5410);
 }
 
 // Epilogue of 4 consecutive channels of one pixel: sums t, residual r (4 floats, or 4 int8 values in its first word), written
@@ -445,15 +464,18 @@ __device__ __forceinline__ void finish_column(const TcvParams &p, int m, int ch,
 {
     float *y = reinterpret_cast<float *>(p.y) + (size_t)m * p.ldc + p.c_off + ch;
 #pragma unroll
-    for (int i = 0; i < U; ++i)
-        if (m + i < p.M) y[(size_t)i * p.ldc] = finish_f(p, t[i], sc, bi, __uint_as_float(r[i]));
+    for (int i = 0; i < U; ++i) {
+        st_word_if(y, finish_f(p, t[i], sc, bi, __uint_as_float(r[i])), m + i < p.M);
+        y += p.ldc;
+    }
 }
 template <int U> __device__ __forceinline__ void load_column_residual(const TcvParams &p, int m, int ch, unsigned (&r)[U])
 {
+    const float *res = reinterpret_cast<const float *>(p.residual) + (size_t)m * p.c_out + ch;
 #pragma unroll
     for (int i = 0; i < U; ++i) {
-        r[i] = 0;
-        if (p.residual && m + i < p.M) r[i] = __float_as_uint(ld_act(reinterpret_cast<const float *>(p.residual) + (size_t)(m + i) * p.c_out + ch));
+        r[i] = ld_word_if(res, p.residual && m + i < p.M);
+        res += p.c_out;
     }
 }
 // Split tile whose rows are channels: a thread takes channel ch (of the tile) and every second group of U pixels of this
