@@ -69,6 +69,14 @@ struct TcvParams {
     Prefetch ahead;
 };
 
+// One lane of a converged warp.  The compiler knows that a single lane runs what stands behind it and keeps the operands of copies and
+// multiply-adds in uniform registers; behind `lane == 0` it emits a loop over the lanes around each of them.
+__device__ __forceinline__ bool elected()
+{
+    unsigned r;
+    asm volatile("{\n.reg .pred q;\nelect.sync _|q, 0xffffffff;\nselp.u32 %0, 1, 0, q;\n}\n" : "=r"(r));
+    return r != 0;
+}
 __device__ __forceinline__ void mb_init(unsigned bar, unsigned count)
 {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
@@ -745,7 +753,8 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, GATHER>::kThreads, Cfg<
                 asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n"
                              ::"l"((const char *)p.ahead.at[lane - 1] + lo), "r"((unsigned)(min(part, n - lo) & ~15ull)) : "memory");
         }
-        if (lane == 0) {
+        __syncwarp();
+        if (elected()) {
             // where the window of the tile's first pixel starts, and the position of the next 64 values of K (copy engine)
             const int at = POOL ? m0 >> 2 : m0, img = (int)fdiv((unsigned)at, p.d_hw), q = at - img * p.h_out * p.w_out;
             const int oy = (int)fdiv((unsigned)q, p.d_wo), ox = q - oy * p.w_out, step = (POOL ? 2 : 1) * p.stride;
@@ -784,7 +793,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, GATHER>::kThreads, Cfg<
                 if (++s == S) { s = 0; ++round; }
             }
         }
-    } else if (lane == 0) {
+    } else if (elected()) {
         asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
         const unsigned tmem = *slot;
         const int N = SWAP ? npx : CH;
