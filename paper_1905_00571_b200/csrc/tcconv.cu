@@ -376,7 +376,7 @@ template <bool POOL> __device__ __forceinline__ int place_of(const TcvParams &p,
     return (2 * r + ((m >> 1) & 1)) * (2 * p.w_out) + 2 * (g - r * p.w_out) + (m & 1);
 }
 
-// act_f32 and requant_s8 without branches: with them in, a value took about 60 clocks wherever 16 stood in a row (the activation is
+// act_f32 without branches: with them in, a value took about 60 clocks wherever 16 stood in a row (the activation is
 // a kernel argument, so each value jumped over what it did not need).  NaN and the sign of zero come out as they do there.
 __device__ __forceinline__ float activate(float z, int act)
 {
@@ -385,29 +385,32 @@ __device__ __forceinline__ float activate(float z, int act)
     z = (z > 0.0f) | none ? z : 0.0f;
     return z > top ? top : z;
 }
-// one int8-layer output value, in the low byte (the rest is undefined): the sum of a value of at most 127 and 1.5 x 2^23 has it
-// there, rounded half to even
-__device__ __forceinline__ unsigned finish_q(const TcvParams &p, int sum, float sc, float bi, int r)
-{
-    float t = __fmaf_rn(__int2float_rn(sum), sc, bi);
-    const float u = __fmaf_rn(__int2float_rn(r), p.res_scale, t);
-    t = p.residual ? u : t;
-    t = (t > 0.0f) | (p.act != CADNN_ACT_RELU) ? t : 0.0f;
-    t = fminf(fmaxf(t, -127.0f), 127.0f);
-    return __float_as_uint(t + 12582912.0f);
-}
 __device__ __forceinline__ float finish_f(const TcvParams &p, unsigned sum, float sc, float bi, float r)
 {
     return activate(__fmaf_rn(__uint_as_float(sum), sc, bi) + r, p.act);
 }
 __device__ __forceinline__ int byte_of(unsigned w, int j) { return (int)(signed char)((w >> (8 * j)) & 0xff); }
+// that byte of a word whose bytes had their top bits turned, as a float: 2^23 + its value + 128 by placing it in a mantissa (a
+// conversion takes four times as long)
+__device__ __forceinline__ float turned_byte(unsigned w, int j) { return __uint_as_float(__byte_perm(w, 0x4b000000u, 0x7540u + j)) - 8388736.0f; }
 
-// four of them, packed
+// Four int8-layer output values, packed: requant_s8 with the activation's lower bound and the clamp's in one (NaN comes out as that
+// bound there too), and rounded by an addition: a value of at most 127 plus 1.5 x 2^23 has it in the low byte, half to even.  The
+// epilogue's instructions bound int8 layers of few stages: 18 a value before, 9 (6 without a residual).
 __device__ __forceinline__ unsigned finish_q4(const TcvParams &p, const uint4 &t, unsigned r, const float4 &sc, const float4 &bi)
 {
-    const unsigned q0 = finish_q(p, (int)t.x, sc.x, bi.x, byte_of(r, 0)), q1 = finish_q(p, (int)t.y, sc.y, bi.y, byte_of(r, 1));
-    const unsigned q2 = finish_q(p, (int)t.z, sc.z, bi.z, byte_of(r, 2)), q3 = finish_q(p, (int)t.w, sc.w, bi.w, byte_of(r, 3));
-    return __byte_perm(__byte_perm(q0, q1, 0x0040), __byte_perm(q2, q3, 0x0040), 0x5410);
+    float v[4] = {__fmaf_rn(__int2float_rn((int)t.x), sc.x, bi.x), __fmaf_rn(__int2float_rn((int)t.y), sc.y, bi.y),
+                  __fmaf_rn(__int2float_rn((int)t.z), sc.z, bi.z), __fmaf_rn(__int2float_rn((int)t.w), sc.w, bi.w)};
+    if (p.residual) {
+        r ^= 0x80808080u;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = __fmaf_rn(turned_byte(r, j), p.res_scale, v[j]);
+    }
+    const float least = p.act == CADNN_ACT_RELU ? 0.0f : -127.0f;
+    unsigned q[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) q[j] = __float_as_uint(fminf(fmaxf(v[j], least), 127.0f) + 12582912.0f);
+    return __byte_perm(__byte_perm(q[0], q[1], 0x0040), __byte_perm(q[2], q[3], 0x0040), 0x5410);
 }
 
 // Epilogue of 4 consecutive channels of one pixel: sums t, residual r (4 floats, or 4 int8 values in its first word), written
