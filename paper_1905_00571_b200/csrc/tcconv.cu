@@ -1078,11 +1078,11 @@ constexpr SmemPlan plan_smem(bool f32, const Pick &k, int nkb, bool res_tile)
 {
     const int PX = tile_pixels(k);
     const bool swap = k.ch == 128;
-    const int stage = (f32 ? 3 : 2) * 64 * (k.px + k.ch), out = k.px * (k.ch + 4) * 4;
+    const int stage = (f32 ? 3 : 2) * 64 * (k.px + k.ch), out = k.px * (k.ch + (f32 && swap ? 0 : 4)) * 4;
     const int res = res_tile ? k.px / k.split * k.ch : 0;
     const int budget = (PX > 128 ? 216 : 108) * 1024 - res;   // two blocks share a multiprocessor but for the largest shape
     SmemPlan s = {};
-    s.stages = std::max(2, std::min(std::min(4, std::max(2, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
+    s.stages = std::max(2, std::min(std::min(f32 ? 4 : 6, std::max(2, ceil_div(nkb, k.split))), (budget - (k.split > 1 ? out : 0)) / stage));
     // sums staged over the stages: int8 tiles, and unsplit float tiles whose rows are pixels
     s.recv_off = std::max(s.stages * stage, !f32 || (!swap && k.split == 1) ? out : 0);
     s.bar_off = (s.recv_off + (k.split > 1 ? out : 0) + 127) / 128 * 128;
