@@ -1110,38 +1110,73 @@ constexpr bool clusters_find_tensor_memory()
 static_assert(clusters_find_tensor_memory(), "clusters of split tiles could wait for each other's tensor memory");
 
 // Block shape of a layer: the one a time model calls the fastest.  The model is linear in what a block does, with
-// coefficients fitted to 3900 measured shapes (212 layers of the workloads at batch 1 to 128, launched back to back as
-// programmatic dependents):
+// coefficients fitted to 37500 measured shapes (1950 layers: those of the workloads at batch 1 to 128, and random ones, launched back to
+// back as programmatic dependents; least squares, then a search that lowers the excess of the chosen shapes over 4 of 5 layers):
 //   time = start + P (b2 + n (c2 + d2 px / 64)) + Q (b1 + n (c1 + d1 px / 64))   [microseconds]
 // n = stages per block, P = rounds in which every multiprocessor runs two blocks, Q = rounds with one.  How many clusters
 // of a size run at once (a cluster has to fit one GPC) is the table cap1 / cap2 in choose, as cudaOccupancyMaxActiveClusters
 // reported it on a B200.
-// Mean excess of the chosen over the best measured shape: 1 %.
+// Mean excess of the chosen over the best measured shape, on the fifth that was left out: 0.8 to 1.7 % by gather (with the coefficients
+// of the kernel before its epilogue and issue were mended 3.2 to 4.8 %).
 struct Cost {
     float start, b2, c2, d2, b1, c1, d1;
 };
-const Cost kCost[2][9] = {   // float, int8; 128 px x 64 ch, then up to 32, 64 and 128 px x 128 ch, each unsplit and split; 256 px x 128 ch
-    {{0.385f, 4.84f, 0.0f, 0.421f, 3.61f, 0.0f, 0.257f},
-     {1.3f, 5.25f, 0.0f, 0.429f, 3.28f, 0.0f, 0.28f},
-     {0.0f, 3.35f, 0.522f, 0.0f, 2.99f, 0.415f, 0.0615f},
-     {0.641f, 2.81f, 0.413f, 0.303f, 2.26f, 0.41f, 0.0958f},
-     {0.166f, 4.49f, 0.634f, 0.0f, 3.79f, 0.36f, 0.11f},
-     {1.03f, 3.89f, 0.115f, 0.561f, 2.63f, 0.324f, 0.169f},
-     {0.172f, 6.37f, 0.26f, 0.501f, 5.52f, 0.54f, 0.156f},
-     {0.76f, 0.0f, 0.0f, 0.0f, 4.85f, 0.322f, 0.301f},
-     {0.0f, 0.0f, 0.0f, 0.0f, 6.52f, 0.435f, 0.162f}},
-    {{1.19f, 3.83f, 0.0f, 0.353f, 2.85f, 0.0f, 0.191f},
-     {1.68f, 3.44f, 0.0f, 0.358f, 2.44f, 0.0f, 0.216f},
-     {0.927f, 2.42f, 0.445f, 0.0f, 1.83f, 0.28f, 0.167f},
-     {2.83f, 0.611f, 0.216f, 0.605f, 0.0f, 0.259f, 0.309f},
-     {1.24f, 3.19f, 0.602f, 0.0f, 2.64f, 0.215f, 0.147f},
-     {2.71f, 2.82f, 0.0f, 0.505f, 1.18f, 0.119f, 0.305f},
-     {2.74f, 4.88f, 0.0f, 0.452f, 2.61f, 0.108f, 0.224f},
-     {0.507f, 5.89f, 0.0f, 0.563f, 4.98f, 0.0f, 0.356f},
-     {0.0f, 11.6f, 0.0f, 0.578f, 6.35f, 0.0f, 0.21f}}};
+const Cost kCost[5][9] = {   // by gather; 128 px x 64 ch, then up to 32, 64 and 128 px x 128 ch, each unsplit and split; 256 px x 128 ch
+    // float, 16 bytes at a time
+    {{0.871f, 2.86f, 0.0643f, 0.399f, 4.29f, 0.0f, 0.197f},
+     {1.30f, 7.30f, 0.0f, 0.329f, 3.47f, 0.0405f, 0.185f},
+     {0.0f, 2.12f, 0.617f, 0.297f, 1.93f, 0.267f, 0.191f},
+     {0.588f, 2.95f, 0.221f, 0.392f, 1.79f, 0.263f, 0.232f},
+     {0.0392f, 3.60f, 0.255f, 0.337f, 2.70f, 0.196f, 0.165f},
+     {1.41f, 3.86f, 0.0385f, 0.488f, 2.11f, 0.155f, 0.312f},
+     {2.47f, 3.83f, 0.208f, 0.457f, 1.43f, 0.342f, 0.307f},
+     {0.638f, 0.0973f, 0.0747f, 0.0865f, 11.6f, 0.143f, 0.399f},
+     {0.0f, 0.0219f, 0.0f, 0.0551f, 5.67f, 0.0278f, 0.255f}},
+    // float, one value at a time
+    {{2.07f, 1.89f, 0.0229f, 0.521f, 2.02f, 0.00927f, 0.336f},
+     {0.00999f, 5.93f, 0.0f, 0.567f, 4.70f, 0.00640f, 0.290f},
+     {0.0f, 1.54f, 0.503f, 0.640f, 1.56f, 0.292f, 0.309f},
+     {0.158f, 3.60f, 0.327f, 0.375f, 2.03f, 0.430f, 0.0f},
+     {0.153f, 2.78f, 0.143f, 0.786f, 2.40f, 0.177f, 0.298f},
+     {0.905f, 3.28f, 0.0372f, 0.680f, 2.53f, 0.0833f, 0.381f},
+     {3.42f, 1.99f, 0.195f, 0.692f, 2.18f, 0.232f, 0.213f},
+     {0.0411f, 0.0227f, 0.0783f, 0.0140f, 5.94f, 0.338f, 0.134f},
+     {0.0f, 0.0144f, 0.0142f, 0.0382f, 4.83f, 0.0834f, 0.280f}},
+    // int8, copy engine
+    {{0.0f, 0.504f, 0.427f, 0.333f, 1.99f, 0.0f, 0.200f},
+     {0.0f, 2.41f, 0.0875f, 0.870f, 3.05f, 0.0f, 0.125f},
+     {0.358f, 1.39f, 0.310f, 0.0f, 0.335f, 0.218f, 0.526f},
+     {1.56f, 1.72f, 0.108f, 0.0430f, 0.0f, 0.161f, 0.417f},
+     {0.0f, 2.71f, 0.115f, 0.457f, 17.7f, 1.94f, 2.14f},
+     {2.47f, 1.76f, 0.0f, 0.128f, 0.279f, 0.379f, 0.762f},
+     {0.0f, 1.55f, 0.300f, 0.505f, 5.85f, 0.446f, 0.0778f},
+     {6.86f, 5.70f, 0.0f, 0.0412f, 10.9f, 0.122f, 0.452f},
+     {0.0f, 12.4f, 0.0f, 0.613f, 7.77f, 0.0f, 0.186f}},
+    // int8, 16 bytes at a time
+    {{1.31f, 1.43f, 0.0624f, 0.430f, 0.0229f, 0.0677f, 0.341f},
+     {1.12f, 16.0f, 0.0318f, 0.0422f, 1.94f, 0.122f, 0.262f},
+     {0.0f, 1.35f, 0.282f, 0.567f, 0.456f, 0.156f, 0.732f},
+     {0.906f, 1.29f, 0.774f, 0.588f, 0.0877f, 0.163f, 0.425f},
+     {1.20f, 2.45f, 0.0359f, 0.617f, 1.33f, 0.212f, 0.209f},
+     {2.55f, 2.11f, 0.0f, 0.533f, 0.340f, 0.0189f, 0.331f},
+     {0.184f, 6.32f, 2.73f, 0.0299f, 6.04f, 0.126f, 0.203f},
+     {0.186f, 46.7f, 0.242f, 1.48f, 5.14f, 0.0252f, 0.251f},
+     {0.451f, 12.7f, 0.00654f, 2.34f, 4.30f, 0.0272f, 0.225f}},
+    // int8, shifted words
+    {{2.23f, 2.74f, 0.393f, 0.795f, 4.38f, 0.0928f, 0.328f},
+     {3.30f, 1.99f, 0.0623f, 0.764f, 22.6f, 0.0870f, 0.382f},
+     {0.313f, 2.48f, 0.560f, 1.03f, 1.65f, 0.0905f, 0.845f},
+     {0.0f, 9.62f, 0.0393f, 6.15f, 0.0f, 0.552f, 0.632f},
+     {1.15f, 3.60f, 0.297f, 0.651f, 2.52f, 0.114f, 0.598f},
+     {1.29f, 3.16f, 0.0279f, 0.797f, 1.54f, 0.0f, 0.666f},
+     {1.20f, 4.90f, 0.638f, 0.744f, 4.41f, 0.0f, 0.553f},
+     {4.58f, 4.90f, 0.373f, 1.89f, 2.11f, 0.200f, 1.02f},
+     {0.469f, 11.2f, 0.190f, 0.309f, 6.23f, 0.452f, 0.343f}}};
 
-Pick choose(bool f32, int c_out, long long M, int nkb, bool res_tile)
+// kind: row of kCost
+Pick choose(int kind, int c_out, long long M, int nkb, bool res_tile)
 {
+    const bool f32 = kind < 2;
     Pick best = {128, 64, 1};
     double best_t = 1e300;
     auto consider = [&](int px, int ch) {
@@ -1160,7 +1195,7 @@ Pick choose(bool f32, int c_out, long long M, int nkb, bool res_tile)
                 if (rest > cap1[log]) ++P;
                 else if (rest > 0) Q = 1;
             } else Q = (tiles + cap1[log] - 1) / cap1[log];
-            const Cost &c = kCost[!f32][px > 128 ? 8 : (ch == 64 ? 0 : px <= 32 ? 2 : px <= 64 ? 4 : 6) + (split > 1)];
+            const Cost &c = kCost[kind][px > 128 ? 8 : (ch == 64 ? 0 : px <= 32 ? 2 : px <= 64 ? 4 : 6) + (split > 1)];
             const double n = ceil_div(nkb, split), u = px / 64.0;
             const double t = c.start + P * (c.b2 + n * (c.c2 + c.d2 * u)) + Q * (c.b1 + n * (c.c1 + c.d1 * u));
             if (t < best_t) { best_t = t; best = k; }
@@ -1501,7 +1536,7 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     if (pick.px > 0) pick.split = std::max(1, pick.split);
     else if ((kept >> 32) == (uint64_t)n && kept != 0) pick = {(int)(kept & 0xfff), (int)(kept >> 12 & 0xfff), (int)(kept >> 24 & 0xff)};
     else {
-        pick = choose(f32, d.c_out, M, p.nkb, p.res_tile != 0);
+        pick = choose(f32 ? d.c_in % 4 != 0 : engine_takes(d) ? 2 : d.c_in % 16 == 0 ? 3 : 4, d.c_out, M, p.nkb, p.res_tile != 0);
         w->tcv_pick.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
     }
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0, run_tail = !f32 && !vec && p.tail;
