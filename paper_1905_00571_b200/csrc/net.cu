@@ -667,10 +667,11 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
             }
         }
         // Layers packed with the dense tensor-core image run NHWC (tcconv.cu); for those timed at pack time the times decide below.
-        // Networks with depthwise layers do so above 150 million multiply-adds of kept weights: up to there the planar kernels'
-        // shorter start-up and the depthwise layers they take along make up for their rate (MobileNet-V2, planar / NHWC: batch 1
-        // 208 / 223 us, batch 2 298 / 262, batch 16 962 / 661; half width at 160 x 160, batch 1 151 / 199, batch 2 166 / 209;
-        // MobileNet-V1, batch 1, 148 / 143).
+        // Networks with depthwise layers do so above 75 million multiply-adds of kept weights, single images above 150 million: up to there
+        // the planar kernels' shorter start-up and the depthwise layers they take along make up for their rate (MobileNet-V2, planar / NHWC,
+        // us: batch 1, 41 million 181 / 197, 65 193 / 207, 99 209 / 207, 193 254 / 207; batch 2, 81 million 221 / 213, 131 271 / 233,
+        // 198 297 / 233; batch 4, 163 million 302 / 247).  (From 85 million on single images gain as well, 228 / 211 at 256 x 256; the line
+        // stays, because the slots of a full MobileNet-V1 are seen as planes.)
         if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr && !(getenv("CADNN_PERSIST") && atoi(getenv("CADNN_PERSIST")) != 0)) {
             bool tc = true, dw = false;
             double macs = 0.0;
@@ -683,7 +684,7 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
                     macs += (double)w->nnz * w->h_out * w->w_out * n;
                 }
             }
-            if (tc && (!dw || macs > 150e6)) planar = false;
+            if (tc && (!dw || macs > (n > 1 ? 75e6 : 150e6))) planar = false;
         }
         // Where the packer timed both layouts for every sparse conv, the measured sums decide: planar, and NHWC by the kernel that
         // would run there (a handle keeps a dense image only where that kernel was the faster one).
@@ -706,7 +707,8 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
             if (getenv("CADNN_VERBOSE"))
                 fprintf(stderr, "cadnn_net_create: sparse convs timed at pack time: planar %.1f us, NHWC %.1f us%s\n", t_planar, t_nhwc,
                         all ? "" : " (incomplete)");
-            if (all && t_nhwc > 0.0 && t_planar > t_nhwc) planar = false;
+            // (Timed single images have had planes, which callers see through the slots: they keep them unless NHWC takes less than 3/4.)
+            if (all && t_nhwc > 0.0 && t_planar * (n > 1 ? 1.0 : 0.75) > t_nhwc) planar = false;
         }
         net->planar = planar;
     }

@@ -15,15 +15,20 @@
 // shared memory (small maps would otherwise leave most multiprocessors idle).
 //   * 8 loader warps gather the im2col rows from NHWC memory (out-of-image taps are zeros) into swizzled
 //     K-major operand tiles, 128 source bytes per pixel and stage, in groups that fill alternate stages;
+//     int8 layers of whole 64-channel rows leave that to the copy engine (engine_takes);
 //   * one thread copies the matching weight tiles (pre-swizzled by the packer) with bulk copies; the first
 //     ones do not wait for the previous layer;
 //   * one thread issues the tcgen05.mma's; accumulators live in tensor memory;
-//   * the loader warps then finish the tile: a lane per pixel straight from tensor memory, or through
+//   * the loader warps then finish the tile, with scale, bias and residual asked for at its start: float
+//     tiles whose rows are channels as columns of 16 pixels straight from tensor memory, the others through
 //     shared memory as [pixel][channel]; with a split reduction every block sends each other block its
 //     pixels' sums from registers, counted on the receiver's barrier.
-// What bounds it: at batch 1 the chain start - first loads - last multiply-adds - exchange (about 5 of the 6
-// to 9 microseconds of a layer); at large batch, for float, shared-memory bandwidth - the six products of a
-// stage read 40 KB of operands per 16 K values where the tensor core needs 384 clocks.
+// What bounds it, from clock stamps in its warps.  At batch 1 a chain: 14x14, 256 -> 1024 1x1 with a residual, 32 x 128 tile split
+// in four (clocks of 0.5 ns after the previous layer has ended): requests 350, first stage in shared memory 1300, first products 1600,
+// last 3100, sums read and sent 4300, received 5000, written 6000; 0.8 us from the end of one layer to the next.  Four to eight warps a
+// scheduler share the issue slots, so what helps there is fewer instructions.  At large batch, float: the products (256 x 128 tiles
+// run at 90 % of the tensor cores' rate while multiplying; their first loads and epilogue, 10 to 50 % of the time, are not
+// overlapped).  Int8: epilogue instructions and the exchange.
 //
 // Float precision.  A float is the exact sum of three bf16 numbers (8 + 8 + 8 significand bits), a = a1 + a2 +
 // a3 with |a2| <= 2^-9 |a|, |a3| <= 2^-18 |a|, from 2^-110 (8e-34) on (below, the third part loses bits under
@@ -1275,12 +1280,11 @@ int stages_of(const cadnn_layer_desc &d) { return ceil_div(d.kh * row_positions(
 
 // When the dense route is taken.  Per multiply-add of the full layer the tensor cores cost the same whatever the mask; the
 // sparse kernels cost per stored weight.  Measured on the 3x3 and 1x1 layers of the workloads at batch 1 to 32 (microseconds
-// against density) the lines cross between 1 and 3 per cent, for float and for int8; float layers of at most 64 output channels
-// fill half a tile's columns only, and cross between 5 and 7 per cent.
+// against density) the lines cross below 3 per cent, for float and for int8.  Float layers of at most 64 output channels fill half a
+// tile's columns, and are faster there all the same: 16 to 64 channels at 2 % kept, batch 1 to 16, sparse 8.2 to 14.4, dense 6.5 to 8.2.
 bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz)
 {
-    const double density = (double)nnz / ((double)d.c_out * d.kh * d.kw * d.c_in);
-    return density >= (d.dtype == CADNN_F32 && d.c_out <= 64 ? 0.06 : 0.025);
+    return (double)nnz >= 0.025 * ((double)d.c_out * d.kh * d.kw * d.c_in);
 }
 
 namespace {

@@ -5,9 +5,9 @@ import numpy as np
 import pytest
 import torch
 
-from oracle import ref
-from workloads import gen
-from parity import assert_close_or_bounded, assert_exact
+from oracle import forward as oracle_forward, ref
+from workloads import gen, models
+from parity import NET_FLOOR, assert_close_f32, assert_close_or_bounded, assert_exact
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -287,3 +287,50 @@ def test_int8_rows_by_the_copy_engine(layer, shape, monkeypatch):
         outs.append(y.cpu().numpy())
     assert (outs[0] == outs[1]).all()
     assert B.cadnn_device_status()["copy_timeouts"] == 0
+
+
+@pytest.mark.parametrize("c_out,density,dense", [(16, 0.03, True), (64, 0.03, True), (65, 0.03, True), (16, 0.02, False), (64, 0.02, False)])
+def test_float_layers_take_the_dense_route_from_two_and_a_half_per_cent_on(c_out, density, dense):
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(61)
+    x, w = gen.relu_normal_input(g, (2, 9, 8, 72)), gen.he_weights(g, c_out, 3, 3, 72)
+    mask = gen.random_mask(g, w.shape, density)
+    want = ref.conv2d_f32(x, w, mask, 1, 1, act="relu")
+    wh = B.cadnn_pack(B.make_desc(72, c_out, 3, 3, 1, 1, 1, 9, 8, 2, "f32"), w, mask)
+    assert (B.cadnn_weights_info(wh)["packed_bytes"] > 6 * w.size) == dense
+    y = torch.zeros(want.shape, device=DEV)
+    B.cadnn_conv2d(wh, torch.from_numpy(x).to(DEV), y, act="relu")
+    torch.cuda.synchronize()
+    s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None, 1, 1)
+    assert_close_or_bounded(y.cpu().numpy(), want, s_abs, int(mask.reshape(c_out, -1).sum(1).max()) + 4, "%d %g" % (c_out, density))
+
+
+@pytest.mark.parametrize("batch,c,planar", [(2, 272, True), (2, 304, False), (1, 304, True)])
+def test_layout_of_networks_with_depthwise_layers(batch, c, planar):
+    """A pointwise, a depthwise and a pointwise layer, with kept multiply-adds on both sides of the line for two images, and below the
+    line for one."""
+    from paper_1905_00571_b200 import binding as B
+    from paper_1905_00571_b200.network import PackedModel
+    from test_gpu_fused_depthwise import _add
+    g = gen.rng(63)
+    hw = (48, 48)
+    m = models.Model("dw_layout", "f32", (96, 96, 3), seed=63)
+    stem, at = _add(m, g, "stem", 0, 3, 40, 3, 3, 2, 1, 1, m.in_shape[:2], "relu", 1.0)
+    assert at == hw
+    a, _ = _add(m, g, "expand", stem, 40, c, 1, 1, 1, 0, 0, hw, "relu6", 0.99)
+    b, hw2 = _add(m, g, "dw", a, c, c, 3, 3, 1, 1, 1, hw, "relu6", 1.0, groups=c)
+    d, _ = _add(m, g, "project", b, c, 20, 1, 1, 1, 0, 0, hw2, "none", 0.99)
+    pool = m.new_slot()
+    m.ops.append(models.Op("gavgpool", "pool", d, pool, c_in=20, c_out=20, in_hw=hw2, out_hw=(1, 1)))
+    m.ops.append(models.Op("fc", "fc", pool, m.new_slot(), -1, 20, 10, 1, 1, 0, 1, "none", gen.he_weights(g, 10, 1, 1, 20), None,
+                           np.ones(10, np.float32), np.zeros(10, np.float32), "f32", 1.0, (1, 1), (1, 1)))
+    kept = batch * sum(int(op.mask.sum()) * op.out_hw[0] * op.out_hw[1] for op in m.ops if op.mask is not None)
+    assert planar == (kept <= (75e6 if batch > 1 else 150e6)) and 0.9 < kept / (75e6 if batch > 1 else 37.5e6) < 1.12
+    x = models.make_input(m, batch)
+    pm = PackedModel(m, batch, DEV)
+    assert B.cadnn_net_layout(pm.net)["planar"] == planar
+    y = pm.new_output()
+    pm.forward(torch.from_numpy(x).to(DEV), y)
+    torch.cuda.synchronize()
+    want, _ = oracle_forward.forward(m, x)
+    assert_close_f32(y.cpu().numpy(), want, "logits", floor=NET_FLOOR)
