@@ -278,7 +278,7 @@ template <bool F32, int PX, int CH, bool SWAP, Gather GATHER> struct Cfg {
     static const int kCols = tensor_columns(F32, kN);
     // Blocks per multiprocessor the registers are cut for (more than tensor memory holds would wait in tcgen05.alloc).  Int8 tiles
     // of 128 columns and layers with few stages are small enough for three (int8 ResNet-50, batch 32: 963 us with 62 to 78
-    // registers and one residual row ahead, 923 us with 64 and two; four rows 947, eight 998).
+    // registers, 923 us with 64).
     static const int kBlocks = PX > 128 ? 1 : F32 || GATHER == Gather::kValues || 3 * kCols > kTensorColumns ? 2 : 3;
     static_assert(kBlocks * kCols <= kTensorColumns, "a block would wait for tensor memory that its neighbours hold");
     static const int kRow = CH + 4;                        // words per pixel of the exchanged sums (conflict-free 16-byte access)

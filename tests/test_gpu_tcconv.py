@@ -334,3 +334,43 @@ def test_layout_of_networks_with_depthwise_layers(batch, c, planar):
     torch.cuda.synchronize()
     want, _ = oracle_forward.forward(m, x)
     assert_close_f32(y.cpu().numpy(), want, "logits", floor=NET_FLOOR)
+
+
+@pytest.mark.parametrize("shape", ["128,64,1", "32,128,1", "64,128,2"])
+@pytest.mark.parametrize("act", ["none", "relu", "relu6"])
+def test_float_epilogue_of_nan_infinities_and_zeros(act, shape, monkeypatch):
+    """The activation as act_f32 defines it (z > 0 ? z : 0, then at most 6), whatever joins through the residual."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(67)
+    w = gen.he_weights(g, 72, 1, 1, 64)
+    monkeypatch.setenv("CADNN_TCV", shape)
+    wh = B.cadnn_pack(B.make_desc(64, 72, 1, 1, 1, 0, 1, 5, 7, 1, "f32"), w, gen.random_mask(g, w.shape, 0.2))
+    r = np.resize(np.array([np.nan, np.inf, -np.inf, -0.0, 0.0, 3.0, -3.0, 7.0, 6.0, 1e-40], np.float32), (1, 5, 7, 72))
+    y = torch.full(r.shape, 9.0, device=DEV)
+    B.cadnn_conv2d(wh, torch.zeros((1, 5, 7, 64), device=DEV), y, residual=torch.from_numpy(r).to(DEV), act=act)
+    torch.cuda.synchronize()
+    want = r + np.float32(0.0)
+    if act != "none":
+        want = np.where(want > 0, want, np.float32(0.0))
+    if act == "relu6":
+        want = np.minimum(want, np.float32(6.0))
+    assert np.array_equal(y.cpu().numpy(), want, equal_nan=True)
+
+
+@pytest.mark.parametrize("act", ["none", "relu"])
+def test_int8_epilogue_of_nan_infinities_and_ties(act):
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(69)
+    b = np.resize(np.array([np.nan, np.inf, -np.inf, 0.5, 1.5, -0.5, -2.5, 126.5, 127.5, -126.5, -200.0, 1e30], np.float32), 96)
+    q = gen.int8_weights(g, (96, 1, 1, 64))
+    wh = B.cadnn_pack_q8(B.make_desc(64, 96, 1, 1, 1, 0, 1, 5, 7, 1, "s8"), q, gen.random_mask(g, q.shape, 0.2))
+    r = gen.int8_weights(g, (1, 5, 7, 96))
+    for res in (None, r):
+        y = torch.full(r.shape, 9, dtype=torch.int8, device=DEV)
+        B.cadnn_conv2d(wh, torch.zeros((1, 5, 7, 64), dtype=torch.int8, device=DEV), y, torch.ones(96, device=DEV), torch.from_numpy(b).to(DEV),
+                       None if res is None else torch.from_numpy(res).to(DEV), act, out_dtype="s8", residual_scale=1.0)
+        torch.cuda.synchronize()
+        t = np.broadcast_to(b, r.shape) if res is None else (b + res.astype(np.float32))   # (sums of halves: exact, or beyond the clamp)
+        t = np.where(t > 0, t, np.float32(0.0)) if act == "relu" else t
+        want = np.rint(np.fmin(np.fmax(t, np.float32(-127.0)), np.float32(127.0))).astype(np.int8)
+        assert (y.cpu().numpy() == want).all()
