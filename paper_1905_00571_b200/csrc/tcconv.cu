@@ -50,7 +50,6 @@ namespace {
 const int kSpin = 1 << 22;
 
 struct TcvParams {
-    CUtensorMap pixels;              // Gather::kCopyEngine: the input as im2col rows
     const void *x;
     void *y;
     const unsigned char *wimg;
@@ -263,6 +262,14 @@ constexpr int tensor_columns(bool f32, int n)
 // How the activations come into shared memory: values one by one or as shifted words (pixels of any number of channels), 16 bytes at a
 // time (whole 16-byte pieces of channels), or by the copy engine (int8, whole 64-channel rows).
 enum class Gather { kValues, kPieces, kCopyEngine };
+
+// Only the copy engine's kernels carry a tensor map among their parameters: with it in all of them a launch took the host 0.55 us longer
+// (small layers called one by one: 4.5 us a call against 4.0).
+struct TcvEngineParams : TcvParams {
+    CUtensorMap pixels;   // the input as im2col rows
+};
+template <Gather GATHER> struct ParamsOf { typedef TcvParams type; };
+template <> struct ParamsOf<Gather::kCopyEngine> { typedef TcvEngineParams type; };
 
 // One kernel shape: PX pixels x CH channels per block.  SWAP: the channels are the 128 rows of the tensor-core tile and
 // the pixels its columns (any multiple of 16 up to PX, so that small maps waste little); otherwise the 128 rows are pixels
@@ -569,7 +576,7 @@ __device__ __forceinline__ void send_columns(const TcvParams &p, unsigned at, un
 // (POOL and TAIL are instantiations of their own: as branches at run time they cost the int8 ResNet-50, which has neither such a pool
 // nor such a tensor, 0.7 and 0.4 %.)
 template <bool F32, int PX, int CH, bool SWAP, Gather GATHER, bool POOL, bool TAIL>
-__global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, GATHER>::kThreads, Cfg<F32, PX, CH, SWAP, GATHER>::kBlocks) tcconv_kernel(const __grid_constant__ TcvParams p)
+__global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, GATHER>::kThreads, Cfg<F32, PX, CH, SWAP, GATHER>::kBlocks) tcconv_kernel(const __grid_constant__ typename ParamsOf<GATHER>::type p)
 {
     const bool VEC = GATHER == Gather::kPieces, ENGINE = GATHER == Gather::kCopyEngine;
     typedef Cfg<F32, PX, CH, SWAP, GATHER> C;
@@ -770,6 +777,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, GATHER>::kThreads, Cfg<
             int ky = (int)fdiv((unsigned)(kb0 * C::kKB), p.d_Rp), ci = kb0 * C::kKB - ky * p.Rp, kx = (int)fdiv((unsigned)ci, p.d_ci);
             ci -= kx * p.c_in;
             auto pixels = [&](int s) {
+                if constexpr (GATHER == Gather::kCopyEngine) {
 #pragma unroll
                 for (int t = 0; t < 2; ++t) {
                     if (ky == p.kh) break;
@@ -784,6 +792,7 @@ __global__ void __launch_bounds__(Cfg<F32, PX, CH, SWAP, GATHER>::kThreads, Cfg<
                         ci = 0;
                         if (++kx == p.kw) { kx = 0; ++ky; }
                     }
+                }
                 }
             };
             const int ahead = ENGINE ? min(S, kb1 - kb0) : 0;
@@ -1221,7 +1230,7 @@ Pick choose(int kind, int c_out, long long M, int nkb, bool res_tile)
 }
 
 template <bool F32, int PX, int CH, bool SWAP, Gather GATHER, bool POOL, bool TAIL>
-cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
+cadnn_status launch_one(typename ParamsOf<GATHER>::type p, int blocks, bool pdl, cudaStream_t st)
 {
     auto kern = tcconv_kernel<F32, PX, CH, SWAP, GATHER, POOL, TAIL>;
     typedef Cfg<F32, PX, CH, SWAP, GATHER> C;
@@ -1258,7 +1267,7 @@ cadnn_status launch_one(TcvParams p, int blocks, bool pdl, cudaStream_t st)
     return CADNN_OK;
 }
 
-template <bool F32, Gather GATHER, bool POOL = false, bool TAIL = false> cadnn_status launch_shape(const TcvParams &p, int ch, int blocks, bool pdl, cudaStream_t st)
+template <bool F32, Gather GATHER, bool POOL = false, bool TAIL = false> cadnn_status launch_shape(const typename ParamsOf<GATHER>::type &p, int ch, int blocks, bool pdl, cudaStream_t st)
 {
     if (ch == 64) return launch_one<F32, 128, 64, false, GATHER, POOL, TAIL>(p, blocks, pdl, st);
     if (p.npx <= 64) return launch_one<F32, 64, 128, true, GATHER, POOL, TAIL>(p, blocks, pdl, st);
@@ -1565,9 +1574,13 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
                         : launch_shape<false, Gather::kValues, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
     // (With a pool the copies of one stage are quarters of the tile, which have to be whole groups of 8 swizzled rows, and blocks of a
     // cluster would share out quarters of windows.)
-    if (engine_takes(d) && !(p.pooled && (p.S > 1 || p.npx % 32)) && encode_pixels(&p.pixels, d, x, n, p.pooled ? p.npx / 4 : p.npx, p.pooled != nullptr))
-        return p.pooled ? launch_shape<false, Gather::kCopyEngine, true>(p, pick.ch, n_blocks, ep.pdl, st)
-                        : launch_shape<false, Gather::kCopyEngine>(p, pick.ch, n_blocks, ep.pdl, st);
+    if (engine_takes(d) && !(p.pooled && (p.S > 1 || p.npx % 32))) {
+        TcvEngineParams e;
+        static_cast<TcvParams &>(e) = p;
+        if (encode_pixels(&e.pixels, d, x, n, p.pooled ? p.npx / 4 : p.npx, p.pooled != nullptr))
+            return p.pooled ? launch_shape<false, Gather::kCopyEngine, true>(e, pick.ch, n_blocks, ep.pdl, st)
+                            : launch_shape<false, Gather::kCopyEngine>(e, pick.ch, n_blocks, ep.pdl, st);
+    }
     if (p.pooled)
         return vec ? launch_shape<false, Gather::kPieces, true>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, Gather::kValues, true>(p, pick.ch, n_blocks, ep.pdl, st);
     return vec ? launch_shape<false, Gather::kPieces>(p, pick.ch, n_blocks, ep.pdl, st) : launch_shape<false, Gather::kValues>(p, pick.ch, n_blocks, ep.pdl, st);
