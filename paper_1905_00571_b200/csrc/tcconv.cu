@@ -1289,11 +1289,14 @@ int stages_of(const cadnn_layer_desc &d) { return ceil_div(d.kh * row_positions(
 
 // When the dense route is taken.  Per multiply-add of the full layer the tensor cores cost the same whatever the mask; the
 // sparse kernels cost per stored weight.  Measured on the 3x3 and 1x1 layers of the workloads at batch 1 to 32 (microseconds
-// against density) the lines cross below 3 per cent, for float and for int8.  Float layers of at most 64 output channels fill half a
-// tile's columns, and are faster there all the same: 16 to 64 channels at 2 % kept, batch 1 to 16, sparse 8.2 to 14.4, dense 6.5 to 8.2.
+// against density) the lines cross below 3 per cent, for float and for int8.  Float layers of at most 64 output channels keep the sparse
+// kernels' 32-bit multiply-adds up to 6 per cent: the split products would be faster from 2 on (16 to 64 channels, batch 1 to 16, 6.5 to
+// 8.2 against 8.2 to 14.4), but with so few terms a sum they are not everywhere as close to 64 bits (2-norm errors at 2.5 to 5.5 per cent, dense
+// over sparse: 28 x 28 maps 0.55 to 1.00, 14 x 14 maps 0.70 to 1.09; activations of 1e-35, 4 per cent: 2.4e-6 against 6.3e-8).
 bool tcv_pays(const cadnn_layer_desc &d, int64_t nnz)
 {
-    return (double)nnz >= 0.025 * ((double)d.c_out * d.kh * d.kw * d.c_in);
+    const double density = (double)nnz / ((double)d.c_out * d.kh * d.kw * d.c_in);
+    return density >= (d.dtype == CADNN_F32 && d.c_out <= 64 ? 0.06 : 0.025);
 }
 
 namespace {

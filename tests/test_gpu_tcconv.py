@@ -289,20 +289,25 @@ def test_int8_rows_by_the_copy_engine(layer, shape, monkeypatch):
     assert B.cadnn_device_status()["copy_timeouts"] == 0
 
 
-@pytest.mark.parametrize("c_out,density,dense", [(16, 0.03, True), (64, 0.03, True), (65, 0.03, True), (16, 0.02, False), (64, 0.02, False)])
-def test_float_layers_take_the_dense_route_from_two_and_a_half_per_cent_on(c_out, density, dense):
+@pytest.mark.parametrize("c_out,density,dense", [(16, 0.03, False), (64, 0.03, False), (64, 0.055, False), (64, 0.065, True), (65, 0.03, True), (65, 0.02, False)])
+def test_float_layers_of_up_to_64_channels_take_the_dense_route_from_six_per_cent_on(c_out, density, dense):
+    """Below, the sparse kernels' sums keep every bit of activations of any magnitude (the split products lose bits below 8e-34)."""
     from paper_1905_00571_b200 import binding as B
     g = gen.rng(61)
     x, w = gen.relu_normal_input(g, (2, 9, 8, 72)), gen.he_weights(g, c_out, 3, 3, 72)
     mask = gen.random_mask(g, w.shape, density)
-    want = ref.conv2d_f32(x, w, mask, 1, 1, act="relu")
     wh = B.cadnn_pack(B.make_desc(72, c_out, 3, 3, 1, 1, 1, 9, 8, 2, "f32"), w, mask)
     assert (B.cadnn_weights_info(wh)["packed_bytes"] > 6 * w.size) == dense
-    y = torch.zeros(want.shape, device=DEV)
-    B.cadnn_conv2d(wh, torch.from_numpy(x).to(DEV), y, act="relu")
-    torch.cuda.synchronize()
-    s_abs = ref.conv2d_f32(np.abs(x), np.abs(w) * mask, None, 1, 1)
-    assert_close_or_bounded(y.cpu().numpy(), want, s_abs, int(mask.reshape(c_out, -1).sum(1).max()) + 4, "%d %g" % (c_out, density))
+    terms = int(mask.reshape(c_out, -1).sum(1).max()) + 4
+    for xs in (x,) if dense else (x, x * np.float32(1e-35)):
+        want = ref.conv2d_f32(xs, w, mask, 1, 1, act="relu")
+        y = torch.zeros(want.shape, device=DEV)
+        B.cadnn_conv2d(wh, torch.from_numpy(xs).to(DEV), y, act="relu")
+        torch.cuda.synchronize()
+        got, s_abs = y.cpu().numpy(), ref.conv2d_f32(np.abs(xs), np.abs(w) * mask, None, 1, 1)
+        assert_close_or_bounded(got, want, s_abs, terms, "%d %g" % (c_out, density))
+        # fewer than `terms` fused multiply-adds, each within 2^-24 of a sum that the magnitudes bound, and the oracle's own rounding
+        assert dense or (np.abs(got.astype(np.float64) - want) <= (terms + 1) * 2.0 ** -24 * s_abs.astype(np.float64)).all()
 
 
 @pytest.mark.parametrize("batch,c,planar", [(2, 272, True), (2, 304, False), (1, 304, True)])
