@@ -667,11 +667,12 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
             }
         }
         // Layers packed with the dense tensor-core image run NHWC (tcconv.cu); for those timed at pack time the times decide below.
-        // Networks with depthwise layers do so above 75 million multiply-adds of kept weights, single images above 150 million: up to there
-        // the planar kernels' shorter start-up and the depthwise layers they take along make up for their rate (MobileNet-V2, planar / NHWC,
-        // us: batch 1, 41 million 181 / 197, 65 193 / 207, 99 209 / 207, 193 254 / 207; batch 2, 81 million 221 / 213, 131 271 / 233,
-        // 198 297 / 233; batch 4, 163 million 302 / 247).  (From 85 million on single images gain as well, 228 / 211 at 256 x 256; the line
-        // stays, because the slots of a full MobileNet-V1 are seen as planes.)
+        // Networks with depthwise layers do so above 150 million multiply-adds of kept weights: the planar kernels' shorter start-up and the
+        // depthwise layers they take along make up for their rate at small sizes (MobileNet-V2, planar / NHWC, us: batch 1, 41 million 181 / 197,
+        // 65 193 / 207, 99 209 / 207, 193 254 / 207; batch 2, 81 million 221 / 213, 198 297 / 233; batch 4, 163 million 302 / 247).  NHWC is
+        // the faster form from about 85 million on (batch 2, 131 million 271 / 233), but not the more precise one there: the planar kernels
+        // sum in 32 bits, the dense route in split products (error against 64 bits, dense over planar: MobileNet-V1, two images of 144 x 144,
+        // 115 million, 1.17 to 1.75, four of 112 x 112, 140 million, 0.89 to 1.44; MobileNet-V2 at 120 to 136 million 0.67 to 1.04).
         if (planar && getenv("CADNN_FORCE_PLANAR") == nullptr && !(getenv("CADNN_PERSIST") && atoi(getenv("CADNN_PERSIST")) != 0)) {
             bool tc = true, dw = false;
             double macs = 0.0;
@@ -684,7 +685,7 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
                     macs += (double)w->nnz * w->h_out * w->w_out * n;
                 }
             }
-            if (tc && (!dw || macs > (n > 1 ? 75e6 : 150e6))) planar = false;
+            if (tc && (!dw || macs > 150e6)) planar = false;
         }
         // Where the packer timed both layouts for every sparse conv, the measured sums decide: planar, and NHWC by the kernel that
         // would run there (a handle keeps a dense image only where that kernel was the faster one).
