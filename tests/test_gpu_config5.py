@@ -59,11 +59,12 @@ def _slot_to_host(B, net, slot):
     return host
 
 
-def test_every_intermediate_tensor_of_the_planar_resnet50():
-    """Walks the slots of the full-size network (channel planes with a zero border) and compares each with
-    the oracle's tensor of the same slot; the assertion names the first layer out of tolerance."""
+def test_every_intermediate_tensor_of_the_planar_resnet50(monkeypatch):
+    """Walks the slots of the full-size network (channel planes with a zero border, asked for: the times would choose NHWC) and compares
+    each with the oracle's tensor of the same slot; the assertion names the first layer out of tolerance."""
     from paper_1905_00571_b200 import binding as B
     from paper_1905_00571_b200.network import PackedModel
+    monkeypatch.setenv("CADNN_FORCE_PLANAR", "1")
     m = models.resnet50()
     x = models.make_input(m, 1)
     pm = PackedModel(m, 1, DEV, autotune=True)

@@ -101,9 +101,10 @@ def test_rectangular_odd_maps_at_stride_2(in_hw, monkeypatch):
 
 
 def test_full_resnet50_takes_the_faster_form(monkeypatch):
-    """With timed schedules the net picks per layer; whatever it picks matches the oracle."""
+    """With timed schedules a planar net picks per layer; whatever it picks matches the oracle."""
     from paper_1905_00571_b200 import binding as B
     from paper_1905_00571_b200.network import PackedModel
+    monkeypatch.setenv("CADNN_FORCE_PLANAR", "1")
     monkeypatch.setenv("CADNN_PERSIST", "0")
     m = models.resnet50()
     x = models.make_input(m, 1)

@@ -42,6 +42,38 @@ def test_a_timed_network_takes_the_dense_route_where_it_is_faster():
         assert_close_f32(y.cpu().numpy(), want, "logits, autotune %s" % autotune, floor=NET_FLOOR)
 
 
+@pytest.mark.parametrize("batch", [1, 2])
+def test_a_timed_network_takes_the_layout_of_the_lower_sum(batch, tmp_path, monkeypatch):
+    """The times of a cache record's layer (its last four numbers: the two planar kernels, the NHWC sparse and the dense kernel) written
+    on both sides of each other: the network's layout follows the sums, a single image's as well."""
+    from paper_1905_00571_b200 import binding as B
+    from paper_1905_00571_b200.network import PackedModel
+    cache = tmp_path / "tune.cache"
+    monkeypatch.setenv("CADNN_TUNE_CACHE", str(cache))
+    g = gen.rng(75)
+    m = models.Model("timed_layout", "f32", (28, 28, 3), seed=75)
+    stem, hw = _conv(m, g, "stem", 0, 3, 32, 3, 2, 1, (28, 28), "relu", 1.0)
+    a, _ = _conv(m, g, "a", stem, 32, 96, 3, 1, 1, hw, "relu", 0.2)
+    b, _ = _conv(m, g, "b", a, 96, 80, 1, 1, 0, hw, "relu", 0.2)
+    pool = m.new_slot()
+    m.ops.append(models.Op("gavgpool", "pool", b, pool, c_in=80, c_out=80, in_hw=hw, out_hw=(1, 1)))
+    m.ops.append(models.Op("fc", "fc", pool, m.new_slot(), -1, 80, 10, 1, 1, 0, 1, "none", gen.he_weights(g, 10, 1, 1, 80), None,
+                           np.ones(10, np.float32), np.zeros(10, np.float32), "f32", 1.0, (1, 1), (1, 1)))
+    x = models.make_input(m, batch)
+    want, _ = oracle_forward.forward(m, x)
+    PackedModel(m, batch, DEV, autotune=True)
+    records = [line.split() for line in cache.read_text().splitlines()]
+    assert records
+    for dense_us, planar in ((9.5, False), (7.0, False), (10.5, True)):
+        cache.write_text("".join("%s %s\n" % (key, r[:-32] + struct.pack("<4f", 10.0, 10.0, 20.0, dense_us).hex()) for key, r in records))
+        pm = PackedModel(m, batch, DEV, autotune=True)
+        assert B.cadnn_net_layout(pm.net)["planar"] == planar, (dense_us, planar)
+        y = pm.new_output()
+        pm.forward(torch.from_numpy(x).to(DEV), y)
+        torch.cuda.synchronize()
+        assert_close_f32(y.cpu().numpy(), want, "logits, dense layers of %g us" % dense_us, floor=NET_FLOOR)
+
+
 @pytest.mark.parametrize("dtype", ["f32", "s8"])
 def test_a_timed_handle_keeps_the_dense_image_only_where_it_was_faster(dtype, tmp_path, monkeypatch):
     """The cache record's last number is the dense kernel's time: with a long one the handle holds no dense image and calls run the
