@@ -1549,14 +1549,16 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     if (ep.prefetch) p.ahead = *ep.prefetch;
     cadnn_status rs = copy_timeout_word(&p.gave_up);
     if (rs != CADNN_OK) return rs;
-    // the last batch size's choice is kept in the handle (one word, so that threads may race on it)
+    // the last batch size's choice is kept in the handle, with and without what else it depends on: a residual tile, which takes shared
+    // memory (one word each, so that threads may race on it)
     Pick pick = {w->tcv_force[0], w->tcv_force[1], w->tcv_force[2]};
-    const uint64_t kept = w->tcv_pick.load(std::memory_order_relaxed);
+    std::atomic<uint64_t> &last = w->tcv_pick[p.res_tile != 0];
+    const uint64_t kept = last.load(std::memory_order_relaxed);
     if (pick.px > 0) pick.split = std::max(1, pick.split);
     else if ((kept >> 32) == (uint64_t)n && kept != 0) pick = {(int)(kept & 0xfff), (int)(kept >> 12 & 0xfff), (int)(kept >> 24 & 0xff)};
     else {
         pick = choose(f32 ? d.c_in % 4 != 0 : engine_takes(d) ? 2 : d.c_in % 16 == 0 ? 3 : 4, d.c_out, M, p.nkb, p.res_tile != 0);
-        w->tcv_pick.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
+        last.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
     }
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0, run_tail = !f32 && !vec && p.tail;
     if (pick.ch == 64 || (run_tail && pick.px > 128)) pick.px = 128;

@@ -6,6 +6,8 @@ or cancellation drives r to 0).  The bound follows from fp32 accumulation in any
 order of at most a few thousand terms against a float64 sum rounded once.
 Integer layers: bit-exact.
 """
+import json
+
 import numpy as np
 
 REL_TOL = 1e-4
@@ -66,3 +68,16 @@ def assert_close_or_bounded(got, ref, abs_sum, terms, what=""):
         what, int(bad.sum()), worst, np.unravel_index(int(bad.argmax()), bad.shape), got.flat[int(bad.argmax())],
         ref.flat[int(bad.argmax())], bound.flat[int(bad.argmax())])
     return worst, int(miss.sum())
+
+
+def launches_of(call, tmp_path):
+    """(name, blocks) of the kernels that call() launches, from the profiler's trace."""
+    import torch
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        call()
+        torch.cuda.synchronize()
+    trace = tmp_path / "trace.json"
+    prof.export_chrome_trace(str(trace))
+    events = [e for e in json.loads(trace.read_text())["traceEvents"] if e.get("cat") == "kernel"]
+    return [(e["name"], e["args"]["grid"][0]) for e in sorted(events, key=lambda e: e["ts"])]

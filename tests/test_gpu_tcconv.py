@@ -7,7 +7,7 @@ import torch
 
 from oracle import forward as oracle_forward, ref
 from workloads import gen, models
-from parity import NET_FLOOR, assert_close_f32, assert_close_or_bounded, assert_exact
+from parity import NET_FLOOR, assert_close_f32, assert_close_or_bounded, assert_exact, launches_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -379,3 +379,29 @@ def test_int8_epilogue_of_nan_infinities_and_ties(act):
         t = np.where(t > 0, t, np.float32(0.0)) if act == "relu" else t
         want = np.rint(np.fmin(np.fmax(t, np.float32(-127.0)), np.float32(127.0))).astype(np.int8)
         assert (y.cpu().numpy() == want).all()
+
+
+def test_one_handle_with_and_without_a_residual(tmp_path):
+    """The residual tile of an int8 layer takes shared memory, so the block shape may differ: whichever call comes first, each runs the
+    shape that a handle of its own would."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(71)
+    n, hw, c_in, c_out = 4, 56, 512, 64
+    x, q = gen.int8_relu_activation(g, (n, hw, hw, c_in)), gen.int8_weights(g, (c_out, 3, 3, c_in))
+    mask = gen.random_mask(g, q.shape, 0.1)
+    r = torch.from_numpy(gen.int8_relu_activation(g, (n, hw, hw, c_out))).to(DEV)
+    xd, m, b = torch.from_numpy(x).to(DEV), torch.full((c_out,), 3e-4, device=DEV), torch.zeros(c_out, device=DEV)
+    ran = {}
+    for order in ((False, True), (True, False)):
+        wh = B.cadnn_pack_q8(B.make_desc(c_in, c_out, 3, 3, 1, 1, 1, hw, hw, n, "s8"), q, mask)
+        for res in order:
+            y = torch.zeros((n, hw, hw, c_out), dtype=torch.int8, device=DEV)
+            call = lambda: B.cadnn_conv2d(wh, xd, y, m, b, r if res else None, "relu", out_dtype="s8", residual_scale=0.5)
+            names = launches_of(call, tmp_path)
+            assert len(names) == 1 and "tcconv_kernel" in names[0][0], names
+            ran.setdefault(res, []).append((names, y.cpu().numpy()))
+    for res in (False, True):
+        (first, a), (second, c) = ran[res]
+        assert first == second, (res, first, second)
+        assert (a == c).all()
+    assert ran[False][0][0] != ran[True][0][0]   # (the layer is one where the two choices differ)
