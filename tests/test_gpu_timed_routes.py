@@ -112,3 +112,38 @@ def test_a_timed_handle_keeps_the_dense_image_only_where_it_was_faster(dtype, tm
     check(pack(d, w, mask), "no time recorded")
     again = cache.read_text().split()
     assert again[2] == key and struct.unpack("<f", bytes.fromhex(again[3][-8:]))[0] > 0.0
+
+
+def test_records_of_earlier_kernels_are_timed_again(tmp_path, monkeypatch):
+    """A record under the key of the kernels before (the same hash without their generation), with a dense time that would drop the dense
+    image: the pack does not take it, times the layer itself and adds a record of its own, which the next pack takes."""
+    from paper_1905_00571_b200 import binding as B
+    cache = tmp_path / "tune.cache"
+    monkeypatch.setenv("CADNN_TUNE_CACHE", str(cache))
+    g = gen.rng(77)
+    c_in, c_out, h, wd, n = 72, 70, 9, 10, 2
+    w = gen.he_weights(g, c_out, 3, 3, c_in)
+    mask = gen.random_mask(g, w.shape, 0.2)
+    d = B.make_desc(c_in, c_out, 3, 3, 1, 1, 1, h, wd, n, "f32", autotune=True)
+    B.cadnn_pack(d, w, mask)
+    key, record = cache.read_text().split()
+    assert len(record) == 2 * (100 + 100 + 6 * 4 + 4 * 4)
+    rows = [int(k) for k in mask.reshape(c_out, -1).astype(bool).sum(1)]
+
+    def digest(*generation):
+        v = 1469598103934665603
+        for byte in struct.pack("<%dq" % (15 + len(generation) + c_out), c_in, c_out, 3, 3, 1, 1, 1, 1, h, wd, n, d.dtype, 100, 100, 240, *generation, *rows):
+            v = (v ^ byte) * 1099511628211 % 2 ** 64
+        return "%016x" % v
+
+    old = digest()
+    assert key != old and key in [digest(i) for i in range(2, 100)]
+    slow = record[:-8] + struct.pack("<f", 1e6).hex()
+    cache.write_text("%s %s\n" % (old, slow))
+    B.cadnn_pack(d, w, mask)
+    lines = [line.split() for line in cache.read_text().splitlines()]
+    assert [k for k, _ in lines] == [old, key]
+    assert 0.0 < struct.unpack("<f", bytes.fromhex(lines[1][1][-8:]))[0] < 1e3
+    cache.write_text("%s %s\n" % (key, slow))
+    B.cadnn_pack(d, w, mask)
+    assert len(cache.read_text().splitlines()) == 1
