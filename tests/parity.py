@@ -6,7 +6,7 @@ or cancellation drives r to 0).  The bound follows from fp32 accumulation in any
 order of at most a few thousand terms against a float64 sum rounded once.
 Integer layers: bit-exact.
 """
-import json
+import ctypes
 
 import numpy as np
 
@@ -70,14 +70,37 @@ def assert_close_or_bounded(got, ref, abs_sum, terms, what=""):
     return worst, int(miss.sum())
 
 
-def launches_of(call, tmp_path):
-    """(name, blocks) of the kernels that call() launches, from the profiler's trace."""
+class _KernelNode(ctypes.Structure):   # CUDA_KERNEL_NODE_PARAMS
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3), ("shared", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p), ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def launches_of(call):
+    """(mangled name, blocks) of the kernels that call() launches, in the order of their launch: read off a CUDA graph that records the
+    call, which is then run once."""
     import torch
-    torch.cuda.synchronize()
-    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+    call()   # (what is set up once per kernel is not for a capture)
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
         call()
-        torch.cuda.synchronize()
-    trace = tmp_path / "trace.json"
-    prof.export_chrome_trace(str(trace))
-    events = [e for e in json.loads(trace.read_text())["traceEvents"] if e.get("cat") == "kernel"]
-    return [(e["name"], e["args"]["grid"][0]) for e in sorted(events, key=lambda e: e["ts"])]
+    cuda = ctypes.CDLL("libcuda.so.1")
+    raw, count = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t()
+    assert cuda.cuGraphGetNodes(raw, None, ctypes.byref(count)) == 0
+    nodes = (ctypes.c_void_p * count.value)()
+    assert cuda.cuGraphGetNodes(raw, nodes, ctypes.byref(count)) == 0
+    out = []
+    for node in nodes:
+        kind, p, name = ctypes.c_int(), _KernelNode(), ctypes.c_char_p()
+        assert cuda.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) == 0
+        if kind.value != 0:   # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        assert cuda.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)) == 0
+        if p.func:
+            assert cuda.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func)) == 0
+        else:
+            assert cuda.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern)) == 0
+        out.append((name.value.decode(), p.grid[0]))
+    graph.instantiate()
+    graph.replay()
+    torch.cuda.synchronize()
+    return out

@@ -8,20 +8,21 @@ import torch
 
 from oracle import forward as oracle_forward
 from workloads import gen, models
-from parity import assert_exact
+from parity import assert_exact, launches_of
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-def _add(m, g, name, src, c_in, c_out, k, stride, hw):
+def _add(m, g, name, src, c_in, c_out, k, stride, hw, pad=None):
     w = np.clip(np.rint(g.standard_normal((c_out, k, k, c_in)) * 40), -127, 127).astype(np.int8)
     mask = gen.random_mask(g, w.shape, 0.3)
     # (negative multipliers too: the pool takes the maximum of finished values)
     scale = (g.uniform(-1.0, 1.5, c_out) * 1.5 / np.sqrt(0.3 * k * k * c_in) / 40).astype(np.float32)
     bias = (g.standard_normal(c_out) * 10).astype(np.float32)
-    ho = tuple((d + 2 * (k // 2) - k) // stride + 1 for d in hw)
-    m.ops.append(models.Op("conv", name, src, m.new_slot(), -1, c_in, c_out, k, stride, k // 2, 1, "none", w, mask, scale, bias, "s8", 0.3, hw, ho))
+    pad = k // 2 if pad is None else pad
+    ho = tuple((d + 2 * pad - k) // stride + 1 for d in hw)
+    m.ops.append(models.Op("conv", name, src, m.new_slot(), -1, c_in, c_out, k, stride, pad, 1, "none", w, mask, scale, bias, "s8", 0.3, hw, ho))
     return m.ops[-1].dst, ho
 
 
@@ -40,12 +41,36 @@ def _add(m, g, name, src, c_in, c_out, k, stride, hw):
     ((14, 14), 16, 36, 3, 1, 1, "128,64,1", False),
 ])
 def test_pool_behind_int8_layer(hw, c_in, c_out, k, stride, batch, shape, fused, monkeypatch):
+    _check(hw, c_in, c_out, k, stride, batch, shape, fused, monkeypatch)
+
+
+@pytest.mark.parametrize("hw,c_in,c_out,k,stride,pad,batch,shape", [
+    ((14, 12), 64, 80, 3, 1, 1, 3, "32,128,1"),       # 42 windows an image: tiles of 8 run over rows and images, the last one is ragged
+    ((14, 12), 192, 96, 3, 1, 1, 3, "96,128,1"),      # 27 halves of a stage: the last stage has one
+    ((10, 6), 64, 48, 1, 1, 0, 5, "192,128,1"),       # one stage of one half; a tile holds three images
+    ((20, 14), 64, 64, 5, 1, 2, 2, "256,128,1"),
+    ((22, 10), 128, 64, 3, 1, 1, 2, "128,64,1"),
+    ((24, 20), 64, 96, 3, 2, 1, 3, "64,128,1"),       # windows 4, 6 and 8 positions apart
+    ((18, 30), 64, 48, 3, 3, 1, 2, "128,128,1"),
+    ((32, 24), 128, 64, 5, 4, 2, 3, "32,128,1"),
+    ((16, 12), 64, 32, 3, 1, 0, 3, "160,128,1"),      # no padding
+    ((9, 13), 64, 64, 4, 1, 3, 2, "96,128,1"),        # more padding than the window's middle, odd maps
+    ((2, 2), 64, 16, 3, 1, 1, 9, "32,128,1"),         # one window an image
+    ((56, 40), 64, 160, 3, 1, 1, 2, None),
+])
+def test_pool_behind_int8_layer_gathered_by_the_copy_engine(hw, c_in, c_out, k, stride, pad, batch, shape, monkeypatch):
+    """Unsplit tiles of whole 64-channel rows, a quarter of a tile's rows for each place in a window."""
+    _check(hw, c_in, c_out, k, stride, batch, shape, True, monkeypatch, pad, True)
+
+
+def _check(hw, c_in, c_out, k, stride, batch, shape, fused, monkeypatch, pad=None, engine=False):
     from paper_1905_00571_b200 import binding as B
     from paper_1905_00571_b200.network import PackedModel
-    monkeypatch.setenv("CADNN_TCV", shape)
+    if shape:
+        monkeypatch.setenv("CADNN_TCV", shape)
     g = gen.rng(83)
     m = models.Model("pool_tail", "s8", (hw[0], hw[1], c_in), seed=83)
-    a, at = _add(m, g, "conv", 0, c_in, c_out, k, stride, hw)
+    a, at = _add(m, g, "conv", 0, c_in, c_out, k, stride, hw, pad)
     pooled = m.new_slot()
     half = (at[0] // 2, at[1] // 2)
     m.ops.append(models.Op("maxpool", "pool", a, pooled, k=2, stride=2, pad=0, c_in=c_out, c_out=c_out, out="s8", in_hw=at, out_hw=half))
@@ -56,6 +81,8 @@ def test_pool_behind_int8_layer(hw, c_in, c_out, k, stride, batch, shape, fused,
     want, slots = oracle_forward.forward(m, x)
     xd = torch.from_numpy(x).to(DEV)
     y = pm.new_output()
+    name, _ = launches_of(lambda: pm.forward(xd, y, use_graph=False))[0]
+    assert "tcconv_kernel" in name and ("6GatherE2ELb1" in name) == engine, name   # (the copy engine's kernel, with a pool)
     for use_graph in (False, True):
         y.zero_()
         pm.forward(xd, y, use_graph=use_graph)

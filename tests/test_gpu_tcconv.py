@@ -257,6 +257,7 @@ def test_shares_of_a_split_tile(shape, dtype, monkeypatch):
 
 # n, h, w, c_in, c_out, kh, kw, stride, pad, pad_w
 ENGINE_LAYERS = [(3, 9, 7, 64, 80, 3, 3, 1, 1, 1), (2, 13, 10, 192, 96, 1, 7, 1, 0, 3), (2, 10, 13, 64, 130, 7, 1, 1, 3, 0), (3, 15, 12, 128, 64, 3, 3, 2, 1, 1),
+                 (2, 17, 20, 64, 48, 3, 5, 3, 1, 2), (2, 23, 21, 128, 72, 7, 7, 4, 6, 5), (1, 12, 9, 64, 80, 1, 9, 1, 0, 8),
                  (5, 9, 11, 64, 64, 1, 1, 2, 0, 0), (1, 8, 8, 64, 48, 5, 5, 1, 0, 0), (2, 6, 5, 128, 70, 3, 5, 1, 2, 0), (33, 1, 1, 320, 200, 1, 1, 1, 0, 0)]
 
 
@@ -264,7 +265,8 @@ ENGINE_LAYERS = [(3, 9, 7, 64, 80, 3, 3, 1, 1, 1), (2, 13, 10, 192, 96, 1, 7, 1,
 @pytest.mark.parametrize("layer", ENGINE_LAYERS)
 def test_int8_rows_by_the_copy_engine(layer, shape, monkeypatch):
     """Layers of whole 64-channel rows: tiles that begin and end inside a row of the map and run over images, rectangular windows with
-    different paddings, strides, a last stage of one half, against float64 sums and against the general gather (one channel more)."""
+    different paddings, strides of up to four, a last stage of one half, against float64 sums and against the general gather (one channel
+    more); the kernels' names tell which ran."""
     from paper_1905_00571_b200 import binding as B
     n, h, wd, c_in, c_out, kh, kw, stride, pad, pad_w = layer
     g = gen.rng(59 + c_in + kw)
@@ -281,8 +283,9 @@ def test_int8_rows_by_the_copy_engine(layer, shape, monkeypatch):
                                           stride, (pad, pad_w)).permute(0, 2, 3, 1).to(torch.int32).numpy()
         wh = B.cadnn_pack_q8(B.make_desc(c_in + extra, c_out, kh, kw, stride, pad, 1, h, wd, n, "s8", pad_w=pad_w), qs, ms)
         y = torch.full(want.shape, 5, dtype=torch.int32, device=DEV)
-        B.cadnn_conv2d(wh, dev(xs), y, out_dtype="s32")
-        torch.cuda.synchronize()
+        xd = dev(xs)
+        names = launches_of(lambda: B.cadnn_conv2d(wh, xd, y, out_dtype="s32"))
+        assert len(names) == 1 and "tcconv_kernel" in names[0][0] and ("6GatherE0" if extra else "6GatherE2") in names[0][0], names
         assert_exact(y.cpu().numpy(), want, "%s %s" % (layer, shape))
         outs.append(y.cpu().numpy())
     assert (outs[0] == outs[1]).all()
@@ -351,15 +354,19 @@ def test_float_epilogue_of_nan_infinities_and_zeros(act, shape, monkeypatch):
     monkeypatch.setenv("CADNN_TCV", shape)
     wh = B.cadnn_pack(B.make_desc(64, 72, 1, 1, 1, 0, 1, 5, 7, 1, "f32"), w, gen.random_mask(g, w.shape, 0.2))
     r = np.resize(np.array([np.nan, np.inf, -np.inf, -0.0, 0.0, 3.0, -3.0, 7.0, 6.0, 1e-40], np.float32), (1, 5, 7, 72))
-    y = torch.full(r.shape, 9.0, device=DEV)
-    B.cadnn_conv2d(wh, torch.zeros((1, 5, 7, 64), device=DEV), y, residual=torch.from_numpy(r).to(DEV), act=act)
-    torch.cuda.synchronize()
-    want = r + np.float32(0.0)
-    if act != "none":
-        want = np.where(want > 0, want, np.float32(0.0))
-    if act == "relu6":
-        want = np.minimum(want, np.float32(6.0))
-    assert np.array_equal(y.cpu().numpy(), want, equal_nan=True)
+    for scale in (1.0, -1.0):   # with -1 the sum is -0 before the residual joins
+        y = torch.full(r.shape, 9.0, device=DEV)
+        B.cadnn_conv2d(wh, torch.zeros((1, 5, 7, 64), device=DEV), y, torch.full((72,), scale, device=DEV), torch.full((72,), -0.0, device=DEV),
+                       torch.from_numpy(r).to(DEV), act)
+        torch.cuda.synchronize()
+        want = r + (np.float32(0.0) * np.float32(scale) + np.float32(-0.0))
+        if act != "none":
+            want = np.where(want > 0, want, np.float32(0.0))
+        if act == "relu6":
+            want = np.minimum(want, np.float32(6.0))
+        got = y.cpu().numpy()
+        assert np.array_equal(got, want, equal_nan=True)
+        assert (np.signbit(got) == np.signbit(want))[want == 0].all() and (want[r == 0] == 0).all()
 
 
 @pytest.mark.parametrize("act", ["none", "relu"])
@@ -381,7 +388,7 @@ def test_int8_epilogue_of_nan_infinities_and_ties(act):
         assert (y.cpu().numpy() == want).all()
 
 
-def test_one_handle_with_and_without_a_residual(tmp_path):
+def test_one_handle_with_and_without_a_residual():
     """The residual tile of an int8 layer takes shared memory, so the block shape may differ: whichever call comes first, each runs the
     shape that a handle of its own would."""
     from paper_1905_00571_b200 import binding as B
@@ -397,7 +404,7 @@ def test_one_handle_with_and_without_a_residual(tmp_path):
         for res in order:
             y = torch.zeros((n, hw, hw, c_out), dtype=torch.int8, device=DEV)
             call = lambda: B.cadnn_conv2d(wh, xd, y, m, b, r if res else None, "relu", out_dtype="s8", residual_scale=0.5)
-            names = launches_of(call, tmp_path)
+            names = launches_of(call)
             assert len(names) == 1 and "tcconv_kernel" in names[0][0], names
             ran.setdefault(res, []).append((names, y.cpu().numpy()))
     for res in (False, True):
