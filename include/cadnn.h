@@ -73,8 +73,8 @@ typedef enum {
                                   overlaps its neighbours in a network does not show.  With
                                   CADNN_TUNE_CACHE=<file> in the environment the choices are appended to that
                                   text file and a later pack of the same layer (geometry, batch hint, nonzeros
-                                  per filter) reads them back instead of timing: tune once per machine, and a
-                                  profiled run executes the schedules of the plain run */
+                                  per filter) by the same kernels reads them back instead of timing: tune once per
+                                  machine and library, and a profiled run executes the schedules of the plain run */
 
 /*
  * One layer.  The packer is the offline stage of Section 4 ("Memory layout
@@ -303,9 +303,11 @@ cadnn_status cadnn_net_create(const cadnn_op *ops, int n_ops, int n, int h, int 
  * max pools, a global average pool and fc layers keep their intermediate feature maps
  * channel-planar with a zero halo (see cadnn_conv2d_planar), unless every sparse conv carries the
  * dense tensor-core image and none was timed at pack time (networks with depthwise layers: and the
- * network is large); others (int8) keep NHWC
- * (CADNN_NO_PLANAR_DW: networks with depthwise layers too).  CADNN_NO_PLANAR in the
- * environment at cadnn_net_create forces NHWC.
+ * sparse convs multiply more than 150 million kept weights with activations), or every sparse conv was
+ * timed and the times of the NHWC kernels sum lower than those of the planar ones; others (int8) keep
+ * NHWC (CADNN_NO_PLANAR_DW: networks with depthwise layers too).  No layout is promised to callers of
+ * cadnn_net_slot: cadnn_net_layout tells it, CADNN_NO_PLANAR and CADNN_FORCE_PLANAR in the environment
+ * at cadnn_net_create ask for one.
  * Layers after the first are launched as programmatic dependents of their predecessor
  * (their weight fetch overlaps its stores); set CADNN_NO_PDL in the environment before
  * cadnn_net_create to use plain stream order instead (CADNN_NO_PDL_GRAPH: only inside

@@ -15,17 +15,17 @@
 // shared memory (small maps would otherwise leave most multiprocessors idle).
 //   * 8 loader warps gather the im2col rows from NHWC memory (out-of-image taps are zeros) into swizzled
 //     K-major operand tiles, 128 source bytes per pixel and stage, in groups that fill alternate stages;
-//     int8 layers of whole 64-channel rows leave that to the copy engine (engine_takes);
+//     int8 layers of whole 64-channel rows leave that to the copy engine (engine_takes; not the split tiles of pooled layers);
 //   * one thread copies the matching weight tiles (pre-swizzled by the packer) with bulk copies; the first
 //     ones do not wait for the previous layer;
 //   * one thread issues the tcgen05.mma's; accumulators live in tensor memory;
 //   * the loader warps then finish the tile, with scale, bias and residual asked for at its start: float
 //     tiles whose rows are channels as columns of 16 pixels straight from tensor memory, the others through
 //     shared memory as [pixel][channel]; with a split reduction every block sends each other block its
-//     pixels' sums from registers, counted on the receiver's barrier.
+//     pixels' sums, float from registers, int8 as bulk copies of the staged tile, counted on the receiver's barrier.
 // What bounds it, from clock stamps in its warps.  At batch 1 a chain: 14x14, 256 -> 1024 1x1 with a residual, 32 x 128 tile split
-// in four (clocks of 0.5 ns after the previous layer has ended): requests 350, first stage in shared memory 1300, first products 1600,
-// last 3100, sums read and sent 4300, received 5000, written 6000; 0.8 us from the end of one layer to the next.  Four to eight warps a
+// in four (clocks of 0.5 ns after the previous layer has ended): first stage in shared memory 1300, first products 2250, last 3330, complete
+// 3610, sums read and sent 4370, received 5030, written 6050; 0.8 us from the end of one layer to the next.  Four to eight warps a
 // scheduler share the issue slots, so what helps there is fewer instructions.  At large batch, float: the products (256 x 128 tiles
 // run at 90 % of the tensor cores' rate while multiplying; their first loads and epilogue, 10 to 50 % of the time, are not
 // overlapped).  Int8: epilogue instructions and the exchange.
@@ -1570,6 +1570,9 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     if (pick.px > 0) pick.split = std::max(1, pick.split);
     else if ((kept >> 32) == (uint64_t)n && kept != 0) pick = {(int)(kept & 0xfff), (int)(kept >> 12 & 0xfff), (int)(kept >> 24 & 0xff)};
     else {
+        // (Pooled layers count as the copy engine's although their split tiles run on the gather: its shapes are within 0.6 us of the best of
+        // 20 on each pooled layer of int8 VGG-16 at batch 1, 2, 4 and 8.  With the gather's coefficients for the split tiles, which know no
+        // pooled epilogue, fewer blocks share the pooling: batch 1 / 2 / 4 / 8 104 / 141 / 207 / 332 us became 108 / 145 / 212 / 336.)
         pick = choose(f32 ? d.c_in % 4 != 0 : engine_takes(d) ? 2 : d.c_in % 16 == 0 ? 3 : 4, d.c_out, M, p.nkb, p.res_tile != 0);
         last.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
     }
