@@ -151,7 +151,7 @@ struct cadnn_weights {
     void *d_tcv = nullptr;
     size_t tcv_bytes = 0;
     int tcv_force[3] = {0, 0, 0};          // CADNN_TCV at pack time: pixels, channels, split (0 = choose)
-    mutable std::atomic<uint64_t> tcv_pick[2] = {{0}, {0}};   // block shape of the last batch size, without and with an int8 residual (tcconv.cu)
+    mutable std::atomic<uint64_t> tcv_pick[4] = {{0}, {0}, {0}, {0}};   // block shapes of the last batch size (tcconv.cu)
 
     // device image (one allocation)
     void *d_blob = nullptr;

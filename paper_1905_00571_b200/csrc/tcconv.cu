@@ -1515,6 +1515,17 @@ bool engine_takes(const cadnn_layer_desc &d)
     return d.dtype == CADNN_S8 && d.c_in % 64 == 0 && d.stride <= 4 && d.pad <= 127 && d.pad_w <= 127 && d.kh <= 128 && d.kw <= 128 && encode_im2col_fn();
 }
 
+// Whether a launch that does not overlap the one before it (pdl) gains by that: the engine's first fetch of the tensor map and of the pixels
+// then stands alone, 0.3 to 0.4 us, which small layers do not make up for.  Launches one after the other in a captured graph, engine /
+// gather, us each: 64 -> 64 1x1 7x7 3.46 / 3.18, 448 -> 384 3x3 8x8 5.26 / 4.71, 1024 -> 256 1x1 14x14 4.70 / 4.39, 2048 -> 1000 fc of 16 images
+// 4.27 / 3.88, 4096 -> 4096 fc of 32 6.97 / 6.01; beyond the lines, 64 -> 256 1x1 56x56 (803 thousand outputs) 4.62 / 4.95, 25088 -> 4096 fc
+// of 9 (925 million multiply-adds) 15.0 / 19.4.  (Of 45 layers within them one is faster by the engine, by 0.02 us.)
+bool engine_pays_alone(long long M, int c_out, long long k)
+{
+    const double outputs = (double)M * ((c_out + 63) / 64 * 64);
+    return outputs > 300e3 || outputs * k > 600e6;
+}
+
 // The input of n images as im2col rows of 64 channels, `rows` output pixels per copy (`pooled`: every second one of every second row).
 bool encode_pixels(CUtensorMap *map, const cadnn_layer_desc &d, const void *x, int n, int rows, bool pooled)
 {
@@ -1562,10 +1573,11 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
     if (ep.prefetch) p.ahead = *ep.prefetch;
     cadnn_status rs = copy_timeout_word(&p.gave_up);
     if (rs != CADNN_OK) return rs;
-    // the last batch size's choice is kept in the handle, with and without what else it depends on: a residual tile, which takes shared
-    // memory (one word each, so that threads may race on it)
     Pick pick = {w->tcv_force[0], w->tcv_force[1], w->tcv_force[2]};
-    std::atomic<uint64_t> &last = w->tcv_pick[p.res_tile != 0];
+    const bool engine = engine_takes(d) && (ep.pdl || p.pooled || pick.px > 0 || engine_pays_alone(M, d.c_out, (long long)d.kh * d.kw * d.c_in));
+    // the last batch size's choice is kept in the handle, for each of what else it depends on: a residual tile, which takes shared memory, and
+    // the gather (one word each, so that threads may race on it)
+    std::atomic<uint64_t> &last = w->tcv_pick[2 * (p.res_tile != 0) + engine];
     const uint64_t kept = last.load(std::memory_order_relaxed);
     if (pick.px > 0) pick.split = std::max(1, pick.split);
     else if ((kept >> 32) == (uint64_t)n && kept != 0) pick = {(int)(kept & 0xfff), (int)(kept >> 12 & 0xfff), (int)(kept >> 24 & 0xff)};
@@ -1573,7 +1585,7 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
         // (Pooled layers count as the copy engine's although their split tiles run on the gather: its shapes are within 0.6 us of the best of
         // 20 on each pooled layer of int8 VGG-16 at batch 1, 2, 4 and 8.  With the gather's coefficients for the split tiles, which know no
         // pooled epilogue, fewer blocks share the pooling: batch 1 / 2 / 4 / 8 104 / 141 / 207 / 332 us became 108 / 145 / 212 / 336.)
-        pick = choose(f32 ? d.c_in % 4 != 0 : engine_takes(d) ? 2 : d.c_in % 16 == 0 ? 3 : 4, d.c_out, M, p.nkb, p.res_tile != 0);
+        pick = choose(f32 ? d.c_in % 4 != 0 : engine ? 2 : d.c_in % 16 == 0 ? 3 : 4, d.c_out, M, p.nkb, p.res_tile != 0);
         last.store((uint64_t)n << 32 | (uint64_t)pick.split << 24 | (uint64_t)pick.ch << 12 | (uint64_t)pick.px, std::memory_order_relaxed);
     }
     const bool vec = d.c_in % (f32 ? 4 : 16) == 0, run_tail = !f32 && !vec && p.tail;
@@ -1595,7 +1607,7 @@ cadnn_status launch_tcv(const cadnn_weights *w, const void *x, int n, void *y, c
                         : launch_shape<false, Gather::kValues, false, true>(p, pick.ch, n_blocks, ep.pdl, st);
     // (With a pool the copies of one stage are quarters of the tile, which have to be whole groups of 8 swizzled rows, and blocks of a
     // cluster would share out quarters of windows.)
-    if (engine_takes(d) && !(p.pooled && (p.S > 1 || p.npx % 32))) {
+    if (engine && !(p.pooled && (p.S > 1 || p.npx % 32))) {
         TcvEngineParams e;
         static_cast<TcvParams &>(e) = p;
         if (encode_pixels(&e.pixels, d, x, n, p.pooled ? p.npx / 4 : p.npx, p.pooled != nullptr))

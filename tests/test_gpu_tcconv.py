@@ -285,7 +285,8 @@ def test_int8_rows_by_the_copy_engine(layer, shape, monkeypatch):
         y = torch.full(want.shape, 5, dtype=torch.int32, device=DEV)
         xd = dev(xs)
         names = launches_of(lambda: B.cadnn_conv2d(wh, xd, y, out_dtype="s32"))
-        assert len(names) == 1 and "tcconv_kernel" in names[0][0] and ("6GatherE0" if extra else "6GatherE2") in names[0][0], names
+        own = "6GatherE0" if extra else "6GatherE2" if shape else "6GatherE1"   # (small layers that do not overlap, as in a graph: the gather)
+        assert len(names) == 1 and "tcconv_kernel" in names[0][0] and own in names[0][0], names
         assert_exact(y.cpu().numpy(), want, "%s %s" % (layer, shape))
         outs.append(y.cpu().numpy())
     assert (outs[0] == outs[1]).all()
@@ -412,3 +413,24 @@ def test_one_handle_with_and_without_a_residual():
         assert first == second, (res, first, second)
         assert (a == c).all()
     assert ran[False][0][0] != ran[True][0][0]   # (the layer is one where the two choices differ)
+
+
+@pytest.mark.parametrize("n,hw,c_in,c_out,k,engine", [(1, 7, 64, 64, 1, False), (16, 1, 2048, 1000, 1, False), (1, 28, 128, 320, 1, False), (1, 28, 128, 384, 1, True),
+                                                      (1, 14, 512, 576, 3, False), (1, 14, 512, 704, 3, True)])
+def test_small_int8_layers_that_overlap_nothing_run_on_the_gather(n, hw, c_in, c_out, k, engine):
+    """On both sides of the two lines, 300 thousand outputs and 600 million multiply-adds, in a captured graph, and called one by one, where a
+    layer's start overlaps the one before it and the copy engine takes them all: the same bytes."""
+    from paper_1905_00571_b200 import binding as B
+    g = gen.rng(79)
+    x, q = gen.int8_relu_activation(g, (n, hw, hw, c_in)), gen.int8_weights(g, (c_out, k, k, c_in))
+    mask = gen.random_mask(g, q.shape, 0.1)
+    wh = B.cadnn_pack_q8(B.make_desc(c_in, c_out, k, k, 1, k // 2, 1, hw, hw, n, "s8"), q, mask)
+    want = ref.conv2d_s8(x, q, mask, 1, k // 2, out="s32")
+    y, xd = torch.zeros(want.shape, dtype=torch.int32, device=DEV), torch.from_numpy(x).to(DEV)
+    B.cadnn_conv2d(wh, xd, y, out_dtype="s32")
+    torch.cuda.synchronize()
+    assert_exact(y.cpu().numpy(), want, "called")
+    y.zero_()
+    names = launches_of(lambda: B.cadnn_conv2d(wh, xd, y, out_dtype="s32"))
+    assert len(names) == 1 and ("6GatherE2" if engine else "6GatherE1") in names[0][0], names
+    assert_exact(y.cpu().numpy(), want, "captured")
